@@ -182,7 +182,12 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     (1..16) warps share the row's kept columns, reading the canonical storage format and
  *                     the input vectors straight from global memory; partial sums are added in a fixed
  *                     order.  Only pixels_per_lane (2, 4, 8; g * pixels_per_lane <= 32) and warps apply;
- *                     the device copy of the storage format is made on its first use with a packed matrix
+ *                     the device copy of the storage format is made on its first use with a packed matrix;
+ *                     4 = fifth-generation tensor cores: the kept blocks of a tile of output channels are expanded
+ *                     (once per packed matrix, on the device) to dense weight tiles and multiplied with 128-pixel
+ *                     tiles of X; fp32 operands are split exactly into three bfloat16 parts each.  Only row_groups
+ *                     (the number of channel tiles, each of at most 128 channels) applies; no scratch is used.  Non-finite
+ *                     values of X reach all channels of the tile's outputs at that pixel, dropped blocks included
  *   consumer_groups   1 = all consumer warps work on one work item at a time; 2 = two halves of the
  *                     consumer warps take the thread block's work items alternately (tensor-core
  *                     kernels only), so that one half multiplies while the other half stores

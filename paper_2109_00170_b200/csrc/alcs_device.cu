@@ -5,6 +5,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <memory>
+#include <queue>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -14,6 +16,7 @@
 #include "alcs_gather.h"
 #include "alcs_internal.h"
 #include "alcs_kernels.cuh"
+#include "alcs_tc_prep.h"
 
 namespace alcs {
 void set_cuda_error_text(const char* s);
@@ -291,6 +294,46 @@ bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const Devic
     return true;
 }
 
+// Fixed cost of a launch of the tcgen05 kernel, first copies and last stores included, in microseconds.
+constexpr double kTcRampUs = 4.5;
+// What the small-problem kernel's latency model comes to on the GPU (seconds = weight * model + ramp).
+constexpr double kGatherWeight = 1.3, kGatherRamp = 2.5e-6;
+
+// The tcgen05 kernel with n output channels per tile as a plan, and its cost: rounds of items over the SMs.
+Plan tc_plan(const alcs_packed* w, int n, long long q, int sms)
+{
+    Plan p;
+    p.n_rg = (w->cout + n - 1) / n;
+    n = ((w->cout + p.n_rg - 1) / p.n_rg + 15) / 16 * 16;       // (the equal split into that many tiles)
+    p.tc_n = n;
+    const long long items = (q + alcs::kTcM - 1) / alcs::kTcM * p.n_rg, rounds = (items + sms - 1) / sms;
+    p.cost = 1e-6 * (kTcRampUs + rounds * alcs::tc_item_us(w->dt, n, (w->cin + 15) / 16));
+    return p;
+}
+
+// Channels per tile worth considering: the equal split of cout into as many tiles as each multiple of 16 asks for.
+int tc_widths(const alcs_packed* w, int (&n)[8])
+{
+    int count = 0;
+    for (int want = alcs::kTcMaxN; want >= 16; want -= 16) {
+        const int tiles = (w->cout + want - 1) / want, v = ((w->cout + tiles - 1) / tiles + 15) / 16 * 16;
+        if (!count || v != n[count - 1]) n[count++] = v;
+    }
+    return count;
+}
+
+Plan tc_best(const alcs_packed* w, long long q, int sms)
+{
+    int n[8];
+    const int count = tc_widths(w, n);
+    Plan best = tc_plan(w, n[0], q, sms);
+    for (int i = 1; i < count; ++i) {
+        const Plan p = tc_plan(w, n[i], q, sms);
+        if (p.cost < best.cost) best = p;
+    }
+    return best;
+}
+
 // Can the producers stage the rows of X as they are, with 8-byte copies, where 16-byte copies would need
 // the rows repacked?
 bool direct_rows_ok(int hw, int elt) { return ((size_t)hw * elt) % 16 == 8; }
@@ -390,6 +433,11 @@ int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>
             }
         }
     }
+    if (hw > 0 && alcs::tc_fits(w->cin, w->cout, q / hw, hw, hw, 1)) {
+        int n[8];
+        const int count = tc_widths(w, n);
+        for (int i = 0; i < count; ++i) out.push_back(tc_plan(w, n[i], q, di.sms));
+    }
     if (allow_small && hw > 0 && q / hw <= 8) {        // small batches only: one thread block per (block row, image, pixel tile)
         for (int p = 8; p >= 2; p /= 2)
             for (int ks = 4; ks <= 16; ks *= 2) {
@@ -410,6 +458,13 @@ void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
         c->math_mode = 3;
         return;
     }
+    if (p.tc_n) {
+        std::memset(c, 0, sizeof *c);
+        c->pixels_per_lane = 1;
+        c->math_mode = 4;
+        c->row_groups = p.n_rg;
+        return;
+    }
     const KernelVariant& v = g_variants[p.variant].v;
     c->pixels_per_lane = v.p;
     c->rows_per_warp = v.rw;
@@ -426,10 +481,37 @@ void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
 }
 
 // Resolve a (possibly partial) configuration into a concrete plan.
-int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg* c, Plan* out, bool allow_small = true)
+int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg* c, Plan* out, bool allow_small = true, long long hw_in = 0)
 {
+    if (hw_in < hw) hw_in = hw;
+    DeviceInfo di;
+    int rc = device_info(w->device, &di);
+    if (rc) return rc;
+    // (strided inputs are staged element by element by the tcgen05 kernel: 135 us against 90 for 256 -> 512 channels,
+    // 56 x 56 at stride 2, batch 32, so it takes them only when asked to)
+    if (hw > 0 && ((!c && hw_in == hw) || (c && c->math_mode == 4)) && alcs::tc_fits(w->cin, w->cout, q / hw, hw_in, hw, 1)) {
+        if (c) {        // the tcgen05 kernel as asked for: row_groups channel tiles
+            const int tiles = c->row_groups ? c->row_groups : tc_best(w, q, di.sms).n_rg;
+            const int n = ((w->cout + std::max(1, tiles) - 1) / std::max(1, tiles) + 15) / 16 * 16;
+            if (n > alcs::kTcMaxN) return ALCS_ERR_UNSUPPORTED;
+            *out = tc_plan(w, n, q, di.sms);
+            return ALCS_OK;
+        }
+        // Nobody asked for anything: the tcgen05 kernel, or the small-problem kernel where a few images leave most
+        // SMs without a tile and the latency of one item's chunk chain is all there is.
+        *out = tc_best(w, q, di.sms);
+        if (allow_small && q / hw <= 8)
+            for (int p = 8; p >= 2; p /= 2)
+                for (int ks = 4; ks <= 16; ks *= 2) {
+                    Plan g;
+                    if (gather_plan(w, (int)(q / hw), hw, p, ks, di, &g) && g.cost * kGatherWeight + kGatherRamp < out->cost &&
+                        (!out->gather || g.cost < out->cost)) *out = g;
+                }
+        return ALCS_OK;
+    }
+    if (c && c->math_mode == 4) return ALCS_ERR_UNSUPPORTED;
     std::vector<Plan> all;
-    int rc = enumerate_plans(w, q, hw, all, allow_small);
+    rc = enumerate_plans(w, q, hw, all, allow_small);
     if (rc) return rc;
     if (!c) { *out = all[0]; return ALCS_OK; }
     if (c->math_mode == 3 && !allow_small) return ALCS_ERR_UNSUPPORTED;
@@ -439,15 +521,12 @@ int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg
                 *out = p;
                 return ALCS_OK;
             }
-        DeviceInfo di;
-        rc = device_info(w->device, &di);
-        if (rc) return rc;
         if (hw > 0 && c->pixels_per_lane && c->warps &&
             gather_plan(w, (int)(q / hw), hw, c->pixels_per_lane, c->warps, di, out)) return ALCS_OK;
         return ALCS_ERR_UNSUPPORTED;
     }
     auto variant_ok = [&](const Plan& p) {
-        if (p.gather) return false;
+        if (p.gather || p.tc_n) return false;
         const KernelVariant& v = g_variants[p.variant].v;
         if (c->pixels_per_lane && c->pixels_per_lane != v.p) return false;
         if (c->rows_per_warp && c->rows_per_warp != v.rw) return false;
@@ -469,9 +548,6 @@ int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg
         if (variant_ok(p) && (!c->row_groups || c->row_groups == p.n_rg)) { *out = p; return ALCS_OK; }
     // a row-group count outside the enumerated range: accept it for a matching variant if it fits
     if (c->row_groups > 0 && c->row_groups <= w->rows) {
-        DeviceInfo di;
-        rc = device_info(w->device, &di);
-        if (rc) return rc;
         for (const Plan& p0 : all) {
             if (!variant_ok(p0)) continue;
             const KernelVariant& v = g_variants[p0.variant].v;
@@ -701,6 +777,29 @@ int launch_gather_plan(const alcs_packed* w, const Plan& p, const void* x, void*
     return ALCS_OK;
 }
 
+alcs::TcProblem tc_problem(const void* x, void* y, int n, int h, int wd, const float* bias, unsigned flags, const void* residual, int stride,
+                           int h_in, int wd_in)
+{
+    return {x, y, bias, residual, n, h, wd, h_in, wd_in, stride, 0, 0, 0, flags};
+}
+
+// Launch the tcgen05 kernel for one layer whose weights are prepared.
+int launch_tc_prepared(const alcs_packed* w, const alcs::TcPrep& t, const alcs::TcProblem& p, cudaStream_t st)
+{
+    alcs::TcArgs<alcs::kTcMaxLayers> a;
+    a.n_layers = 1;
+    alcs::tc_fill(w, t, p, &a.layer[0]);
+    const int rc = alcs::tc_finish(w, a);
+    return rc ? rc : alcs::tc_launch(w, a, false, st);
+}
+
+int launch_tc_plan(const alcs_packed* w, const Plan& p, const alcs::TcProblem& pr, cudaStream_t st)
+{
+    alcs::TcPrep* t = nullptr;
+    const int rc = alcs::tc_prepare(w, {p.tc_n, 0, 0, 0, 0}, st, &t);
+    return rc ? rc : launch_tc_prepared(w, *t, pr, st);
+}
+
 // scratch / scratch_bytes: where X is repacked when its rows are not 16-byte multiples.  nullptr means
 // the scratch that w owns (allocated or grown here); a layer stack passes its own, fixed for the
 // stack's lifetime, so that a captured graph never refers to memory a later call may free.
@@ -717,6 +816,7 @@ int launch_plan(const alcs_packed* w, const Plan& p, const void* x, void* y, int
         const int rc = ensure_canonical_on_device(w, st);
         return rc ? rc : launch_gather_plan(w, p, x, y, n, h, wd, bias, flags, st);
     }
+    if (p.tc_n) return launch_tc_plan(w, p, tc_problem(x, y, n, h, wd, bias, flags, residual, stride, h_in, wd_in), st);
     const KernelVariant& v = g_variants[p.variant].v;
     Schedule* sc = get_schedule(w, p.kc, p.n_rg, true, flavour_of(v));
     if (!sc) return ALCS_ERR_ALLOC;
@@ -827,7 +927,7 @@ int check_device(const alcs_packed* w)
 }
 
 int resolve_plan(const alcs_packed* w, int n, int h, int wd, unsigned flags, long long q,
-                 const alcs_launch_cfg* cfg, Plan* plan)
+                 const alcs_launch_cfg* cfg, Plan* plan, long long hw_in = 0)
 {
     alcs::ShapeKey key{n, h, wd, flags};
     if (cfg) {
@@ -846,7 +946,7 @@ int resolve_plan(const alcs_packed* w, int n, int h, int wd, unsigned flags, lon
         auto it = w->tuned.find(alcs::ShapeKey{n, h, wd, flags & ~kStagedOnly});
         if (it != w->tuned.end() && !((flags & kStagedOnly) && it->second.math_mode == 3)) use = &it->second;
     }
-    const int rc = cfg_to_plan(w, q, h * wd, use, plan, !(flags & kStagedOnly));
+    const int rc = cfg_to_plan(w, q, h * wd, use, plan, !(flags & kStagedOnly), hw_in);
     if (rc) return rc;
     std::lock_guard<std::mutex> lk(w->mu);
     w->plan_cache[key] = *plan;
@@ -873,6 +973,11 @@ int schedule_upload(const alcs_packed* w, Schedule* sc, void* cuda_stream)
     return upload_schedule(w, sc, static_cast<cudaStream_t>(cuda_stream));
 }
 
+int canonical_on_device(const alcs_packed* w, void* cuda_stream)
+{
+    return ensure_canonical_on_device(w, static_cast<cudaStream_t>(cuda_stream));
+}
+
 int require_current_device(const alcs_packed* w) { return check_device(w); }
 
 }  // namespace alcs
@@ -889,6 +994,15 @@ struct alcs_stack {
         int oh, ow;         // output size (= h, wd unless the layer has a stride)
     };
     std::vector<Item> items;
+    // What one pass launches, in order: a layer by its plan, or (args) consecutive layers on the tcgen05 kernel, none
+    // of which reads or writes what another one writes, in one launch.  Made from the items by build_runs().
+    struct Run {
+        int first, count;
+        std::unique_ptr<alcs::TcArgs<alcs::kTcMaxLayers>> args;
+        int* sched = nullptr;       // device
+    };
+    std::vector<Run> runs;
+    bool runs_valid = false;
     unsigned flags = 0;
     cudaGraphExec_t exec = nullptr;
     // repack scratch of the stack's own (the layers run one after the other, so they share it):
@@ -949,6 +1063,7 @@ ALCS_API void alcs_packed_free(alcs_packed* p)
         if (cudaGetDevice(&prev) == cudaSuccess && cudaSetDevice(p->device) == cudaSuccess) {
             for (auto& kv : p->sched) free_schedule_device(kv.second);
             for (auto& kv : p->sched2d) free_schedule_device(kv.second);
+            for (auto& kv : p->tc) alcs::tc_free(kv.second);
             cudaFree(p->d_err);
             cudaFree(p->d_xpad);
             cudaFree(p->d_row_ptr); cudaFree(p->d_col_idx); cudaFree(p->d_vals);
@@ -1037,7 +1152,7 @@ ALCS_API int alcs_spconv1x1_ex(const alcs_packed* w, const void* x, void* y, int
         if (rb < yend && yb < rend) return ALCS_ERR_INVALID_ARG;     // the residual may not overlap y
     }
     Plan plan;
-    rc = resolve_plan(w, n, oh, ow, flags | kStagedOnly, q, cfg, &plan);
+    rc = resolve_plan(w, n, oh, ow, flags | kStagedOnly, q, cfg, &plan, (long long)h * wd);
     if (rc) return rc;
     return launch_plan(w, plan, x, y, n, oh, ow, bias, flags, static_cast<cudaStream_t>(cuda_stream), nullptr, 0,
                        residual, stride, h, wd);
@@ -1154,8 +1269,8 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
     }
     {   // release the device copies of the schedules that did not win
         std::lock_guard<std::mutex> lk(w->mu);
-        auto key_of = [&](const Plan& pl) {      // (the small-problem kernel uses no schedule: a key that matches none)
-            return pl.gather ? std::make_pair(0, 0) : alcs::sched_key(pl.kc, pl.n_rg, flavour_of(g_variants[pl.variant].v));
+        auto key_of = [&](const Plan& pl) {      // (kernels that use no schedule: a key that matches none)
+            return pl.gather || pl.tc_n ? std::make_pair(0, 0) : alcs::sched_key(pl.kc, pl.n_rg, flavour_of(g_variants[pl.variant].v));
         };
         for (auto& kv : w->sched)
             if (kv.second.uploaded && kv.first != key_of(all[best_i])) {
@@ -1227,6 +1342,258 @@ ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void*
     return ALCS_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Bytes [first, last) of a layer's buffers.
+struct Extent {
+    uintptr_t b, e;
+    bool meets(const Extent& o) const { return b < o.e && o.b < e; }
+};
+
+struct LayerExtents {
+    Extent x, y, res;
+};
+
+LayerExtents extents(const alcs_stack::Item& it)
+{
+    const alcs_layer& L = it.layer;
+    const size_t xe = L.w->elt(), ye = (L.w->dt != ALCS_F32 && !(L.flags & ALCS_Y_F32)) ? 2 : 4;
+    const size_t yb = (size_t)it.q * L.w->cout * ye;
+    LayerExtents r;
+    r.x = {(uintptr_t)L.x, (uintptr_t)L.x + (size_t)L.n * L.w->cin * L.h * L.wd * xe};
+    r.y = {(uintptr_t)L.y, (uintptr_t)L.y + yb};
+    r.res = {(uintptr_t)L.residual, L.residual ? (uintptr_t)L.residual + yb : 0};
+    return r;
+}
+
+// May the two layers run at the same time?
+bool independent(const LayerExtents& a, const LayerExtents& b)
+{
+    return !(a.y.meets(b.x) || a.y.meets(b.res) || a.y.meets(b.y) || b.y.meets(a.x) || b.y.meets(a.res));
+}
+
+alcs::TcProblem tc_problem(const alcs_stack::Item& it)
+{
+    const alcs_layer& L = it.layer;
+    return tc_problem(L.x, L.y, L.n, it.oh, it.ow, L.bias, L.flags, L.residual, L.stride > 1 ? L.stride : 1, L.h, L.wd);
+}
+
+// Layers [first, end) that one launch of the tcgen05 kernel could take, starting at `first`; eligible(i) says
+// whether layer i may be part of it.
+template <typename F>
+size_t merge_end(const alcs_stack* s, size_t first, F eligible)
+{
+    std::vector<LayerExtents> ext;
+    size_t end = first;
+    for (; end < s->items.size() && end - first < (size_t)alcs::kTcMaxLayers; ++end) {
+        const alcs_stack::Item& it = s->items[end];
+        if (it.q == 0 || !eligible(it) || it.layer.w->dt != s->items[first].layer.w->dt || it.layer.w->device != s->items[first].layer.w->device) break;
+        const LayerExtents e = extents(it);
+        bool free = true;
+        for (const LayerExtents& o : ext) free = free && independent(e, o);
+        if (!free) break;
+        ext.push_back(e);
+    }
+    return end;
+}
+
+// Consecutive independent layers whose configuration nobody fixed: one launch of the tcgen05 kernel for all of
+// them, where its estimate is below the sum of the layers' own.  With few items in all, narrower tiles shorten
+// the longest SM's share; with many, wide ones do the least work.
+void stack_merge(alcs_stack* s)
+{
+    auto open = [&](const alcs_stack::Item& it) {
+        const alcs_layer& L = it.layer;
+        if (L.stride > 1 || !alcs::tc_fits(L.w->cin, L.w->cout, L.n, (long long)L.h * L.wd, (long long)it.oh * it.ow, 1)) return false;
+        std::lock_guard<std::mutex> lk(L.w->mu);
+        return L.w->tuned.find(alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}) == L.w->tuned.end();
+    };
+    for (size_t i = 0; i < s->items.size();) {
+        const size_t end = s->items[i].q ? merge_end(s, i, open) : i;
+        DeviceInfo di;
+        if (end - i < 2 || device_info(s->items[i].layer.w->device, &di)) { i = std::max(end, i + 1); continue; }
+        double best = 0;
+        for (size_t k = i; k < end; ++k) best += s->items[k].plan.cost * 1e6;
+        std::vector<int> choice, widths(end - i);
+        for (int cap = alcs::kTcMaxN; cap >= 16; cap /= 2) {
+            double total = 0, longest = 0;
+            for (size_t k = i; k < end; ++k) {
+                const alcs_stack::Item& it = s->items[k];
+                const alcs_packed* w = it.layer.w;
+                int n[8], at = 0;
+                const int count = tc_widths(w, n);
+                while (at + 1 < count && n[at] > cap) ++at;
+                const double us = alcs::tc_item_us(w->dt, n[at], (w->cin + 15) / 16);
+                total += us * ((it.q + alcs::kTcM - 1) / alcs::kTcM) * ((w->cout + n[at] - 1) / n[at]);
+                longest = std::max(longest, us);
+                widths[k - i] = n[at];
+            }
+            const double t = kTcRampUs + std::max(total / di.sms, longest) + 0.25 * longest;
+            if (t < best) { best = t; choice = widths; }
+        }
+        for (size_t k = i; k < end && !choice.empty(); ++k) {
+            alcs_stack::Item& it = s->items[k];
+            it.plan = tc_plan(it.layer.w, choice[k - i], it.q, di.sms);
+        }
+        i = end;
+    }
+}
+
+// What the layers' plans need on the device must be there before any launch is captured.
+int stack_make_resident(alcs_stack* s)
+{
+    for (auto& it : s->items) {
+        if (it.q == 0) continue;
+        const alcs_packed* w = it.layer.w;
+        int rc = ALCS_OK;
+        if (it.plan.gather) {
+            rc = ensure_canonical_on_device(w, nullptr);
+        } else if (it.plan.tc_n) {
+            alcs::TcPrep* t = nullptr;
+            rc = alcs::tc_prepare(w, {it.plan.tc_n, 0, 0, 0, 0}, nullptr, &t);
+        } else {
+            Schedule* sc = get_schedule(w, it.plan.kc, it.plan.n_rg, true, flavour_of(g_variants[it.plan.variant].v));
+            rc = sc ? upload_schedule(w, sc, nullptr) : ALCS_ERR_ALLOC;
+        }
+        if (rc) return rc;
+    }
+    return ALCS_OK;
+}
+
+// Scratch for the repacked inputs of the staged kernels: of the layers that run on one, or (any_plan) of every
+// layer, with room for copy mode 4 at any tile width, so that alcs_stack_tune may switch a layer to it.
+int stack_scratch(alcs_stack* s, bool any_plan)
+{
+    size_t need = 0;
+    for (const auto& it : s->items) {
+        if (it.q == 0 || (!any_plan && (it.plan.gather || it.plan.tc_n))) continue;
+        const alcs_layer& L = it.layer;
+        const int elt = (int)L.w->elt();
+        const long long hw = (long long)it.oh * it.ow;
+        const size_t px = (size_t)L.n * padded_hw((int)hw, elt);
+        if (px > (1ull << 30)) continue;
+        if ((hw * elt) % 16 != 0 || L.stride > 1) need = std::max(need, px * L.w->cin * elt);
+        if (it.q > 8 * hw) need = std::max(need, (px + 512) * L.w->cin * (elt + 1));
+    }
+    if (need <= s->xpad_bytes) return ALCS_OK;
+    if (s->xpad) cudaFree(s->xpad);
+    s->xpad = nullptr;
+    s->xpad_bytes = 0;
+    if (cudaMalloc(&s->xpad, need) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ALCS_ERR_ALLOC;
+    }
+    s->xpad_bytes = need;
+    return ALCS_OK;
+}
+
+void drop_runs(alcs_stack* s)
+{
+    for (auto& r : s->runs)
+        if (r.sched) cudaFree(r.sched);
+    s->runs.clear();
+    s->runs_valid = false;
+}
+
+// One launch for items [first, end): arguments, and which SM takes which items.  Items of different layers take
+// different times, so they are dealt out by a greedy list: in order, the next item to the SM that is free first;
+// where each SM gets only a few, the longest ones go first.
+int build_merged(alcs_stack* s, size_t first, size_t end)
+{
+    const alcs_packed* w0 = s->items[first].layer.w;
+    DeviceInfo di;
+    int rc = device_info(w0->device, &di);
+    if (rc) return rc;
+    alcs_stack::Run run;
+    run.first = (int)first;
+    run.count = (int)(end - first);
+    run.args.reset(new alcs::TcArgs<alcs::kTcMaxLayers>());
+    alcs::TcArgs<alcs::kTcMaxLayers>& a = *run.args;
+    a.n_layers = run.count;
+    std::vector<std::vector<double>> us(run.count);       // per layer and channel tile
+    for (int i = 0; i < run.count; ++i) {
+        const auto& it = s->items[first + i];
+        alcs::TcPrep* t = nullptr;
+        rc = alcs::tc_prepare(it.layer.w, {it.plan.tc_n, 0, 0, 0, 0}, nullptr, &t);
+        if (rc) return rc;
+        alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
+        for (int k16 : t->k16) us[i].push_back(alcs::tc_item_us(it.layer.w->dt, t->n, k16));
+    }
+    rc = alcs::tc_finish(w0, a);
+    if (rc) return rc;
+    if (run.count > 1) {
+        const int blocks = std::min(a.n_items, di.sms);
+        std::vector<std::pair<double, int>> items;
+        items.reserve(a.n_items);
+        for (int i = 0; i < run.count; ++i) {
+            const alcs::TcLayer& y = a.layer[i];
+            for (int k = 0; k < y.n_tiles.d * y.px_tiles.d; ++k)
+                items.emplace_back(us[i][y.tile_major ? k / y.px_tiles.d : k % y.n_tiles.d], y.first_item + k);
+        }
+        if (a.n_items <= 16 * blocks)
+            std::stable_sort(items.begin(), items.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
+        std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<std::pair<double, int>>> idle;
+        for (int b = 0; b < blocks; ++b) idle.emplace(0.0, b);
+        std::vector<std::vector<int>> list(blocks);
+        size_t longest = 0;
+        for (const auto& it : items) {
+            auto b = idle.top();
+            idle.pop();
+            list[b.second].push_back(it.second);
+            longest = std::max(longest, list[b.second].size());
+            idle.emplace(b.first + it.first, b.second);
+        }
+        std::vector<int> table((longest + 1) * blocks, -1);
+        for (int b = 0; b < blocks; ++b)
+            for (size_t k = 0; k < list[b].size(); ++k) table[k * blocks + b] = list[b][k];
+        if (cudaMalloc(&run.sched, table.size() * 4) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ALCS_ERR_ALLOC;
+        }
+        a.sched = run.sched;
+        const cudaError_t e = cudaMemcpy(run.sched, table.data(), table.size() * 4, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            cudaFree(run.sched);
+            alcs::set_cuda_error_text(cudaGetErrorString(e));
+            (void)cudaGetLastError();
+            return ALCS_ERR_CUDA;
+        }
+    }
+    s->runs.push_back(std::move(run));
+    return ALCS_OK;
+}
+
+int build_runs(alcs_stack* s)
+{
+    drop_runs(s);
+    auto on_tc = [](const alcs_stack::Item& it) { return it.plan.tc_n != 0; };
+    for (size_t i = 0; i < s->items.size();) {
+        if (s->items[i].q == 0) { ++i; continue; }
+        const size_t end = merge_end(s, i, on_tc);
+        if (end > i) {
+            const int rc = build_merged(s, i, end);
+            if (rc) { drop_runs(s); return rc; }
+            i = end;
+        } else {
+            alcs_stack::Run run;
+            run.first = (int)i;
+            run.count = 1;
+            s->runs.push_back(std::move(run));
+            ++i;
+        }
+    }
+    s->runs_valid = true;
+    return ALCS_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+ALCS_API int alcs_stack_destroy(alcs_stack* s);
+
 ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned stack_flags, alcs_stack** out)
 {
     if (!out) return ALCS_ERR_INVALID_ARG;
@@ -1235,7 +1602,6 @@ ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned 
     alcs_stack* s = new (std::nothrow) alcs_stack();
     if (!s) return ALCS_ERR_ALLOC;
     s->flags = stack_flags;
-    size_t scratch_need = 0;
     for (int i = 0; i < n_layers; ++i) {
         const alcs_layer& L = layers[i];
         alcs_stack::Item it;
@@ -1247,51 +1613,34 @@ ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned 
         it.ow = (L.wd + stride - 1) / stride;
         int rc = check_conv_args(L.w, L.x, L.y, L.n, it.oh, it.ow, L.flags, &it.q);
         if (!rc) rc = check_device(L.w);
-        if (!rc && it.q > 0) rc = resolve_plan(L.w, L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u), it.q, nullptr, &it.plan);
-        if (!rc && it.q > 0 && it.plan.gather) {
-            rc = ensure_canonical_on_device(L.w, nullptr);
-        } else if (!rc && it.q > 0) {   // the schedule must be resident before any launch is captured
-            Schedule* sc = get_schedule(L.w, it.plan.kc, it.plan.n_rg, true, flavour_of(g_variants[it.plan.variant].v));
-            rc = sc ? upload_schedule(L.w, sc, nullptr) : ALCS_ERR_ALLOC;
-            const int elt = (int)L.w->elt();
-            const long long hw = (long long)it.oh * it.ow;
-            if (!rc && ((hw * elt) % 16 != 0 || stride > 1) && (long long)L.n * padded_hw((int)hw, elt) <= (1ll << 30))
-                scratch_need = std::max(scratch_need, (size_t)L.n * L.w->cin * padded_hw((int)hw, elt) * elt);
-            // room for the tile-major copy of X that copy mode 4 makes, for any tile width (alcs_stack_tune
-            // may switch a layer to it)
-            if (!rc && (long long)L.n * padded_hw((int)hw, elt) <= (1ll << 30) && it.q > 8 * hw)
-                scratch_need = std::max(scratch_need, ((size_t)L.n * padded_hw((int)hw, elt) + 512) * L.w->cin * (elt + 1));
-        }
+        if (!rc && it.q > 0) rc = resolve_plan(L.w, L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u), it.q, nullptr, &it.plan, (long long)L.h * L.wd);
         if (rc) { delete s; return rc; }
         s->items.push_back(it);
     }
-    if (scratch_need) {
-        if (cudaMalloc(&s->xpad, scratch_need) != cudaSuccess) {
-            (void)cudaGetLastError();
-            delete s;
-            return ALCS_ERR_ALLOC;
-        }
-        s->xpad_bytes = scratch_need;
-    }
+    stack_merge(s);
+    int rc = stack_make_resident(s);
+    if (!rc) rc = stack_scratch(s, false);
+    if (!rc) rc = build_runs(s);
+    if (rc) { alcs_stack_destroy(s); return rc; }
     *out = s;
     return ALCS_OK;
 }
 
 static int stack_enqueue(alcs_stack* s, cudaStream_t st)
 {
-    int index = 0;
-    for (auto& it : s->items) {
-        ++index;
-        if (it.q == 0) continue;
+    for (auto& run : s->runs) {
+        const auto& it = s->items[run.first];
         const alcs_layer& L = it.layer;
-        // one named range per layer: a timeline then shows the per-layer run times T^(l) whose sum the
+        // one named range per launch: a timeline then shows the per-layer run times T^(l) whose sum the
         // paper's latency model is about (a no-op unless a profiler has attached itself to the process)
         char name[96];
-        std::snprintf(name, sizeof name, "alcs layer %d: %d->%d @%dx%d n=%d", index, L.w->cin, L.w->cout, L.h, L.wd, L.n);
+        if (run.count > 1) std::snprintf(name, sizeof name, "alcs layers %d to %d", run.first + 1, run.first + run.count);
+        else std::snprintf(name, sizeof name, "alcs layer %d: %d->%d @%dx%d n=%d", run.first + 1, L.w->cin, L.w->cout, L.h, L.wd, L.n);
         nvtxRangePushA(name);
         struct Pop { ~Pop() { nvtxRangePop(); } } pop;
-        int rc = launch_plan(L.w, it.plan, L.x, L.y, L.n, it.oh, it.ow, L.bias, L.flags, st, s->xpad, s->xpad_bytes,
-                             L.residual, L.stride > 1 ? L.stride : 1, L.h, L.wd);
+        const int rc = run.args ? alcs::tc_launch(L.w, *run.args, false, st)
+                                : launch_plan(L.w, it.plan, L.x, L.y, L.n, it.oh, it.ow, L.bias, L.flags, st, s->xpad, s->xpad_bytes,
+                                              L.residual, L.stride > 1 ? L.stride : 1, L.h, L.wd);
         if (rc) return rc;
     }
     return ALCS_OK;
@@ -1300,6 +1649,10 @@ static int stack_enqueue(alcs_stack* s, cudaStream_t st)
 ALCS_API int alcs_stack_run(alcs_stack* s, void* cuda_stream)
 {
     if (!s) return ALCS_ERR_INVALID_ARG;
+    if (!s->runs_valid) {
+        const int rc = build_runs(s);
+        if (rc) return rc;
+    }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (!(s->flags & ALCS_STACK_GRAPH)) return stack_enqueue(s, st);
     if (!s->exec) {
@@ -1333,7 +1686,7 @@ namespace {
 bool same_plan(const Plan& a, const Plan& b)
 {
     return a.variant == b.variant && a.kc == b.kc && a.n_rg == b.n_rg && a.stages == b.stages && a.bulk == b.bulk &&
-           a.gather == b.gather && a.gp == b.gp && a.gks == b.gks;
+           a.gather == b.gather && a.gp == b.gp && a.gks == b.gks && a.tc_n == b.tc_n;
 }
 
 // Run time of one pass over the whole stack in microseconds, as alcs_stack_run runs it (a graph stack
@@ -1342,6 +1695,7 @@ bool same_plan(const Plan& a, const Plan& b)
 double time_stack(alcs_stack* s, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int reps)
 {
     if (s->exec) { cudaGraphExecDestroy(s->exec); s->exec = nullptr; }
+    s->runs_valid = false;
     for (int i = 0; i < 2; ++i)
         if (alcs_stack_run(s, st) != ALCS_OK) return -1.0;
     double best = 1e30;
@@ -1402,6 +1756,8 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
         return ALCS_ERR_CUDA;
     }
     struct Done { cudaEvent_t a, b; ~Done() { cudaEventDestroy(a); cudaEventDestroy(b); } } done{e0, e1};
+    const int scratch_rc = stack_scratch(s, true);
+    if (scratch_rc) return scratch_rc;
     double cur = time_stack(s, st, e0, e1, 3);
     if (cur < 0) return ALCS_ERR_CUDA;
     const int reps = (int)std::min(100.0, std::max(3.0, 3000.0 / std::max(cur, 1.0)));     // batches of about 3 ms
@@ -1424,7 +1780,7 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
                 if (same_plan(c, best) || same_plan(c, it.plan)) continue;
                 if (c.gather) {
                     if (ensure_canonical_on_device(L.w, nullptr) != ALCS_OK) continue;
-                } else {
+                } else if (!c.tc_n) {
                     const KernelVariant& v = g_variants[c.variant].v;
                     Schedule* sc = get_schedule(L.w, c.kc, c.n_rg, true, flavour_of(v));
                     if (!sc || (v.split && sc->max_x == 0) || upload_schedule(L.w, sc, nullptr) != ALCS_OK) continue;
@@ -1440,15 +1796,19 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
                 it.plan = best;
                 cur = best_t;
                 changed = true;
-                alcs_launch_cfg c;
-                plan_to_cfg(best, &c);
-                const bool extra = (L.stride > 1) || L.residual;
-                std::lock_guard<std::mutex> lk(L.w->mu);
-                L.w->tuned[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}] = c;
-                L.w->plan_cache[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u)}] = best;
             }
         }
         if (!changed) break;
+    }
+    for (auto& it : s->items) {
+        if (it.q == 0) continue;
+        const alcs_layer& L = it.layer;
+        alcs_launch_cfg c;
+        plan_to_cfg(it.plan, &c);
+        const bool extra = (L.stride > 1) || L.residual;
+        std::lock_guard<std::mutex> lk(L.w->mu);
+        L.w->tuned[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}] = c;
+        L.w->plan_cache[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u)}] = it.plan;
     }
     cur = time_stack(s, st, e0, e1, reps);      // (also leaves a graph stack captured with the chosen plans)
     if (cur < 0) return ALCS_ERR_CUDA;
@@ -1469,6 +1829,7 @@ ALCS_API int alcs_stack_destroy(alcs_stack* s)
 {
     if (!s) return ALCS_OK;
     if (s->exec) cudaGraphExecDestroy(s->exec);
+    drop_runs(s);
     if (s->xpad) cudaFree(s->xpad);     // waits for the device, so no replay can still be using it
     delete s;
     return ALCS_OK;
@@ -1530,6 +1891,12 @@ extern "C" ALCS_API int alcs_spconv1x1_noalloc(const alcs_packed* w, const void*
         if (plan.gather) {      // the small-problem kernel: needs only its resident copy of the storage format
             if (!w->d_row_ptr) return ALCS_ERR_STATE;
             return launch_gather_plan(w, plan, x, y, n, h, wd, bias, flags, st);
+        }
+        if (plan.tc_n) {        // needs no scratch, but what does not fit it is refused whatever kernel the plan names
+            const size_t row = (size_t)h * wd * w->elt();
+            if (row % 16 != 0 && (size_t)n * w->cin * ((row + 15) / 16 * 16) > ALCS_NOALLOC_SCRATCH_BYTES) return ALCS_ERR_TOO_LARGE;
+            const alcs::TcPrep* t = alcs::tc_find(w, {plan.tc_n, 0, 0, 0, 0});
+            return t ? launch_tc_prepared(w, *t, tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd), st) : ALCS_ERR_STATE;
         }
         auto si = w->sched.find(alcs::sched_key(plan.kc, plan.n_rg, flavour_of(g_variants[plan.variant].v)));
         if (si == w->sched.end() || !si->second.uploaded) return ALCS_ERR_STATE;

@@ -15,6 +15,8 @@
 
 namespace alcs {
 
+struct TcPrep;      // alcs_tc_prep.h
+
 // Chunk sizes (input channels per pipeline stage) the planner considers.  0 stands for "the
 // whole Cin in one chunk" (used when Cin is small).
 constexpr int kNumChunkings = 6;
@@ -86,6 +88,8 @@ struct Plan {
     // the small-problem kernel (no staging, reads the canonical format): variant is -1, and
     int gather = 0;        // 1 selects it,
     int gp = 0, gks = 0;   // pixels per lane and warps per thread block (shares of one block row's columns)
+    // the tcgen05 kernel (alcs_tc.cu): variant is -1, and
+    int tc_n = 0;          // output channels per tile (0: not this kernel)
 };
 
 // Key of the plan cache: the problem shape plus the requested configuration (all zero = automatic).
@@ -126,6 +130,8 @@ struct alcs_packed {
     // plane, plane pitch, stride, kh, kw, channels per chunk}: the column offsets baked into them depend
     // on the geometry
     mutable std::map<std::array<int, 8>, alcs::Schedule> sched2d;
+    // expanded weights of the tcgen05 kernel, by {channels per tile, kh, kw, h, wd} (alcs_tc_prep.h)
+    mutable std::map<std::array<int, 5>, alcs::TcPrep*> tc;
     mutable std::map<alcs::ShapeKey, alcs_launch_cfg> tuned;   // filled by alcs_spconv1x1_tune, alcs_spconv1x1_set_cfg, alcs_stack_tune
     // the best few plans of the last alcs_spconv1x1_tune per shape, best first: what alcs_stack_tune tries in context
     mutable std::map<alcs::ShapeKey, std::vector<alcs::Plan>> finalists;
@@ -162,6 +168,7 @@ inline std::pair<int, int> sched_key(int kc, int n_rg, int flavour)
 // Device-side helpers implemented in alcs_device.cu, for the library's other translation units.
 int device_limits(int device, int* sms, int* smem_optin);                 // SM count, opt-in shared memory per block
 int schedule_upload(const alcs_packed* w, Schedule* sc, void* cuda_stream); // copy a schedule to w's device (once)
+int canonical_on_device(const alcs_packed* w, void* cuda_stream);           // device copy of row_ptr / col_idx / vals (once)
 int require_current_device(const alcs_packed* w);                          // ALCS_OK if w is uploaded and its device is current
 // bytes of one step record of the tensor-core flavour
 constexpr int step_record_bytes(int g) { return 32 + 32 * (g < 8 ? 8 : g); }

@@ -1,0 +1,870 @@
+// Convolution on the fifth-generation tensor cores (tcgen05), sm_100a.
+//
+// A work item is (128 output pixels) x (n output channels).  The item's pruned weights are expanded
+// to a dense [columns][n] tile (columns that no row of the tile keeps are left out), so that the item
+// is a plain contraction
+//     D[128 pixels][n] += A[128 pixels][64 columns] * B[64 columns][n]
+// per chunk of 64 columns, with D and A in tensor memory and B in shared memory.
+//
+// fp32 operands are split exactly into three bfloat16 parts (8 + 8 + 8 significant bits) and six of
+// the nine partial products are formed, which leaves out terms below 2^-24 of a product; they are
+// summed smallest first into a fresh accumulator per chunk, and the chunk sums are added in fp32
+// (round to nearest) in registers.  The tensor core truncates when it adds to its fp32 accumulator;
+// with four full-size additions per chunk the result is closer to the exact sum than a chain of fp32
+// FMAs (relative error 7e-8 against 2.3e-7 at 512 columns, 30 % of them kept).
+// 16-bit operands are used as they are, 256 columns per accumulator.
+//
+// Roles (32 warps, one thread block per SM, persistent over items):
+//   warps 27-30  producers: copy chunks of X ([64 columns][128 pixels]) into a ring in shared memory, several
+//                chunks ahead; 16-byte copies where images allow it, single elements otherwise (any image
+//                size, stride, channel list or tap offset costs only address arithmetic)
+//   warps 0-15   converters: a lane is a pixel, a warp takes 16 of a chunk's columns; split the values and write them to tensor memory as
+//                the A operand (double-buffered)
+//   warps 24-25  issue the MMAs: in fp32 the chunks, which have an accumulator each, in turn, so that one waits for
+//                its next chunk while the other's instructions run; in 16 bits the first alone
+//   warp 26      copies the weight tiles (bulk copies into a ring)
+//   warps 16-23  epilogue: add the chunk sums up, then bias, residual, ReLU and stores, while the next
+//                item is already being multiplied (two accumulators)
+#include "alcs_tc.h"
+
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+namespace alcs {
+namespace {
+
+constexpr int kConvWarps = 16, kEpiWarps = 8, kProdWarps = 4;
+constexpr int kMmaWarp = kConvWarps + kEpiWarps, kLoadWarp = kMmaWarp + 2, kProdWarp0 = kMmaWarp + 3;
+constexpr int kThreads = 1024;      // eight warpgroups (one warp idle)
+// Registers per thread: 1024 threads start with 64; the epilogue, which holds 64 sums, takes from the
+// others: 4 * 40 + 2 * 128 + 2 * 48 <= 8 * 64.
+constexpr int kConvRegs = 40, kEpiRegs = 128, kProdRegs = 48;
+// Shared memory: barriers and the TMEM address; the bias of the items being stored (two copies of 128 words per
+// half of the epilogue); weight stages; X ring.
+constexpr int kBarBytes = kTcHeaderBytes, kEpiOff = 1024, kEpiBytes = 512;
+static_assert(kEpiOff + 4 * kEpiBytes <= kBarBytes, "header");
+constexpr int kMaxStages = 8;
+constexpr int kMaxTcSmem = 227 * 1024;
+constexpr unsigned kPolls = 1u << 18;
+
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void bar_init(unsigned bar, unsigned count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(unsigned bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity)
+{
+#pragma unroll 1
+    for (unsigned i = 0; i < kPolls; ++i) {
+        unsigned ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+__device__ __forceinline__ bool elect_one()
+{
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+    return ok != 0;
+}
+__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+__device__ __forceinline__ void mma_f16(unsigned d, unsigned a, unsigned long long b, unsigned idesc, unsigned acc)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+                 ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void mma_commit(unsigned bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_st4(unsigned addr, const unsigned (&v)[4])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(unsigned addr, float* v)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]) : "r"(addr));
+}
+
+__device__ __forceinline__ void tmem_ld32(unsigned addr, float (&v)[32])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]),
+                   "=f"(v[16]), "=f"(v[17]), "=f"(v[18]), "=f"(v[19]), "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]),
+                   "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29]), "=f"(v[30]), "=f"(v[31])
+                 : "r"(addr));
+}
+
+// One element of X: read once per item, so it takes no room in L1.
+__device__ __forceinline__ unsigned short ld_x(const unsigned short* p)
+{
+    unsigned short v;
+    asm volatile("ld.global.nc.L1::no_allocate.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
+// Wait for loads from tensor memory; the values may not be touched before (they are tied to the wait here).
+template <int N>
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[N])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
+}
+
+template <typename XT> struct Elem;
+template <> struct Elem<float> {
+    using raw = float;
+    static constexpr int planes = 3, fmt = 1;
+    static constexpr int group = 1;       // chunks per accumulator
+    static constexpr int abufs = 2;       // chunks in tensor memory
+};
+template <> struct Elem<__half> {
+    using raw = unsigned short;
+    static constexpr int planes = 1, fmt = 0, group = 2, abufs = 3;
+};
+template <> struct Elem<__nv_bfloat16> {
+    using raw = unsigned short;
+    static constexpr int planes = 1, fmt = 1, group = 2, abufs = 3;
+};
+
+__device__ __forceinline__ int div_of(int n, const TcDiv& d) { return (int)((unsigned long long)(unsigned)n * d.mul >> d.shift); }
+
+// A role's walk over the block's items.  Where the tiles differ, what the next item needs from the tile table
+// is loaded one item ahead.
+template <int L>
+struct Cursor {
+    const TcArgs<L>& a;
+    int item, next_item, at, layer = 0, next_layer = 0;
+    TcTile t, next;
+
+    __device__ __forceinline__ explicit Cursor(const TcArgs<L>& a_) : a(a_), at(blockIdx.x)
+    {
+        next_item = L > 1 && a.sched ? __ldg(a.sched + at) : at;
+        peek();
+    }
+    __device__ __forceinline__ const TcLayer& of() const { return a.layer[L > 1 ? layer : 0]; }
+    __device__ __forceinline__ const TcLayer& next_of() const { return a.layer[L > 1 ? next_layer : 0]; }
+    __device__ __forceinline__ bool has_next() const { return (unsigned)next_item < (unsigned)a.n_items; }
+    static __device__ __forceinline__ int channel_tile(const TcLayer& y, int i)
+    {
+        if (y.tile_major) return div_of(i - y.first_item, y.px_tiles);
+        const int r = i - y.first_item;
+        return r - div_of(r, y.n_tiles) * y.n_tiles.d;
+    }
+    __device__ __forceinline__ int nt() const { return channel_tile(of(), item); }
+    __device__ __forceinline__ int next_nt() const { return channel_tile(next_of(), next_item); }
+    __device__ __forceinline__ int pt() const
+    {
+        const TcLayer& y = of();
+        const int r = item - y.first_item;
+        return y.tile_major ? r - div_of(r, y.px_tiles) * y.px_tiles.d : div_of(r, y.n_tiles);
+    }
+    __device__ __forceinline__ void peek()
+    {
+        if (!has_next()) return;
+        if (L > 1) {
+            next_layer = 0;
+#pragma unroll 1
+            while (next_layer + 1 < a.n_layers && next_item >= a.layer[next_layer + 1].first_item) ++next_layer;
+        }
+        const TcLayer& y = next_of();
+        if (y.tiles) {
+            const TcTile* p = y.tiles + next_nt();
+            next.b16 = __ldg(&p->b16);
+            next.k16 = __ldg(&p->k16);
+            next.kstart = __ldg(&p->kstart);
+        } else {
+            next.k16 = y.k16;
+            next.kstart = 0;
+        }
+    }
+    __device__ __forceinline__ bool step()
+    {
+        if (!has_next()) return false;
+        item = next_item;
+        at += gridDim.x;
+        next_item = L > 1 && a.sched ? __ldg(a.sched + at) : at;
+        layer = next_layer;
+        t = next;
+        peek();
+        return true;
+    }
+};
+
+// Subtract from each of two fp32 values what its upper 16 bits stand for (exact).
+__device__ __forceinline__ void cut2(unsigned& u0, unsigned& u1)
+{
+    asm("{\n\t.reg .b32 h0, h1;\n\t.reg .b64 x, h;\n\tand.b32 h0, %0, 0xffff0000;\n\tand.b32 h1, %1, 0xffff0000;\n\t"
+        "mov.b64 x, {%0, %1};\n\tmov.b64 h, {h0, h1};\n\tsub.rn.f32x2 x, x, h;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "+r"(u0), "+r"(u1));
+}
+
+// Three bfloat16 parts of two fp32 values, packed two to a word: x = part 0 + part 1 + part 2 exactly.
+// Cutting off the low bits (instead of rounding) needs no conversion instructions and cannot overflow;
+// the weights' parts are rounded, so the partial products that are left out have no common sign.
+__device__ __forceinline__ void split2(float x0, float x1, unsigned& p0, unsigned& p1, unsigned& p2)
+{
+    unsigned u0 = __float_as_uint(x0), u1 = __float_as_uint(x1);
+    p0 = __byte_perm(u0, u1, 0x7632);
+    cut2(u0, u1);
+    p1 = __byte_perm(u0, u1, 0x7632);
+    cut2(u0, u1);
+    p2 = __byte_perm(u0, u1, 0x7632);
+}
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+template <int B>
+__device__ __forceinline__ void cp_async_small(unsigned dst, const void* src, unsigned bytes)      // bytes = B, or 0: write zeros
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(B), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void st_slot(unsigned addr, unsigned short v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory"); }
+
+__device__ __forceinline__ void cp_async_arrive(unsigned bar)      // one arrival once this thread's copies so far have landed
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes, unsigned bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
+// Where a producer warp finds the pixels of one item.
+template <typename XT, bool TAPS>
+struct Source {
+    using raw = typename Elem<XT>::raw;
+    static constexpr int kRow = kTcM * (int)sizeof(raw);      // bytes of a column of a chunk in shared memory
+    const raw* x;
+    const int* cols;
+    int off[4];                    // element offset of this lane's first column entry: [0] alone for vector copies
+    unsigned mask[TAPS ? 4 : 1];   // TAPS: which taps of the pixel lie inside the image
+    int hw_in, cin, vb;
+    int img0, n_img = 0, hw;       // whole images (TcLayer::images): first, how many, pixels
+
+    __device__ __forceinline__ int pixel(const TcLayer& y, int q, unsigned& m) const
+    {
+        const int img = div_of(q, y.hw), p = q - img * y.hw.d;
+        const int img_off = img * cin * hw_in;
+        if (TAPS) {
+            const int oy = div_of(p, y.ow), ox = p - oy * y.ow.d;
+            const int ih = oy * y.stride - y.pad, iw = ox * y.stride - y.pad;
+            unsigned row = 0;
+            m = 0;
+#pragma unroll 1
+            for (int s = 0; s < y.kw; ++s) row |= ((unsigned)(iw + s) < (unsigned)y.w_in ? 1u : 0u) << s;
+#pragma unroll 1
+            for (int r = 0; r < y.kh; ++r)
+                if ((unsigned)(ih + r) < (unsigned)y.h_in) m |= row << (r * y.kw);
+            return img_off + ih * y.w_in + iw;
+        }
+        if (y.stride == 1) return img_off + p;
+        const int oy = div_of(p, y.ow);
+        return img_off + oy * y.stride * y.w_in + (p - oy * y.ow.d) * y.stride;
+    }
+
+    __device__ __forceinline__ void open(const TcLayer& y, const TcTile& t, int pt, int lane)
+    {
+        x = static_cast<const raw*>(y.x);
+        hw_in = y.hw_in;
+        cin = y.cin;
+        vb = y.vec_bytes;
+        cols = TAPS ? y.cols + 2 * (size_t)t.kstart : y.cols ? y.cols + t.kstart : nullptr;
+        // (pixels past the end repeat the last ones and are not stored)
+        if (!TAPS && y.images) {
+            img0 = pt * y.images;
+            n_img = min(y.images, y.n_img - img0);
+            hw = y.hw.d;
+        } else if (!TAPS && vb) {
+            const int ppl = vb / (int)sizeof(raw);      // pixels per copy; a column's 128 pixels take 128 / ppl copies
+            off[0] = pixel(y, min(pt * y.ppt + (lane * ppl & (kTcM - 1)), y.q - ppl), mask[0]);
+            if (vb == 4) off[1] = pixel(y, min(pt * y.ppt + 64 + (lane * ppl & 63), y.q - ppl), mask[0]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) off[j] = pixel(y, min(pt * y.ppt + j * 32 + lane, y.q - 1), mask[TAPS ? j : 0]);
+        }
+    }
+
+    // Element offsets of columns k .. k + 3 (past the last channel they meet zero weights: any valid one will do).
+    __device__ __forceinline__ int4 cols4(int k) const
+    {
+        int4 c;
+        if (cols) {
+            c = __ldg(reinterpret_cast<const int4*>(cols + k));
+        } else {
+            c = make_int4(k, k + 1, k + 2, k + 3);
+            if (k + 4 > cin) c = make_int4(min(c.x, cin - 1), min(c.y, cin - 1), min(c.z, cin - 1), min(c.w, cin - 1));
+        }
+        return make_int4(c.x * hw_in, c.y * hw_in, c.z * hw_in, c.w * hw_in);
+    }
+
+    // Copy the chunk that starts at column k0 (kk columns, a multiple of 16) into `slot`; one arrival per lane on `bar`.
+    __device__ __forceinline__ void chunk(unsigned slot, int k0, int kk, int lane, unsigned bar) const
+    {
+        if (!TAPS && n_img) {
+            // whole small images: the chunk's columns of an image are one run of memory
+            if (lane == 0) {
+                const unsigned bytes = (unsigned)(kk * hw) * (unsigned)sizeof(raw);
+                asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes * n_img) : "memory");
+#pragma unroll 1
+                for (int i = 0; i < n_img; ++i)
+                    bulk_load(slot + i * bytes, x + ((size_t)(img0 + i) * cin + k0) * hw, bytes, bar);
+            }
+            __syncwarp();
+            bar_arrive(bar);
+            return;
+        }
+        slot += lane * (TAPS || vb == 0 ? (int)sizeof(raw) : vb);
+#pragma unroll 1
+        for (int k = 0; k < kk; k += 4, slot += 4 * kRow) {
+            if constexpr (TAPS) {
+                const int4 c0 = __ldg(reinterpret_cast<const int4*>(cols + 2 * (k0 + k))), c1 = __ldg(reinterpret_cast<const int4*>(cols + 2 * (k0 + k)) + 1);
+                const int at[4] = {c0.x, c0.z, c1.x, c1.z}, tap[4] = {c0.y, c0.w, c1.y, c1.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const bool in = (mask[j] >> tap[i]) & 1u;
+                        cp_async_small<4>(slot + i * kRow + j * 128, in ? x + (off[j] + at[i]) : x, in ? 4 : 0);
+                    }
+            } else {
+                const int4 c = cols4(k0 + k);
+                const int at[4] = {c.x, c.y, c.z, c.w};
+                if (vb == 16) {
+                    if constexpr (sizeof(raw) == 4) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) cp_async16(slot + i * kRow, x + (at[i] + off[0]));
+                    } else {        // two columns per instruction
+#pragma unroll
+                        for (int i = 0; i < 4; i += 2) cp_async16(slot + i * kRow, x + ((lane < 16 ? at[i] : at[i + 1]) + off[0]));
+                    }
+                } else if constexpr (sizeof(raw) == 4) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) cp_async_small<4>(slot + i * kRow + j * 128, x + (at[i] + off[j]), 4);
+                } else if (vb == 8) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) cp_async_small<8>(slot + i * kRow, x + (at[i] + off[0]), 8);
+                } else if (vb == 4) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        cp_async_small<4>(slot + i * kRow, x + (at[i] + off[0]), 4);
+                        cp_async_small<4>(slot + i * kRow + 128, x + (at[i] + off[1]), 4);
+                    }
+                } else {            // rows that start on odd element boundaries: through registers
+                    raw v[4][4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[i][j] = ld_x(x + (at[i] + off[j]));
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) st_slot(slot + i * kRow + j * 64, v[i][j]);
+                }
+            }
+        }
+        if (sizeof(raw) == 2 && vb == 0) bar_arrive(bar);
+        else cp_async_arrive(bar);
+    }
+};
+
+__device__ __forceinline__ void ld_slot(unsigned addr, float& v) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr)); }
+__device__ __forceinline__ void ld_slot(unsigned addr, unsigned short& v) { asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr)); }
+
+__device__ __forceinline__ void put(float* p, float v) { *p = v; }
+__device__ __forceinline__ void put(__half* p, float v) { *p = __float2half_rn(v); }
+__device__ __forceinline__ void put(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+
+// Output channel of row r of the channel tiles (-1: none).
+__device__ __forceinline__ int channel_of(const TcLayer& y, int r) { return y.chan ? __ldg(y.chan + r) : r < y.cout ? r : -1; }
+
+// The end of an item, 32 rows at a time: bias, residual, ReLU, one rounding, stores.  A warp stores 32 consecutive
+// pixels of one channel per instruction.  `lane_off` is the byte offset of this lane's pixel from `out` (and from
+// `res`, if there is one), which are the same for the whole warp, so that an address is one 32-bit addition.
+// any = false: rows row0 .. are channels row0 .. , and out points at row0; otherwise every row's channel is
+// looked up and out points at channel 0.
+template <typename YT>
+__device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* out, const char* res, unsigned lane_off, unsigned bias, int row0,
+                                        int rows, bool live, bool any)
+{
+    const float floor = y.relu ? 0.0f : __int_as_float(0x7fffffff);      // (NaN: fmaxf returns the other operand)
+    const unsigned pitch = (unsigned)y.hw.d * (unsigned)sizeof(YT);
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) {
+        float b[4];
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3]) : "r"(bias + j * 4));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[j + k] += b[k];
+    }
+    if (!any) {
+        if (!live) return;
+        if (res) {
+#pragma unroll
+            for (int h = 0; h < 32; h += 8) {
+                if (h >= rows) break;
+                YT r[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) r[j] = __ldg(reinterpret_cast<const YT*>(res + (lane_off + (h + j) * pitch)));
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[h + j] += (float)r[j];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 32; j += 8) {
+            if (j >= rows) break;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) put(reinterpret_cast<YT*>(out + (lane_off + (j + k) * pitch)), fmaxf(v[j + k], floor));
+        }
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+        if (j >= rows) break;
+        int c[8];
+        float r[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) c[k] = channel_of(y, row0 + j + k);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) r[k] = res && live && c[k] >= 0 ? (float)__ldg(reinterpret_cast<const YT*>(res + (lane_off + c[k] * pitch))) : 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (live && c[k] >= 0) put(reinterpret_cast<YT*>(out + (lane_off + c[k] * pitch)), fmaxf(v[j + k] + r[k], floor));
+    }
+}
+
+// An item whose tile keeps no block: bias and residual alone.
+template <typename YT>
+__device__ __forceinline__ void store_bias(const TcLayer& y, char* out, const char* res, unsigned lane_off, int row0, int rows, bool live)
+{
+    const unsigned pitch = (unsigned)y.hw.d * (unsigned)sizeof(YT);
+#pragma unroll 1
+    for (int j = 0; j < rows; ++j) {
+        const int c = channel_of(y, row0 + j);
+        if (live && c >= 0) {
+            float v = y.bias ? __ldg(y.bias + c) : 0.0f;
+            if (res) v += (float)__ldg(reinterpret_cast<const YT*>(res + (lane_off + c * pitch)));
+            put(reinterpret_cast<YT*>(out + (lane_off + c * pitch)), y.relu ? fmaxf(v, 0.0f) : v);
+        }
+    }
+}
+
+template <typename XT, bool TAPS, int L>
+__global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__ TcArgs<L> a)
+{
+    using E = Elem<XT>;
+    using raw = typename E::raw;
+    constexpr int P = E::planes;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const unsigned s0 = smem_u32(smem);
+    const unsigned a_full = s0, a_empty = s0 + 32, d_full = s0 + 64, d_empty = s0 + 80, x_full = s0 + 128, x_empty = s0 + 192;
+    const unsigned b_full = s0 + 256, b_empty = s0 + 320, turn = s0 + 384, tmem_slot = s0 + 400;
+    const unsigned stage0 = s0 + kBarBytes, ring0 = stage0 + a.stages * a.stage_bytes;
+    constexpr int NA = E::abufs, KC = P == 3 ? kTcKC32 : kTcKC16, NS = KC / 16, AB = KC / 2 * P;      // AB: TMEM columns of a chunk of A
+    constexpr int S = kProdWarps, kSlot = KC * kTcM * (int)sizeof(raw);      // (every producer owns a slot)
+    static_assert(S * kSlot == kTcRingBytes && NA * AB <= 256, "ring and A buffers");
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (warp == kMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(tmem_slot) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    } else if (warp == kLoadWarp && lane == 0) {
+#pragma unroll 1
+        for (int i = 0; i < NA; ++i) {
+            bar_init(a_full + 8 * i, kConvWarps);
+            bar_init(a_empty + 8 * i, 1);
+        }
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+            bar_init(turn + 8 * i, 1);
+            bar_init(d_full + 8 * i, 1);
+            bar_init(d_empty + 8 * i, kEpiWarps);
+        }
+#pragma unroll 1
+        for (int i = 0; i < kMaxStages; ++i) {
+            bar_init(b_full + 8 * i, 1);
+            bar_init(b_empty + 8 * i, 1);
+        }
+#pragma unroll 1
+        for (int i = 0; i < S; ++i) {
+            bar_init(x_full + 8 * i, 32);
+            bar_init(x_empty + 8 * i, kConvWarps);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
+    unsigned tmem;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem) : "r"(tmem_slot));
+    // tensor memory: D in columns [0, 256), two accumulators of up to 128; A behind, NA buffers
+    const unsigned tmem_a = tmem + 256;
+    bool ok = true;
+
+    if (warp < kConvWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConvRegs));
+        const unsigned quad = (unsigned)(warp & 3);
+        const int s0_ = warp >> 2, row = quad * 32 + lane;       // a warp takes every fourth 16-column step
+        unsigned i = 0, buf = 0, aph = 1;
+        Cursor<L> cur(a);
+#pragma unroll 1
+        while (ok && cur.step()) {
+            const int images = cur.of().images;
+            int hw = kTcM, img = 0, px = row;
+            if (images) {
+                hw = cur.of().hw.d;
+                img = min(div_of(row, cur.of().hw), images - 1);
+                px = min(row - img * hw, hw - 1);
+            }
+#pragma unroll 1
+            for (int k16 = cur.t.k16; k16 > 0; k16 -= NS, ++i) {
+                const unsigned slot = i % S, my_a = tmem_a + (quad << 21) + buf * AB;      // lanes 32 * quad ...
+                const int ns = min(NS, k16);
+                const unsigned src = ring0 + slot * kSlot + (img * ns * 16 * hw + px) * (unsigned)sizeof(raw);
+                ok = __all_sync(0xffffffffu, bar_wait(x_full + 8 * slot, (i / S) & 1u) && bar_wait(a_empty + 8 * buf, aph));
+                if (!ok) break;
+                tc_after();
+#pragma unroll 1
+                for (int s = s0_; s < ns; s += 4) {
+                    raw v[16];
+                    if (images) {
+                        const unsigned at = src + s * 16 * hw * (unsigned)sizeof(raw);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) ld_slot(at + j * hw * (unsigned)sizeof(raw), v[j]);
+                    } else {
+                        const unsigned at = src + s * 16 * kTcM * (unsigned)sizeof(raw);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) ld_slot(at + j * kTcM * (unsigned)sizeof(raw), v[j]);
+                    }
+#pragma unroll
+                    for (int h = 0; h < 8; h += 4) {
+                        unsigned w[P][4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const raw x0 = v[2 * (h + j)], x1 = v[2 * (h + j) + 1];
+                            if constexpr (P == 3) split2(x0, x1, w[0][j], w[1][j], w[2][j]);
+                            else w[0][j] = (unsigned)x0 | ((unsigned)x1 << 16);
+                        }
+#pragma unroll
+                        for (int p = 0; p < P; ++p) tmem_st4(my_a + p * (KC / 2) + s * 8 + h, w[p]);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) bar_arrive(x_empty + 8 * slot);
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_before();
+                __syncwarp();
+                if (lane == 0) bar_arrive(a_full + 8 * buf);
+                if (++buf == NA) { buf = 0; aph ^= 1u; }
+            }
+        }
+    } else if (warp < kConvWarps + kEpiWarps) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
+        const unsigned quad = (unsigned)(warp & 3);
+        // An item of one chunk sum is stored by the four warps that own its accumulator, so that consecutive items
+        // overlap; the sums of the others are added up by all eight warps, half of the channels each.
+        const int e = (warp - kConvWarps) >> 2;
+        unsigned n_grp = 0, bias = s0 + kEpiOff + e * (2 * kEpiBytes);
+        int key = -1, key_layer = -1;       // whose bias is in shared memory
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        Cursor<L> cur(a);
+#pragma unroll 1
+        while (ok && cur.step()) {
+            const TcLayer& y = cur.of();
+            const int groups = (cur.t.k16 + NS * E::group - 1) / (NS * E::group);
+            const bool whole = groups <= 1;
+            if (whole && (groups ? (int)(n_grp & 1u) : 0) != e) {
+                n_grp += groups;
+                continue;
+            }
+            const int nr = whole ? y.n : y.n >> 1, part = whole ? 0 : e * nr, row0 = cur.nt() * y.n + part;
+            // the bias of these rows goes through shared memory; consecutive items of one channel tile share it
+            const int want = row0 * 2 + whole;
+            const bool fresh = groups && (want != key || cur.layer != key_layer);
+            float b[4];
+            if (fresh) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = row0 + i * 32 + lane, c = !y.bias || i * 32 + lane >= nr ? -1 : y.chan ? __ldg(y.chan + r) : r;
+                    b[i] = c >= 0 && c < y.cout ? __ldg(y.bias + c) : 0.0f;
+                }
+                key = want;
+                key_layer = cur.layer;
+            }
+            const int row = (int)quad * 32 + lane, q0 = cur.pt() * y.ppt, q = q0 + row;
+            const bool live = row < y.ppt && q < y.q;
+            const int img0 = div_of(q0, y.hw), img = div_of(live ? q : q0, y.hw), p = (live ? q : q0) - img * y.hw.d;
+            const bool wide = sizeof(XT) == 4 || y.y32, any = y.chan || row0 + nr > y.cout;
+            const unsigned ye = wide ? 4 : sizeof(XT);
+            const unsigned lane_off = ((unsigned)(img - img0) * (unsigned)y.cout * (unsigned)y.hw.d + (unsigned)p) * ye;
+            const size_t item_off = ((size_t)img0 * y.cout + (any ? 0 : row0)) * y.hw.d * ye;
+            char* const out = static_cast<char*>(y.y) + item_off;
+            const char* const res = y.res ? static_cast<const char*>(y.res) + item_off : nullptr;
+            if (groups == 0) {      // nothing kept: the sum is zero, and there is no accumulator to read it from
+                const char* r = y.res ? static_cast<const char*>(y.res) + (size_t)img0 * y.cout * y.hw.d * ye : nullptr;
+                char* o = static_cast<char*>(y.y) + (size_t)img0 * y.cout * y.hw.d * ye;
+                if (wide) store_bias<float>(y, o, r, lane_off, row0, nr, live);
+                else store_bias<XT>(y, o, r, lane_off, row0, nr, live);
+                __syncwarp();
+                continue;
+            }
+            if (res && live) {      // what the end of the item will add: on its way while the item is multiplied
+#pragma unroll 1
+                for (int k = 0; k < nr; ++k) {
+                    const int c = any ? channel_of(y, row0 + k) : k;
+                    if (c >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(res + (lane_off + (unsigned)c * (unsigned)y.hw.d * ye)));
+                }
+            }
+            __syncwarp();
+            float lo[32], hi[32];               // rows 0 .. 31 and 32 .. 63
+            if (!whole) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) lo[j] = hi[j] = 0.0f;
+            }
+            const unsigned src = tmem + (quad << 21) + part;
+#pragma unroll 1
+            for (int g = 0; g < groups; ++g, ++n_grp) {
+                const unsigned d = n_grp & 1u;
+                ok = __all_sync(0xffffffffu, bar_wait(d_full + 8 * d, (n_grp >> 1) & 1u));
+                if (!ok) break;
+                tc_after();
+                if (whole) break;               // (stored from where it is)
+                const unsigned from = src + d * 128;
+#pragma unroll
+                for (int j = 0; j < 64; j += 16) {
+                    if (j >= nr) break;
+                    float t[16];
+                    tmem_ld16(from + j, t);         // (rows past nr: other columns of the accumulators, never stored)
+                    tmem_wait_ld(t);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) (j < 32 ? lo : hi)[(j & 31) + k] += t[k];
+                }
+                tc_before();
+                __syncwarp();
+                if (lane == 0) bar_arrive(d_empty + 8 * d);
+            }
+            if (!ok) break;
+            if (fresh) {
+                // The four warps of a half write the same values.  Whoever has seen the item's last accumulator full knows
+                // that all have stored the item that they stored before the last one, whose copy this is: an accumulator
+                // is full only after the one two before it has been drained, and nobody drains for an item before the
+                // item before it is stored.
+                bias ^= kEpiBytes;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) asm volatile("st.shared.f32 [%0], %1;" ::"r"(bias + (i * 32 + lane) * 4), "f"(b[i]) : "memory");
+                __syncwarp();
+            }
+            const unsigned d = n_grp & 1u;
+            if (whole) tmem_ld32(src + d * 128, lo);
+#pragma unroll 1
+            for (int h = 0; h < nr; h += 32) {
+                if (whole) tmem_wait_ld(lo);
+                const unsigned off = lane_off + (any ? 0 : (unsigned)h * (unsigned)y.hw.d * ye);
+                const int rows = min(32, nr - h);
+                if (wide) store32<float>(lo, y, out, res, off, bias + h * 4, row0 + h, rows, live, any);
+                else store32<XT>(lo, y, out, res, off, bias + h * 4, row0 + h, rows, live, any);
+                __syncwarp();
+                if (whole && h + 32 < nr) {
+                    tmem_ld32(src + d * 128 + h + 32, lo);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) lo[j] = hi[j];
+                }
+            }
+            if (whole) {
+                tc_before();
+                __syncwarp();
+                if (lane == 0) {        // (once more for the half that has no part in it)
+                    bar_arrive(d_empty + 8 * d);
+                    bar_arrive(d_empty + 8 * d);
+                }
+                ++n_grp;
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProdRegs));
+        constexpr int kIssuers = E::group == 1 ? 2 : 1;
+        if (warp >= kMmaWarp && warp < kMmaWarp + kIssuers && elect_one()) {
+            const unsigned me = warp - kMmaWarp;
+            unsigned n_chunk = 0, n_grp = 0, stage = 0, ph = 0, buf = 0, aph = 0;
+            Cursor<L> cur(a);
+#pragma unroll 1
+            while (ok && cur.step()) {
+                const int k16 = cur.t.k16, n = cur.of().n;
+                const unsigned idesc = (1u << 4) | ((unsigned)E::fmt << 7) | ((unsigned)E::fmt << 10) | ((unsigned)(n >> 3) << 17) |
+                                       ((unsigned)(kTcM >> 4) << 24);
+                // shared-memory descriptor of B: K-major, no swizzle; 8 columns x n channels are n * 16
+                // contiguous bytes, so neighbouring column groups are n * 16 and channel groups 128 bytes apart
+                const unsigned long long desc0 = ((unsigned long long)n << 16) | (8ull << 32) | (1ull << 46);
+                const unsigned step = 2u * n;      // in 16-byte units
+                const int nch = (k16 + NS - 1) / NS;
+#pragma unroll 1
+                for (int c = 0; c < nch; ++c, ++n_chunk) {
+                    const bool first = c % E::group == 0, last = (c + 1) % E::group == 0 || c + 1 == nch;
+                    if (kIssuers == 1 || (n_chunk & 1u) == me) {
+                        const int ns = min(NS, k16 - NS * c);
+                        const unsigned d = n_grp & 1u;
+                        ok = (!first || bar_wait(d_empty + 8 * d, ((n_grp >> 1) & 1u) ^ 1u)) && bar_wait(b_full + 8 * stage, ph) &&
+                             bar_wait(a_full + 8 * buf, aph);
+                        // all a chunk needs is there: when the other issuer's chunk has been issued, this one follows it
+                        // without a gap, and whatever surrounds it here costs the tensor cores nothing
+                        if (kIssuers == 2) ok = ok && bar_wait(turn + 8 * me, ((n_chunk >> 1) & 1u) ^ (me ^ 1u));
+                        if (!ok) break;
+                        tc_after();
+                        const unsigned dst = tmem + d * 128, at = tmem_a + buf * AB, plane = step * ns;
+                        const unsigned long long bt = desc0 | ((stage0 + stage * a.stage_bytes) >> 4);
+                        if constexpr (P == 3) {
+                            const int pa[5] = {2, 0, 1, 1, 0}, pb[5] = {0, 2, 1, 0, 1};
+#pragma unroll 1
+                            for (int s = 0; s < ns; ++s)
+#pragma unroll
+                                for (int m = 0; m < 5; ++m)
+                                    mma_f16(dst, at + pa[m] * (KC / 2) + s * 8, bt + pb[m] * plane + s * step, idesc, (s | m) != 0);
+#pragma unroll 1
+                            for (int s = 0; s < ns; ++s) mma_f16(dst, at + s * 8, bt + s * step, idesc, 1u);
+                        } else {
+#pragma unroll 1
+                            for (int s = 0; s < ns; ++s) mma_f16(dst, at + s * 8, bt + s * step, idesc, !(first && s == 0));
+                        }
+                        if (kIssuers == 2) bar_arrive(turn + 8 * (me ^ 1u));
+                        mma_commit(a_empty + 8 * buf);
+                        mma_commit(b_empty + 8 * stage);
+                        if (last) mma_commit(d_full + 8 * d);
+                    }
+                    n_grp += last;
+                    if (++buf == NA) { buf = 0; aph ^= 1u; }
+                    if (++stage == (unsigned)a.stages) { stage = 0; ph ^= 1u; }
+                }
+            }
+        }
+        if (warp >= kProdWarp0 && warp < kProdWarp0 + kProdWarps) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            // every producer copies whole chunks, the block's chunks in turn
+            unsigned n = 0, mine = warp - kProdWarp0;
+            Source<XT, TAPS> src;
+            Cursor<L> cur(a);
+#pragma unroll 1
+            while (ok && cur.step()) {
+                const int k16 = cur.t.k16;
+                const unsigned end = n + (k16 + NS - 1) / NS;
+                if (mine < end) src.open(cur.of(), cur.t, cur.pt(), lane);
+#pragma unroll 1
+                for (; mine < end; mine += kProdWarps) {
+                    const unsigned slot = mine % S;
+                    const int k = (mine - n) * NS;
+                    ok = __all_sync(0xffffffffu, bar_wait(x_empty + 8 * slot, ((mine / S) & 1u) ^ 1u));
+                    if (!ok) break;
+                    src.chunk(ring0 + slot * kSlot, k * 16, min(NS, k16 - k) * 16, lane, x_full + 8 * slot);
+                }
+                n = end;
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        }
+        if (warp == kLoadWarp && elect_one()) {
+            unsigned stage = 0, ph = 0, used = 0;
+            Cursor<L> cur(a);
+#pragma unroll 1
+            while (ok && cur.step()) {
+                const TcLayer& y = cur.of();
+                const TcTile t = cur.t;
+                const unsigned char* src = y.b + (y.tiles ? (size_t)t.b16 * 16 : (size_t)cur.nt() * y.k16 * (32 * P) * y.n);
+#pragma unroll 1
+                for (int k = 0; k < t.k16 && ok; k += NS) {
+                    const unsigned bytes = (unsigned)(min(NS, t.k16 - k) * 16 * y.n * 2 * P);
+                    ok = bar_wait(b_empty + 8 * stage, ph ^ 1u);
+                    if (!ok) break;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b_full + 8 * stage), "r"(bytes) : "memory");
+                    bulk_load(stage0 + stage * a.stage_bytes, src, bytes, b_full + 8 * stage);
+                    src += bytes;
+                    ++used;
+                    if (++stage == (unsigned)a.stages) { stage = 0; ph ^= 1u; }
+                }
+            }
+            if (!ok)        // gave up: see the copies in flight land before shared memory goes away
+#pragma unroll 1
+                for (unsigned i = 0; i < min(used, (unsigned)a.stages); ++i) {
+                    const unsigned at = (stage + a.stages - 1 - i) % a.stages;
+                    (void)bar_wait(b_full + 8 * at, at < stage ? ph : ph ^ 1u);
+                }
+        }
+    }
+    if (!ok)
+#pragma unroll 1
+        for (int l = 0; l < a.n_layers; ++l) atomicExch(a.layer[l].err, warp == kLoadWarp || warp >= kProdWarp0 ? 2 : 1);
+    tc_before();
+    __syncthreads();
+    if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
+
+template <typename XT, bool TAPS, int L>
+cudaError_t launch(const TcArgs<L>& a, int blocks, cudaStream_t st)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)blocks);
+    lc.blockDim = dim3(kThreads);
+    lc.dynamicSmemBytes = kBarBytes + (size_t)a.stages * a.stage_bytes + kTcRingBytes;
+    lc.stream = st;
+    // programmatic dependent launch: set-up overlaps the tail of the kernel before it on the stream
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, tc_kernel<XT, TAPS, L>, a);
+}
+
+template <typename XT, bool TAPS>
+cudaError_t launch_any(const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
+{
+    if (a.n_layers > 1) return launch<XT, TAPS, kTcMaxLayers>(a, blocks, st);
+    TcArgs<1> one;      // (a launch's arguments are copied by the driver: few layers, few bytes)
+    one.n_layers = 1; one.n_items = a.n_items; one.sched = nullptr; one.stages = a.stages; one.stage_bytes = a.stage_bytes;
+    one.layer[0] = a.layer[0];
+    return launch<XT, TAPS, 1>(one, blocks, st);
+}
+
+template <typename XT, bool TAPS>
+cudaError_t prepare()
+{
+    cudaError_t e = cudaFuncSetAttribute(tc_kernel<XT, TAPS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_kernel<XT, TAPS, kTcMaxLayers>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
+    return e;
+}
+
+}  // namespace
+
+cudaError_t launch_tc(int dt, bool taps, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
+{
+    if (taps) return dt == 0 ? launch_any<float, true>(a, blocks, st) : cudaErrorInvalidValue;
+    return dt == 0 ? launch_any<float, false>(a, blocks, st)
+                   : dt == 1 ? launch_any<__half, false>(a, blocks, st) : launch_any<__nv_bfloat16, false>(a, blocks, st);
+}
+
+cudaError_t prepare_tc(int dt, bool taps)
+{
+    if (taps) return dt == 0 ? prepare<float, true>() : cudaErrorInvalidValue;
+    return dt == 0 ? prepare<float, false>() : dt == 1 ? prepare<__half, false>() : prepare<__nv_bfloat16, false>();
+}
+
+}  // namespace alcs

@@ -1,0 +1,89 @@
+// The tensor-core path of the convolutions (fifth-generation tensor cores, tcgen05): launch arguments
+// shared by the kernel (alcs_tc.cu) and the host code that prepares it.
+#ifndef ALCS_TC_H_
+#define ALCS_TC_H_
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace alcs {
+
+constexpr int kTcM = 128;            // pixels per tile = rows of one MMA (TMEM lanes)
+constexpr int kTcMaxN = 128;         // output channels per tile
+constexpr int kTcKC32 = 64, kTcKC16 = 128;      // input columns per pipeline step (chunk): fp32, 16 bits
+constexpr int tc_kc(int dt) { return dt == 0 ? kTcKC32 : kTcKC16; }
+constexpr int kTcHeaderBytes = 3072;     // shared memory in front of the weight stages
+constexpr int kTcMaxLayers = 16;     // layers one launch can take
+
+// One channel tile of a layer: the `n` output channels one work item computes.
+struct TcTile {
+    unsigned b16;      // start of its weight tiles, in 16-byte units from TcLayer::b
+    int k16;           // 16-column steps (0: the tile keeps nothing, output = bias)
+    int kstart;        // start of its column list
+};
+
+// Division of 0 <= n < 2^31 by a fixed d >= 1 as a multiplication: with 2^(s-1) < d <= 2^s and
+// mul = floor(2^(31+s) / d) + 1 the error of n * mul / 2^(31+s) is below n / 2^(31+s) < 1 / d.
+struct TcDiv {
+    unsigned mul, shift;
+    int d;
+};
+inline TcDiv tc_div(int d)
+{
+    unsigned s = 0;
+    while ((1ull << s) < (unsigned long long)d) ++s;
+    return {(unsigned)((1ull << (31 + s)) / (unsigned)d + 1), 31 + s, d};
+}
+
+struct TcLayer {
+    const void* x;
+    void* y;
+    const float* bias;
+    const void* res;
+    const unsigned char* b;      // weight tiles, in the layout the MMA reads from shared memory
+    const TcTile* tiles;         // null: every tile takes k16 steps, the tiles' weights one after the other
+    int k16;
+    const int* cols;             // 1x1: input channel per entry of the tile's column list (null: all channels in order);
+                                 // k x k: {element offset of the column from the pixel's window, tap number} per entry
+    const int* chan;             // output channel of row i of the tiles (null: i itself; -1: padding)
+    int* err;
+    int first_item;              // items of this layer start here
+    TcDiv n_tiles, px_tiles;     // channel tiles, pixel tiles
+    int tile_major;              // item order: 0 = channel tiles of one pixel tile together, 1 = pixel tiles together
+    int n;                       // output channels per tile (a multiple of 16)
+    int q;                       // output pixels, all images
+    TcDiv hw;                    // output pixels per image
+    int cin, cout;
+    int hw_in, w_in, h_in;       // input image
+    TcDiv ow;
+    int stride, pad;
+    int kh, kw;                  // k x k only: tap = r * kw + s
+    int vec_bytes;               // bytes of one copy of X: 16, 8, 4; 0: element by element
+    int ppt;                     // pixels per tile: kTcM, or those of ...
+    int images;                  // ... this many whole images, staged as runs of memory (0: not so)
+    int n_img;
+    int relu, y32;               // y32: fp32 output of 16-bit operands
+};
+
+template <int L>
+struct TcArgs {
+    int n_layers, n_items;
+    const int* sched;            // null: thread block b takes items b, b + grid, ...; else its items are sched[b], sched[b + grid], ... until -1
+    int stages;                  // weight stages in shared memory
+    int stage_bytes;
+    TcLayer layer[L];
+};
+
+// Launch a (n_layers <= kTcMaxLayers; one launch with elements of type dt) on `blocks` thread
+// blocks; taps: k x k convolution (fp32 only).
+cudaError_t launch_tc(int dt, bool taps, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st);
+cudaError_t prepare_tc(int dt, bool taps);      // once per device: shared-memory attribute
+constexpr int tc_planes(int dt) { return dt == 0 ? 3 : 1; }      // 16-bit planes an operand is split into
+// ring of X chunks: 4 of 128 pixels x 64 columns in fp32, x 128 columns in 16 bits
+constexpr int kTcRingBytes = 4 * kTcM * 64 * 4;
+constexpr int tc_stage_bytes(int dt, int n) { return tc_planes(dt) * tc_kc(dt) * n * 2; }
+
+}  // namespace alcs
+
+#endif  // ALCS_TC_H_

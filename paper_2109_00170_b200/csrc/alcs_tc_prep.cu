@@ -1,0 +1,341 @@
+// Host side of the tensor-core path: which output channels form a tile, which columns a tile needs,
+// the expanded weight tiles (built on the device from the storage format) and the launch arguments.
+#include "alcs_tc_prep.h"
+
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cstring>
+#include <new>
+#include <numeric>
+
+namespace alcs {
+void set_cuda_error_text(const char* s);
+
+namespace {
+
+int cuda_fail(cudaError_t e)
+{
+    set_cuda_error_text(cudaGetErrorString(e));
+    (void)cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? ALCS_ERR_ALLOC : ALCS_ERR_CUDA;
+}
+
+// Expand the kept blocks into the weight tiles (zeroed before): tile of n channels, chunks of KC
+// columns, per chunk the planes one after the other, in a plane [8-column group][channel][8 columns]
+// 16-bit values, which is what the MMA's shared-memory descriptor describes.  One warp per block row;
+// `place` is where the row's first channel stands (tile * n + channel inside the tile).
+template <typename T, int P>
+__global__ void expand_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col_idx, const T* __restrict__ vals,
+                              const int* __restrict__ place, const TcTile* __restrict__ tiles, const int* __restrict__ inv,
+                              int rows, int g, int n, int cols, unsigned char* __restrict__ b)
+{
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (r >= rows) return;
+    const int at = place[r], tile = at / n, n0 = at - tile * n;
+    const TcTile t = tiles[tile];
+    unsigned char* const bt = b + (size_t)t.b16 * 16;
+    const int beg = row_ptr[r], cnt = row_ptr[r + 1] - beg;
+    for (int i = threadIdx.x & 31; i < cnt * g; i += 32) {
+        const int blk = i / g, j = i - blk * g;
+        int k = col_idx[beg + blk];
+        if (inv) k = inv[(size_t)tile * cols + k];
+        constexpr int KC = P == 3 ? kTcKC32 : kTcKC16;
+        const int chunk = k / KC, ns = min(KC / 16, t.k16 - KC / 16 * chunk);
+        unsigned char* d = bt + (size_t)chunk * (P * KC * 2) * n + ((size_t)((k % KC) >> 3) * n + n0 + j) * 16 + (k & 7) * 2;
+        const size_t plane = (size_t)ns * 32 * n;
+        const T v = vals[(size_t)beg * g + i];
+        if constexpr (P == 3) {
+            // three bfloat16 parts, rounded to nearest: v = part 0 + part 1 + part 2 exactly
+            __nv_bfloat16 h = __float2bfloat16(v);
+            if (__hisinf(h) && !isinf(v)) h = __float2bfloat16_rz(v);
+            const float rest = v - __bfloat162float(h);
+            const __nv_bfloat16 m = __float2bfloat16(rest);
+            *reinterpret_cast<__nv_bfloat16*>(d) = h;
+            *reinterpret_cast<__nv_bfloat16*>(d + plane) = m;
+            *reinterpret_cast<__nv_bfloat16*>(d + 2 * plane) = __float2bfloat16(rest - __bfloat162float(m));
+        } else {
+            *reinterpret_cast<T*>(d) = v;
+        }
+    }
+}
+
+// Union of the columns that rows order[i0 .. i1) keep, ascending.
+void union_of(const alcs_packed& w, const std::vector<int>& order, int i0, int i1, std::vector<unsigned char>& mark, std::vector<int>& out)
+{
+    out.clear();
+    std::fill(mark.begin(), mark.end(), 0);
+    for (int i = i0; i < i1; ++i)
+        for (int k = w.row_ptr[order[i]]; k < w.row_ptr[order[i] + 1]; ++k) mark[w.col_idx[k]] = 1;
+    for (int c = 0; c < w.cin; ++c)
+        if (mark[c]) out.push_back(c);
+}
+
+struct Layout {
+    std::vector<int> order;
+    std::vector<std::vector<int>> cols;      // per tile
+    long long k16 = 0;
+};
+
+void layout_of(const alcs_packed& w, int rows_per_tile, bool sorted, Layout& L)
+{
+    L.order.resize(w.rows);
+    std::iota(L.order.begin(), L.order.end(), 0);
+    if (sorted)
+        std::stable_sort(L.order.begin(), L.order.end(), [&](int a, int b) {
+            return w.row_ptr[a + 1] - w.row_ptr[a] > w.row_ptr[b + 1] - w.row_ptr[b];
+        });
+    const int tiles = (w.rows + rows_per_tile - 1) / rows_per_tile;
+    L.cols.resize(tiles);
+    std::vector<unsigned char> mark(w.cin);
+    L.k16 = 0;
+    for (int t = 0; t < tiles; ++t) {
+        union_of(w, L.order, t * rows_per_tile, std::min(w.rows, (t + 1) * rows_per_tile), mark, L.cols[t]);
+        L.k16 += (L.cols[t].size() + 15) / 16;
+    }
+}
+
+// Are the rows so unequal that sorting them by length may empty columns of whole tiles?
+bool skewed(const alcs_packed& w)
+{
+    double s = 0, s2 = 0;
+    for (int r = 0; r < w.rows; ++r) {
+        const double c = w.row_ptr[r + 1] - w.row_ptr[r];
+        s += c;
+        s2 += c * c;
+    }
+    const double mean = s / w.rows;
+    return s2 / w.rows - mean * mean > 0.25 * mean * mean + mean;
+}
+
+}  // namespace
+
+TcPrep* tc_find(const alcs_packed* w, const TcKey& key)
+{
+    auto it = w->tc.find({key.n, key.kh, key.kw, key.h, key.wd});
+    return it == w->tc.end() ? nullptr : it->second;
+}
+
+void tc_free(TcPrep* p)
+{
+    if (!p) return;
+    cudaFree(p->b);
+    delete p;
+}
+
+int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep** out)
+{
+    {
+        std::lock_guard<std::mutex> lk(w->mu);
+        if ((*out = tc_find(w, key)) != nullptr) return ALCS_OK;
+    }
+    int rc = canonical_on_device(w, st);
+    if (rc) return rc;
+    {
+        // the shared-memory attribute belongs to the kernel as loaded on a device
+        static std::mutex mu;
+        static bool ready[64][4] = {};
+        std::lock_guard<std::mutex> lk(mu);
+        bool& r = ready[w->device & 63][key.kh ? 3 : (int)w->dt];
+        if (!r) {
+            const cudaError_t e = prepare_tc(w->dt, key.kh > 0);
+            if (e != cudaSuccess) return cuda_fail(e);
+            r = true;
+        }
+    }
+    std::lock_guard<std::mutex> lk(w->mu);
+    if ((*out = tc_find(w, key)) != nullptr) return ALCS_OK;
+    try {
+        const int P = tc_planes(w->dt), n = key.n, rpt = n / w->g;
+        const bool taps = key.kh > 0;
+        const int dense16 = (w->cin + 15) / 16;
+        Layout L;
+        layout_of(*w, rpt, false, L);
+        bool sorted = false;
+        if (skewed(*w)) {
+            Layout S;
+            layout_of(*w, rpt, true, S);
+            if (S.k16 * 20 <= L.k16 * 19) { L = std::move(S); sorted = true; }
+        }
+        const int n_tiles = (int)L.cols.size();
+        // A column list costs the converters its loads: without at least a tenth of the steps to save,
+        // take all columns in order.
+        const bool list = taps || L.k16 * 10 <= (long long)dense16 * n_tiles * 9;
+        std::vector<TcTile> tiles(n_tiles);
+        std::vector<int> cols, inv, chan, place(w->rows);
+        size_t bytes = 0;
+        TcPrep p;
+        p.n = n;
+        p.n_tiles = n_tiles;
+        p.k16_min = 1 << 30;
+        for (int t = 0; t < n_tiles; ++t) {
+            const int used = (int)L.cols[t].size();
+            const int k16 = !list ? (used ? dense16 : 0) : (used + 15) / 16;
+            tiles[t] = {(unsigned)(bytes / 16), k16, (int)(cols.size() / (taps ? 2 : 1))};
+            if (list && used) {
+                const int kk = key.kh * key.kw;
+                for (int i = 0; i < k16 * 16; ++i) {
+                    const int c = L.cols[t][std::min(i, used - 1)];
+                    if (taps) {
+                        const int tap = c % kk, r = tap / key.kw, s = tap % key.kw;
+                        cols.push_back(c / kk * key.h * key.wd + r * key.wd + s);
+                        cols.push_back(tap);
+                    } else {
+                        cols.push_back(c);
+                    }
+                }
+            }
+            if (list) {
+                inv.resize((size_t)(t + 1) * w->cin, 0);
+                for (int i = 0; i < used; ++i) inv[(size_t)t * w->cin + L.cols[t][i]] = i;
+            }
+            bytes += (size_t)P * k16 * 16 * n * 2;
+            p.k16.push_back(k16);
+            p.k16_max = std::max(p.k16_max, k16);
+            p.k16_min = std::min(p.k16_min, k16);
+        }
+        if (bytes / 16 > 0xffffffffull) return ALCS_ERR_SHAPE;
+        for (int i = 0; i < w->rows; ++i) place[L.order[i]] = i / rpt * n + i % rpt * w->g;
+        if (sorted || rpt * w->g != n) {
+            chan.assign((size_t)n_tiles * n, -1);
+            for (int r = 0; r < w->rows; ++r)
+                for (int j = 0; j < w->g; ++j)
+                    if (r * w->g + j < w->cout) chan[place[r] + j] = r * w->g + j;
+        }
+        // one device block: weights, then the small arrays (each on a 256-byte boundary); the inverse
+        // column map and the places are needed by the expansion only
+        auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+        const size_t o_tiles = up(bytes), o_cols = o_tiles + up(tiles.size() * sizeof(TcTile)), o_chan = o_cols + up(cols.size() * 4);
+        const size_t o_place = o_chan + up(chan.size() * 4), o_inv = o_place + up(place.size() * 4), end = o_inv + up(inv.size() * 4);
+        std::vector<unsigned char> small(end - o_tiles);
+        std::memcpy(small.data(), tiles.data(), tiles.size() * sizeof(TcTile));
+        std::memcpy(small.data() + (o_cols - o_tiles), cols.data(), cols.size() * 4);
+        std::memcpy(small.data() + (o_chan - o_tiles), chan.data(), chan.size() * 4);
+        std::memcpy(small.data() + (o_place - o_tiles), place.data(), place.size() * 4);
+        std::memcpy(small.data() + (o_inv - o_tiles), inv.data(), inv.size() * 4);
+        unsigned char* d = nullptr;
+        cudaError_t e = cudaMalloc(&d, std::max<size_t>(end, 256));
+        if (e != cudaSuccess) return cuda_fail(e);
+        e = cudaMemcpyAsync(d + o_tiles, small.data(), small.size(), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess && bytes) e = cudaMemsetAsync(d, 0, bytes, st);
+        if (e == cudaSuccess && w->nb > 0) {
+            const int* dp = reinterpret_cast<const int*>(d + o_place);
+            const int* di = list ? reinterpret_cast<const int*>(d + o_inv) : nullptr;
+            const TcTile* dt = reinterpret_cast<const TcTile*>(d + o_tiles);
+            const unsigned blocks = (unsigned)((w->rows + 3) / 4);
+            if (w->dt == ALCS_F32)
+                expand_kernel<float, 3><<<blocks, 128, 0, st>>>(w->d_row_ptr, w->d_col_idx, static_cast<const float*>(w->d_vals), dp, dt, di,
+                                                               w->rows, w->g, n, w->cin, d);
+            else
+                expand_kernel<unsigned short, 1><<<blocks, 128, 0, st>>>(w->d_row_ptr, w->d_col_idx,
+                                                                        static_cast<const unsigned short*>(w->d_vals), dp, dt, di,
+                                                                        w->rows, w->g, n, w->cin, d);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);      // (the host arrays go away; other streams may use the tiles)
+        if (e != cudaSuccess) {
+            cudaFree(d);
+            return cuda_fail(e);
+        }
+        p.b = d;
+        p.tiles = reinterpret_cast<TcTile*>(d + o_tiles);
+        p.cols = list ? reinterpret_cast<int*>(d + o_cols) : nullptr;
+        p.chan = chan.empty() ? nullptr : reinterpret_cast<int*>(d + o_chan);
+        p.uploaded = true;
+        TcPrep* kept = new TcPrep(p);
+        w->tc[{key.n, key.kh, key.kw, key.h, key.wd}] = kept;
+        *out = kept;
+    } catch (const std::bad_alloc&) {
+        return ALCS_ERR_ALLOC;
+    }
+    return ALCS_OK;
+}
+
+void tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out)
+{
+    TcLayer& y = *out;
+    y.x = p.x; y.y = p.y; y.bias = p.bias; y.res = p.res;
+    y.b = t.b; y.tiles = t.cols || t.k16_min != t.k16_max ? t.tiles : nullptr; y.k16 = t.k16_max; y.cols = t.cols; y.chan = t.chan;
+    y.err = w->d_err;
+    y.hw = tc_div(p.oh * p.ow);
+    y.q = p.n * y.hw.d;
+    y.n_tiles = tc_div(t.n_tiles);
+    
+    // tiles of unequal work: all pixel tiles of the heaviest channel tile first, so that the light ones
+    // fill the end; otherwise the channel tiles of a pixel tile run together and share its reads of X
+    y.tile_major = t.k16_max > t.k16_min + t.k16_min / 4 ? 1 : 0;
+    y.n = t.n;
+    y.cin = p.kh ? w->cin / (p.kh * p.kw) : w->cin;
+    y.cout = w->cout;
+    y.hw_in = p.h_in * p.w_in; y.w_in = p.w_in; y.h_in = p.h_in;
+    y.ow = tc_div(p.ow); y.stride = p.stride; y.pad = p.pad;
+    y.kh = p.kh; y.kw = p.kw;
+    // the widest copy that keeps to one image and to its alignment
+    const int elt = w->dt == ALCS_F32 ? 4 : 2;
+    int vb = 16;
+    while (vb > elt && (p.stride != 1 || p.kh || ((size_t)y.hw.d * elt) % vb || (uintptr_t)p.x % vb)) vb >>= 1;
+    y.vec_bytes = vb == 16 || (elt == 2 && vb > elt) ? vb : 0;      // (8 bytes of fp32: as single elements)
+    // Small images whose rows do not start on copy boundaries (7x7): a tile takes whole images, of which the
+    // columns of a chunk are one run of memory, if those runs keep to 16 bytes
+    y.n_img = p.n;
+    y.images = 0;
+    if (y.vec_bytes == 0 && !p.kh && p.stride == 1 && !t.cols && y.hw.d <= kTcM && (uintptr_t)p.x % 16 == 0 &&
+        (size_t)y.cin * y.hw.d * elt % 16 == 0 && (size_t)16 * y.hw.d * elt % 16 == 0 && y.cin % 16 == 0)
+        y.images = kTcM / y.hw.d;
+    y.ppt = y.images ? y.images * y.hw.d : kTcM;
+    y.px_tiles = tc_div((y.q + y.ppt - 1) / y.ppt);
+    y.relu = (p.flags & ALCS_RELU) ? 1 : 0;
+    y.y32 = (p.flags & ALCS_Y_F32) ? 1 : 0;
+}
+
+// How long one item takes, in microseconds, by type, channels per tile and 16-column steps: per chunk the MMAs
+// (24 of n / 2 cycles in fp32; the tensor cores run at about 1.55 GHz under that load) or the staging and
+// conversion of X, whichever is longer, plus the part of the store that nothing overlaps.  Measured: 1.33 / 1.03 /
+// 0.95 us per fp32 chunk at n = 128 / 64 / 32.
+double tc_item_us(int dt, int n, int k16)
+{
+    const int nch = (k16 * 16 + tc_kc(dt) - 1) / tc_kc(dt);
+    const double chunk = dt == ALCS_F32 ? std::max(0.95, 0.1 + 0.0096 * n) : std::max(0.9, 0.3 + 0.006 * n);
+    return nch * chunk + 0.3 + 0.005 * n;
+}
+
+// Number items and choose the ring depth for the a.n_layers layers filled in.
+int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a)
+{
+    int sms = 0, smem = 0;
+    const int rc = device_limits(w->device, &sms, &smem);
+    if (rc) return rc;
+    int n = 16;
+    long long items = 0;
+    for (int i = 0; i < a.n_layers; ++i) {
+        a.layer[i].first_item = (int)items;
+        items += (long long)a.layer[i].n_tiles.d * a.layer[i].px_tiles.d;
+        n = std::max(n, a.layer[i].n);
+    }
+    if (items > 0x7fffffffll) return ALCS_ERR_SHAPE;
+    a.n_items = (int)items;
+    a.sched = nullptr;
+    a.stage_bytes = tc_stage_bytes(w->dt, n);
+    // (an even number: of two MMA issuers each then always meets the same stages)
+    a.stages = ~1 & std::min(8, (std::min(smem, 227 * 1024) - kTcHeaderBytes - kTcRingBytes) / a.stage_bytes);
+    return a.stages >= 2 ? ALCS_OK : ALCS_ERR_UNSUPPORTED;
+}
+
+int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool taps, cudaStream_t st)
+{
+    int sms = 0, smem = 0;
+    const int rc = device_limits(w->device, &sms, &smem);
+    if (rc) return rc;
+    const cudaError_t e = launch_tc(w->dt, taps, a, std::min(a.n_items, sms), st);
+    return e == cudaSuccess ? ALCS_OK : cuda_fail(e);
+}
+
+// 32-bit arithmetic of the kernel: element offsets into X, byte offsets inside the images one tile touches.
+bool tc_fits(int cin, int cout, long long n, long long hw_in, long long hw, int k)
+{
+    return n * hw_in * cin < (1ll << 31) - 4096 && ((long long)kTcM / std::max(1ll, hw) + 2) * hw * cout * 4 < (1ll << 32) &&
+           (long long)cin * k < (1 << 20) && n * hw <= (1ll << 30);
+}
+
+}  // namespace alcs

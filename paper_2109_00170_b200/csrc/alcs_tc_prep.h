@@ -1,0 +1,48 @@
+// Host side of the tensor-core path (alcs_tc_prep.cu): channel tiles, expanded weights, launch arguments.
+#ifndef ALCS_TC_PREP_H_
+#define ALCS_TC_PREP_H_
+
+#include <vector>
+
+#include "alcs_internal.h"
+#include "alcs_tc.h"
+
+namespace alcs {
+
+// What the expanded weights depend on: channels per tile and, for k x k kernels (kh > 0), the image
+// and kernel sizes the columns' element offsets are computed from.
+struct TcKey {
+    int n, kh, kw, h, wd;
+};
+
+struct TcPrep {
+    int n = 0, n_tiles = 0;
+    std::vector<int> k16;        // steps of each tile
+    int k16_max = 0, k16_min = 0;
+    bool uploaded = false;
+    // device; one allocation, `b` first
+    unsigned char* b = nullptr;
+    TcTile* tiles = nullptr;
+    int* cols = nullptr;         // null: every tile takes all columns in order
+    int* chan = nullptr;         // null: identity
+};
+
+// The problem a launch solves (one layer), everything but the weights.
+struct TcProblem {
+    const void* x; void* y; const float* bias; const void* res;
+    int n, oh, ow, h_in, w_in, stride, pad, kh, kw;      // kh = 0: pointwise
+    unsigned flags;
+};
+
+int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep** out);
+TcPrep* tc_find(const alcs_packed* w, const TcKey& key);       // already prepared, or null; caller holds w->mu
+void tc_free(TcPrep* p);
+void tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out);
+double tc_item_us(int dt, int n, int k16);
+int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a);
+int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool taps, cudaStream_t st);
+bool tc_fits(int cin, int cout, long long n, long long hw_in, long long hw, int k);
+
+}  // namespace alcs
+
+#endif  // ALCS_TC_PREP_H_
