@@ -8,6 +8,7 @@
 #include <new>
 
 #include "alcs_internal.h"
+#include "alcs_tc_prep.h"
 
 namespace alcs {
 void set_cuda_error_text(const char* s);
@@ -283,6 +284,10 @@ extern "C" ALCS_API int alcs_spconv2d_cfg(const alcs_packed* w, const void* x, v
     if (rc) return rc;
     if (n == 0) return ALCS_OK;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (!cfg) {     // the tcgen05 kernel, unless its patches do not fit shared memory (or cannot be copied by words)
+        rc = alcs::tc_conv2d(w, {x, y, bias, nullptr, n, g.oh, g.ow, h, wd, stride, pad, kh, kw, flags}, st);
+        if (rc != ALCS_ERR_UNSUPPORTED) return rc;
+    }
     int sms = 0, smem_optin = 0;
     rc = alcs::device_limits(w->device, &sms, &smem_optin);
     if (rc) return rc;

@@ -345,6 +345,8 @@ constexpr size_t kFinalists = 12;
 // Internal flag, only ever seen in plan-cache keys: the call has a residual operand or a stride, which
 // the small-problem kernel does not take, so only the staged kernels are listed.
 constexpr unsigned kStagedOnly = 0x10000u;
+// Another one: a strided input that the tcgen05 kernel cannot stage.
+constexpr unsigned kNoTc = 0x20000u;
 
 int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>& out, bool allow_small = true)
 {
@@ -481,15 +483,13 @@ void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
 }
 
 // Resolve a (possibly partial) configuration into a concrete plan.
-int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg* c, Plan* out, bool allow_small = true, long long hw_in = 0)
+int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg* c, Plan* out, bool allow_small = true, long long hw_in = 0, bool allow_tc = true)
 {
     if (hw_in < hw) hw_in = hw;
     DeviceInfo di;
     int rc = device_info(w->device, &di);
     if (rc) return rc;
-    // (strided inputs are staged element by element by the tcgen05 kernel: 135 us against 90 for 256 -> 512 channels,
-    // 56 x 56 at stride 2, batch 32, so it takes them only when asked to)
-    if (hw > 0 && ((!c && hw_in == hw) || (c && c->math_mode == 4)) && alcs::tc_fits(w->cin, w->cout, q / hw, hw_in, hw, 1)) {
+    if (hw > 0 && allow_tc && (!c || c->math_mode == 4) && alcs::tc_fits(w->cin, w->cout, q / hw, hw_in, hw, 1)) {
         if (c) {        // the tcgen05 kernel as asked for: row_groups channel tiles
             const int tiles = c->row_groups ? c->row_groups : tc_best(w, q, di.sms).n_rg;
             const int n = ((w->cout + std::max(1, tiles) - 1) / std::max(1, tiles) + 15) / 16 * 16;
@@ -780,24 +780,28 @@ int launch_gather_plan(const alcs_packed* w, const Plan& p, const void* x, void*
 alcs::TcProblem tc_problem(const void* x, void* y, int n, int h, int wd, const float* bias, unsigned flags, const void* residual, int stride,
                            int h_in, int wd_in)
 {
-    return {x, y, bias, residual, n, h, wd, h_in, wd_in, stride, 0, 0, 0, flags};
+    const int k = stride > 1 ? 1 : 0;
+    return {x, y, bias, residual, n, h, wd, h_in, wd_in, stride, 0, k, k, flags};
 }
 
-// Launch the tcgen05 kernel for one layer whose weights are prepared.
-int launch_tc_prepared(const alcs_packed* w, const alcs::TcPrep& t, const alcs::TcProblem& p, cudaStream_t st)
+alcs::TcKey tc_key(const Plan& p, int stride)
 {
-    alcs::TcArgs<alcs::kTcMaxLayers> a;
-    a.n_layers = 1;
-    alcs::tc_fill(w, t, p, &a.layer[0]);
-    const int rc = alcs::tc_finish(w, a);
-    return rc ? rc : alcs::tc_launch(w, a, false, st);
+    const int k = stride > 1 ? 1 : 0;
+    return {p.tc_n, k, k};
 }
 
+// Can the tcgen05 kernel take a strided layer (whatever the channels per tile)?
+bool tc_strided_ok(const alcs_packed* w, const void* x, int n, int oh, int ow, int stride, int h_in, int wd_in)
+{
+    return alcs::tc_patch_fits(w, tc_problem(x, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
+}
+
+// Launch the tcgen05 kernel for one layer; strided layers run by patch staging.
 int launch_tc_plan(const alcs_packed* w, const Plan& p, const alcs::TcProblem& pr, cudaStream_t st)
 {
     alcs::TcPrep* t = nullptr;
-    const int rc = alcs::tc_prepare(w, {p.tc_n, 0, 0, 0, 0}, st, &t);
-    return rc ? rc : launch_tc_prepared(w, *t, pr, st);
+    const int rc = alcs::tc_prepare(w, tc_key(p, pr.stride), st, &t);
+    return rc ? rc : alcs::tc_run(w, *t, pr, st);
 }
 
 // scratch / scratch_bytes: where X is repacked when its rows are not 16-byte multiples.  nullptr means
@@ -943,10 +947,11 @@ int resolve_plan(const alcs_packed* w, int n, int h, int wd, unsigned flags, lon
     }
     const alcs_launch_cfg* use = cfg;
     if (!use) {     // a configuration tuned or set for the shape (stored under the public flags)
-        auto it = w->tuned.find(alcs::ShapeKey{n, h, wd, flags & ~kStagedOnly});
-        if (it != w->tuned.end() && !((flags & kStagedOnly) && it->second.math_mode == 3)) use = &it->second;
+        auto it = w->tuned.find(alcs::ShapeKey{n, h, wd, flags & ~(kStagedOnly | kNoTc)});
+        if (it != w->tuned.end() && !((flags & kStagedOnly) && it->second.math_mode == 3) &&
+            !((flags & kNoTc) && it->second.math_mode == 4)) use = &it->second;
     }
-    const int rc = cfg_to_plan(w, q, h * wd, use, plan, !(flags & kStagedOnly), hw_in);
+    const int rc = cfg_to_plan(w, q, h * wd, use, plan, !(flags & kStagedOnly), hw_in, !(flags & kNoTc));
     if (rc) return rc;
     std::lock_guard<std::mutex> lk(w->mu);
     w->plan_cache[key] = *plan;
@@ -1152,7 +1157,8 @@ ALCS_API int alcs_spconv1x1_ex(const alcs_packed* w, const void* x, void* y, int
         if (rb < yend && yb < rend) return ALCS_ERR_INVALID_ARG;     // the residual may not overlap y
     }
     Plan plan;
-    rc = resolve_plan(w, n, oh, ow, flags | kStagedOnly, q, cfg, &plan, (long long)h * wd);
+    const bool tc = stride == 1 || tc_strided_ok(w, x, n, oh, ow, stride, h, wd);
+    rc = resolve_plan(w, n, oh, ow, flags | kStagedOnly | (tc ? 0u : kNoTc), q, cfg, &plan, (long long)h * wd);
     if (rc) return rc;
     return launch_plan(w, plan, x, y, n, oh, ow, bias, flags, static_cast<cudaStream_t>(cuda_stream), nullptr, 0,
                        residual, stride, h, wd);
@@ -1452,7 +1458,7 @@ int stack_make_resident(alcs_stack* s)
             rc = ensure_canonical_on_device(w, nullptr);
         } else if (it.plan.tc_n) {
             alcs::TcPrep* t = nullptr;
-            rc = alcs::tc_prepare(w, {it.plan.tc_n, 0, 0, 0, 0}, nullptr, &t);
+            rc = alcs::tc_prepare(w, tc_key(it.plan, it.layer.stride), nullptr, &t);
         } else {
             Schedule* sc = get_schedule(w, it.plan.kc, it.plan.n_rg, true, flavour_of(g_variants[it.plan.variant].v));
             rc = sc ? upload_schedule(w, sc, nullptr) : ALCS_ERR_ALLOC;
@@ -1516,12 +1522,12 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
     for (int i = 0; i < run.count; ++i) {
         const auto& it = s->items[first + i];
         alcs::TcPrep* t = nullptr;
-        rc = alcs::tc_prepare(it.layer.w, {it.plan.tc_n, 0, 0, 0, 0}, nullptr, &t);
+        rc = alcs::tc_prepare(it.layer.w, {it.plan.tc_n, 0, 0}, nullptr, &t);
         if (rc) return rc;
         alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
         for (int k16 : t->k16) us[i].push_back(alcs::tc_item_us(it.layer.w->dt, t->n, k16));
     }
-    rc = alcs::tc_finish(w0, a);
+    rc = alcs::tc_finish(w0, a, false);
     if (rc) return rc;
     if (run.count > 1) {
         const int blocks = std::min(a.n_items, di.sms);
@@ -1568,7 +1574,7 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
 int build_runs(alcs_stack* s)
 {
     drop_runs(s);
-    auto on_tc = [](const alcs_stack::Item& it) { return it.plan.tc_n != 0; };
+    auto on_tc = [](const alcs_stack::Item& it) { return it.plan.tc_n != 0 && it.layer.stride <= 1; };
     for (size_t i = 0; i < s->items.size();) {
         if (s->items[i].q == 0) { ++i; continue; }
         const size_t end = merge_end(s, i, on_tc);
@@ -1613,7 +1619,8 @@ ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned 
         it.ow = (L.wd + stride - 1) / stride;
         int rc = check_conv_args(L.w, L.x, L.y, L.n, it.oh, it.ow, L.flags, &it.q);
         if (!rc) rc = check_device(L.w);
-        if (!rc && it.q > 0) rc = resolve_plan(L.w, L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u), it.q, nullptr, &it.plan, (long long)L.h * L.wd);
+        const bool tc = !rc && it.q > 0 && (stride == 1 || tc_strided_ok(L.w, L.x, L.n, it.oh, it.ow, stride, L.h, L.wd));
+        if (!rc && it.q > 0) rc = resolve_plan(L.w, L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u) | (tc ? 0u : kNoTc), it.q, nullptr, &it.plan, (long long)L.h * L.wd);
         if (rc) { delete s; return rc; }
         s->items.push_back(it);
     }
@@ -1724,7 +1731,7 @@ int stack_candidates(const alcs_stack::Item& it, std::vector<Plan>& out)
         auto f = L.w->finalists.find(alcs::ShapeKey{L.n, it.oh, it.ow, L.flags});
         if (f != L.w->finalists.end())
             for (const Plan& p : f->second)
-                if (!(extra && p.gather)) out.push_back(p);
+                if (!(extra && p.gather) && !(L.stride > 1 && p.tc_n)) out.push_back(p);
     }
     const bool had = !out.empty();
     const bool small = !extra && it.oh * it.ow > 0 && it.q / ((long long)it.oh * it.ow) <= 8;
@@ -1733,7 +1740,7 @@ int stack_candidates(const alcs_stack::Item& it, std::vector<Plan>& out)
     const int rc = enumerate_plans(L.w, it.q, it.oh * it.ow, all, !extra);
     if (rc) return rc;
     for (size_t i = 0; i < all.size(); ++i) {
-        if (!((!had && i < 8) || all[i].gather)) continue;
+        if (!((!had && i < 8) || all[i].gather) || (L.stride > 1 && all[i].tc_n)) continue;
         bool dup = false;
         for (const Plan& p : out) dup |= same_plan(p, all[i]);
         if (!dup) out.push_back(all[i]);
@@ -1895,8 +1902,8 @@ extern "C" ALCS_API int alcs_spconv1x1_noalloc(const alcs_packed* w, const void*
         if (plan.tc_n) {        // needs no scratch, but what does not fit it is refused whatever kernel the plan names
             const size_t row = (size_t)h * wd * w->elt();
             if (row % 16 != 0 && (size_t)n * w->cin * ((row + 15) / 16 * 16) > ALCS_NOALLOC_SCRATCH_BYTES) return ALCS_ERR_TOO_LARGE;
-            const alcs::TcPrep* t = alcs::tc_find(w, {plan.tc_n, 0, 0, 0, 0});
-            return t ? launch_tc_prepared(w, *t, tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd), st) : ALCS_ERR_STATE;
+            const alcs::TcPrep* t = alcs::tc_find(w, {plan.tc_n, 0, 0});
+            return t ? alcs::tc_run(w, *t, tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd), st) : ALCS_ERR_STATE;
         }
         auto si = w->sched.find(alcs::sched_key(plan.kc, plan.n_rg, flavour_of(g_variants[plan.variant].v)));
         if (si == w->sched.end() || !si->second.uploaded) return ALCS_ERR_STATE;

@@ -130,8 +130,8 @@ struct alcs_packed {
     // plane, plane pitch, stride, kh, kw, channels per chunk}: the column offsets baked into them depend
     // on the geometry
     mutable std::map<std::array<int, 8>, alcs::Schedule> sched2d;
-    // expanded weights of the tcgen05 kernel, by {channels per tile, kh, kw, h, wd} (alcs_tc_prep.h)
-    mutable std::map<std::array<int, 5>, alcs::TcPrep*> tc;
+    // expanded weights of the tcgen05 kernel, by {channels per tile, kh, kw} (alcs_tc_prep.h)
+    mutable std::map<std::array<int, 3>, alcs::TcPrep*> tc;
     mutable std::map<alcs::ShapeKey, alcs_launch_cfg> tuned;   // filled by alcs_spconv1x1_tune, alcs_spconv1x1_set_cfg, alcs_stack_tune
     // the best few plans of the last alcs_spconv1x1_tune per shape, best first: what alcs_stack_tune tries in context
     mutable std::map<alcs::ShapeKey, std::vector<alcs::Plan>> finalists;

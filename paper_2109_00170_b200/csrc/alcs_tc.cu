@@ -250,36 +250,20 @@ __device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigne
 }
 
 // Where a producer warp finds the pixels of one item.
-template <typename XT, bool TAPS>
+template <typename XT>
 struct Source {
     using raw = typename Elem<XT>::raw;
     static constexpr int kRow = kTcM * (int)sizeof(raw);      // bytes of a column of a chunk in shared memory
     const raw* x;
     const int* cols;
     int off[4];                    // element offset of this lane's first column entry: [0] alone for vector copies
-    unsigned mask[TAPS ? 4 : 1];   // TAPS: which taps of the pixel lie inside the image
     int hw_in, cin, vb;
     int img0, n_img = 0, hw;       // whole images (TcLayer::images): first, how many, pixels
 
-    __device__ __forceinline__ int pixel(const TcLayer& y, int q, unsigned& m) const
+    __device__ __forceinline__ int pixel(const TcLayer& y, int q) const
     {
-        const int img = div_of(q, y.hw), p = q - img * y.hw.d;
-        const int img_off = img * cin * hw_in;
-        if (TAPS) {
-            const int oy = div_of(p, y.ow), ox = p - oy * y.ow.d;
-            const int ih = oy * y.stride - y.pad, iw = ox * y.stride - y.pad;
-            unsigned row = 0;
-            m = 0;
-#pragma unroll 1
-            for (int s = 0; s < y.kw; ++s) row |= ((unsigned)(iw + s) < (unsigned)y.w_in ? 1u : 0u) << s;
-#pragma unroll 1
-            for (int r = 0; r < y.kh; ++r)
-                if ((unsigned)(ih + r) < (unsigned)y.h_in) m |= row << (r * y.kw);
-            return img_off + ih * y.w_in + iw;
-        }
-        if (y.stride == 1) return img_off + p;
-        const int oy = div_of(p, y.ow);
-        return img_off + oy * y.stride * y.w_in + (p - oy * y.ow.d) * y.stride;
+        const int img = div_of(q, y.hw);
+        return img * cin * hw_in + (q - img * y.hw.d);
     }
 
     __device__ __forceinline__ void open(const TcLayer& y, const TcTile& t, int pt, int lane)
@@ -288,19 +272,19 @@ struct Source {
         hw_in = y.hw_in;
         cin = y.cin;
         vb = y.vec_bytes;
-        cols = TAPS ? y.cols + 2 * (size_t)t.kstart : y.cols ? y.cols + t.kstart : nullptr;
+        cols = y.cols ? y.cols + t.kstart : nullptr;
         // (pixels past the end repeat the last ones and are not stored)
-        if (!TAPS && y.images) {
+        if (y.images) {
             img0 = pt * y.images;
             n_img = min(y.images, y.n_img - img0);
             hw = y.hw.d;
-        } else if (!TAPS && vb) {
+        } else if (vb) {
             const int ppl = vb / (int)sizeof(raw);      // pixels per copy; a column's 128 pixels take 128 / ppl copies
-            off[0] = pixel(y, min(pt * y.ppt + (lane * ppl & (kTcM - 1)), y.q - ppl), mask[0]);
-            if (vb == 4) off[1] = pixel(y, min(pt * y.ppt + 64 + (lane * ppl & 63), y.q - ppl), mask[0]);
+            off[0] = pixel(y, min(pt * y.ppt + (lane * ppl & (kTcM - 1)), y.q - ppl));
+            if (vb == 4) off[1] = pixel(y, min(pt * y.ppt + 64 + (lane * ppl & 63), y.q - ppl));
         } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) off[j] = pixel(y, min(pt * y.ppt + j * 32 + lane, y.q - 1), mask[TAPS ? j : 0]);
+            for (int j = 0; j < 4; ++j) off[j] = pixel(y, min(pt * y.ppt + j * 32 + lane, y.q - 1));
         }
     }
 
@@ -320,7 +304,7 @@ struct Source {
     // Copy the chunk that starts at column k0 (kk columns, a multiple of 16) into `slot`; one arrival per lane on `bar`.
     __device__ __forceinline__ void chunk(unsigned slot, int k0, int kk, int lane, unsigned bar) const
     {
-        if (!TAPS && n_img) {
+        if (n_img) {
             // whole small images: the chunk's columns of an image are one run of memory
             if (lane == 0) {
                 const unsigned bytes = (unsigned)(kk * hw) * (unsigned)sizeof(raw);
@@ -333,20 +317,9 @@ struct Source {
             bar_arrive(bar);
             return;
         }
-        slot += lane * (TAPS || vb == 0 ? (int)sizeof(raw) : vb);
+        slot += lane * (vb == 0 ? (int)sizeof(raw) : vb);
 #pragma unroll 1
         for (int k = 0; k < kk; k += 4, slot += 4 * kRow) {
-            if constexpr (TAPS) {
-                const int4 c0 = __ldg(reinterpret_cast<const int4*>(cols + 2 * (k0 + k))), c1 = __ldg(reinterpret_cast<const int4*>(cols + 2 * (k0 + k)) + 1);
-                const int at[4] = {c0.x, c0.z, c1.x, c1.z}, tap[4] = {c0.y, c0.w, c1.y, c1.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool in = (mask[j] >> tap[i]) & 1u;
-                        cp_async_small<4>(slot + i * kRow + j * 128, in ? x + (off[j] + at[i]) : x, in ? 4 : 0);
-                    }
-            } else {
                 const int4 c = cols4(k0 + k);
                 const int at[4] = {c.x, c.y, c.z, c.w};
                 if (vb == 16) {
@@ -382,12 +355,74 @@ struct Source {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) st_slot(slot + i * kRow + j * 64, v[i][j]);
                 }
-            }
         }
         if (sizeof(raw) == 2 && vb == 0) bar_arrive(bar);
         else cp_async_arrive(bar);
     }
 };
+
+// The input rows a tile of consecutive output pixels needs, by patch staging: the tile touches images img0 .. ; of
+// each, rows first .. of every channel lie one after the other in the slot.
+struct Patch {
+    int img0, n_img;
+    int y0, first0, rows0;         // of the first image (y0: its first output row here)
+    int rows, rows_last;           // of a whole image, and of the last one (if it is not the first)
+
+    __device__ __forceinline__ Patch(const TcLayer& y, int pt)
+    {
+        const int q0 = pt * y.ppt, q1 = min(q0 + kTcM, y.q) - 1;
+        img0 = div_of(q0, y.hw);
+        n_img = div_of(q1, y.hw) - img0 + 1;
+        y0 = div_of(q0 - img0 * y.hw.d, y.ow);
+        const int y1 = div_of(q1 - (img0 + n_img - 1) * y.hw.d, y.ow);
+        first0 = max(0, y0 * y.stride - y.pad);
+        rows0 = count(y, first0, n_img > 1 ? y.oh - 1 : y1);
+        rows = count(y, 0, y.oh - 1);
+        rows_last = count(y, 0, y1);
+    }
+    // input rows from `first` to the last one that output row `last` needs
+    static __device__ __forceinline__ int count(const TcLayer& y, int first, int last)
+    {
+        const int n = min(y.h_in - 1, last * y.stride - y.pad + y.kh - 1) - first;
+        return max(0, y.row_step == 1 ? n + 1 : last - first / y.stride + 1);
+    }
+};
+
+// Copy one slot of patches: channels c0 .. c0 + nc, all images of the tile.
+template <typename XT>
+__device__ __forceinline__ void copy_patch(const TcLayer& y, const Patch& t, unsigned slot, int c0, int nc, int lane, unsigned bar)
+{
+    using raw = typename Elem<XT>::raw;
+    const int vb = y.vec_bytes, epv = vb / (int)sizeof(raw);
+    const raw* const x = static_cast<const raw*>(y.x);
+    const unsigned pitch = y.pitch * (unsigned)sizeof(raw);
+#pragma unroll 1
+    for (int i = 0; i < t.n_img; ++i) {
+        const int rows = i == 0 ? t.rows0 : i + 1 == t.n_img ? t.rows_last : t.rows;
+        const raw* const src = x + (((t.img0 + i) * y.cin + c0) * y.hw_in + (i == 0 ? t.first0 : 0) * y.w_in);
+        const int pieces = rows * y.w_vec.d;
+#pragma unroll 1
+        for (int p = lane; p < pieces; p += 32) {
+            int at = p * epv;
+            if (y.row_step != 1) {
+                const int r = div_of(p, y.w_vec);
+                at += r * (y.row_step - 1) * y.w_in;
+            }
+            const raw* from = src + at;
+            unsigned to = slot + p * vb;
+#pragma unroll 4
+            for (int c = 0; c < nc; ++c) {
+                if (vb == 16) cp_async16(to, from);
+                else if (vb == 8) cp_async_small<8>(to, from, 8);
+                else cp_async_small<4>(to, from, 4);
+                to += pitch;
+                from += y.hw_in;
+            }
+        }
+        slot += rows * y.w_in * (unsigned)sizeof(raw);
+    }
+    cp_async_arrive(bar);
+}
 
 __device__ __forceinline__ void ld_slot(unsigned addr, float& v) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr)); }
 __device__ __forceinline__ void ld_slot(unsigned addr, unsigned short& v) { asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr)); }
@@ -469,7 +504,7 @@ __device__ __forceinline__ void store_bias(const TcLayer& y, char* out, const ch
     }
 }
 
-template <typename XT, bool TAPS, int L>
+template <typename XT, bool PATCH, int L>
 __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__ TcArgs<L> a)
 {
     using E = Elem<XT>;
@@ -481,8 +516,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     const unsigned b_full = s0 + 256, b_empty = s0 + 320, turn = s0 + 384, tmem_slot = s0 + 400;
     const unsigned stage0 = s0 + kBarBytes, ring0 = stage0 + a.stages * a.stage_bytes;
     constexpr int NA = E::abufs, KC = P == 3 ? kTcKC32 : kTcKC16, NS = KC / 16, AB = KC / 2 * P;      // AB: TMEM columns of a chunk of A
-    constexpr int S = kProdWarps, kSlot = KC * kTcM * (int)sizeof(raw);      // (every producer owns a slot)
-    static_assert(S * kSlot == kTcRingBytes && NA * AB <= 256, "ring and A buffers");
+    // every producer owns a slot
+    const unsigned S = PATCH ? (unsigned)a.slots : (unsigned)kProdWarps, kSlot = PATCH ? (unsigned)a.slot_bytes : KC * kTcM * (unsigned)sizeof(raw);
+    static_assert(kProdWarps * KC * kTcM * (int)sizeof(raw) == kTcRingBytes && NA * AB <= 256, "ring and A buffers");
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -507,7 +543,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             bar_init(b_empty + 8 * i, 1);
         }
 #pragma unroll 1
-        for (int i = 0; i < S; ++i) {
+        for (int i = 0; i < kProdWarps; ++i) {
             bar_init(x_full + 8 * i, 32);
             bar_init(x_empty + 8 * i, kConvWarps);
         }
@@ -526,34 +562,81 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConvRegs));
         const unsigned quad = (unsigned)(warp & 3);
         const int s0_ = warp >> 2, row = quad * 32 + lane;       // a warp takes every fourth 16-column step
-        unsigned i = 0, buf = 0, aph = 1;
+        unsigned i = 0, slot = 0, xph = 0, buf = 0, aph = 1;
+        bool opened = false;            // PATCH: whether the slot in use has been waited for
         Cursor<L> cur(a);
 #pragma unroll 1
         while (ok && cur.step()) {
-            const int images = cur.of().images;
+            const TcLayer& y = cur.of();
+            const int images = PATCH ? 0 : y.images;
             int hw = kTcM, img = 0, px = row;
-            if (images) {
-                hw = cur.of().hw.d;
-                img = min(div_of(row, cur.of().hw), images - 1);
+            // PATCH: this pixel's window in the patch, which taps of it lie inside the image, and the walk over the steps
+            int block = 0, tap = s0_, in_slot = 0;
+            unsigned mask = 0;
+            if constexpr (PATCH) {
+                const Patch t(y, cur.pt());
+                const int q = min(cur.pt() * y.ppt + row, y.q - 1);
+                img = div_of(q, y.hw);
+                const int p = q - img * y.hw.d, oy = div_of(p, y.ow), ox = p - oy * y.ow.d;
+                const int ih = oy * y.stride - y.pad, iw = ox * y.stride - y.pad, seg = img - t.img0;
+                unsigned bits = 0;
+#pragma unroll 1
+                for (int s = 0; s < y.kw; ++s) bits |= ((unsigned)(iw + s) < (unsigned)y.w_in ? 1u : 0u) << s;
+#pragma unroll 1
+                for (int r = 0; r < y.kh; ++r)
+                    if ((unsigned)(ih + r) < (unsigned)y.h_in) mask |= bits << (r * y.kw);
+                const int line = y.row_step == 1 ? ih - (seg ? 0 : t.first0) : oy - (seg ? 0 : t.y0);
+                px = ((seg ? t.rows0 + (seg - 1) * t.rows : 0) + line) * y.w_in + iw;
+            } else if (images) {
+                hw = y.hw.d;
+                img = min(div_of(row, y.hw), images - 1);
                 px = min(row - img * hw, hw - 1);
             }
 #pragma unroll 1
             for (int k16 = cur.t.k16; k16 > 0; k16 -= NS, ++i) {
-                const unsigned slot = i % S, my_a = tmem_a + (quad << 21) + buf * AB;      // lanes 32 * quad ...
+                const unsigned my_a = tmem_a + (quad << 21) + buf * AB;      // lanes 32 * quad ...
                 const int ns = min(NS, k16);
-                const unsigned src = ring0 + slot * kSlot + (img * ns * 16 * hw + px) * (unsigned)sizeof(raw);
-                ok = __all_sync(0xffffffffu, bar_wait(x_full + 8 * slot, (i / S) & 1u) && bar_wait(a_empty + 8 * buf, aph));
+                ok = (PATCH || bar_wait(x_full + 8 * slot, xph)) && bar_wait(a_empty + 8 * buf, aph);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_after();
 #pragma unroll 1
                 for (int s = s0_; s < ns; s += 4) {
                     raw v[16];
-                    if (images) {
-                        const unsigned at = src + s * 16 * hw * (unsigned)sizeof(raw);
+                    if constexpr (PATCH) {
+                        while (tap >= y.taps.d) { tap -= y.taps.d; ++block; ++in_slot; }
+                        // on to the slot that holds the block; every slot is waited for and given back in turn
+                        while (in_slot >= y.blocks || !opened) {
+                            if (in_slot >= y.blocks) {
+                                in_slot -= y.blocks;
+                                if (!opened) ok = ok && bar_wait(x_full + 8 * slot, xph);
+                                __syncwarp();
+                                if (lane == 0) bar_arrive(x_empty + 8 * slot);
+                                if (++slot == S) { slot = 0; xph ^= 1u; }
+                                opened = false;
+                            } else {
+                                ok = ok && bar_wait(x_full + 8 * slot, xph);
+                                opened = true;
+                            }
+                        }
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                        const int r = div_of(tap, y.kwd), nv = y.cin - block * 16;
+                        const bool in = (mask >> tap) & 1u;
+                        const int pitch = y.pitch * (int)sizeof(raw);
+                        const unsigned at = ring0 + slot * kSlot + in_slot * 16 * pitch + (px + r * y.w_in + (tap - r * y.kw)) * (int)sizeof(raw);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            v[j] = raw(0);
+                            if (in && j < nv) ld_slot(at + j * pitch, v[j]);
+                        }
+                        tap += 4;
+                    } else if (images) {
+                        const unsigned at = ring0 + slot * kSlot + ((img * ns + s) * 16 * hw + px) * (unsigned)sizeof(raw);
 #pragma unroll
                         for (int j = 0; j < 16; ++j) ld_slot(at + j * hw * (unsigned)sizeof(raw), v[j]);
                     } else {
-                        const unsigned at = src + s * 16 * kTcM * (unsigned)sizeof(raw);
+                        const unsigned at = ring0 + slot * kSlot + (s * 16 * kTcM + px) * (unsigned)sizeof(raw);
 #pragma unroll
                         for (int j = 0; j < 16; ++j) ld_slot(at + j * kTcM * (unsigned)sizeof(raw), v[j]);
                     }
@@ -570,13 +653,29 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         for (int p = 0; p < P; ++p) tmem_st4(my_a + p * (KC / 2) + s * 8 + h, w[p]);
                     }
                 }
-                __syncwarp();
-                if (lane == 0) bar_arrive(x_empty + 8 * slot);
+                if (!ok) break;
+                if constexpr (!PATCH) {
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(x_empty + 8 * slot);
+                    if (++slot == S) { slot = 0; xph ^= 1u; }
+                }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_before();
                 __syncwarp();
                 if (lane == 0) bar_arrive(a_full + 8 * buf);
                 if (++buf == NA) { buf = 0; aph ^= 1u; }
+            }
+            if constexpr (PATCH) {      // give back the slots that are left of the item
+                if (!ok) break;
+                const int n_blocks = cur.t.k16 ? div_of(cur.t.k16, y.taps) : 0;
+#pragma unroll 1
+                for (int b = block - in_slot; b < n_blocks; b += y.blocks) {
+                    if (!opened) ok = ok && __all_sync(0xffffffffu, bar_wait(x_full + 8 * slot, xph));
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(x_empty + 8 * slot);
+                    if (++slot == S) { slot = 0; xph ^= 1u; }
+                    opened = false;
+                }
             }
         }
     } else if (warp < kConvWarps + kEpiWarps) {
@@ -758,26 +857,42 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 }
             }
         }
-        if (warp >= kProdWarp0 && warp < kProdWarp0 + kProdWarps) {
+        if (warp >= kProdWarp0 && warp < kProdWarp0 + (int)S) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             // every producer copies whole chunks, the block's chunks in turn
             unsigned n = 0, mine = warp - kProdWarp0;
-            Source<XT, TAPS> src;
             Cursor<L> cur(a);
 #pragma unroll 1
             while (ok && cur.step()) {
+                const TcLayer& y = cur.of();
                 const int k16 = cur.t.k16;
-                const unsigned end = n + (k16 + NS - 1) / NS;
-                if (mine < end) src.open(cur.of(), cur.t, cur.pt(), lane);
+                if constexpr (PATCH) {
+                    const int n_blocks = k16 ? div_of(k16, y.taps) : 0;
+                    const unsigned end = n + (n_blocks + y.blocks - 1) / y.blocks;
+                    const Patch t(y, cur.pt());
 #pragma unroll 1
-                for (; mine < end; mine += kProdWarps) {
-                    const unsigned slot = mine % S;
-                    const int k = (mine - n) * NS;
-                    ok = __all_sync(0xffffffffu, bar_wait(x_empty + 8 * slot, ((mine / S) & 1u) ^ 1u));
-                    if (!ok) break;
-                    src.chunk(ring0 + slot * kSlot, k * 16, min(NS, k16 - k) * 16, lane, x_full + 8 * slot);
+                    for (; mine < end; mine += S) {
+                        const unsigned slot = mine % S;
+                        const int c0 = (mine - n) * y.blocks * 16;
+                        ok = __all_sync(0xffffffffu, bar_wait(x_empty + 8 * slot, ((mine / S) & 1u) ^ 1u));
+                        if (!ok) break;
+                        copy_patch<XT>(y, t, ring0 + slot * kSlot, c0, min(y.blocks * 16, y.cin - c0), lane, x_full + 8 * slot);
+                    }
+                    n = end;
+                } else {
+                    Source<XT> src;
+                    const unsigned end = n + (k16 + NS - 1) / NS;
+                    if (mine < end) src.open(y, cur.t, cur.pt(), lane);
+#pragma unroll 1
+                    for (; mine < end; mine += S) {
+                        const unsigned slot = mine % S;
+                        const int k = (mine - n) * NS;
+                        ok = __all_sync(0xffffffffu, bar_wait(x_empty + 8 * slot, ((mine / S) & 1u) ^ 1u));
+                        if (!ok) break;
+                        src.chunk(ring0 + slot * kSlot, k * 16, min(NS, k16 - k) * 16, lane, x_full + 8 * slot);
+                    }
+                    n = end;
                 }
-                n = end;
             }
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
@@ -817,13 +932,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-template <typename XT, bool TAPS, int L>
+template <typename XT, bool PATCH, int L>
 cudaError_t launch(const TcArgs<L>& a, int blocks, cudaStream_t st)
 {
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)blocks);
     lc.blockDim = dim3(kThreads);
-    lc.dynamicSmemBytes = kBarBytes + (size_t)a.stages * a.stage_bytes + kTcRingBytes;
+    lc.dynamicSmemBytes = kBarBytes + (size_t)a.stages * a.stage_bytes + (PATCH ? (size_t)a.slots * a.slot_bytes : kTcRingBytes);
     lc.stream = st;
     // programmatic dependent launch: set-up overlaps the tail of the kernel before it on the stream
     cudaLaunchAttribute attr[1];
@@ -831,39 +946,42 @@ cudaError_t launch(const TcArgs<L>& a, int blocks, cudaStream_t st)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, tc_kernel<XT, TAPS, L>, a);
+    return cudaLaunchKernelEx(&lc, tc_kernel<XT, PATCH, L>, a);
 }
 
-template <typename XT, bool TAPS>
+template <typename XT, bool PATCH>
 cudaError_t launch_any(const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
 {
-    if (a.n_layers > 1) return launch<XT, TAPS, kTcMaxLayers>(a, blocks, st);
+    if (a.n_layers > 1) return launch<XT, PATCH, kTcMaxLayers>(a, blocks, st);
     TcArgs<1> one;      // (a launch's arguments are copied by the driver: few layers, few bytes)
     one.n_layers = 1; one.n_items = a.n_items; one.sched = nullptr; one.stages = a.stages; one.stage_bytes = a.stage_bytes;
+    one.slots = a.slots; one.slot_bytes = a.slot_bytes;
     one.layer[0] = a.layer[0];
-    return launch<XT, TAPS, 1>(one, blocks, st);
+    return launch<XT, PATCH, 1>(one, blocks, st);
 }
 
-template <typename XT, bool TAPS>
+template <typename XT, bool PATCH>
 cudaError_t prepare()
 {
-    cudaError_t e = cudaFuncSetAttribute(tc_kernel<XT, TAPS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_kernel<XT, TAPS, kTcMaxLayers>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
+    cudaError_t e = cudaFuncSetAttribute(tc_kernel<XT, PATCH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_kernel<XT, PATCH, kTcMaxLayers>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
     return e;
 }
 
 }  // namespace
 
-cudaError_t launch_tc(int dt, bool taps, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
+cudaError_t launch_tc(int dt, bool patch, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
 {
-    if (taps) return dt == 0 ? launch_any<float, true>(a, blocks, st) : cudaErrorInvalidValue;
+    if (patch)
+        return dt == 0 ? launch_any<float, true>(a, blocks, st)
+                       : dt == 1 ? launch_any<__half, true>(a, blocks, st) : launch_any<__nv_bfloat16, true>(a, blocks, st);
     return dt == 0 ? launch_any<float, false>(a, blocks, st)
                    : dt == 1 ? launch_any<__half, false>(a, blocks, st) : launch_any<__nv_bfloat16, false>(a, blocks, st);
 }
 
-cudaError_t prepare_tc(int dt, bool taps)
+cudaError_t prepare_tc(int dt, bool patch)
 {
-    if (taps) return dt == 0 ? prepare<float, true>() : cudaErrorInvalidValue;
+    if (patch) return dt == 0 ? prepare<float, true>() : dt == 1 ? prepare<__half, true>() : prepare<__nv_bfloat16, true>();
     return dt == 0 ? prepare<float, false>() : dt == 1 ? prepare<__half, false>() : prepare<__nv_bfloat16, false>();
 }
 

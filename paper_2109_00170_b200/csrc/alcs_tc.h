@@ -44,8 +44,7 @@ struct TcLayer {
     const unsigned char* b;      // weight tiles, in the layout the MMA reads from shared memory
     const TcTile* tiles;         // null: every tile takes k16 steps, the tiles' weights one after the other
     int k16;
-    const int* cols;             // 1x1: input channel per entry of the tile's column list (null: all channels in order);
-                                 // k x k: {element offset of the column from the pixel's window, tap number} per entry
+    const int* cols;             // input channel per entry of the tile's column list (null: all channels in order)
     const int* chan;             // output channel of row i of the tiles (null: i itself; -1: padding)
     int* err;
     int first_item;              // items of this layer start here
@@ -58,7 +57,13 @@ struct TcLayer {
     int hw_in, w_in, h_in;       // input image
     TcDiv ow;
     int stride, pad;
-    int kh, kw;                  // k x k only: tap = r * kw + s
+    // Patch staging (k x k kernels, strides): columns run [block of 16 channels][tap = r * kw + s][channel]; a ring slot
+    // holds `blocks` blocks of the input rows a tile needs, `pitch` elements per channel
+    int kh, kw;
+    TcDiv taps, kwd;
+    TcDiv w_vec;                 // copies per image row
+    int oh, row_step;            // input rows are taken every row_step
+    int blocks, pitch;
     int vec_bytes;               // bytes of one copy of X: 16, 8, 4; 0: element by element
     int ppt;                     // pixels per tile: kTcM, or those of ...
     int images;                  // ... this many whole images, staged as runs of memory (0: not so)
@@ -72,13 +77,14 @@ struct TcArgs {
     const int* sched;            // null: thread block b takes items b, b + grid, ...; else its items are sched[b], sched[b + grid], ... until -1
     int stages;                  // weight stages in shared memory
     int stage_bytes;
+    int slots, slot_bytes;       // patch staging: X ring
     TcLayer layer[L];
 };
 
 // Launch a (n_layers <= kTcMaxLayers; one launch with elements of type dt) on `blocks` thread
-// blocks; taps: k x k convolution (fp32 only).
-cudaError_t launch_tc(int dt, bool taps, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st);
-cudaError_t prepare_tc(int dt, bool taps);      // once per device: shared-memory attribute
+// blocks; patch: all layers by patch staging.
+cudaError_t launch_tc(int dt, bool patch, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st);
+cudaError_t prepare_tc(int dt, bool patch);      // once per device: shared-memory attribute
 constexpr int tc_planes(int dt) { return dt == 0 ? 3 : 1; }      // 16-bit planes an operand is split into
 // ring of X chunks: 4 of 128 pixels x 64 columns in fp32, x 128 columns in 16 bits
 constexpr int kTcRingBytes = 4 * kTcM * 64 * 4;

@@ -29,7 +29,7 @@ int cuda_fail(cudaError_t e)
 template <typename T, int P>
 __global__ void expand_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col_idx, const T* __restrict__ vals,
                               const int* __restrict__ place, const TcTile* __restrict__ tiles, const int* __restrict__ inv,
-                              int rows, int g, int n, int cols, unsigned char* __restrict__ b)
+                              int rows, int g, int n, int cols, int taps, unsigned char* __restrict__ b)
 {
     const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (r >= rows) return;
@@ -41,6 +41,7 @@ __global__ void expand_kernel(const int* __restrict__ row_ptr, const int* __rest
         const int blk = i / g, j = i - blk * g;
         int k = col_idx[beg + blk];
         if (inv) k = inv[(size_t)tile * cols + k];
+        else if (taps > 1) k = (k / taps / 16 * taps + k % taps) * 16 + k / taps % 16;      // [16 channels][tap]
         constexpr int KC = P == 3 ? kTcKC32 : kTcKC16;
         const int chunk = k / KC, ns = min(KC / 16, t.k16 - KC / 16 * chunk);
         unsigned char* d = bt + (size_t)chunk * (P * KC * 2) * n + ((size_t)((k % KC) >> 3) * n + n0 + j) * 16 + (k & 7) * 2;
@@ -113,7 +114,7 @@ bool skewed(const alcs_packed& w)
 
 TcPrep* tc_find(const alcs_packed* w, const TcKey& key)
 {
-    auto it = w->tc.find({key.n, key.kh, key.kw, key.h, key.wd});
+    auto it = w->tc.find({key.n, key.kh, key.kw});
     return it == w->tc.end() ? nullptr : it->second;
 }
 
@@ -135,9 +136,9 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
     {
         // the shared-memory attribute belongs to the kernel as loaded on a device
         static std::mutex mu;
-        static bool ready[64][4] = {};
+        static bool ready[64][6] = {};
         std::lock_guard<std::mutex> lk(mu);
-        bool& r = ready[w->device & 63][key.kh ? 3 : (int)w->dt];
+        bool& r = ready[w->device & 63][(key.kh ? 3 : 0) + (int)w->dt];
         if (!r) {
             const cudaError_t e = prepare_tc(w->dt, key.kh > 0);
             if (e != cudaSuccess) return cuda_fail(e);
@@ -148,12 +149,12 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
     if ((*out = tc_find(w, key)) != nullptr) return ALCS_OK;
     try {
         const int P = tc_planes(w->dt), n = key.n, rpt = n / w->g;
-        const bool taps = key.kh > 0;
-        const int dense16 = (w->cin + 15) / 16;
+        const int taps = std::max(1, key.kh * key.kw);
+        const int dense16 = (w->cin / taps + 15) / 16 * taps;
         Layout L;
         layout_of(*w, rpt, false, L);
         bool sorted = false;
-        if (skewed(*w)) {
+        if (!key.kh && skewed(*w)) {
             Layout S;
             layout_of(*w, rpt, true, S);
             if (S.k16 * 20 <= L.k16 * 19) { L = std::move(S); sorted = true; }
@@ -161,7 +162,7 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         const int n_tiles = (int)L.cols.size();
         // A column list costs the converters its loads: without at least a tenth of the steps to save,
         // take all columns in order.
-        const bool list = taps || L.k16 * 10 <= (long long)dense16 * n_tiles * 9;
+        const bool list = !key.kh && L.k16 * 10 <= (long long)dense16 * n_tiles * 9;
         std::vector<TcTile> tiles(n_tiles);
         std::vector<int> cols, inv, chan, place(w->rows);
         size_t bytes = 0;
@@ -172,20 +173,9 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         for (int t = 0; t < n_tiles; ++t) {
             const int used = (int)L.cols[t].size();
             const int k16 = !list ? (used ? dense16 : 0) : (used + 15) / 16;
-            tiles[t] = {(unsigned)(bytes / 16), k16, (int)(cols.size() / (taps ? 2 : 1))};
-            if (list && used) {
-                const int kk = key.kh * key.kw;
-                for (int i = 0; i < k16 * 16; ++i) {
-                    const int c = L.cols[t][std::min(i, used - 1)];
-                    if (taps) {
-                        const int tap = c % kk, r = tap / key.kw, s = tap % key.kw;
-                        cols.push_back(c / kk * key.h * key.wd + r * key.wd + s);
-                        cols.push_back(tap);
-                    } else {
-                        cols.push_back(c);
-                    }
-                }
-            }
+            tiles[t] = {(unsigned)(bytes / 16), k16, (int)cols.size()};
+            if (list && used)
+                for (int i = 0; i < k16 * 16; ++i) cols.push_back(L.cols[t][std::min(i, used - 1)]);
             if (list) {
                 inv.resize((size_t)(t + 1) * w->cin, 0);
                 for (int i = 0; i < used; ++i) inv[(size_t)t * w->cin + L.cols[t][i]] = i;
@@ -226,11 +216,11 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
             const unsigned blocks = (unsigned)((w->rows + 3) / 4);
             if (w->dt == ALCS_F32)
                 expand_kernel<float, 3><<<blocks, 128, 0, st>>>(w->d_row_ptr, w->d_col_idx, static_cast<const float*>(w->d_vals), dp, dt, di,
-                                                               w->rows, w->g, n, w->cin, d);
+                                                               w->rows, w->g, n, w->cin, taps, d);
             else
                 expand_kernel<unsigned short, 1><<<blocks, 128, 0, st>>>(w->d_row_ptr, w->d_col_idx,
                                                                         static_cast<const unsigned short*>(w->d_vals), dp, dt, di,
-                                                                        w->rows, w->g, n, w->cin, d);
+                                                                        w->rows, w->g, n, w->cin, taps, d);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);      // (the host arrays go away; other streams may use the tiles)
@@ -244,7 +234,7 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         p.chan = chan.empty() ? nullptr : reinterpret_cast<int*>(d + o_chan);
         p.uploaded = true;
         TcPrep* kept = new TcPrep(p);
-        w->tc[{key.n, key.kh, key.kw, key.h, key.wd}] = kept;
+        w->tc[{key.n, key.kh, key.kw}] = kept;
         *out = kept;
     } catch (const std::bad_alloc&) {
         return ALCS_ERR_ALLOC;
@@ -252,7 +242,49 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
     return ALCS_OK;
 }
 
-void tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out)
+namespace {
+
+// Patch staging of one problem: copy width, elements per channel of the largest patch, input rows taken.
+struct PatchPlan {
+    int vec_bytes, pitch, row_step;
+};
+
+PatchPlan patch_plan(const alcs_packed* w, const TcProblem& p)
+{
+    const int elt = (int)w->elt();
+    PatchPlan r;
+    r.vec_bytes = 16;
+    while (r.vec_bytes > 2 && ((size_t)p.w_in * elt % r.vec_bytes || (uintptr_t)p.x % r.vec_bytes)) r.vec_bytes >>= 1;
+    r.row_step = p.kh == 1 && p.pad == 0 ? p.stride : 1;
+    // A tile of 128 consecutive output pixels touches at most (126 / ow) + 2 output rows and (126 / hw) + 2 images.
+    const long long hw = (long long)p.oh * p.ow, images = std::min<long long>(p.n, (kTcM - 2) / hw + 2);
+    const long long out_rows = std::min<long long>((kTcM - 2) / p.ow + 2, images * p.oh);
+    long long rows = r.row_step > 1 ? out_rows : (out_rows - images) * p.stride + images * std::max(p.kh, p.stride);
+    rows = std::min(rows, images * p.h_in);
+    r.pitch = (int)((rows * p.w_in + 7) / 8 * 8);
+    return r;
+}
+
+// Blocks of 16 channels per slot: as many as a chunk has steps, if at least three slots then fit.
+int patch_blocks(const alcs_packed* w, const TcProblem& p, const PatchPlan& pl, int room)
+{
+    const int want = std::max(1, tc_kc(w->dt) / 16 / (p.kh * p.kw));
+    const long long block = 16ll * pl.pitch * w->elt();
+    return (int)std::max(1ll, std::min<long long>(want, room / 3 / block));
+}
+
+int patch_room(int dt, int n) { return 227 * 1024 - kTcHeaderBytes - 2 * tc_stage_bytes(dt, n); }
+
+}  // namespace
+
+bool tc_patch_fits(const alcs_packed* w, const TcProblem& p, int n)
+{
+    if (p.kh * p.kw > 32 || w->cin % (p.kh * p.kw)) return false;
+    const PatchPlan pl = patch_plan(w, p);
+    return pl.vec_bytes >= 4 && 2 * 16ll * pl.pitch * (long long)w->elt() <= patch_room(w->dt, n);
+}
+
+int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out)
 {
     TcLayer& y = *out;
     y.x = p.x; y.y = p.y; y.bias = p.bias; y.res = p.res;
@@ -261,7 +293,6 @@ void tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer*
     y.hw = tc_div(p.oh * p.ow);
     y.q = p.n * y.hw.d;
     y.n_tiles = tc_div(t.n_tiles);
-    
     // tiles of unequal work: all pixel tiles of the heaviest channel tile first, so that the light ones
     // fill the end; otherwise the channel tiles of a pixel tile run together and share its reads of X
     y.tile_major = t.k16_max > t.k16_min + t.k16_min / 4 ? 1 : 0;
@@ -269,24 +300,35 @@ void tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer*
     y.cin = p.kh ? w->cin / (p.kh * p.kw) : w->cin;
     y.cout = w->cout;
     y.hw_in = p.h_in * p.w_in; y.w_in = p.w_in; y.h_in = p.h_in;
-    y.ow = tc_div(p.ow); y.stride = p.stride; y.pad = p.pad;
+    y.ow = tc_div(p.ow); y.oh = p.oh; y.stride = p.stride; y.pad = p.pad;
     y.kh = p.kh; y.kw = p.kw;
-    // the widest copy that keeps to one image and to its alignment
-    const int elt = w->dt == ALCS_F32 ? 4 : 2;
-    int vb = 16;
-    while (vb > elt && (p.stride != 1 || p.kh || ((size_t)y.hw.d * elt) % vb || (uintptr_t)p.x % vb)) vb >>= 1;
-    y.vec_bytes = vb == 16 || (elt == 2 && vb > elt) ? vb : 0;      // (8 bytes of fp32: as single elements)
-    // Small images whose rows do not start on copy boundaries (7x7): a tile takes whole images, of which the
-    // columns of a chunk are one run of memory, if those runs keep to 16 bytes
     y.n_img = p.n;
     y.images = 0;
-    if (y.vec_bytes == 0 && !p.kh && p.stride == 1 && !t.cols && y.hw.d <= kTcM && (uintptr_t)p.x % 16 == 0 &&
-        (size_t)y.cin * y.hw.d * elt % 16 == 0 && (size_t)16 * y.hw.d * elt % 16 == 0 && y.cin % 16 == 0)
-        y.images = kTcM / y.hw.d;
+    const int elt = (int)w->elt();
+    if (p.kh) {
+        const PatchPlan pl = patch_plan(w, p);
+        y.taps = tc_div(p.kh * p.kw); y.kwd = tc_div(p.kw);
+        y.vec_bytes = pl.vec_bytes;
+        y.w_vec = tc_div(p.w_in * elt / pl.vec_bytes);
+        y.row_step = pl.row_step;
+        y.pitch = pl.pitch;
+        y.blocks = patch_blocks(w, p, pl, patch_room(w->dt, t.n));
+    } else {
+        // the widest copy that keeps to one image and to its alignment
+        int vb = 16;
+        while (vb > elt && (((size_t)y.hw.d * elt) % vb || (uintptr_t)p.x % vb)) vb >>= 1;
+        y.vec_bytes = vb == 16 || (elt == 2 && vb > elt) ? vb : 0;      // (8 bytes of fp32: as single elements)
+        // Small images whose rows do not start on copy boundaries (7x7): a tile takes whole images, of which the
+        // columns of a chunk are one run of memory, if those runs keep to 16 bytes
+        if (y.vec_bytes == 0 && !t.cols && y.hw.d <= kTcM && (uintptr_t)p.x % 16 == 0 && (size_t)y.cin * y.hw.d * elt % 16 == 0 &&
+            (size_t)16 * y.hw.d * elt % 16 == 0 && y.cin % 16 == 0)
+            y.images = kTcM / y.hw.d;
+    }
     y.ppt = y.images ? y.images * y.hw.d : kTcM;
     y.px_tiles = tc_div((y.q + y.ppt - 1) / y.ppt);
     y.relu = (p.flags & ALCS_RELU) ? 1 : 0;
     y.y32 = (p.flags & ALCS_Y_F32) ? 1 : 0;
+    return ALCS_OK;
 }
 
 // How long one item takes, in microseconds, by type, channels per tile and 16-column steps: per chunk the MMAs
@@ -301,7 +343,7 @@ double tc_item_us(int dt, int n, int k16)
 }
 
 // Number items and choose the ring depth for the a.n_layers layers filled in.
-int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a)
+int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a, bool patch)
 {
     int sms = 0, smem = 0;
     const int rc = device_limits(w->device, &sms, &smem);
@@ -317,18 +359,61 @@ int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a)
     a.n_items = (int)items;
     a.sched = nullptr;
     a.stage_bytes = tc_stage_bytes(w->dt, n);
+    int room = std::min(smem, 227 * 1024) - kTcHeaderBytes;
+    a.slots = a.slot_bytes = 0;
+    if (patch) {
+        for (int i = 0; i < a.n_layers; ++i) a.slot_bytes = std::max(a.slot_bytes, a.layer[i].blocks * 16 * a.layer[i].pitch * (int)w->elt());
+        a.slots = std::min(4, (room - 2 * a.stage_bytes) / a.slot_bytes);
+        if (a.slots < 2) return ALCS_ERR_UNSUPPORTED;
+        room -= a.slots * a.slot_bytes;
+    } else {
+        room -= kTcRingBytes;
+    }
     // (an even number: of two MMA issuers each then always meets the same stages)
-    a.stages = ~1 & std::min(8, (std::min(smem, 227 * 1024) - kTcHeaderBytes - kTcRingBytes) / a.stage_bytes);
+    a.stages = ~1 & std::min(8, room / a.stage_bytes);
     return a.stages >= 2 ? ALCS_OK : ALCS_ERR_UNSUPPORTED;
 }
 
-int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool taps, cudaStream_t st)
+int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool patch, cudaStream_t st)
 {
     int sms = 0, smem = 0;
     const int rc = device_limits(w->device, &sms, &smem);
     if (rc) return rc;
-    const cudaError_t e = launch_tc(w->dt, taps, a, std::min(a.n_items, sms), st);
+    const cudaError_t e = launch_tc(w->dt, patch, a, std::min(a.n_items, sms), st);
     return e == cudaSuccess ? ALCS_OK : cuda_fail(e);
+}
+
+int tc_run(const alcs_packed* w, const TcPrep& t, const TcProblem& p, cudaStream_t st)
+{
+    TcArgs<kTcMaxLayers> a;
+    a.n_layers = 1;
+    tc_fill(w, t, p, &a.layer[0]);
+    const int rc = tc_finish(w, a, p.kh > 0);
+    return rc ? rc : tc_launch(w, a, p.kh > 0, st);
+}
+
+int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st)
+{
+    const long long hw = (long long)p.oh * p.ow;
+    const int taps = p.kh * p.kw;
+    if (!tc_fits(w->cin / taps, w->cout, p.n, (long long)p.h_in * p.w_in, hw, taps)) return ALCS_ERR_UNSUPPORTED;
+    int sms = 0, smem = 0;
+    int rc = device_limits(w->device, &sms, &smem);
+    if (rc) return rc;
+    // the width whose rounds of items over the SMs take the least time
+    const int k16 = (w->cin / taps + 15) / 16 * taps;
+    int n = 0;
+    double best = 0;
+    for (int want = kTcMaxN; want >= 16; want -= 16) {
+        const int tiles = (w->cout + want - 1) / want, v = ((w->cout + tiles - 1) / tiles + 15) / 16 * 16;
+        const long long items = (p.n * hw + kTcM - 1) / kTcM * ((w->cout + v - 1) / v);
+        const double us = (double)((items + sms - 1) / sms) * tc_item_us(w->dt, v, k16);
+        if ((n == 0 || us < best) && tc_patch_fits(w, p, v)) { n = v; best = us; }
+    }
+    if (n == 0) return ALCS_ERR_UNSUPPORTED;
+    TcPrep* t = nullptr;
+    rc = tc_prepare(w, {n, p.kh, p.kw}, st, &t);
+    return rc ? rc : tc_run(w, *t, p, st);
 }
 
 // 32-bit arithmetic of the kernel: element offsets into X, byte offsets inside the images one tile touches.

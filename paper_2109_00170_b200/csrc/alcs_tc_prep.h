@@ -9,10 +9,10 @@
 
 namespace alcs {
 
-// What the expanded weights depend on: channels per tile and, for k x k kernels (kh > 0), the image
-// and kernel sizes the columns' element offsets are computed from.
+// What the expanded weights depend on: channels per tile and, for patch staging (kh > 0), the kernel size, by
+// which the columns are reordered.
 struct TcKey {
-    int n, kh, kw, h, wd;
+    int n, kh, kw;
 };
 
 struct TcPrep {
@@ -23,24 +23,27 @@ struct TcPrep {
     // device; one allocation, `b` first
     unsigned char* b = nullptr;
     TcTile* tiles = nullptr;
-    int* cols = nullptr;         // null: every tile takes all columns in order
+    int* cols = nullptr;         // null: every tile takes all columns
     int* chan = nullptr;         // null: identity
 };
 
 // The problem a launch solves (one layer), everything but the weights.
 struct TcProblem {
     const void* x; void* y; const float* bias; const void* res;
-    int n, oh, ow, h_in, w_in, stride, pad, kh, kw;      // kh = 0: pointwise
+    int n, oh, ow, h_in, w_in, stride, pad, kh, kw;      // kh = 0: no patch staging
     unsigned flags;
 };
 
 int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep** out);
 TcPrep* tc_find(const alcs_packed* w, const TcKey& key);       // already prepared, or null; caller holds w->mu
 void tc_free(TcPrep* p);
-void tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out);
+int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out);
 double tc_item_us(int dt, int n, int k16);
-int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a);
-int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool taps, cudaStream_t st);
+int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a, bool patch);
+int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool patch, cudaStream_t st);
+int tc_run(const alcs_packed* w, const TcPrep& t, const TcProblem& p, cudaStream_t st);      // one layer, prepared
+int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st);      // UNSUPPORTED where patch staging cannot
+bool tc_patch_fits(const alcs_packed* w, const TcProblem& p, int n);     // can the problem be run by patch staging, n channels per tile?
 bool tc_fits(int cin, int cout, long long n, long long hw_in, long long hw, int k);
 
 }  // namespace alcs
