@@ -270,9 +270,11 @@ void set_unit_args(ConvArgs& a, const Schedule& sc, int mma)
     a.xch_slots = sc.max_x;
 }
 
-// The small-problem kernel as a plan.  Its cost estimate is a latency model: a warp issues the loads of
-// a few blocks at a time and waits about one L2 round trip for each batch; the arithmetic term makes it
-// lose against the staged kernels as soon as there is enough work to keep the SMs busy.
+// The small-problem kernel as a plan.  Its cost: a launch, then the longer of two times: the rounds of dependent
+// loads (a warp issues the input vectors of four blocks and waits for them; a thread block's columns take `batches`
+// such rounds) and the bytes of X, which every block row fetches for itself from L2.  The constants are fits to one
+// B200: 4.5 us for 512 -> 512 @14 at batch 1, 3.8 for 731 -> 95 @7, 12 for 512 -> 512 @14 at batch 4, 24 for
+// 512 -> 512 @7 at batch 16.
 bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const DeviceInfo& di, Plan* out)
 {
     const int sms = di.sms;
@@ -283,21 +285,23 @@ bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const Devic
     if (blocks > (1ll << 22)) return false;
     Plan pl;
     pl.variant = -1; pl.gather = 1; pl.gp = p; pl.gks = ks;
+    const bool vec = hw % 4 == 0 && p >= 4;
     const double per_row = w->rows ? (double)w->nb / w->rows : 0.0;
     const double batches = std::ceil(per_row / ks / 4.0);
-    const double resident = std::max(1.0, std::floor(2048.0 / (ks * 32)));          // thread blocks per SM
+    const double resident = std::max(1, (w->g * p > 16 ? 512 : 1024) / (ks * 32));          // thread blocks per SM
     const double rounds = std::ceil((double)blocks / (sms * resident));
-    const double latency = rounds * (batches * 900.0 + 2500.0);
-    const double alu = (double)w->nb * w->g * n * tiles * 32.0 * p / (sms * 128.0 * 0.25);
-    pl.cost = std::max(latency, alu) / di.sm_hz;
+    const double batch_us = (p == 2 ? 0.55 : p == 4 ? 0.7 : 0.9) * (vec || p == 2 ? 1.0 : 1.3);
+    const double bytes = (double)w->nb * n * tiles * 32.0 * p * 4;
+    pl.cost = 1e-6 * (2.6 + std::max(rounds * batches * batch_us, bytes / (vec ? 5.5e6 : 3.3e6)));
     *out = pl;
     return true;
 }
 
 // Fixed cost of a launch of the tcgen05 kernel, first copies and last stores included, in microseconds.
-constexpr double kTcRampUs = 4.5;
-// What the small-problem kernel's latency model comes to on the GPU (seconds = weight * model + ramp).
-constexpr double kGatherWeight = 1.3, kGatherRamp = 2.5e-6;
+constexpr double kTcRampUs = 5.0;
+
+// Most images for which the small-problem kernel is considered (beyond, the bytes of X decide against it anyway).
+constexpr long long kGatherImages = 64;
 
 // The tcgen05 kernel with n output channels per tile as a plan, and its cost: rounds of items over the SMs.
 Plan tc_plan(const alcs_packed* w, int n, long long q, int sms)
@@ -500,12 +504,11 @@ int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg
         // Nobody asked for anything: the tcgen05 kernel, or the small-problem kernel where a few images leave most
         // SMs without a tile and the latency of one item's chunk chain is all there is.
         *out = tc_best(w, q, di.sms);
-        if (allow_small && q / hw <= 8)
+        if (allow_small && q / hw <= kGatherImages)
             for (int p = 8; p >= 2; p /= 2)
                 for (int ks = 4; ks <= 16; ks *= 2) {
                     Plan g;
-                    if (gather_plan(w, (int)(q / hw), hw, p, ks, di, &g) && g.cost * kGatherWeight + kGatherRamp < out->cost &&
-                        (!out->gather || g.cost < out->cost)) *out = g;
+                    if (gather_plan(w, (int)(q / hw), hw, p, ks, di, &g) && g.cost < out->cost) *out = g;
                 }
         return ALCS_OK;
     }

@@ -1,11 +1,11 @@
 // Latency model (paper, Section 3.3) and projection with bisection (Section 3.4, Algorithm 1).
 //
 // Host part: the linear interpolation over a layer's measured (non-zero count, run time) pairs and
-// the network sum.  Device part, the data-parallel steps of Algorithm 1: the ranking key of every
-// group of g adjacent filters (its squared L2 norm), the ranking of all groups of all layers (a
-// radix sort from the CUDA toolkit's CUB, a library primitive), the layer of every ranked group with
-// per-bucket layer histograms, and the final mask / projected tensor.  The search over the length of
-// the kept prefix of the ranked list runs on the host from one copy of those two arrays.
+// the network sum.  Algorithm 1 runs on the device from end to end, in one stream and with one wait at the
+// end: the ranking key of every group of g adjacent filters (its squared L2 norm), the ranking of all
+// groups of all layers (a radix sort from the CUDA toolkit's CUB, a library primitive), per-bucket layer
+// histograms of the ranked list, the search over the length of the kept prefix (one thread block, five
+// bisection steps per round), and the mask and the projected tensors from the key of the last kept group.
 #include <cuda_runtime.h>
 
 #include <cub/device/device_radix_sort.cuh>
@@ -54,87 +54,268 @@ int check_table(const alcs_latency_table* tab)
     return ALCS_OK;
 }
 
+// Layers of one launch of the per-group kernels.
+constexpr int kLayersPerLaunch = 64;
+struct LayerTable {
+    int n_layers, g;
+    long long total;                        // groups in this launch
+    const float* u[kLayersPerLaunch];
+    float* out[kLayersPerLaunch];           // may be null
+    int cout[kLayersPerLaunch], cols[kLayersPerLaunch];
+    long long off[kLayersPerLaunch + 1];    // first group of each layer, counted over all layers of the call
+};
+
+// Layer of group i (binary search over the layers' group offsets).
+__device__ __forceinline__ int layer_of_group(const long long* off, int n_layers, long long i)
+{
+    int lo = 0, hi = n_layers - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= i) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
 // key[group] = sum over the g filters of the group of the squared element: fp32, one rounded
 // multiply and one rounded add per element, filters in ascending order (no fused multiply-add, so
 // that the ranking is reproducible bit for bit).  Group (r, c) of a [cout][cols] layer covers
 // elements (r*g + j, c); a missing filter of a ragged last group counts as zero.  Also writes the
-// identity permutation that the sort carries along.
-__global__ void group_keys_kernel(const float* __restrict__ u, int cout, int cols, int g, long long base,
-                                  unsigned* __restrict__ keys, unsigned* __restrict__ idx)
+// identity permutation that the sort carries along.  One launch for (up to 64) layers: reads the weights
+// once, at the memory's rate for large networks; small ones are a launch's latency.
+__global__ void group_keys_kernel(const __grid_constant__ LayerTable t, unsigned* __restrict__ keys, unsigned* __restrict__ idx)
 {
-    const int rows = (cout + g - 1) / g;
-    const long long n = (long long)rows * cols;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(i / cols);
-        const int c = (int)(i - (long long)r * cols);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < t.total; i += (long long)gridDim.x * blockDim.x) {
+        const long long id = t.off[0] + i;
+        const int l = layer_of_group(t.off, t.n_layers, id);
+        const int cols = t.cols[l];
+        const unsigned in = (unsigned)(id - t.off[l]);
+        const int r = in / (unsigned)cols, c = in - r * cols;
+        const float* p = t.u[l] + (size_t)r * t.g * cols + c;
+        const int nj = min(t.g, t.cout[l] - r * t.g);
         float acc = 0.0f;
-        for (int j = 0; j < g; ++j) {
-            const int co = r * g + j;
-            if (co >= cout) break;
-            const float v = __ldg(u + (size_t)co * cols + c);
+#pragma unroll 8
+        for (int j = 0; j < nj; ++j) {
+            const float v = __ldg(p + (size_t)j * cols);
             acc = __fadd_rn(acc, __fmul_rn(v, v));
         }
-        keys[base + i] = __float_as_uint(acc);      // non-negative floats order like their bit patterns
-        idx[base + i] = (unsigned)(base + i);
+        keys[id] = __float_as_uint(acc);      // non-negative floats order like their bit patterns
+        idx[id] = (unsigned)id;
     }
 }
 
-// layer_of[i] = layer of the i-th ranked group (binary search over the layers' group offsets)
-__global__ void ranked_layer_kernel(const unsigned* __restrict__ idx, long long total, const long long* __restrict__ off,
-                                    int n_layers, unsigned short* __restrict__ layer_of)
+// The result: a group is kept if it ranks before the n_keep-th, i.e. if its key is larger than that of the last
+// kept group, or equal and its number not larger (the sort is stable).  u_out = u where kept, +0 elsewhere.
+__global__ void apply_kernel(const __grid_constant__ LayerTable t, const unsigned* __restrict__ keys, const unsigned* __restrict__ ranked_keys,
+                             const unsigned* __restrict__ ranked_idx, const long long* __restrict__ n_keep, uint8_t* __restrict__ mask)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const long long gidx = idx[i];
-        int lo = 0, hi = n_layers - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (off[mid] <= gidx) lo = mid; else hi = mid - 1;
-        }
-        layer_of[i] = (unsigned short)lo;
+    const long long n = *n_keep;
+    const unsigned last_key = n > 0 ? ranked_keys[n - 1] : 0u, last_id = n > 0 ? ranked_idx[n - 1] : 0u;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < t.total; i += (long long)gridDim.x * blockDim.x) {
+        const long long id = t.off[0] + i;
+        const unsigned k = keys[id];
+        const bool keep = n > 0 && (k > last_key || (k == last_key && (unsigned)id <= last_id));
+        mask[id] = keep ? 1 : 0;
+        const int l = layer_of_group(t.off, t.n_layers, id);
+        if (!t.out[l]) continue;
+        const int cols = t.cols[l];
+        const unsigned in = (unsigned)(id - t.off[l]);
+        const int r = in / (unsigned)cols, c = in - r * cols;
+        const size_t at = (size_t)r * t.g * cols + c;
+        const int nj = min(t.g, t.cout[l] - r * t.g);
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) t.out[l][at + (size_t)j * cols] = keep ? t.u[l][at + (size_t)j * cols] : 0.0f;
     }
 }
 
 constexpr int kMaxLayers = 4096;
+constexpr long long kRankBucket = 1024;
 
-constexpr long long kRankBucket = 4096;
-
-// page-locked host staging area of alcs_project_bisection, shared by all calls (one call at a time uses it)
-std::mutex g_staging_mu;
-void* g_staging = nullptr;
-size_t g_staging_bytes = 0;
-
-// hist[b][l] = how many of the ranked entries b*kRankBucket .. (b+1)*kRankBucket - 1 belong to layer l
-// (one thread block per bucket, a shared-memory histogram)
-__global__ void bucket_histogram_kernel(const unsigned short* __restrict__ layer_of, long long total, int n_layers,
-                                        unsigned* __restrict__ hist)
+// layer_of[i] = layer of the i-th ranked group; hist[b][l] = how many of the ranked entries
+// b*kRankBucket .. (b+1)*kRankBucket - 1 belong to layer l (one thread block per bucket).
+__global__ void ranked_layers_kernel(const unsigned* __restrict__ idx, long long total, const long long* __restrict__ off, int n_layers,
+                                     unsigned short* __restrict__ layer_of, unsigned* __restrict__ hist)
 {
     extern __shared__ unsigned int h[];
     for (int i = threadIdx.x; i < n_layers; i += blockDim.x) h[i] = 0;
     __syncthreads();
     const long long b0 = (long long)blockIdx.x * kRankBucket;
     const long long b1 = b0 + kRankBucket < total ? b0 + kRankBucket : total;
-    for (long long i = b0 + threadIdx.x; i < b1; i += blockDim.x) atomicAdd(&h[layer_of[i]], 1u);
+    for (long long i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
+        const int l = layer_of_group(off, n_layers, idx[i]);
+        layer_of[i] = (unsigned short)l;
+        atomicAdd(&h[l], 1u);
+    }
     __syncthreads();
     for (int i = threadIdx.x; i < n_layers; i += blockDim.x) hist[(size_t)blockIdx.x * n_layers + i] = h[i];
 }
 
-// mask[group] = 1 for the n best-ranked groups, 0 for the others
-__global__ void write_mask_kernel(const unsigned* __restrict__ idx, long long total, long long n, uint8_t* __restrict__ mask)
+// hist[b][l] becomes the number of entries of layer l in the buckets before b (one warp per layer).
+__global__ void prefix_kernel(unsigned* __restrict__ hist, long long n_buckets, int n_layers)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
-        mask[idx[i]] = i < n ? 1 : 0;
+    const int l = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (l >= n_layers) return;
+    unsigned before = 0;
+    for (long long b0 = 0; b0 < n_buckets; b0 += 32) {
+        const long long b = b0 + lane;
+        const unsigned v = b < n_buckets ? hist[(size_t)b * n_layers + l] : 0u;
+        unsigned s = v;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned o = __shfl_up_sync(0xffffffffu, s, d);
+            if (lane >= d) s += o;
+        }
+        if (b < n_buckets) hist[(size_t)b * n_layers + l] = before + s - v;
+        before += __shfl_sync(0xffffffffu, s, 31);
+    }
 }
 
-// u_out = u where the element's group is kept, +0 elsewhere
-__global__ void apply_mask_kernel(const float* __restrict__ u, const uint8_t* __restrict__ mask, int cout, int cols, int g,
-                                  float* __restrict__ out)
+// What the search returns; written to page-locked host memory.
+struct SearchResult {
+    long long n_keep, lo, hi;
+    int iters;
+    double latency;
+};
+
+struct SearchArgs {
+    const unsigned short* layer_of;
+    const unsigned* prefix;             // [bucket][layer]
+    const int* first_knot;              // [n_layers + 1]
+    const long long* k;                 // knots of all layers
+    const double* t;
+    const double* alpha;                // slope of the interval that starts at a knot
+    long long total;
+    int n_layers, g, depth;
+    double tau, t_budget, eps;
+    long long* n_keep;                  // device
+    SearchResult* result;               // host
+    long long* kept;                    // host, [n_layers]
+};
+
+// T(W) of "the n best-ranked groups kept", by one warp: per-layer counts from the bucket's prefix and a walk over
+// at most one bucket, then Eq. for T^(s) term by term and the sum over the layers in order, every operation
+// rounded as the host's (no fused multiply-add).
+__device__ double latency_of_top(const SearchArgs& a, long long n, unsigned* counts, double* terms, int lane)
 {
-    const long long n = (long long)cout * cols;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int co = (int)(i / cols);
-        const int c = (int)(i - (long long)co * cols);
-        out[i] = mask[(size_t)(co / g) * cols + c] ? u[i] : 0.0f;
+    const long long bk = n / kRankBucket < (a.total + kRankBucket - 1) / kRankBucket ? n / kRankBucket : (a.total + kRankBucket - 1) / kRankBucket - 1;
+    __syncwarp();
+    for (int l = lane; l < a.n_layers; l += 32) counts[l] = a.prefix[(size_t)bk * a.n_layers + l];
+    __syncwarp();
+    for (long long i = bk * kRankBucket + lane; i < n; i += 32) atomicAdd(&counts[a.layer_of[i]], 1u);
+    __syncwarp();
+    double t = a.tau;
+    for (int l0 = 0; l0 < a.n_layers; l0 += 32) {
+        const int l = l0 + lane;
+        if (l < a.n_layers) {
+            const long long s = (long long)counts[l] * a.g;
+            const int f = a.first_knot[l], e = a.first_knot[l + 1] - 1;
+            double sum = a.t[f];
+            for (int i = f; i < e; ++i) {
+                const double delta = s >= a.k[i] ? 1.0 : 0.0;
+                const double width = __dsub_rn((double)a.k[i + 1], (double)a.k[i]);
+                const double in = __dsub_rn((double)s, (double)a.k[i]);
+                sum = __dadd_rn(sum, __dmul_rn(__dmul_rn(delta, a.alpha[i]), in < width ? in : width));
+            }
+            terms[lane] = sum;
+        }
+        __syncwarp();
+        for (int i = 0; i < min(32, a.n_layers - l0); ++i) t = __dadd_rn(t, terms[i]);
+        __syncwarp();
     }
+    return t;
+}
+
+// Search (Section 3.4, Algorithm 1): the bracket [lo, hi] of prefix lengths is halved until the latencies of its
+// two ends are within eps of each other or it has width 1.  A round evaluates every prefix length the next
+// `depth` steps may ask for (2^depth - 1, a warp each), then the steps are taken one by one as printed:
+// a step costs a fifth of a round trip through the ranked list instead of a whole one.
+__global__ void __launch_bounds__(1024) search_kernel(const __grid_constant__ SearchArgs a)
+{
+    extern __shared__ __align__(16) unsigned char shared[];
+    __shared__ double node[32];
+    __shared__ long long bracket[2];
+    __shared__ double ends[2];
+    __shared__ int state[2];                // iterations, finished
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double* const terms = reinterpret_cast<double*>(shared) + warp * 32;
+    unsigned* const counts = reinterpret_cast<unsigned*>(shared + (blockDim.x >> 5) * 256) + (size_t)warp * a.n_layers;
+    if (warp < 2) {
+        const double t = latency_of_top(a, warp ? a.total : 0, counts, terms, lane);
+        if (lane == 0) { ends[warp] = t; bracket[warp] = warp ? a.total : 0; }
+    }
+    if (threadIdx.x == 0) state[0] = state[1] = 0;
+    __syncthreads();
+    for (;;) {
+        if (threadIdx.x == 0) state[1] = !(ends[1] - ends[0] > a.eps && bracket[1] - bracket[0] > 1);
+        __syncthreads();
+        if (state[1]) break;
+        const int id = warp + 1;            // node of the tree of possible steps: 1 is the next one, 2i / 2i + 1 follow "lower half" / "upper half"
+        if (id < 1 << a.depth) {
+            long long lo = bracket[0], hi = bracket[1];
+            for (int bit = 30 - __clz(id); bit >= 0; --bit) {
+                const long long mid = (lo + hi) / 2;
+                if ((id >> bit) & 1) lo = mid; else hi = mid;
+            }
+            const double t = hi - lo > 1 ? latency_of_top(a, (lo + hi) / 2, counts, terms, lane) : 0.0;
+            if (lane == 0) node[id] = t;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            long long lo = bracket[0], hi = bracket[1];
+            double t_lo = ends[0], t_hi = ends[1];
+            int id2 = 1, iters = state[0];
+            for (int d = 0; d < a.depth && t_hi - t_lo > a.eps && hi - lo > 1; ++d) {
+                const long long mid = (lo + hi) / 2;
+                const double t = node[id2];
+                if (t < a.t_budget) { t_lo = t; lo = mid; id2 = 2 * id2 + 1; } else { t_hi = t; hi = mid; id2 = 2 * id2; }
+                ++iters;
+            }
+            bracket[0] = lo; bracket[1] = hi;
+            ends[0] = t_lo; ends[1] = t_hi;
+            state[0] = iters;
+        }
+        __syncthreads();
+    }
+    if (warp == 0) {
+        const long long n = (bracket[0] + bracket[1]) / 2;
+        const double t = latency_of_top(a, n, counts, terms, lane);
+        for (int l = lane; l < a.n_layers; l += 32) a.kept[l] = counts[l];
+        if (lane == 0) {
+            *a.n_keep = n;
+            *a.result = {n, bracket[0], bracket[1], state[0], t};
+        }
+    }
+}
+
+// Page-locked staging of alcs_project_bisection (tables in, result out), shared by all calls: one call at a time.
+std::mutex g_staging_mu;
+void* g_staging = nullptr;
+size_t g_staging_bytes = 0;
+
+// Device memory of the calls: a pool of the library's own per device, which keeps up to kPoolKeep bytes between
+// calls (the device's default pool gives everything back at the first synchronisation, and a call then spends
+// more time in the driver than on the GPU).
+constexpr unsigned long long kPoolKeep = 64ull << 20;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[64] = {};
+
+cudaError_t pool_of(int dev, cudaMemPool_t* out)
+{
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pools[dev]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        cudaError_t e = cudaMemPoolCreate(&pool, &props);
+        unsigned long long keep = kPoolKeep;
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) return e;
+        g_pools[dev] = pool;
+    }
+    *out = g_pools[dev];
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -186,120 +367,125 @@ ALCS_API int alcs_project_bisection(const float* const* u_tilde, const int* cout
     auto blocks_for = [&](long long n) {
         return (unsigned)std::max<long long>(1, std::min<long long>((n + 255) / 256, (long long)sms * 16));
     };
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
 
-    // One stream-ordered allocation for everything: after the first call the memory comes back from
-    // the runtime's pool without touching the driver.
-    const long long n_buckets = (total + kRankBucket - 1) / kRankBucket;
+    // Host tables: group offsets, knots, slopes.
+    size_t knots = 0;
+    for (int l = 0; l < n_layers; ++l) knots += tabs[l].n_knots;
+    const size_t h_first = up((n_layers + 1) * 8), h_k = h_first + up((n_layers + 1) * 4), h_t = h_k + up(knots * 8), h_alpha = h_t + up(knots * 8);
+    const size_t h_tables = h_alpha + up(knots * 8), h_result = h_tables, h_kept = h_result + up(sizeof(SearchResult));
+    const size_t host_bytes = h_kept + up((size_t)n_layers * 8);
+    std::unique_lock<std::mutex> staging_lock(g_staging_mu);
+    if (g_staging_bytes < host_bytes) {
+        if (g_staging) cudaFreeHost(g_staging);
+        g_staging = nullptr;
+        g_staging_bytes = 0;
+        if (cudaMallocHost(&g_staging, host_bytes) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ALCS_ERR_ALLOC;
+        }
+        g_staging_bytes = host_bytes;
+    }
+    unsigned char* const host = static_cast<unsigned char*>(g_staging);
+    std::copy(off.begin(), off.end(), reinterpret_cast<long long*>(host));
+    {
+        int* first = reinterpret_cast<int*>(host + h_first);
+        long long* k = reinterpret_cast<long long*>(host + h_k);
+        double *t = reinterpret_cast<double*>(host + h_t), *alpha = reinterpret_cast<double*>(host + h_alpha);
+        int at = 0;
+        for (int l = 0; l < n_layers; ++l) {
+            first[l] = at;
+            for (int i = 0; i < tabs[l].n_knots; ++i, ++at) {
+                k[at] = tabs[l].k[i];
+                t[at] = tabs[l].t[i];
+                alpha[at] = i + 1 < tabs[l].n_knots ? (tabs[l].t[i + 1] - tabs[l].t[i]) / ((double)tabs[l].k[i + 1] - (double)tabs[l].k[i]) : 0.0;
+            }
+        }
+        first[n_layers] = at;
+    }
+
+    // One stream-ordered allocation for everything.
+    const long long n_buckets = std::max(1ll, (total + kRankBucket - 1) / kRankBucket);
     size_t sort_bytes = 0;
     ALCS_CUDA(cub::DeviceRadixSort::SortPairsDescending(nullptr, sort_bytes, (unsigned*)nullptr, (unsigned*)nullptr,
                                                        (unsigned*)nullptr, (unsigned*)nullptr, (int)total, 0, 32, st));
-    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-    const size_t b_keys = up((size_t)total * 4), b_lay = up((size_t)total * 2), b_off = up((size_t)(n_layers + 1) * 8);
-    const size_t b_hist = up((size_t)std::max<long long>(n_buckets, 1) * n_layers * 4);
-    const size_t bytes = 4 * b_keys + b_lay + b_off + b_hist + up(sort_bytes) + 256;
+    const size_t b_keys = up((size_t)total * 4), b_lay = up((size_t)total * 2), b_hist = up((size_t)n_buckets * n_layers * 4);
+    const size_t bytes = 4 * b_keys + b_lay + b_hist + h_tables + 256 + up(sort_bytes);
+    cudaMemPool_t mem = nullptr;
+    ALCS_CUDA(pool_of(dev, &mem));
     unsigned char* pool = nullptr;
-    if (cudaMallocAsync(&pool, bytes, st) != cudaSuccess) {
+    if (cudaMallocFromPoolAsync(reinterpret_cast<void**>(&pool), bytes, mem, st) != cudaSuccess) {
         (void)cudaGetLastError();
         return ALCS_ERR_ALLOC;
     }
+    // (an error on the way out: nothing may still write to the staging memory when the lock goes)
     struct Release {
-        unsigned char* p; cudaStream_t s;
-        ~Release() { cudaFreeAsync(p, s); }
-    } release{pool, st};
+        unsigned char* p; cudaStream_t s; bool waited;
+        ~Release() { cudaFreeAsync(p, s); if (!waited) cudaStreamSynchronize(s); }
+    } release{pool, st, false};
     unsigned* keys = (unsigned*)pool;
     unsigned* idx = (unsigned*)(pool + b_keys);
     unsigned* keys2 = (unsigned*)(pool + 2 * b_keys);
     unsigned* idx2 = (unsigned*)(pool + 3 * b_keys);
     unsigned short* layer_of = (unsigned short*)(pool + 4 * b_keys);
-    long long* d_off = (long long*)(pool + 4 * b_keys + b_lay);
-    unsigned* d_hist = (unsigned*)(pool + 4 * b_keys + b_lay + b_off);
-    void* sort_tmp = pool + 4 * b_keys + b_lay + b_off + b_hist;
+    unsigned* hist = (unsigned*)(pool + 4 * b_keys + b_lay);
+    unsigned char* tables = pool + 4 * b_keys + b_lay + b_hist;
+    long long* d_keep = (long long*)(tables + h_tables);
+    void* sort_tmp = tables + h_tables + 256;
 
     // Ranking (Algorithm 1: the groups of all layers sorted together by norm, largest first).  The radix
     // sort is stable, so equal keys stay in (layer, group) order.  Then, for the ranked list, the layer
-    // of every entry and, per bucket of kRankBucket consecutive ranks, how many entries each layer has.
-    for (int l = 0; l < n_layers; ++l) {
-        const long long n = off[l + 1] - off[l];
-        group_keys_kernel<<<blocks_for(n), 256, 0, st>>>(u_tilde[l], cout[l], cols[l], g, off[l], keys, idx);
+    // of every entry and, per bucket of kRankBucket consecutive ranks, how many entries each layer has
+    // before it: the latency of "the N best-ranked groups kept" depends on N through those counts only.
+    ALCS_CUDA(cudaMemcpyAsync(tables, host, h_tables, cudaMemcpyHostToDevice, st));
+    std::vector<LayerTable> launches((n_layers + kLayersPerLaunch - 1) / kLayersPerLaunch);
+    for (size_t i = 0; i < launches.size(); ++i) {
+        LayerTable& t = launches[i];
+        const int l0 = (int)i * kLayersPerLaunch;
+        t.n_layers = std::min(kLayersPerLaunch, n_layers - l0);
+        t.g = g;
+        for (int l = 0; l < t.n_layers; ++l) {
+            t.u[l] = u_tilde[l0 + l];
+            t.out[l] = u_out ? u_out[l0 + l] : nullptr;
+            t.cout[l] = cout[l0 + l];
+            t.cols[l] = cols[l0 + l];
+            t.off[l] = off[l0 + l];
+        }
+        t.off[t.n_layers] = off[l0 + t.n_layers];
+        t.total = t.off[t.n_layers] - t.off[0];
+        group_keys_kernel<<<blocks_for(t.total), 256, 0, st>>>(t, keys, idx);
     }
     ALCS_CUDA(cudaGetLastError());
     ALCS_CUDA(cub::DeviceRadixSort::SortPairsDescending(sort_tmp, sort_bytes, keys, keys2, idx, idx2, (int)total, 0, 32, st));
-    ALCS_CUDA(cudaMemcpyAsync(d_off, off.data(), (n_layers + 1) * 8, cudaMemcpyHostToDevice, st));
-    ranked_layer_kernel<<<blocks_for(total), 256, 0, st>>>(idx2, total, d_off, n_layers, layer_of);
+    ranked_layers_kernel<<<(unsigned)n_buckets, 256, n_layers * 4, st>>>(idx2, total, (const long long*)tables, n_layers, layer_of, hist);
+    prefix_kernel<<<(unsigned)((n_layers + 3) / 4), 128, 0, st>>>(hist, n_buckets, n_layers);
     ALCS_CUDA(cudaGetLastError());
-    if (n_buckets > 0) {
-        bucket_histogram_kernel<<<(unsigned)n_buckets, 256, n_layers * 4, st>>>(layer_of, total, n_layers, d_hist);
-        ALCS_CUDA(cudaGetLastError());
-    }
 
-    // The latency of "the N best-ranked groups kept" depends on N only through the number of kept
-    // groups per layer, a monotone step function of N.  One copy brings what is needed to evaluate it
-    // for any N on the host: the bucket histograms (turned into prefix counts) and the ranked list's
-    // layers, of which at most one bucket is scanned per evaluation.  No device work per search step.
-    // (page-locked staging memory, kept between calls: a copy into pageable memory is several times slower)
-    const size_t hist_bytes = (size_t)n_buckets * n_layers * 4, lay_bytes = (size_t)total * 2;
-    std::unique_lock<std::mutex> staging_lock(g_staging_mu);
-    if (g_staging_bytes < up(hist_bytes) + lay_bytes + 16) {
-        if (g_staging) cudaFreeHost(g_staging);
-        g_staging = nullptr;
-        g_staging_bytes = 0;
-        const size_t want = (up(hist_bytes) + lay_bytes + 16) * 5 / 4;
-        if (cudaMallocHost(&g_staging, want) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return ALCS_ERR_ALLOC;
-        }
-        g_staging_bytes = want;
-    }
-    const unsigned* hist = reinterpret_cast<const unsigned*>(g_staging);
-    const unsigned short* lay = reinterpret_cast<const unsigned short*>(static_cast<unsigned char*>(g_staging) + up(hist_bytes));
-    if (total > 0) {
-        ALCS_CUDA(cudaMemcpyAsync(g_staging, d_hist, hist_bytes, cudaMemcpyDeviceToHost, st));
-        ALCS_CUDA(cudaMemcpyAsync(static_cast<unsigned char*>(g_staging) + up(hist_bytes), layer_of, lay_bytes, cudaMemcpyDeviceToHost, st));
-    }
-    ALCS_CUDA(cudaStreamSynchronize(st));
-    std::vector<long long> prefix((size_t)(n_buckets + 1) * n_layers, 0);     // groups of layer l among ranks < b*kRankBucket
-    for (long long bk = 0; bk < n_buckets; ++bk)
-        for (int l = 0; l < n_layers; ++l)
-            prefix[(size_t)(bk + 1) * n_layers + l] = prefix[(size_t)bk * n_layers + l] + hist[(size_t)bk * n_layers + l];
-    std::vector<long long> counts(n_layers);
-    auto latency_of_top = [&](long long n) {
-        const long long bk = n / kRankBucket;
-        for (int l = 0; l < n_layers; ++l) counts[l] = prefix[(size_t)bk * n_layers + l];
-        for (long long i = bk * kRankBucket; i < n; ++i) ++counts[lay[(size_t)i]];
-        double t = tau;
-        for (int l = 0; l < n_layers; ++l) t += interpolate(tabs[l], (int64_t)counts[l] * g);
-        return t;
-    };
-
-    // Search: the bracket [lo, hi] of prefix lengths always has latency(lo) on the budget's near side
-    // as far as it is known and is halved until the latencies of its two ends are within eps of each
-    // other (Section 3.4, Algorithm 1); a bracket of width 1 cannot shrink further and also ends it.
-    long long lo = 0, hi = total;
-    double t_lo = latency_of_top(lo), t_hi = latency_of_top(hi);
-    int iters = 0;
-    while (t_hi - t_lo > eps && hi - lo > 1) {
-        const long long mid = (lo + hi) / 2;
-        const double t = latency_of_top(mid);
-        if (t < t_budget) { t_lo = t; lo = mid; } else { t_hi = t; hi = mid; }
-        ++iters;
-    }
-    const long long n_keep = (lo + hi) / 2;
-    const double t_final = latency_of_top(n_keep);      // (leaves the kept counts of the result in `counts`)
-
-    write_mask_kernel<<<blocks_for(total), 256, 0, st>>>(idx2, total, n_keep, mask_out);
+    SearchArgs a;
+    a.layer_of = layer_of; a.prefix = hist;
+    a.first_knot = (const int*)(tables + h_first); a.k = (const long long*)(tables + h_k);
+    a.t = (const double*)(tables + h_t); a.alpha = (const double*)(tables + h_alpha);
+    a.total = total; a.n_layers = n_layers; a.g = g;
+    a.tau = tau; a.t_budget = t_budget; a.eps = eps;
+    a.n_keep = d_keep;
+    a.result = reinterpret_cast<SearchResult*>(host + h_result);
+    a.kept = reinterpret_cast<long long*>(host + h_kept);
+    // as many warps as have room for their counts, in full levels of the tree of steps
+    const size_t per_warp = 256 + (size_t)n_layers * 4;
+    a.depth = 5;
+    while (a.depth > 1 && ((1u << a.depth) - 1) * per_warp > 40 * 1024) --a.depth;
+    const unsigned warps = std::max(2u, (1u << a.depth) - 1);
+    search_kernel<<<1, warps * 32, warps * per_warp, st>>>(a);
     ALCS_CUDA(cudaGetLastError());
-    if (u_out) {
-        for (int l = 0; l < n_layers; ++l) {
-            if (!u_out[l]) continue;
-            apply_mask_kernel<<<blocks_for((long long)cout[l] * cols[l]), 256, 0, st>>>(u_tilde[l], mask_out + off[l], cout[l], cols[l], g, u_out[l]);
-        }
-        ALCS_CUDA(cudaGetLastError());
-    }
+    for (const LayerTable& t : launches) apply_kernel<<<blocks_for(t.total), 256, 0, st>>>(t, keys, keys2, idx2, d_keep, mask_out);
+    ALCS_CUDA(cudaGetLastError());
     ALCS_CUDA(cudaStreamSynchronize(st));
+    release.waited = true;
+    const SearchResult& r = *a.result;
     if (kept_per_layer)
-        for (int l = 0; l < n_layers; ++l) kept_per_layer[l] = (int64_t)counts[l];
+        for (int l = 0; l < n_layers; ++l) kept_per_layer[l] = (int64_t)a.kept[l];
     if (result) {
-        result->n_keep = n_keep; result->n0 = lo; result->n1 = hi; result->iters = iters; result->latency = t_final;
+        result->n_keep = r.n_keep; result->n0 = r.lo; result->n1 = r.hi; result->iters = r.iters; result->latency = r.latency;
         result->n_groups = total;
     }
     return ALCS_OK;

@@ -437,8 +437,8 @@ __device__ __forceinline__ int channel_of(const TcLayer& y, int r) { return y.ch
 // The end of an item, 32 rows at a time: bias, residual, ReLU, one rounding, stores.  A warp stores 32 consecutive
 // pixels of one channel per instruction.  `lane_off` is the byte offset of this lane's pixel from `out` (and from
 // `res`, if there is one), which are the same for the whole warp, so that an address is one 32-bit addition.
-// any = false: rows row0 .. are channels row0 .. , and out points at row0; otherwise every row's channel is
-// looked up and out points at channel 0.
+// any = false: rows row0 .. row0 + rows are channels row0 .. , and out points at row0; otherwise every row's channel
+// is looked up and out points at channel 0.
 template <typename YT>
 __device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* out, const char* res, unsigned lane_off, unsigned bias, int row0,
                                         int rows, bool live, bool any)
@@ -460,7 +460,8 @@ __device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* 
                 if (h >= rows) break;
                 YT r[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) r[j] = __ldg(reinterpret_cast<const YT*>(res + (lane_off + (h + j) * pitch)));
+                for (int j = 0; j < 8; ++j)
+                    if (h + j < rows) r[j] = __ldg(reinterpret_cast<const YT*>(res + (lane_off + (h + j) * pitch)));
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[h + j] += (float)r[j];
             }
@@ -469,7 +470,8 @@ __device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* 
         for (int j = 0; j < 32; j += 8) {
             if (j >= rows) break;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) put(reinterpret_cast<YT*>(out + (lane_off + (j + k) * pitch)), fmaxf(v[j + k], floor));
+            for (int k = 0; k < 8; ++k)
+                if (j + k < rows) put(reinterpret_cast<YT*>(out + (lane_off + (j + k) * pitch)), fmaxf(v[j + k], floor));
         }
         return;
     }
@@ -714,7 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             const int row = (int)quad * 32 + lane, q0 = cur.pt() * y.ppt, q = q0 + row;
             const bool live = row < y.ppt && q < y.q;
             const int img0 = div_of(q0, y.hw), img = div_of(live ? q : q0, y.hw), p = (live ? q : q0) - img * y.hw.d;
-            const bool wide = sizeof(XT) == 4 || y.y32, any = y.chan || row0 + nr > y.cout;
+            const bool wide = sizeof(XT) == 4 || y.y32, any = y.chan;
             const unsigned ye = wide ? 4 : sizeof(XT);
             const unsigned lane_off = ((unsigned)(img - img0) * (unsigned)y.cout * (unsigned)y.hw.d + (unsigned)p) * ye;
             const size_t item_off = ((size_t)img0 * y.cout + (any ? 0 : row0)) * y.hw.d * ye;
@@ -731,7 +733,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             if (res && live) {      // what the end of the item will add: on its way while the item is multiplied
 #pragma unroll 1
                 for (int k = 0; k < nr; ++k) {
-                    const int c = any ? channel_of(y, row0 + k) : k;
+                    const int c = any ? channel_of(y, row0 + k) : row0 + k < y.cout ? k : -1;
                     if (c >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(res + (lane_off + (unsigned)c * (unsigned)y.hw.d * ye)));
                 }
             }
@@ -780,7 +782,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             for (int h = 0; h < nr; h += 32) {
                 if (whole) tmem_wait_ld(lo);
                 const unsigned off = lane_off + (any ? 0 : (unsigned)h * (unsigned)y.hw.d * ye);
-                const int rows = min(32, nr - h);
+                const int rows = min(32, any ? nr - h : min(nr, y.cout - row0) - h);      // (may be negative: nothing to store)
                 if (wide) store32<float>(lo, y, out, res, off, bias + h * 4, row0 + h, rows, live, any);
                 else store32<XT>(lo, y, out, res, off, bias + h * 4, row0 + h, rows, live, any);
                 __syncwarp();
