@@ -787,9 +787,11 @@ alcs::TcProblem tc_problem(const void* x, void* y, int n, int h, int wd, const f
     return {x, y, bias, residual, n, h, wd, h_in, wd_in, stride, 0, k, k, flags};
 }
 
-alcs::TcKey tc_key(const Plan& p, int stride)
+// Which form of the expanded weights a problem takes: strided layers, and small images that are staged as runs of
+// all columns, cannot use a tile's column list.
+alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& pr)
 {
-    const int k = stride > 1 ? 1 : 0;
+    const int k = pr.kh || alcs::tc_whole_images(w, pr) ? 1 : 0;
     return {p.tc_n, k, k};
 }
 
@@ -803,7 +805,7 @@ bool tc_strided_ok(const alcs_packed* w, const void* x, int n, int oh, int ow, i
 int launch_tc_plan(const alcs_packed* w, const Plan& p, const alcs::TcProblem& pr, cudaStream_t st)
 {
     alcs::TcPrep* t = nullptr;
-    const int rc = alcs::tc_prepare(w, tc_key(p, pr.stride), st, &t);
+    const int rc = alcs::tc_prepare(w, tc_key(w, p, pr), st, &t);
     return rc ? rc : alcs::tc_run(w, *t, pr, st);
 }
 
@@ -1461,7 +1463,7 @@ int stack_make_resident(alcs_stack* s)
             rc = ensure_canonical_on_device(w, nullptr);
         } else if (it.plan.tc_n) {
             alcs::TcPrep* t = nullptr;
-            rc = alcs::tc_prepare(w, tc_key(it.plan, it.layer.stride), nullptr, &t);
+            rc = alcs::tc_prepare(w, tc_key(w, it.plan, tc_problem(it)), nullptr, &t);
         } else {
             Schedule* sc = get_schedule(w, it.plan.kc, it.plan.n_rg, true, flavour_of(g_variants[it.plan.variant].v));
             rc = sc ? upload_schedule(w, sc, nullptr) : ALCS_ERR_ALLOC;
@@ -1525,7 +1527,7 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
     for (int i = 0; i < run.count; ++i) {
         const auto& it = s->items[first + i];
         alcs::TcPrep* t = nullptr;
-        rc = alcs::tc_prepare(it.layer.w, {it.plan.tc_n, 0, 0}, nullptr, &t);
+        rc = alcs::tc_prepare(it.layer.w, tc_key(it.layer.w, it.plan, tc_problem(it)), nullptr, &t);
         if (rc) return rc;
         alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
         for (int k16 : t->k16) us[i].push_back(alcs::tc_item_us(it.layer.w->dt, t->n, k16));
@@ -1905,8 +1907,9 @@ extern "C" ALCS_API int alcs_spconv1x1_noalloc(const alcs_packed* w, const void*
         if (plan.tc_n) {        // needs no scratch, but what does not fit it is refused whatever kernel the plan names
             const size_t row = (size_t)h * wd * w->elt();
             if (row % 16 != 0 && (size_t)n * w->cin * ((row + 15) / 16 * 16) > ALCS_NOALLOC_SCRATCH_BYTES) return ALCS_ERR_TOO_LARGE;
-            const alcs::TcPrep* t = alcs::tc_find(w, {plan.tc_n, 0, 0});
-            return t ? alcs::tc_run(w, *t, tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd), st) : ALCS_ERR_STATE;
+            const alcs::TcProblem pr = tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd);
+            const alcs::TcPrep* t = alcs::tc_find(w, tc_key(w, plan, pr));
+            return t ? alcs::tc_run(w, *t, pr, st) : ALCS_ERR_STATE;
         }
         auto si = w->sched.find(alcs::sched_key(plan.kc, plan.n_rg, flavour_of(g_variants[plan.variant].v)));
         if (si == w->sched.end() || !si->second.uploaded) return ALCS_ERR_STATE;

@@ -284,6 +284,15 @@ bool tc_patch_fits(const alcs_packed* w, const TcProblem& p, int n)
     return pl.vec_bytes >= 4 && 2 * 16ll * pl.pitch * (long long)w->elt() <= patch_room(w->dt, n);
 }
 
+// Small images whose rows do not start on copy boundaries (7x7): a tile takes whole images, of which the columns of
+// a chunk are one run of memory, if those runs keep to 16 bytes.
+bool tc_whole_images(const alcs_packed* w, const TcProblem& p)
+{
+    const size_t elt = w->elt(), row = (size_t)p.oh * p.ow * elt;
+    return !p.kh && row % 16 != 0 && (elt == 4 || row % 4 != 0 || (uintptr_t)p.x % 4 != 0) && row <= kTcM * elt && (uintptr_t)p.x % 16 == 0 &&
+           w->cin % 16 == 0;
+}
+
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out)
 {
     TcLayer& y = *out;
@@ -318,11 +327,7 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
         int vb = 16;
         while (vb > elt && (((size_t)y.hw.d * elt) % vb || (uintptr_t)p.x % vb)) vb >>= 1;
         y.vec_bytes = vb == 16 || (elt == 2 && vb > elt) ? vb : 0;      // (8 bytes of fp32: as single elements)
-        // Small images whose rows do not start on copy boundaries (7x7): a tile takes whole images, of which the
-        // columns of a chunk are one run of memory, if those runs keep to 16 bytes
-        if (y.vec_bytes == 0 && !t.cols && y.hw.d <= kTcM && (uintptr_t)p.x % 16 == 0 && (size_t)y.cin * y.hw.d * elt % 16 == 0 &&
-            (size_t)16 * y.hw.d * elt % 16 == 0 && y.cin % 16 == 0)
-            y.images = kTcM / y.hw.d;
+        if (!t.cols && tc_whole_images(w, p)) y.images = kTcM / y.hw.d;
     }
     y.ppt = y.images ? y.images * y.hw.d : kTcM;
     y.px_tiles = tc_div((y.q + y.ppt - 1) / y.ppt);
