@@ -136,11 +136,12 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
     {
         // the shared-memory attribute belongs to the kernel as loaded on a device
         static std::mutex mu;
-        static bool ready[64][6] = {};
+        static bool ready[64][3] = {};
         std::lock_guard<std::mutex> lk(mu);
-        bool& r = ready[w->device & 63][(key.kh ? 3 : 0) + (int)w->dt];
+        bool& r = ready[w->device & 63][(int)w->dt];
         if (!r) {
-            const cudaError_t e = prepare_tc(w->dt, key.kh > 0);
+            cudaError_t e = prepare_tc(w->dt, false);
+            if (e == cudaSuccess) e = prepare_tc(w->dt, true);
             if (e != cudaSuccess) return cuda_fail(e);
             r = true;
         }
