@@ -437,14 +437,13 @@ __device__ __forceinline__ int channel_of(const TcLayer& y, int r) { return y.ch
 // The end of an item, 32 rows at a time: bias, residual, ReLU, one rounding, stores.  A warp stores 32 consecutive
 // pixels of one channel per instruction.  `lane_off` is the byte offset of this lane's pixel from `out` (and from
 // `res`, if there is one), which are the same for the whole warp, so that an address is one 32-bit addition.
+// floor: 0 with ReLU, else NaN (fmaxf then returns the other operand); pitch: bytes from one channel to the next.
 // any = false: rows row0 .. row0 + rows are channels row0 .. , and out points at row0; otherwise every row's channel
 // is looked up and out points at channel 0.
 template <typename YT>
-__device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* out, const char* res, unsigned lane_off, unsigned bias, int row0,
-                                        int rows, bool live, bool any)
+__device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* out, const char* res, unsigned lane_off, unsigned pitch, float floor,
+                                        unsigned bias, int row0, int rows, bool live, bool any)
 {
-    const float floor = y.relu ? 0.0f : __int_as_float(0x7fffffff);      // (NaN: fmaxf returns the other operand)
-    const unsigned pitch = (unsigned)y.hw.d * (unsigned)sizeof(YT);
 #pragma unroll
     for (int j = 0; j < 32; j += 4) {
         float b[4];
@@ -469,9 +468,14 @@ __device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* 
 #pragma unroll
         for (int j = 0; j < 32; j += 8) {
             if (j >= rows) break;
+            if (j + 8 <= rows) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (j + k < rows) put(reinterpret_cast<YT*>(out + (lane_off + (j + k) * pitch)), fmaxf(v[j + k], floor));
+                for (int k = 0; k < 8; ++k) put(reinterpret_cast<YT*>(out + (lane_off + (j + k) * pitch)), fmaxf(v[j + k], floor));
+            } else {
+#pragma unroll
+                for (int k = 0; k < 7; ++k)
+                    if (j + k < rows) put(reinterpret_cast<YT*>(out + (lane_off + (j + k) * pitch)), fmaxf(v[j + k], floor));
+            }
         }
         return;
     }
@@ -506,7 +510,9 @@ __device__ __forceinline__ void store_bias(const TcLayer& y, char* out, const ch
     }
 }
 
-template <typename XT, bool PATCH, int L>
+// GENERAL: layers with a residual, sorted rows or fp32 output of 16-bit operands among them.  What they add to the
+// epilogue is a third of the kernel's code, and the roles' loops compete for the instruction caches as it is.
+template <typename XT, bool PATCH, bool GENERAL, int L>
 __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__ TcArgs<L> a)
 {
     using E = Elem<XT>;
@@ -716,16 +722,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             const int row = (int)quad * 32 + lane, q0 = cur.pt() * y.ppt, q = q0 + row;
             const bool live = row < y.ppt && q < y.q;
             const int img0 = div_of(q0, y.hw), img = div_of(live ? q : q0, y.hw), p = (live ? q : q0) - img * y.hw.d;
-            const bool wide = sizeof(XT) == 4 || y.y32, any = y.chan;
-            const unsigned ye = wide ? 4 : sizeof(XT);
+            const bool wide = sizeof(XT) == 4 || (GENERAL && y.y32), any = GENERAL && y.chan;
+            const unsigned ye = wide ? 4 : sizeof(XT), pitch = (unsigned)y.hw.d * ye;
+            const float floor = y.relu ? 0.0f : __int_as_float(0x7fffffff);
+            const int out_rows = any ? nr : min(nr, y.cout - row0);       // (may be negative: nothing to store)
             const unsigned lane_off = ((unsigned)(img - img0) * (unsigned)y.cout * (unsigned)y.hw.d + (unsigned)p) * ye;
             const size_t item_off = ((size_t)img0 * y.cout + (any ? 0 : row0)) * y.hw.d * ye;
             char* const out = static_cast<char*>(y.y) + item_off;
-            const char* const res = y.res ? static_cast<const char*>(y.res) + item_off : nullptr;
+            const char* const res = GENERAL && y.res ? static_cast<const char*>(y.res) + item_off : nullptr;
             if (groups == 0) {      // nothing kept: the sum is zero, and there is no accumulator to read it from
-                const char* r = y.res ? static_cast<const char*>(y.res) + (size_t)img0 * y.cout * y.hw.d * ye : nullptr;
+                const char* r = GENERAL && y.res ? static_cast<const char*>(y.res) + (size_t)img0 * y.cout * y.hw.d * ye : nullptr;
                 char* o = static_cast<char*>(y.y) + (size_t)img0 * y.cout * y.hw.d * ye;
-                if (wide) store_bias<float>(y, o, r, lane_off, row0, nr, live);
+                if (GENERAL && sizeof(XT) == 2 && wide) store_bias<float>(y, o, r, lane_off, row0, nr, live);
                 else store_bias<XT>(y, o, r, lane_off, row0, nr, live);
                 __syncwarp();
                 continue;
@@ -779,14 +787,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             const unsigned d = n_grp & 1u;
             if (whole) tmem_ld32(src + d * 128, lo);
 #pragma unroll 1
-            for (int h = 0; h < nr; h += 32) {
+            for (int h = 0; h < out_rows; h += 32) {
                 if (whole) tmem_wait_ld(lo);
-                const unsigned off = lane_off + (any ? 0 : (unsigned)h * (unsigned)y.hw.d * ye);
-                const int rows = min(32, any ? nr - h : min(nr, y.cout - row0) - h);      // (may be negative: nothing to store)
-                if (wide) store32<float>(lo, y, out, res, off, bias + h * 4, row0 + h, rows, live, any);
-                else store32<XT>(lo, y, out, res, off, bias + h * 4, row0 + h, rows, live, any);
+                const unsigned off = lane_off + (any ? 0 : (unsigned)h * pitch);
+                const int rows = min(32, out_rows - h);
+                if (GENERAL && sizeof(XT) == 2 && wide) store32<float>(lo, y, out, res, off, pitch, floor, bias + h * 4, row0 + h, rows, live, any);
+                else store32<XT>(lo, y, out, res, off, pitch, floor, bias + h * 4, row0 + h, rows, live, any);
                 __syncwarp();
-                if (whole && h + 32 < nr) {
+                if (whole && h + 32 < out_rows) {
                     tmem_ld32(src + d * 128 + h + 32, lo);
                 } else {
 #pragma unroll
@@ -934,7 +942,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-template <typename XT, bool PATCH, int L>
+template <typename XT, bool PATCH, bool GENERAL, int L>
 cudaError_t launch(const TcArgs<L>& a, int blocks, cudaStream_t st)
 {
     cudaLaunchConfig_t lc = {};
@@ -948,43 +956,46 @@ cudaError_t launch(const TcArgs<L>& a, int blocks, cudaStream_t st)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, tc_kernel<XT, PATCH, L>, a);
+    return cudaLaunchKernelEx(&lc, tc_kernel<XT, PATCH, GENERAL, L>, a);
 }
 
-template <typename XT, bool PATCH>
-cudaError_t launch_any(const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
+template <typename XT>
+cudaError_t launch_any(bool patch, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
 {
-    if (a.n_layers > 1) return launch<XT, PATCH, kTcMaxLayers>(a, blocks, st);
+    bool general = false;
+    for (int i = 0; i < a.n_layers; ++i) general = general || a.layer[i].res || a.layer[i].chan || (sizeof(XT) == 2 && a.layer[i].y32);
+    if (a.n_layers > 1) {
+        if (patch) return cudaErrorInvalidValue;      // (such layers are not merged)
+        return general ? launch<XT, false, true, kTcMaxLayers>(a, blocks, st) : launch<XT, false, false, kTcMaxLayers>(a, blocks, st);
+    }
     TcArgs<1> one;      // (a launch's arguments are copied by the driver: few layers, few bytes)
     one.n_layers = 1; one.n_items = a.n_items; one.sched = nullptr; one.stages = a.stages; one.stage_bytes = a.stage_bytes;
     one.slots = a.slots; one.slot_bytes = a.slot_bytes;
     one.layer[0] = a.layer[0];
-    return launch<XT, PATCH, 1>(one, blocks, st);
+    if (patch) return general ? launch<XT, true, true, 1>(one, blocks, st) : launch<XT, true, false, 1>(one, blocks, st);
+    return general ? launch<XT, false, true, 1>(one, blocks, st) : launch<XT, false, false, 1>(one, blocks, st);
 }
 
-template <typename XT, bool PATCH>
+template <typename XT>
 cudaError_t prepare()
 {
-    cudaError_t e = cudaFuncSetAttribute(tc_kernel<XT, PATCH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_kernel<XT, PATCH, kTcMaxLayers>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
-    return e;
+    const void* const fn[] = {(const void*)tc_kernel<XT, false, false, 1>, (const void*)tc_kernel<XT, false, true, 1>,
+                              (const void*)tc_kernel<XT, false, false, kTcMaxLayers>, (const void*)tc_kernel<XT, false, true, kTcMaxLayers>,
+                              (const void*)tc_kernel<XT, true, false, 1>, (const void*)tc_kernel<XT, true, true, 1>};
+    for (const void* f : fn) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTcSmem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
 
 cudaError_t launch_tc(int dt, bool patch, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
 {
-    if (patch)
-        return dt == 0 ? launch_any<float, true>(a, blocks, st)
-                       : dt == 1 ? launch_any<__half, true>(a, blocks, st) : launch_any<__nv_bfloat16, true>(a, blocks, st);
-    return dt == 0 ? launch_any<float, false>(a, blocks, st)
-                   : dt == 1 ? launch_any<__half, false>(a, blocks, st) : launch_any<__nv_bfloat16, false>(a, blocks, st);
+    return dt == 0 ? launch_any<float>(patch, a, blocks, st) : dt == 1 ? launch_any<__half>(patch, a, blocks, st) : launch_any<__nv_bfloat16>(patch, a, blocks, st);
 }
 
-cudaError_t prepare_tc(int dt, bool patch)
-{
-    if (patch) return dt == 0 ? prepare<float, true>() : dt == 1 ? prepare<__half, true>() : prepare<__nv_bfloat16, true>();
-    return dt == 0 ? prepare<float, false>() : dt == 1 ? prepare<__half, false>() : prepare<__nv_bfloat16, false>();
-}
+cudaError_t prepare_tc(int dt) { return dt == 0 ? prepare<float>() : dt == 1 ? prepare<__half>() : prepare<__nv_bfloat16>(); }
 
 }  // namespace alcs

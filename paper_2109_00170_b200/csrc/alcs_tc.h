@@ -84,7 +84,7 @@ struct TcArgs {
 // Launch a (n_layers <= kTcMaxLayers; one launch with elements of type dt) on `blocks` thread
 // blocks; patch: all layers by patch staging.
 cudaError_t launch_tc(int dt, bool patch, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st);
-cudaError_t prepare_tc(int dt, bool patch);      // once per device: shared-memory attribute
+cudaError_t prepare_tc(int dt);      // once per device: shared-memory attribute
 constexpr int tc_planes(int dt) { return dt == 0 ? 3 : 1; }      // 16-bit planes an operand is split into
 // ring of X chunks: 4 of 128 pixels x 64 columns in fp32, x 128 columns in 16 bits
 constexpr int kTcRingBytes = 4 * kTcM * 64 * 4;

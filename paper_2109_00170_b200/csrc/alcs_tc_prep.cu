@@ -140,8 +140,7 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         std::lock_guard<std::mutex> lk(mu);
         bool& r = ready[w->device & 63][(int)w->dt];
         if (!r) {
-            cudaError_t e = prepare_tc(w->dt, false);
-            if (e == cudaSuccess) e = prepare_tc(w->dt, true);
+            const cudaError_t e = prepare_tc(w->dt);
             if (e != cudaSuccess) return cuda_fail(e);
             r = true;
         }
