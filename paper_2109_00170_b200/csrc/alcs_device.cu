@@ -798,7 +798,11 @@ alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& p
 // Can the tcgen05 kernel take a strided layer (whatever the channels per tile)?
 bool tc_strided_ok(const alcs_packed* w, const void* x, int n, int oh, int ow, int stride, int h_in, int wd_in)
 {
-    return alcs::tc_patch_fits(w, tc_problem(x, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
+    // (rows of 4-byte copies only, as 16-bit 14x14 images have them, cost more than the gather pass of the other
+    // kernels: 31 us against 15 for 231 -> 604 channels, 14 x 14 at stride 2, batch 15, fp16)
+    const size_t row = (size_t)wd_in * w->elt();
+    return row % 8 == 0 && (uintptr_t)x % 8 == 0 &&
+           alcs::tc_patch_fits(w, tc_problem(x, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
 }
 
 // Launch the tcgen05 kernel for one layer; strided layers run by patch staging.
@@ -1020,6 +1024,73 @@ struct alcs_stack {
     void* xpad = nullptr;
     size_t xpad_bytes = 0;
 };
+
+namespace {
+
+// Streams and events with which one alcs_spconv1x1_host call overlaps its uploads, convolutions and downloads.
+// A call takes one from the device's list (or makes one) while it enqueues and puts it back; the list keeps at
+// most kMaxPipes.  Re-recording an event does not disturb waits that were enqueued on its earlier state.
+constexpr int kPipePieces = 4;
+constexpr size_t kMaxPipes = 8;
+struct CopyPipe {
+    cudaStream_t in = nullptr, out = nullptr;
+    cudaEvent_t start = nullptr, done = nullptr, uploaded[kPipePieces] = {}, computed[kPipePieces] = {};
+    bool make()
+    {
+        bool ok = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) == cudaSuccess;
+        auto event = [&](cudaEvent_t& e) { ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
+        event(start); event(done);
+        for (int i = 0; i < kPipePieces; ++i) { event(uploaded[i]); event(computed[i]); }
+        return ok;
+    }
+    ~CopyPipe()
+    {
+        for (cudaEvent_t e : {start, done}) if (e) cudaEventDestroy(e);
+        for (int i = 0; i < kPipePieces; ++i) {
+            if (uploaded[i]) cudaEventDestroy(uploaded[i]);
+            if (computed[i]) cudaEventDestroy(computed[i]);
+        }
+        if (in) cudaStreamDestroy(in);
+        if (out) cudaStreamDestroy(out);
+    }
+};
+std::mutex g_pipe_mu;
+std::vector<std::unique_ptr<CopyPipe>>* const g_pipes = new std::vector<std::unique_ptr<CopyPipe>>[64];     // (never destroyed: the CUDA runtime may be gone by then)
+
+struct PipeLease {
+    int dev;
+    std::unique_ptr<CopyPipe> pipe;
+    explicit PipeLease(int d) : dev(d)
+    {
+        {
+            std::lock_guard<std::mutex> lk(g_pipe_mu);
+            if (!g_pipes[dev].empty()) { pipe = std::move(g_pipes[dev].back()); g_pipes[dev].pop_back(); }
+        }
+        if (!pipe) {
+            pipe.reset(new (std::nothrow) CopyPipe());
+            if (pipe && !pipe->make()) { pipe.reset(); (void)cudaGetLastError(); }
+        }
+    }
+    ~PipeLease()
+    {
+        std::lock_guard<std::mutex> lk(g_pipe_mu);
+        if (pipe && g_pipes[dev].size() < kMaxPipes) g_pipes[dev].push_back(std::move(pipe));
+    }
+};
+
+// Images per piece of a host-buffer call: four pieces of at least half a megabyte whose X starts on 16-byte
+// boundaries; n if the call is too small to gain from overlapping its copies (a piece costs about 10 us of calls).
+int images_per_piece(int n, size_t x_image, size_t y_image)
+{
+    const size_t total = (x_image + y_image) * n;
+    const int pieces = (int)std::min<size_t>({(size_t)kPipePieces, total >> 19, (size_t)n});
+    if (pieces < 2) return n;
+    for (int p = (n + pieces - 1) / pieces; p < n; ++p)
+        if (x_image * p % 16 == 0 && y_image * p % 16 == 0) return p;
+    return n;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -1345,8 +1416,46 @@ ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void*
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     int rc = check_device(w);
     if (rc) return rc;
-    ALCS_CUDA(cudaMemcpyAsync(dx, x_host, xb, cudaMemcpyHostToDevice, st));
     if (bias_host) ALCS_CUDA(cudaMemcpyAsync(db, bias_host, (size_t)w->cout * 4, cudaMemcpyHostToDevice, st));
+    const size_t x_image = xb / n, y_image = yb / n;
+    const int per = images_per_piece(n, x_image, y_image);
+    const unsigned char* const xh = static_cast<const unsigned char*>(x_host);
+    unsigned char* const yh = static_cast<unsigned char*>(y_host);
+    if (per < n) {
+        // The bus carries both directions at once: piece i is downloaded while piece i + 1 is multiplied and piece
+        // i + 2 uploaded.  Everything is ordered after what is on cuda_stream now and before what comes next.
+        PipeLease lease(w->device);
+        if (CopyPipe* const pipe = lease.pipe.get()) {
+            ALCS_CUDA(cudaEventRecord(pipe->start, st));
+            ALCS_CUDA(cudaStreamWaitEvent(pipe->in, pipe->start, 0));
+            rc = ALCS_OK;
+            cudaError_t e = cudaSuccess;
+            auto ok = [&](cudaError_t c) { if (e == cudaSuccess) e = c; return e == cudaSuccess; };
+            for (int i = 0, at = 0; at < n && rc == ALCS_OK && e == cudaSuccess; ++i, at += per) {
+                const int m = std::min(per, n - at);
+                unsigned char* const px = dx + x_image * at;
+                unsigned char* const py = dy + y_image * at;
+                ok(cudaMemcpyAsync(px, xh + x_image * at, x_image * m, cudaMemcpyHostToDevice, pipe->in));
+                ok(cudaEventRecord(pipe->uploaded[i], pipe->in));
+                ok(cudaStreamWaitEvent(st, pipe->uploaded[i], 0));
+                if (e == cudaSuccess) rc = alcs_spconv1x1(w, px, py, m, h, wd, bias_host ? db : nullptr, flags, cuda_stream);
+                if (rc) break;
+                ok(cudaEventRecord(pipe->computed[i], st));
+                ok(cudaStreamWaitEvent(pipe->out, pipe->computed[i], 0));
+                ok(cudaMemcpyAsync(yh + y_image * at, py, y_image * m, cudaMemcpyDeviceToHost, pipe->out));
+            }
+            // (also on an error: the caller's stream must not run ahead of the copies that were enqueued)
+            for (cudaStream_t s : {pipe->in, pipe->out}) {
+                const cudaError_t a1 = cudaEventRecord(pipe->done, s), a2 = cudaStreamWaitEvent(st, pipe->done, 0);
+                ok(a1);
+                ok(a2);
+            }
+            if (rc) return rc;
+            ALCS_CUDA(e);
+            return ALCS_OK;
+        }
+    }
+    ALCS_CUDA(cudaMemcpyAsync(dx, x_host, xb, cudaMemcpyHostToDevice, st));
     rc = alcs_spconv1x1(w, dx, dy, n, h, wd, bias_host ? db : nullptr, flags, cuda_stream);
     if (rc) return rc;
     ALCS_CUDA(cudaMemcpyAsync(y_host, dy, yb, cudaMemcpyDeviceToHost, st));
