@@ -382,20 +382,28 @@ def alcs_spconv2d_plan(w: Packed, n: int, cin: int, h: int, wd: int, kh: int, kw
     return out.as_dict()
 
 
+_TABLE_DTYPE = np.dtype([("n", np.int32), ("pad", np.int32), ("k", np.uintp), ("t", np.uintp)])
+
+
 def _tables(tables):
-    """[(k, t), ...] -> (ctypes array of LatencyTable, keep-alive list)."""
+    """[(k, t), ...] -> (ctypes array of LatencyTable, keep-alive list).  The knots of all tables go into two
+    arrays and the structs are filled as one numpy array: a ctypes pointer per table costs several microseconds."""
     arr = (LatencyTable * len(tables))()
-    keep = []
-    for j, (k, t) in enumerate(tables):
-        ka = np.ascontiguousarray(k, dtype=np.int64)
-        ta = np.ascontiguousarray(t, dtype=np.float64)
-        if ka.shape != ta.shape or ka.ndim != 1:
+    if not tables:
+        return arr, []
+    ks, ts = [np.asarray(k) for k, _ in tables], [np.asarray(t) for _, t in tables]
+    for k, t in zip(ks, ts):
+        if k.shape != t.shape or k.ndim != 1:
             raise ValueError("latency table: k and t must be 1-D of equal length")
-        keep += [ka, ta]
-        arr[j].n_knots = ka.size
-        arr[j].k = ka.ctypes.data_as(C.POINTER(C.c_int64))
-        arr[j].t = ta.ctypes.data_as(C.POINTER(C.c_double))
-    return arr, keep
+    ka = np.concatenate(ks).astype(np.int64, copy=False)
+    ta = np.concatenate(ts).astype(np.float64, copy=False)
+    n = np.array([k.size for k in ks])
+    first = np.cumsum(n) - n
+    view = np.frombuffer(arr, dtype=_TABLE_DTYPE)
+    view["n"] = n
+    view["k"] = ka.ctypes.data + 8 * first
+    view["t"] = ta.ctypes.data + 8 * first
+    return arr, [ka, ta]
 
 
 def alcs_layer_latency(k, t, s: int) -> float:

@@ -149,14 +149,15 @@ __global__ void ranked_layers_kernel(const unsigned* __restrict__ idx, long long
     for (int i = threadIdx.x; i < n_layers; i += blockDim.x) hist[(size_t)blockIdx.x * n_layers + i] = h[i];
 }
 
-// hist[b][l] becomes the number of entries of layer l in the buckets before b (one warp per layer).
-__global__ void prefix_kernel(unsigned* __restrict__ hist, long long n_buckets, int n_layers)
+// hist[b][l] becomes the number of entries of layer l in the buckets before b (one thread block per layer, 1024
+// buckets per round: a warp per layer took 16 us for 767 buckets).
+__global__ void __launch_bounds__(1024) prefix_kernel(unsigned* __restrict__ hist, long long n_buckets, int n_layers)
 {
-    const int l = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (l >= n_layers) return;
+    __shared__ unsigned sums[32];
+    const int l = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned before = 0;
-    for (long long b0 = 0; b0 < n_buckets; b0 += 32) {
-        const long long b = b0 + lane;
+    for (long long b0 = 0; b0 < n_buckets; b0 += 1024) {
+        const long long b = b0 + threadIdx.x;
         const unsigned v = b < n_buckets ? hist[(size_t)b * n_layers + l] : 0u;
         unsigned s = v;
 #pragma unroll
@@ -164,8 +165,18 @@ __global__ void prefix_kernel(unsigned* __restrict__ hist, long long n_buckets, 
             const unsigned o = __shfl_up_sync(0xffffffffu, s, d);
             if (lane >= d) s += o;
         }
-        if (b < n_buckets) hist[(size_t)b * n_layers + l] = before + s - v;
-        before += __shfl_sync(0xffffffffu, s, 31);
+        if (lane == 31) sums[warp] = s;
+        __syncthreads();
+        unsigned w = sums[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned o = __shfl_up_sync(0xffffffffu, w, d);
+            if (lane >= d) w += o;
+        }
+        const unsigned mine = warp ? __shfl_sync(0xffffffffu, w, warp - 1) : 0u;
+        if (b < n_buckets) hist[(size_t)b * n_layers + l] = before + mine + s - v;
+        before += __shfl_sync(0xffffffffu, w, 31);
+        __syncthreads();
     }
 }
 
@@ -458,7 +469,7 @@ ALCS_API int alcs_project_bisection(const float* const* u_tilde, const int* cout
     ALCS_CUDA(cudaGetLastError());
     ALCS_CUDA(cub::DeviceRadixSort::SortPairsDescending(sort_tmp, sort_bytes, keys, keys2, idx, idx2, (int)total, 0, 32, st));
     ranked_layers_kernel<<<(unsigned)n_buckets, 256, n_layers * 4, st>>>(idx2, total, (const long long*)tables, n_layers, layer_of, hist);
-    prefix_kernel<<<(unsigned)((n_layers + 3) / 4), 128, 0, st>>>(hist, n_buckets, n_layers);
+    prefix_kernel<<<(unsigned)n_layers, 1024, 0, st>>>(hist, n_buckets, n_layers);
     ALCS_CUDA(cudaGetLastError());
 
     SearchArgs a;
