@@ -299,7 +299,9 @@ ALCS_API int alcs_spconv1x1_set_cfg(alcs_packed* w, int n, int h, int wd, unsign
  * alcs_spconv1x1_host: the same operation on HOST buffers x_host / y_host / bias_host, staged
  * through a caller-provided device workspace of at least alcs_spconv1x1_host_workspace() bytes
  * (256-byte aligned).  Enqueues H2D copies, the kernel and the D2H copy on cuda_stream and
- * returns without synchronising; use pinned host memory for truly asynchronous copies.
+ * returns without synchronising; use pinned host memory for truly asynchronous copies.  A call of a megabyte or
+ * more is cut into up to four pieces by images, whose uploads and downloads run on two streams of the library's own
+ * beside the convolutions, ordered by events after what is on cuda_stream and before what follows on it.
  */
 ALCS_API size_t alcs_spconv1x1_host_workspace(const alcs_packed* w, int n, int h, int wd, unsigned flags);
 ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void* y_host, int n, int h,
@@ -397,7 +399,10 @@ ALCS_API int alcs_probe_segment_loop(int g, int pixels_per_lane, int rows_per_wa
  * kernels wider than 8*stride+1, or so many input channels that not even a one-row strip of all of
  * them fits in shared memory), STATE, ALLOC, CUDA.
  *
- * alcs_spconv2d_plan reports the launch configuration alcs_spconv2d would use (host only).
+ * alcs_spconv2d runs on the fifth-generation tensor cores (as math_mode 4 of alcs_launch_cfg) wherever the input
+ * rows that 128 output pixels need fit shared memory for 16 channels at a time, kernels of at most 32 taps; else, and
+ * with an explicit configuration, on the CUDA-core kernel.  alcs_spconv2d_plan reports the CUDA-core kernel's launch
+ * configuration (host only).
  * ------------------------------------------------------------------------------------------- */
 typedef struct {
     int positions_per_lane;     /* output positions per lane (2, 4 or 8)                           */
@@ -463,8 +468,8 @@ ALCS_API int alcs_network_latency(double tau, const alcs_latency_table* tabs, in
  * DEVICE pointers, u_out[l] (may be NULL) receives u_tilde[l] with the dropped groups set to +0;
  * kept_per_layer (host, may be NULL) the number of kept groups per layer; *result (host, may be
  * NULL).  The call takes temporary device memory (about 18 bytes per group plus the sort's
- * workspace) from the device's stream-ordered memory pool and returns it there, copies 2 bytes per
- * group to the host for the search, and synchronises cuda_stream.
+ * workspace) from a stream-ordered pool of the library's own, which keeps up to 64 MB between calls, searches on
+ * the device, and synchronises cuda_stream once, at its end.
  * Errors: INVALID_ARG, SHAPE (2^31 or more groups), UNSUPPORTED (more than 4096 layers), ALLOC, CUDA.
  */
 typedef struct {
@@ -506,7 +511,11 @@ typedef struct {
  * Layers whose input rows are not a multiple of 16 bytes long are repacked into scratch memory that
  * the STACK owns (allocated by alcs_stack_create with the layers' device current, sized for its
  * largest such layer, released by alcs_stack_destroy): nothing a captured graph refers to is freed
- * or moved by later alcs_spconv1x1 calls with the same packed matrices, at any batch size.  Two runs
+ * or moved by later alcs_spconv1x1 calls with the same packed matrices, at any batch size.
+ * Consecutive layers on the fifth-generation tensor-core kernel (math_mode 4, up to 16 of one element type) none of
+ * which reads or writes what another one writes run as ONE launch, whose items (128 pixels x a channel tile) are
+ * dealt to the SMs by a list made when the stack is created; layers that do touch each other's buffers keep
+ * their order.  Two runs
  * of the same stack must not overlap on the GPU (they share that scratch and the outputs).
  */
 ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned stack_flags,

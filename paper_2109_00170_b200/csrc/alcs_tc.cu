@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     extern __shared__ __align__(1024) unsigned char smem[];
     const unsigned s0 = smem_u32(smem);
     const unsigned a_full = s0, a_empty = s0 + 32, d_full = s0 + 64, d_empty = s0 + 80, x_full = s0 + 128, x_empty = s0 + 192;
-    const unsigned b_full = s0 + 256, b_empty = s0 + 320, turn = s0 + 384, tmem_slot = s0 + 400;
+    const unsigned b_full = s0 + 256, b_empty = s0 + 320, turn = s0 + 384, tmem_slot = s0 + 400, drained = s0 + 408;
     const unsigned stage0 = s0 + kBarBytes, ring0 = stage0 + a.stages * a.stage_bytes;
     constexpr int NA = E::abufs, KC = P == 3 ? kTcKC32 : kTcKC16, NS = KC / 16, AB = KC / 2 * P;      // AB: TMEM columns of a chunk of A
     // every producer owns a slot
@@ -542,6 +542,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
             bar_init(turn + 8 * i, 1);
+            bar_init(drained + 8 * i, 1);
             bar_init(d_full + 8 * i, 1);
             bar_init(d_empty + 8 * i, kEpiWarps);
         }
@@ -865,6 +866,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     if (++buf == NA) { buf = 0; aph ^= 1u; }
                     if (++stage == (unsigned)a.stages) { stage = 0; ph ^= 1u; }
                 }
+            }
+            if (!ok) {      // gave up: see the MMAs in flight end before tensor memory is given back
+                mma_commit(drained + 8 * me);
+                (void)bar_wait(drained + 8 * me, 0);
             }
         }
         if (warp >= kProdWarp0 && warp < kProdWarp0 + (int)S) {

@@ -86,3 +86,44 @@ def test_merged_stack(alcs, graph):
         prev = Y
     assert all(alcs.alcs_packed_status(L["w"]) == 0 for L in layers)
     alcs.alcs_stack_destroy(st)
+
+
+# n, cin, cout, h, w, kh, kw, stride, pad: patches of one and of several images, rows copied by 16, 8 and 4 bytes,
+# channel blocks with a remainder, fewer taps than steps per chunk, borders on every side, more slots than one item uses
+PATCHES = [(2, 16, 16, 5, 6, 3, 3, 1, 1), (5, 33, 40, 7, 7, 3, 3, 1, 1), (3, 20, 130, 14, 14, 3, 3, 2, 1), (2, 70, 24, 28, 30, 1, 3, 1, 1),
+           (1, 17, 16, 9, 56, 5, 3, 2, 2), (9, 8, 12, 4, 3, 2, 2, 2, 0), (2, 130, 16, 11, 8, 1, 1, 1, 0)]
+
+
+@pytest.mark.parametrize("n,cin,cout,h,w,kh,kw,stride,pad", PATCHES)
+def test_patch_staging(alcs, n, cin, cout, h, w, kh, kw, stride, pad):
+    import torch
+    g, taps = 4, kh * kw
+    W, M, _, b = _case(3 * n + cin + h, n, cin * taps, cout, 1, g, 0.4)
+    X = rng.normal(n + cin, 2, n * cin * h * w).reshape(n, cin, h, w).astype(np.float32)
+    oh, ow = (h + 2 * pad - kh) // stride + 1, (w + 2 * pad - kw) // stride + 1
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    y = torch.full((n, cout, oh, ow), float("nan"), device="cuda:0")
+    alcs.alcs_spconv2d(p, torch.from_numpy(X).cuda(), y, n, cin, h, w, kh, kw, stride, pad, torch.from_numpy(b).cuda(),
+                       alcs.ALCS_RELU, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    Yref, A = oracle.conv2d(W.reshape(cout, cin, kh, kw), M, X, b, True, g, stride, pad, want_scale=True)
+    assert_parity(y.cpu().numpy(), Yref, A, "f32")
+    assert alcs.alcs_packed_status(p) == 0
+
+
+@pytest.mark.parametrize("n,cin,cout,h", [(3, 64, 96, 28), (16, 128, 160, 14), (13, 61, 300, 7), (41, 96, 96, 7)])
+def test_host_call_in_pieces(alcs, n, cin, cout, h):
+    """Calls large enough to be cut into pieces, among them sizes whose pieces cannot start on 16-byte boundaries."""
+    import torch
+    W, M, X, b = _case(n + cin, n, cin, cout, h * h, 4, 0.3)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+    size = alcs.alcs_spconv1x1_host_workspace(p, n, h, h, alcs.ALCS_RELU)
+    ws = torch.empty(size, dtype=torch.uint8, device="cuda:0")
+    xh, bh = torch.from_numpy(X).pin_memory(), torch.from_numpy(b).pin_memory()
+    yh = torch.full((n, cout, h * h), float("nan")).pin_memory()
+    stream = torch.cuda.Stream()
+    for _ in range(3):
+        alcs.alcs_spconv1x1_host(p, xh, yh, n, h, h, bh, alcs.ALCS_RELU, ws, size, stream)
+    stream.synchronize()
+    Yref, A = oracle.conv1x1(W, M, X, b, True, 4, want_scale=True)
+    assert_parity(yh.numpy(), Yref, A, "f32")
