@@ -79,7 +79,8 @@ struct Layout {
     long long k16 = 0;
 };
 
-void layout_of(const alcs_packed& w, int rows_per_tile, bool sorted, Layout& L)
+// all: take every column, where a tile keeps any (its column list is then not wanted, only whether it is empty)
+void layout_of(const alcs_packed& w, int rows_per_tile, bool sorted, bool all, Layout& L)
 {
     L.order.resize(w.rows);
     std::iota(L.order.begin(), L.order.end(), 0);
@@ -92,7 +93,12 @@ void layout_of(const alcs_packed& w, int rows_per_tile, bool sorted, Layout& L)
     std::vector<unsigned char> mark(w.cin);
     L.k16 = 0;
     for (int t = 0; t < tiles; ++t) {
-        union_of(w, L.order, t * rows_per_tile, std::min(w.rows, (t + 1) * rows_per_tile), mark, L.cols[t]);
+        const int r0 = t * rows_per_tile, r1 = std::min(w.rows, r0 + rows_per_tile);
+        if (all) {
+            if (w.row_ptr[r1] > w.row_ptr[r0]) L.cols[t].push_back(0);
+            continue;
+        }
+        union_of(w, L.order, r0, r1, mark, L.cols[t]);
         L.k16 += (L.cols[t].size() + 15) / 16;
     }
 }
@@ -152,11 +158,11 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         const int taps = std::max(1, key.kh * key.kw);
         const int dense16 = (w->cin / taps + 15) / 16 * taps;
         Layout L;
-        layout_of(*w, rpt, false, L);
+        layout_of(*w, rpt, false, key.kh > 0, L);
         bool sorted = false;
         if (!key.kh && skewed(*w)) {
             Layout S;
-            layout_of(*w, rpt, true, S);
+            layout_of(*w, rpt, true, false, S);
             if (S.k16 * 20 <= L.k16 * 19) { L = std::move(S); sorted = true; }
         }
         const int n_tiles = (int)L.cols.size();
