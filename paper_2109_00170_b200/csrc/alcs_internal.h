@@ -168,6 +168,9 @@ inline std::pair<int, int> sched_key(int kc, int n_rg, int flavour)
 // Device-side helpers implemented in alcs_device.cu, for the library's other translation units.
 int device_limits(int device, int* sms, int* smem_optin);                 // SM count, opt-in shared memory per block
 int schedule_upload(const alcs_packed* w, Schedule* sc, void* cuda_stream); // copy a schedule to w's device (once)
+// Stream-ordered device memory from a pool of the library's own (alcs_project.cu).
+int scratch_alloc(int device, size_t bytes, void* cuda_stream, void** out);
+void scratch_free(void* p, void* cuda_stream);
 int canonical_on_device(const alcs_packed* w, void* cuda_stream);           // device copy of row_ptr / col_idx / vals (once)
 int require_current_device(const alcs_packed* w);                          // ALCS_OK if w is uploaded and its device is current
 // bytes of one step record of the tensor-core flavour

@@ -15,7 +15,7 @@
 #include <mutex>
 #include <vector>
 
-#include "alcs.h"
+#include "alcs_internal.h"
 
 namespace alcs {
 void set_cuda_error_text(const char* s);
@@ -331,6 +331,23 @@ cudaError_t pool_of(int dev, cudaMemPool_t* out)
 
 }  // namespace
 
+namespace alcs {
+
+int scratch_alloc(int device, size_t bytes, void* cuda_stream, void** out)
+{
+    cudaMemPool_t mem = nullptr;
+    ALCS_CUDA(pool_of(device, &mem));
+    if (cudaMallocFromPoolAsync(out, bytes, mem, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ALCS_ERR_ALLOC;
+    }
+    return ALCS_OK;
+}
+
+void scratch_free(void* p, void* cuda_stream) { cudaFreeAsync(p, static_cast<cudaStream_t>(cuda_stream)); }
+
+}  // namespace alcs
+
 extern "C" {
 
 ALCS_API int alcs_layer_latency(const alcs_latency_table* tab, int64_t s, double* out)
@@ -422,13 +439,8 @@ ALCS_API int alcs_project_bisection(const float* const* u_tilde, const int* cout
                                                        (unsigned*)nullptr, (unsigned*)nullptr, (int)total, 0, 32, st));
     const size_t b_keys = up((size_t)total * 4), b_lay = up((size_t)total * 2), b_hist = up((size_t)n_buckets * n_layers * 4);
     const size_t bytes = 4 * b_keys + b_lay + b_hist + h_tables + 256 + up(sort_bytes);
-    cudaMemPool_t mem = nullptr;
-    ALCS_CUDA(pool_of(dev, &mem));
     unsigned char* pool = nullptr;
-    if (cudaMallocFromPoolAsync(reinterpret_cast<void**>(&pool), bytes, mem, st) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ALCS_ERR_ALLOC;
-    }
+    if (const int rc = alcs::scratch_alloc(dev, bytes, st, reinterpret_cast<void**>(&pool))) return rc;
     // (an error on the way out: nothing may still write to the staging memory when the lock goes)
     struct Release {
         unsigned char* p; cudaStream_t s; bool waited;

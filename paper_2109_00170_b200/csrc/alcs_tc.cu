@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         }
                         ok = __all_sync(0xffffffffu, ok);
                         if (!ok) break;
-                        const int r = div_of(tap, y.kwd), nv = y.cin - block * 16;
+                        const int r = div_of(tap, y.kwd), nv = y.cin - (cur.t.kstart + block) * 16;
                         const bool in = (mask >> tap) & 1u;
                         const int pitch = y.pitch * (int)sizeof(raw);
                         const unsigned at = ring0 + slot * kSlot + in_slot * 16 * pitch + (px + r * y.w_in + (tap - r * y.kw)) * (int)sizeof(raw);
@@ -888,7 +888,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 #pragma unroll 1
                     for (; mine < end; mine += S) {
                         const unsigned slot = mine % S;
-                        const int c0 = (mine - n) * y.blocks * 16;
+                        const int c0 = (cur.t.kstart + (int)(mine - n) * y.blocks) * 16;
                         ok = __all_sync(0xffffffffu, bar_wait(x_empty + 8 * slot, ((mine / S) & 1u) ^ 1u));
                         if (!ok) break;
                         copy_patch<XT>(y, t, ring0 + slot * kSlot, c0, min(y.blocks * 16, y.cin - c0), lane, x_full + 8 * slot);
@@ -947,6 +947,25 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
+// Memory-bound and short: one output per thread and step, consecutive threads on consecutive pixels.
+__global__ void __launch_bounds__(256) tc_reduce_kernel(const __grid_constant__ TcReduce a)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int hw = a.hw.d, n = a.width.d;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < (int)a.total; i += gridDim.x * 256) {
+        const int row = div_of(i, a.hw), p = i - row * hw;       // row = image * cout + channel
+        const int img = row / a.cout, c = row - img * a.cout;
+        const int tile = div_of(c, a.width), r = c - tile * n;
+        const float* q = a.part + (((size_t)img * a.tiles + tile) * a.splits * n + r) * hw + p;
+        float v = 0.0f;
+#pragma unroll 4
+        for (int s = 0; s < a.splits; ++s) v += __ldcg(q + (size_t)s * n * hw);
+        if (a.bias) v += __ldg(a.bias + c);
+        a.y[i] = a.relu ? fmaxf(v, 0.0f) : v;
+    }
+}
+
 template <typename XT, bool PATCH, bool GENERAL, int L>
 cudaError_t launch(const TcArgs<L>& a, int blocks, cudaStream_t st)
 {
@@ -999,6 +1018,21 @@ cudaError_t prepare()
 cudaError_t launch_tc(int dt, bool patch, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st)
 {
     return dt == 0 ? launch_any<float>(patch, a, blocks, st) : dt == 1 ? launch_any<__half>(patch, a, blocks, st) : launch_any<__nv_bfloat16>(patch, a, blocks, st);
+}
+
+cudaError_t launch_tc_reduce(const TcReduce& a, int sms, cudaStream_t st)
+{
+    cudaLaunchConfig_t lc = {};
+    const long long blocks = (a.total + 255) / 256;
+    lc.gridDim = dim3((unsigned)(blocks < 8ll * sms ? blocks : 8ll * sms));
+    lc.blockDim = dim3(256);
+    lc.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, tc_reduce_kernel, a);
 }
 
 cudaError_t prepare_tc(int dt) { return dt == 0 ? prepare<float>() : dt == 1 ? prepare<__half>() : prepare<__nv_bfloat16>(); }

@@ -20,7 +20,7 @@ constexpr int kTcMaxLayers = 16;     // layers one launch can take
 struct TcTile {
     unsigned b16;      // start of its weight tiles, in 16-byte units from TcLayer::b
     int k16;           // 16-column steps (0: the tile keeps nothing, output = bias)
-    int kstart;        // start of its column list
+    int kstart;        // start of its column list; patch staging: its first block of 16 channels
 };
 
 // Division of 0 <= n < 2^31 by a fixed d >= 1 as a multiplication: with 2^(s-1) < d <= 2^s and
@@ -80,6 +80,18 @@ struct TcArgs {
     int slots, slot_bytes;       // patch staging: X ring
     TcLayer layer[L];
 };
+
+// Sum of the partial results of a layer whose columns were split: part[image][tile][split][n][hw] over the splits in
+// order, bias, ReLU.
+struct TcReduce {
+    const float* part;
+    float* y;
+    const float* bias;
+    int n, splits, tiles, cout, relu;
+    TcDiv hw, width;             // width: channels per tile
+    long long total;             // outputs
+};
+cudaError_t launch_tc_reduce(const TcReduce& a, int sms, cudaStream_t st);
 
 // Launch a (n_layers <= kTcMaxLayers; one launch with elements of type dt) on `blocks` thread
 // blocks; patch: all layers by patch staging.

@@ -29,19 +29,22 @@ int cuda_fail(cudaError_t e)
 template <typename T, int P>
 __global__ void expand_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col_idx, const T* __restrict__ vals,
                               const int* __restrict__ place, const TcTile* __restrict__ tiles, const int* __restrict__ inv,
-                              int rows, int g, int n, int cols, int taps, unsigned char* __restrict__ b)
+                              int rows, int g, int n, int cols, int taps, int splits, int split_blocks, unsigned char* __restrict__ b)
 {
     const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (r >= rows) return;
     const int at = place[r], tile = at / n, n0 = at - tile * n;
-    const TcTile t = tiles[tile];
-    unsigned char* const bt = b + (size_t)t.b16 * 16;
     const int beg = row_ptr[r], cnt = row_ptr[r + 1] - beg;
     for (int i = threadIdx.x & 31; i < cnt * g; i += 32) {
         const int blk = i / g, j = i - blk * g;
         int k = col_idx[beg + blk];
         if (inv) k = inv[(size_t)tile * cols + k];
         else if (taps > 1) k = (k / taps / 16 * taps + k % taps) * 16 + k / taps % 16;      // [16 channels][tap]
+        // (a split tile: the part that has this block of channels, columns counted from its first)
+        const int part = splits > 1 ? k / (16 * taps) / split_blocks : 0;
+        k -= part * split_blocks * 16 * taps;
+        const TcTile t = tiles[tile * splits + part];
+        unsigned char* const bt = b + (size_t)t.b16 * 16;
         constexpr int KC = P == 3 ? kTcKC32 : kTcKC16;
         const int chunk = k / KC, ns = min(KC / 16, t.k16 - KC / 16 * chunk);
         unsigned char* d = bt + (size_t)chunk * (P * KC * 2) * n + ((size_t)((k % KC) >> 3) * n + n0 + j) * 16 + (k & 7) * 2;
@@ -120,7 +123,7 @@ bool skewed(const alcs_packed& w)
 
 TcPrep* tc_find(const alcs_packed* w, const TcKey& key)
 {
-    auto it = w->tc.find({key.n, key.kh, key.kw});
+    auto it = w->tc.find({key.n + key.splits * 1024, key.kh, key.kw});
     return it == w->tc.end() ? nullptr : it->second;
 }
 
@@ -165,31 +168,37 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
             layout_of(*w, rpt, true, false, S);
             if (S.k16 * 20 <= L.k16 * 19) { L = std::move(S); sorted = true; }
         }
-        const int n_tiles = (int)L.cols.size();
+        const int n_tiles = (int)L.cols.size(), splits = key.splits, n_blocks = dense16 / taps, split_blocks = (n_blocks + splits - 1) / splits;
         // A column list costs the converters its loads: without at least a tenth of the steps to save,
         // take all columns in order.
         const bool list = !key.kh && L.k16 * 10 <= (long long)dense16 * n_tiles * 9;
-        std::vector<TcTile> tiles(n_tiles);
+        std::vector<TcTile> tiles;
         std::vector<int> cols, inv, chan, place(w->rows);
         size_t bytes = 0;
         TcPrep p;
         p.n = n;
-        p.n_tiles = n_tiles;
+        p.n_tiles = n_tiles * splits;
+        p.splits = splits;
         p.k16_min = 1 << 30;
         for (int t = 0; t < n_tiles; ++t) {
             const int used = (int)L.cols[t].size();
             const int k16 = !list ? (used ? dense16 : 0) : (used + 15) / 16;
-            tiles[t] = {(unsigned)(bytes / 16), k16, (int)cols.size()};
+            const int list_start = (int)cols.size();
             if (list && used)
                 for (int i = 0; i < k16 * 16; ++i) cols.push_back(L.cols[t][std::min(i, used - 1)]);
             if (list) {
                 inv.resize((size_t)(t + 1) * w->cin, 0);
                 for (int i = 0; i < used; ++i) inv[(size_t)t * w->cin + L.cols[t][i]] = i;
             }
-            bytes += (size_t)P * k16 * 16 * n * 2;
-            p.k16.push_back(k16);
-            p.k16_max = std::max(p.k16_max, k16);
-            p.k16_min = std::min(p.k16_min, k16);
+            for (int part = 0; part < splits; ++part) {
+                const int first = part * split_blocks;
+                const int steps = splits == 1 || k16 == 0 ? k16 : std::max(0, std::min(split_blocks, n_blocks - first)) * taps;
+                tiles.push_back({(unsigned)(bytes / 16), steps, list ? list_start : splits > 1 ? first : 0});
+                bytes += (size_t)P * steps * 16 * n * 2;
+                p.k16.push_back(steps);
+                p.k16_max = std::max(p.k16_max, steps);
+                p.k16_min = std::min(p.k16_min, steps);
+            }
         }
         if (bytes / 16 > 0xffffffffull) return ALCS_ERR_SHAPE;
         for (int i = 0; i < w->rows; ++i) place[L.order[i]] = i / rpt * n + i % rpt * w->g;
@@ -222,11 +231,11 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
             const unsigned blocks = (unsigned)((w->rows + 3) / 4);
             if (w->dt == ALCS_F32)
                 expand_kernel<float, 3><<<blocks, 128, 0, st>>>(w->d_row_ptr, w->d_col_idx, static_cast<const float*>(w->d_vals), dp, dt, di,
-                                                               w->rows, w->g, n, w->cin, taps, d);
+                                                               w->rows, w->g, n, w->cin, taps, splits, split_blocks, d);
             else
                 expand_kernel<unsigned short, 1><<<blocks, 128, 0, st>>>(w->d_row_ptr, w->d_col_idx,
                                                                         static_cast<const unsigned short*>(w->d_vals), dp, dt, di,
-                                                                        w->rows, w->g, n, w->cin, taps, d);
+                                                                        w->rows, w->g, n, w->cin, taps, splits, split_blocks, d);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);      // (the host arrays go away; other streams may use the tiles)
@@ -240,7 +249,7 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         p.chan = chan.empty() ? nullptr : reinterpret_cast<int*>(d + o_chan);
         p.uploaded = true;
         TcPrep* kept = new TcPrep(p);
-        w->tc[{key.n, key.kh, key.kw}] = kept;
+        w->tc[{key.n + key.splits * 1024, key.kh, key.kw}] = kept;
         *out = kept;
     } catch (const std::bad_alloc&) {
         return ALCS_ERR_ALLOC;
@@ -303,7 +312,7 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
 {
     TcLayer& y = *out;
     y.x = p.x; y.y = p.y; y.bias = p.bias; y.res = p.res;
-    y.b = t.b; y.tiles = t.cols || t.k16_min != t.k16_max ? t.tiles : nullptr; y.k16 = t.k16_max; y.cols = t.cols; y.chan = t.chan;
+    y.b = t.b; y.tiles = t.cols || t.k16_min != t.k16_max || t.splits > 1 ? t.tiles : nullptr; y.k16 = t.k16_max; y.cols = t.cols; y.chan = t.chan;
     y.err = w->d_err;
     y.hw = tc_div(p.oh * p.ow);
     y.q = p.n * y.hw.d;
@@ -411,20 +420,57 @@ int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st)
     int sms = 0, smem = 0;
     int rc = device_limits(w->device, &sms, &smem);
     if (rc) return rc;
-    // the width whose rounds of items over the SMs take the least time
-    const int k16 = (w->cin / taps + 15) / 16 * taps;
-    int n = 0;
+    // The width, and the number of parts the channels are split into, that take the least time: rounds of items over
+    // the SMs, and for split columns the partial sums' way through memory and one more launch (3 us, then 2 TB/s each
+    // way).  Small batches leave most SMs idle otherwise: one 7 x 7 image of 512 channels is a chain of 72 chunks.
+    const int blocks = (w->cin / taps + 15) / 16;
+    const long long px = (p.n * hw + kTcM - 1) / kTcM;
+    int n = 0, splits = 1;
     double best = 0;
     for (int want = kTcMaxN; want >= 16; want -= 16) {
-        const int tiles = (w->cout + want - 1) / want, v = ((w->cout + tiles - 1) / tiles + 15) / 16 * 16;
-        const long long items = (p.n * hw + kTcM - 1) / kTcM * ((w->cout + v - 1) / v);
-        const double us = (double)((items + sms - 1) / sms) * tc_item_us(w->dt, v, k16);
-        if ((n == 0 || us < best) && tc_patch_fits(w, p, v)) { n = v; best = us; }
+        const int want_tiles = (w->cout + want - 1) / want, v = ((w->cout + want_tiles - 1) / want_tiles + 15) / 16 * 16;
+        if (!tc_patch_fits(w, p, v)) continue;
+        const int tiles = (w->cout + v - 1) / v;
+        for (int s = 1; s <= std::min(8, blocks); ++s) {
+            const int part = (blocks + s - 1) / s;
+            if ((blocks + part - 1) / part != s) continue;
+            const double bytes = (double)s * tiles * v * p.n * hw * 4;
+            if (s > 1 && (bytes > (32 << 20) || (double)p.n * hw * w->cout > 1e9)) break;
+            const long long items = px * tiles * s;
+            const double us = (double)((items + sms - 1) / sms) * tc_item_us(w->dt, v, part * taps) + (s > 1 ? 3.0 + bytes / 1.0e6 : 0.0);
+            if (n == 0 || us < best * 0.95) { n = v; splits = s; best = us; }
+        }
     }
     if (n == 0) return ALCS_ERR_UNSUPPORTED;
     TcPrep* t = nullptr;
-    rc = tc_prepare(w, {n, p.kh, p.kw}, st, &t);
-    return rc ? rc : tc_run(w, *t, p, st);
+    rc = tc_prepare(w, {n, p.kh, p.kw, splits}, st, &t);
+    if (rc) return rc;
+    if (splits == 1) return tc_run(w, *t, p, st);
+    const int tiles = t->n_tiles / splits;
+    void* part = nullptr;
+    rc = scratch_alloc(w->device, (size_t)t->n_tiles * n * p.n * hw * 4, st, &part);
+    if (rc) return rc;
+    TcProblem q = p;
+    q.y = part;
+    q.bias = nullptr;
+    q.flags = 0;
+    TcArgs<kTcMaxLayers> a;
+    a.n_layers = 1;
+    tc_fill(w, *t, q, &a.layer[0]);
+    a.layer[0].cout = t->n_tiles * n;       // every part of a tile writes rows of its own
+    rc = tc_finish(w, a, true);
+    if (!rc) rc = tc_launch(w, a, true, st);
+    if (!rc) {
+        TcReduce r;
+        r.part = static_cast<const float*>(part); r.y = static_cast<float*>(p.y); r.bias = p.bias;
+        r.n = p.n; r.splits = splits; r.tiles = tiles; r.cout = w->cout; r.relu = (p.flags & ALCS_RELU) ? 1 : 0;
+        r.hw = tc_div((int)hw); r.width = tc_div(n);
+        r.total = (long long)p.n * w->cout * hw;
+        const cudaError_t e = launch_tc_reduce(r, sms, st);
+        if (e != cudaSuccess) rc = cuda_fail(e);
+    }
+    scratch_free(part, st);
+    return rc;
 }
 
 // 32-bit arithmetic of the kernel: element offsets into X, byte offsets inside the images one tile touches.

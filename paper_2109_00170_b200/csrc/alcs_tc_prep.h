@@ -13,10 +13,12 @@ namespace alcs {
 // which the columns are reordered.
 struct TcKey {
     int n, kh, kw;
+    int splits = 1;      // patch staging: parts the channel blocks are split into, a tile of its own each
 };
 
 struct TcPrep {
-    int n = 0, n_tiles = 0;
+    int n = 0, n_tiles = 0;      // channels per tile; tiles, parts counted
+    int splits = 1;
     std::vector<int> k16;        // steps of each tile
     int k16_max = 0, k16_min = 0;
     bool uploaded = false;
