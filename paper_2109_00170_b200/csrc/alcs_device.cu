@@ -292,7 +292,8 @@ bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const Devic
     const double rounds = std::ceil((double)blocks / (sms * resident));
     const double batch_us = (p == 2 ? 0.55 : p == 4 ? 0.7 : 0.9) * (vec || p == 2 ? 1.0 : 1.3);
     const double bytes = (double)w->nb * n * tiles * 32.0 * p * 4;
-    pl.cost = 1e-6 * (2.6 + std::max(rounds * batches * batch_us, bytes / (vec ? 5.5e6 : 3.3e6)));
+    // (every further round of thread blocks pays its own start and its stores: 49 us for 20,000 blocks of 17 -> 169 @56)
+    pl.cost = 1e-6 * (2.6 + std::max(rounds * batches * batch_us + (rounds - 1) * 1.4, bytes / (vec ? 5.5e6 : 3.3e6)));
     *out = pl;
     return true;
 }
@@ -737,22 +738,25 @@ int ensure_canonical_on_device(const alcs_packed* w, cudaStream_t st)
 {
     std::lock_guard<std::mutex> lk(w->mu);
     if (w->d_row_ptr) return ALCS_OK;
-    int32_t *rp = nullptr, *ci = nullptr;
-    void* va = nullptr;
-    cudaError_t e = cudaMalloc(&rp, w->row_ptr.size() * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&ci, std::max<size_t>(w->col_idx.size() * 4, 16));
-    if (e == cudaSuccess) e = cudaMalloc(&va, std::max<size_t>(w->vals.size(), 16));
-    if (e == cudaSuccess) e = cudaMemcpyAsync(rp, w->row_ptr.data(), w->row_ptr.size() * 4, cudaMemcpyHostToDevice, st);
+    // one block for the three arrays: an allocation costs more than the copies
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t o_col = up(w->row_ptr.size() * 4), o_val = o_col + up(w->col_idx.size() * 4);
+    unsigned char* base = nullptr;
+    cudaError_t e = cudaMalloc(&base, o_val + std::max<size_t>(w->vals.size(), 16));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(base, w->row_ptr.data(), w->row_ptr.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !w->col_idx.empty())
-        e = cudaMemcpyAsync(ci, w->col_idx.data(), w->col_idx.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && !w->vals.empty()) e = cudaMemcpyAsync(va, w->vals.data(), w->vals.size(), cudaMemcpyHostToDevice, st);
+        e = cudaMemcpyAsync(base + o_col, w->col_idx.data(), w->col_idx.size() * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !w->vals.empty()) e = cudaMemcpyAsync(base + o_val, w->vals.data(), w->vals.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         alcs::set_cuda_error_text(cudaGetErrorString(e));
-        cudaFree(rp); cudaFree(ci); cudaFree(va);
+        cudaFree(base);
         (void)cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? ALCS_ERR_ALLOC : ALCS_ERR_CUDA;
     }
+    int32_t* const rp = reinterpret_cast<int32_t*>(base);
+    int32_t* const ci = reinterpret_cast<int32_t*>(base + o_col);
+    void* const va = base + o_val;
     w->d_col_idx = ci; w->d_vals = va;
     w->d_row_ptr = rp;
     return ALCS_OK;
@@ -1078,12 +1082,12 @@ struct PipeLease {
     }
 };
 
-// Images per piece of a host-buffer call: four pieces of at least half a megabyte whose X starts on 16-byte
+// Images per piece of a host-buffer call: four pieces of at least a megabyte whose X starts on 16-byte
 // boundaries; n if the call is too small to gain from overlapping its copies (a piece costs about 10 us of calls).
 int images_per_piece(int n, size_t x_image, size_t y_image)
 {
     const size_t total = (x_image + y_image) * n;
-    const int pieces = (int)std::min<size_t>({(size_t)kPipePieces, total >> 19, (size_t)n});
+    const int pieces = (int)std::min<size_t>({(size_t)kPipePieces, total >> 20, (size_t)n});
     if (pieces < 2) return n;
     for (int p = (n + pieces - 1) / pieces; p < n; ++p)
         if (x_image * p % 16 == 0 && y_image * p % 16 == 0) return p;
@@ -1147,7 +1151,7 @@ ALCS_API void alcs_packed_free(alcs_packed* p)
             for (auto& kv : p->tc) alcs::tc_free(kv.second);
             cudaFree(p->d_err);
             cudaFree(p->d_xpad);
-            cudaFree(p->d_row_ptr); cudaFree(p->d_col_idx); cudaFree(p->d_vals);
+            cudaFree(p->d_row_ptr);      // (the other two arrays lie in the same block)
             cudaSetDevice(prev);
         }
         (void)cudaGetLastError();

@@ -89,8 +89,9 @@ def test_merged_stack(alcs, graph):
 
 
 # n, cin, cout, h, w, kh, kw, stride, pad: patches of one and of several images, rows copied by 16, 8 and 4 bytes,
-# channel blocks with a remainder, fewer taps than steps per chunk, borders on every side, more slots than one item uses
-PATCHES = [(2, 16, 16, 5, 6, 3, 3, 1, 1), (5, 33, 40, 7, 7, 3, 3, 1, 1), (3, 20, 130, 14, 14, 3, 3, 2, 1), (2, 70, 24, 28, 30, 1, 3, 1, 1),
+# channel blocks with a remainder, fewer taps than steps per chunk, borders on every side, more slots than one item uses;
+# the first two have few pixels and many channels, so that their columns are split
+PATCHES = [(1, 200, 20, 7, 7, 3, 3, 1, 1), (2, 129, 150, 9, 8, 3, 3, 2, 1), (2, 16, 16, 5, 6, 3, 3, 1, 1), (5, 33, 40, 7, 7, 3, 3, 1, 1), (3, 20, 130, 14, 14, 3, 3, 2, 1), (2, 70, 24, 28, 30, 1, 3, 1, 1),
            (1, 17, 16, 9, 56, 5, 3, 2, 2), (9, 8, 12, 4, 3, 2, 2, 2, 0), (2, 130, 16, 11, 8, 1, 1, 1, 0)]
 
 
