@@ -453,17 +453,12 @@ __device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* 
     }
     if (!any) {
         if (!live) return;
-        if (res) {
+        if (res) {      // all loads, then all additions: one round trip to L2 per 32 rows
+            YT r[32];
 #pragma unroll
-            for (int h = 0; h < 32; h += 8) {
-                if (h >= rows) break;
-                YT r[8];
+            for (int j = 0; j < 32; ++j) r[j] = __ldg(reinterpret_cast<const YT*>(res + (lane_off + (j < rows ? j : 0) * pitch)));
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (h + j < rows) r[j] = __ldg(reinterpret_cast<const YT*>(res + (lane_off + (h + j) * pitch)));
-#pragma unroll
-                for (int j = 0; j < 8; ++j) v[h + j] += (float)r[j];
-            }
+            for (int j = 0; j < 32; ++j) v[j] += (float)r[j];
         }
 #pragma unroll
         for (int j = 0; j < 32; j += 8) {
