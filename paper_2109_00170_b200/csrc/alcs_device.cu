@@ -1526,11 +1526,13 @@ size_t merge_end(const alcs_stack* s, size_t first, F eligible)
 // Consecutive independent layers whose configuration nobody fixed: one launch of the tcgen05 kernel for all of
 // them, where its estimate is below the sum of the layers' own.  With few items in all, narrower tiles shorten
 // the longest SM's share; with many, wide ones do the least work.
-void stack_merge(alcs_stack* s)
+// fixed_too: of whatever was fixed, too (alcs_stack_tune).
+void stack_merge(alcs_stack* s, bool fixed_too = false)
 {
     auto open = [&](const alcs_stack::Item& it) {
         const alcs_layer& L = it.layer;
         if (L.stride > 1 || !alcs::tc_fits(L.w->cin, L.w->cout, L.n, (long long)L.h * L.wd, (long long)it.oh * it.ow, 1)) return false;
+        if (fixed_too) return true;
         std::lock_guard<std::mutex> lk(L.w->mu);
         return L.w->tuned.find(alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}) == L.w->tuned.end();
     };
@@ -1889,6 +1891,15 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
     cur = time_stack(s, st, e0, e1, reps);
     if (cur < 0) return ALCS_ERR_CUDA;
     if (us_before) *us_before = cur;
+    {   // one launch for all independent layers: no sequence of single-layer changes leads there
+        std::vector<Plan> keep;
+        for (const auto& it : s->items) keep.push_back(it.plan);
+        stack_merge(s, true);
+        const double t = time_stack(s, st, e0, e1, reps);
+        if (t > 0 && t < cur * 0.996) cur = t;
+        else
+            for (size_t i = 0; i < keep.size(); ++i) s->items[i].plan = keep[i];
+    }
     for (int pass = 0; pass < passes; ++pass) {
         bool changed = false;
         for (auto& it : s->items) {
