@@ -353,7 +353,8 @@ constexpr unsigned kStagedOnly = 0x10000u;
 // Another one: a strided input that the tcgen05 kernel cannot stage.
 constexpr unsigned kNoTc = 0x20000u;
 
-int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>& out, bool allow_small = true)
+// allow_tc: may the tcgen05 kernel be listed (its limits depend on the input, which this function does not see)?
+int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>& out, bool allow_small = true, bool allow_tc = true)
 {
     DeviceInfo di;
     int rc = device_info(w->device, &di);
@@ -440,7 +441,7 @@ int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>
             }
         }
     }
-    if (hw > 0 && alcs::tc_fits(w->cin, w->cout, q / hw, hw, hw, 1)) {
+    if (allow_tc && hw > 0 && alcs::tc_fits(w->cin, w->cout, q / hw, hw, hw, 1)) {
         int n[8];
         const int count = tc_widths(w, n);
         for (int i = 0; i < count; ++i) out.push_back(tc_plan(w, n[i], q, di.sms));
@@ -515,7 +516,7 @@ int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg
     }
     if (c && c->math_mode == 4) return ALCS_ERR_UNSUPPORTED;
     std::vector<Plan> all;
-    rc = enumerate_plans(w, q, hw, all, allow_small);
+    rc = enumerate_plans(w, q, hw, all, allow_small, allow_tc);
     if (rc) return rc;
     if (!c) { *out = all[0]; return ALCS_OK; }
     if (c->math_mode == 3 && !allow_small) return ALCS_ERR_UNSUPPORTED;
@@ -799,7 +800,8 @@ alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& p
     return {p.tc_n, k, k};
 }
 
-// Can the tcgen05 kernel take a strided layer (whatever the channels per tile)?
+// Can the tcgen05 kernel take a strided layer (whatever the channels per tile)?  The answer is part of the plan's key
+// (kNoTc), which holds the output size alone.
 bool tc_strided_ok(const alcs_packed* w, const void* x, int n, int oh, int ow, int stride, int h_in, int wd_in)
 {
     // (rows of 4-byte copies only, as 16-bit 14x14 images have them, cost more than the gather pass of the other
@@ -1644,7 +1646,8 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
         alcs::TcPrep* t = nullptr;
         rc = alcs::tc_prepare(it.layer.w, tc_key(it.layer.w, it.plan, tc_problem(it)), nullptr, &t);
         if (rc) return rc;
-        alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
+        rc = alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
+        if (rc) return rc;
         for (int k16 : t->k16) us[i].push_back(alcs::tc_item_us(it.layer.w->dt, t->n, k16));
     }
     rc = alcs::tc_finish(w0, a, false);

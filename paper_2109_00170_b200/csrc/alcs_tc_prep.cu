@@ -308,8 +308,12 @@ bool tc_whole_images(const alcs_packed* w, const TcProblem& p)
            w->cin % 16 == 0;
 }
 
+// UNSUPPORTED: beyond the kernel's 32-bit offsets, or rows that patch staging cannot copy (see tc_fits, tc_patch_fits).
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out)
 {
+    const int taps = std::max(1, p.kh * p.kw);
+    if (!tc_fits(w->cin / taps, w->cout, p.n, (long long)p.h_in * p.w_in, (long long)p.oh * p.ow, taps) || (p.kh && !tc_patch_fits(w, p, t.n)))
+        return ALCS_ERR_UNSUPPORTED;
     TcLayer& y = *out;
     y.x = p.x; y.y = p.y; y.bias = p.bias; y.res = p.res;
     y.b = t.b; y.tiles = t.cols || t.k16_min != t.k16_max || t.splits > 1 ? t.tiles : nullptr; y.k16 = t.k16_max; y.cols = t.cols; y.chan = t.chan;
@@ -407,8 +411,8 @@ int tc_run(const alcs_packed* w, const TcPrep& t, const TcProblem& p, cudaStream
 {
     TcArgs<kTcMaxLayers> a;
     a.n_layers = 1;
-    tc_fill(w, t, p, &a.layer[0]);
-    const int rc = tc_finish(w, a, p.kh > 0);
+    int rc = tc_fill(w, t, p, &a.layer[0]);
+    if (!rc) rc = tc_finish(w, a, p.kh > 0);
     return rc ? rc : tc_launch(w, a, p.kh > 0, st);
 }
 
@@ -456,9 +460,9 @@ int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st)
     q.flags = 0;
     TcArgs<kTcMaxLayers> a;
     a.n_layers = 1;
-    tc_fill(w, *t, q, &a.layer[0]);
+    rc = tc_fill(w, *t, q, &a.layer[0]);
     a.layer[0].cout = t->n_tiles * n;       // every part of a tile writes rows of its own
-    rc = tc_finish(w, a, true);
+    if (!rc) rc = tc_finish(w, a, true);
     if (!rc) rc = tc_launch(w, a, true, st);
     if (!rc) {
         TcReduce r;

@@ -1,0 +1,52 @@
+"""Which kernel a call is given, and what it does there: calls at the edge of what the tcgen05 kernel takes must run on
+another kernel (or be refused), and give what the oracle gives."""
+import numpy as np
+import pytest
+
+import oracle
+from alcs_workloads import rng
+from gpu_util import TOL, assert_parity, check_layer
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(seed, n, cin, cout, hw, g, density, dtype=np.float32):
+    rows = (cout + g - 1) // g
+    W = (rng.normal(seed, 1, cout * cin) * cin ** -0.5).reshape(cout, cin).astype(dtype)
+    X = rng.normal(seed, 2, n * cin * hw).reshape(n, cin, hw).astype(dtype)
+    M = (rng.uniform01(seed, 3, rows * cin) < density).astype(np.uint8).reshape(rows, cin)
+    return W, M, X, (0.1 * rng.normal(seed, 4, cout)).astype(np.float32)
+
+
+# n, cin, cout, h, wd, stride: rows of 26, 14 and 18 bytes; the first is large enough for the tensor cores to be the
+# planner's first choice where they can be had
+@pytest.mark.parametrize("n,cin,cout,h,wd,stride", [(64, 1024, 512, 13, 13, 2), (16, 512, 512, 7, 7, 2), (9, 300, 260, 11, 9, 3)])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_strided_rows_that_cannot_be_copied_by_words(alcs, n, cin, cout, h, wd, stride, bf16):
+    """16-bit rows of odd length: no tcgen05 plan, neither by default nor from a stride-1 call of the same output size."""
+    import torch
+    g = 8
+    W, M, X, b = _case(n + cin, n, cin, cout, h * wd, g, 0.5, np.float32 if bf16 else np.float16)
+    if bf16:
+        wb, xb = rng.to_bf16_bits(W), rng.to_bf16_bits(X)
+        W, X = oracle.bf16_decode(wb), oracle.bf16_decode(xb)
+        p = alcs.alcs_pack(wb, M, g, bf16=True)
+        xd = torch.from_numpy(xb.view(np.int16)).cuda().view(torch.bfloat16)
+    else:
+        p = alcs.alcs_pack(W, M, g)
+        xd = torch.from_numpy(X).cuda()
+    p = alcs.alcs_packed_upload(p, 0)
+    st, oh, ow = torch.cuda.current_stream(), -(-h // stride), -(-wd // stride)
+    xs = torch.zeros((n, cin, oh * ow), dtype=xd.dtype, device="cuda")
+    res = torch.zeros((n, cout, oh * ow), device="cuda")
+    y = torch.full((n, cout, oh * ow), float("nan"), device="cuda")
+    alcs.alcs_spconv1x1_ex(p, xs, y, n, oh, ow, 1, None, res, alcs.ALCS_Y_F32, st)
+    y.fill_(float("nan"))
+    alcs.alcs_spconv1x1_ex(p, xd, y, n, h, wd, stride, torch.from_numpy(b).cuda(), None, alcs.ALCS_Y_F32, st)
+    with pytest.raises(alcs.AlcsError) as e:
+        alcs.alcs_spconv1x1_ex(p, xd, y, n, h, wd, stride, None, None, alcs.ALCS_Y_F32, st, dict(math_mode=4))
+    assert e.value.status == alcs.ALCS_ERR_UNSUPPORTED
+    torch.cuda.synchronize()
+    Yref, A = oracle.conv1x1_ex(W, M, X.reshape(n, cin, h, wd), b, None, False, g, stride, want_scale=True)
+    assert_parity(y.cpu().numpy(), Yref, A, "f32")      # exact 16-bit products, fp32 sums and output
+    assert alcs.alcs_packed_status(p) == 0
