@@ -807,7 +807,7 @@ bool tc_strided_ok(const alcs_packed* w, const void* x, int n, int oh, int ow, i
     // (rows of 4-byte copies only, as 16-bit 14x14 images have them, cost more than the gather pass of the other
     // kernels: 31 us against 15 for 231 -> 604 channels, 14 x 14 at stride 2, batch 15, fp16)
     const size_t row = (size_t)wd_in * w->elt();
-    return row % 8 == 0 && (uintptr_t)x % 8 == 0 &&
+    return row % 8 == 0 && (uintptr_t)x % 8 == 0 && alcs::tc_fits(w->cin, w->cout, n, (long long)h_in * wd_in, (long long)oh * ow, 1) &&
            alcs::tc_patch_fits(w, tc_problem(x, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
 }
 

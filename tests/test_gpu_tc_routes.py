@@ -50,3 +50,25 @@ def test_strided_rows_that_cannot_be_copied_by_words(alcs, n, cin, cout, h, wd, 
     Yref, A = oracle.conv1x1_ex(W, M, X.reshape(n, cin, h, wd), b, None, False, g, stride, want_scale=True)
     assert_parity(y.cpu().numpy(), Yref, A, "f32")      # exact 16-bit products, fp32 sums and output
     assert alcs.alcs_packed_status(p) == 0
+
+
+def test_strided_input_beyond_32_bit_offsets(alcs):
+    """2.2e9 input elements: the plan cached for a stride-1 call of the same output size must not be taken."""
+    import torch
+    n, cin, cout, h, g, s = 688, 256, 16, 112, 8, 2
+    W, M, _, _ = _case(3, 1, cin, cout, 1, g, 0.5, np.float16)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    st, o = torch.cuda.current_stream(), h // s
+    small = torch.ones((n, cin, o * o), dtype=torch.float16, device="cuda")
+    y = torch.empty((n, cout, o * o), dtype=torch.float16, device="cuda")
+    alcs.alcs_spconv1x1_ex(p, small, y, n, o, o, 1, None, torch.zeros_like(y), 0, st)
+    torch.cuda.synchronize()
+    del small
+    x = torch.empty((n, cin, h * h), dtype=torch.float16, device="cuda").normal_()
+    assert x.numel() > 2 ** 31
+    alcs.alcs_spconv1x1_ex(p, x, y, n, h, h, s, None, None, 0, st)
+    torch.cuda.synchronize()
+    for i in (0, n // 2, n - 1):
+        Yref, A = oracle.conv1x1_ex(W, M, x[i:i + 1].cpu().numpy().reshape(1, cin, h, h), None, None, False, g, s, want_scale=True)
+        assert_parity(y[i:i + 1].cpu().numpy(), Yref, A, "f16")
+    assert alcs.alcs_packed_status(p) == 0
