@@ -45,7 +45,9 @@ constexpr int kBarBytes = kTcHeaderBytes, kEpiOff = 1024, kEpiBytes = 512;
 static_assert(kEpiOff + 4 * kEpiBytes <= kBarBytes, "header");
 constexpr int kMaxStages = 8;
 constexpr int kMaxTcSmem = 227 * 1024;
-constexpr unsigned kPolls = 1u << 18;
+// A bounded wait gives up after this many polls, about a second (the limit of the library's other kernels).  It is
+// only ever started behind griddepcontrol.wait, so that the time a predecessor still runs does not count against it.
+constexpr unsigned kPolls = 1u << 21;
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -564,6 +566,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 
     if (warp < kConvWarps) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConvRegs));
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         const unsigned quad = (unsigned)(warp & 3);
         const int s0_ = warp >> 2, row = quad * 32 + lane;       // a warp takes every fourth 16-column step
         unsigned i = 0, slot = 0, xph = 0, buf = 0, aph = 1;
@@ -811,6 +814,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProdRegs));
         constexpr int kIssuers = E::group == 1 ? 2 : 1;
         if (warp >= kMmaWarp && warp < kMmaWarp + kIssuers && elect_one()) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             const unsigned me = warp - kMmaWarp;
             unsigned n_chunk = 0, n_grp = 0, stage = 0, ph = 0, buf = 0, aph = 0;
             Cursor<L> cur(a);
@@ -917,6 +921,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 #pragma unroll 1
                 for (int k = 0; k < t.k16 && ok; k += NS) {
                     const unsigned bytes = (unsigned)(min(NS, t.k16 - k) * 16 * y.n * 2 * P);
+                    // (the weights do not depend on the kernel before this one: the first copies run ahead of its end)
+                    if (used == (unsigned)a.stages) asm volatile("griddepcontrol.wait;" ::: "memory");
                     ok = bar_wait(b_empty + 8 * stage, ph ^ 1u);
                     if (!ok) break;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b_full + 8 * stage), "r"(bytes) : "memory");

@@ -72,3 +72,27 @@ def test_strided_input_beyond_32_bit_offsets(alcs):
         Yref, A = oracle.conv1x1_ex(W, M, x[i:i + 1].cpu().numpy().reshape(1, cin, h, h), None, None, False, g, s, want_scale=True)
         assert_parity(y[i:i + 1].cpu().numpy(), Yref, A, "f16")
     assert alcs.alcs_packed_status(p) == 0
+
+
+def test_long_predecessor_does_not_exhaust_the_waits_of_its_successor(alcs):
+    """One pixel tile of many columns keeps one SM busy for milliseconds while the next launch, whose thread blocks
+    start on the idle SMs, has nothing to multiply yet; several in a row."""
+    import torch
+    cin, g = 1 << 18, 16
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(np.ones((16, cin), np.float32), np.ones((1, cin), np.uint8), g), 0)
+    x, y = torch.ones((1, cin, 16), device="cuda"), torch.empty((1, 16, 16), device="cuda")
+    W, M, X, _ = _case(8, 40, 64, 32, 196, 4, 0.5)
+    q = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+    xs, ys = torch.from_numpy(X).cuda(), torch.empty((40, 32, 196), device="cuda")
+    st = torch.cuda.current_stream()
+    for _ in range(3):
+        for _ in range(4):
+            alcs.alcs_spconv1x1(p, x, y, 1, 4, 4, None, 0, st, dict(math_mode=4))
+        ys.fill_(float("nan"))
+        alcs.alcs_spconv1x1(p, x, y, 1, 4, 4, None, 0, st, dict(math_mode=4))
+        alcs.alcs_spconv1x1(q, xs, ys, 40, 14, 14, None, 0, st, dict(math_mode=4))
+    torch.cuda.synchronize()
+    assert (y.cpu().numpy() == cin).all()
+    Yref, A = oracle.conv1x1(W, M, X, None, False, 4, want_scale=True)
+    assert_parity(ys.cpu().numpy(), Yref, A, "f32")
+    assert alcs.alcs_packed_status(p) == 0 and alcs.alcs_packed_status(q) == 0
