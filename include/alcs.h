@@ -186,8 +186,9 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     4 = fifth-generation tensor cores: the kept blocks of a tile of output channels are expanded
  *                     (once per packed matrix, on the device) to dense weight tiles and multiplied with 128-pixel
  *                     tiles of X; fp32 operands are split exactly into three bfloat16 parts each.  Only row_groups
- *                     (the number of channel tiles, each of at most 128 channels) applies; no scratch is used.  Non-finite
- *                     values of X reach all channels of the tile's outputs at that pixel, dropped blocks included
+ *                     (the number of channel tiles, each of at most 128 channels) applies; no scratch is used.  Outputs of
+ *                     pixels with infinite or NaN inputs are computed from the storage format instead, so that such values
+ *                     reach the channels that keep a block of theirs and no others, as with the other kernels (slowly)
  *   consumer_groups   1 = all consumer warps work on one work item at a time; 2 = two halves of the
  *                     consumer warps take the thread block's work items alternately (tensor-core
  *                     kernels only), so that one half multiplies while the other half stores

@@ -507,6 +507,103 @@ __device__ __forceinline__ void store_bias(const TcLayer& y, char* out, const ch
     }
 }
 
+template <typename XT> __device__ __forceinline__ bool special(typename Elem<XT>::raw v);      // infinite or not a number?
+template <> __device__ __forceinline__ bool special<float>(float v) { return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u; }
+template <> __device__ __forceinline__ bool special<__half>(unsigned short v) { return (v & 0x7c00u) == 0x7c00u; }
+template <> __device__ __forceinline__ bool special<__nv_bfloat16>(unsigned short v) { return (v & 0x7f80u) == 0x7f80u; }
+
+template <typename XT> __device__ __forceinline__ float value(typename Elem<XT>::raw v);
+template <> __device__ __forceinline__ float value<float>(float v) { return v; }
+template <> __device__ __forceinline__ float value<__half>(unsigned short v) { return __half2float(__ushort_as_half(v)); }
+template <> __device__ __forceinline__ float value<__nv_bfloat16>(unsigned short v) { return __uint_as_float((unsigned)v << 16); }
+
+// Where output pixel q reads X: the value of (channel, tap) is at base + channel * hw_in + r * w_in + s, inside the image
+// for taps whose (iy + r, ix + s) is.  (Not PATCH: one tap.)
+template <bool PATCH>
+struct Window {
+    int img, p, iy, ix;
+    size_t base;
+    __device__ __forceinline__ Window(const TcLayer& y, int q)
+    {
+        img = div_of(q, y.hw);
+        p = q - img * y.hw.d;
+        const int oy = PATCH ? div_of(p, y.ow) : 0;
+        iy = PATCH ? oy * y.stride - y.pad : 0;
+        ix = PATCH ? (p - oy * y.ow.d) * y.stride - y.pad : p;
+        base = (size_t)img * y.cin * y.hw_in;
+    }
+    __device__ __forceinline__ bool inside(const TcLayer& y, int r, int s) const
+    {
+        return !PATCH || ((unsigned)(iy + r) < (unsigned)y.h_in && (unsigned)(ix + s) < (unsigned)y.w_in);
+    }
+    __device__ __forceinline__ size_t at(const TcLayer& y, int c, int r, int s) const
+    {
+        return base + (size_t)c * y.hw_in + (PATCH ? (iy + r) * y.w_in + ix + s : ix);
+    }
+};
+
+// The block's items once more, for pixels with an infinite or NaN input.  The expanded weights multiply such a value with the
+// zeros of dropped blocks, too, and its parts do not add up to it: the whole tile is NaN there (which is how the
+// epilogue notices).  Here the pixel's outputs are computed from the storage format, which touches kept blocks alone,
+// and stored over what the epilogue stored.  At the end of the block, where no bounded wait of another role can run
+// out meanwhile.  Slow, one pixel per warp at a time, and of use only to outputs that are then mostly not finite.
+template <typename XT, bool PATCH, bool GENERAL, int L>
+__device__ __forceinline__ void recompute(const TcArgs<L>& a, unsigned layers, int quad, int half, int lane)
+{
+    using raw = typename Elem<XT>::raw;
+    Cursor<L> cur(a);
+#pragma unroll 1
+    while (cur.step()) {
+        const TcLayer& y = cur.of();
+        if (!(layers >> (L > 1 ? cur.layer : 0) & 1u) || cur.t.k16 == 0) continue;
+        const raw* const x = static_cast<const raw*>(y.x);
+        const int row = quad * 32 + lane, q0 = cur.pt() * y.ppt;
+        // channels of the item: all, or those of its part
+        const int c0 = PATCH ? cur.t.kstart * 16 : 0, c1 = PATCH ? min(y.cin, c0 + div_of(cur.t.k16, y.taps) * 16) : y.cin;
+        bool bad = false;
+        if (row < y.ppt && q0 + row < y.q) {
+            const Window<PATCH> w(y, q0 + row);
+#pragma unroll 1
+            for (int r = 0; r < (PATCH ? y.kh : 1); ++r)
+#pragma unroll 1
+                for (int s = 0; s < (PATCH ? y.kw : 1); ++s)
+                    if (w.inside(y, r, s))
+#pragma unroll 4
+                        for (int c = c0; c < c1; ++c) bad = bad || special<XT>(__ldg(x + w.at(y, c, r, s)));
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, bad);
+        if (!todo) continue;
+        const TcSparse sp = *y.sparse;
+        const int img0 = div_of(q0, y.hw), nt = cur.nt(), tile = nt / sp.splits;
+        const bool wide = sizeof(XT) == 4 || (GENERAL && y.y32);
+#pragma unroll 1
+        for (; todo; todo &= todo - 1) {
+            const Window<PATCH> w(y, q0 + quad * 32 + __ffs(todo) - 1);
+#pragma unroll 1
+            for (int j = half * 32 + lane; j < y.n; j += 64) {
+                const int c = GENERAL && y.chan ? __ldg(y.chan + nt * y.n + j) : tile * y.n + j;
+                if (c < 0 || c >= sp.cout) continue;
+                const int r = c / sp.g, in_block = c - r * sp.g;
+                float sum = 0.0f;
+#pragma unroll 2
+                for (int k = __ldg(sp.row_ptr + r), end = __ldg(sp.row_ptr + r + 1); k < end; ++k) {
+                    const int col = __ldg(sp.col_idx + k), ch = PATCH ? div_of(col, y.taps) : col, tap = PATCH ? col - ch * y.taps.d : 0;
+                    const int tr = PATCH ? div_of(tap, y.kwd) : 0, ts = PATCH ? tap - tr * y.kwd.d : 0;
+                    if (PATCH && (ch < c0 || ch >= c1 || !w.inside(y, tr, ts))) continue;
+                    sum = fmaf(value<XT>(__ldg(x + w.at(y, ch, tr, ts))), value<XT>(__ldg(static_cast<const raw*>(sp.vals) + (size_t)k * sp.g + in_block)), sum);
+                }
+                const int o = sp.splits > 1 ? nt * y.n + j : c;       // (parts write rows of their own)
+                const size_t at = ((size_t)w.img * y.cout + o) * y.hw.d + w.p;
+                if (y.bias) sum += __ldg(y.bias + c);
+                if (GENERAL && y.res) sum += wide ? __ldg(static_cast<const float*>(y.res) + at) : (float)__ldg(static_cast<const XT*>(y.res) + at);
+                if (y.relu) sum = fmaxf(sum, 0.0f);
+                if (wide) static_cast<float*>(y.y)[at] = sum;
+                else put(static_cast<XT*>(y.y) + at, sum);
+            }
+        }
+    }
+}
+
 // GENERAL: layers with a residual, sorted rows or fp32 output of 16-bit operands among them.  What they add to the
 // epilogue is a third of the kernel's code, and the roles' loops compete for the instruction caches as it is.
 template <typename XT, bool PATCH, bool GENERAL, int L>
@@ -519,6 +616,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     const unsigned s0 = smem_u32(smem);
     const unsigned a_full = s0, a_empty = s0 + 32, d_full = s0 + 64, d_empty = s0 + 80, x_full = s0 + 128, x_empty = s0 + 192;
     const unsigned b_full = s0 + 256, b_empty = s0 + 320, turn = s0 + 384, tmem_slot = s0 + 400, drained = s0 + 408;
+    const unsigned not_finite = s0 + 424;      // layers whose items had sums that are not finite, a bit each
     const unsigned stage0 = s0 + kBarBytes, ring0 = stage0 + a.stages * a.stage_bytes;
     constexpr int NA = E::abufs, KC = P == 3 ? kTcKC32 : kTcKC16, NS = KC / 16, AB = KC / 2 * P;      // AB: TMEM columns of a chunk of A
     // every producer owns a slot
@@ -553,6 +651,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             bar_init(x_full + 8 * i, 32);
             bar_init(x_empty + 8 * i, kConvWarps);
         }
+        asm volatile("st.shared.u32 [%0], 0;" ::"r"(not_finite) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_before();
@@ -788,6 +887,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 #pragma unroll 1
             for (int h = 0; h < out_rows; h += 32) {
                 if (whole) tmem_wait_ld(lo);
+                // (an input that is not finite reaches every channel of the tile, so one of them tells)
+                if (h == 0 && special<float>(lo[0])) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(not_finite), "r"(1u << (L > 1 ? cur.layer : 0)) : "memory");
                 const unsigned off = lane_off + (any ? 0 : (unsigned)h * pitch);
                 const int rows = min(32, out_rows - h);
                 if (GENERAL && sizeof(XT) == 2 && wide) store32<float>(lo, y, out, res, off, pitch, floor, bias + h * 4, row0 + h, rows, live, any);
@@ -810,6 +911,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 ++n_grp;
             }
         }
+        // (whichever warp stored an output, all have)
+        asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+        unsigned layers;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(layers) : "r"(not_finite));
+        if (layers) recompute<XT, PATCH, GENERAL, L>(a, layers, (int)quad, e, lane);
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProdRegs));
         constexpr int kIssuers = E::group == 1 ? 2 : 1;

@@ -36,6 +36,14 @@ inline TcDiv tc_div(int d)
     return {(unsigned)((1ull << (31 + s)) / (unsigned)d + 1), 31 + s, d};
 }
 
+// The layer's packed weights as they are stored, for the outputs that the tensor cores cannot give (see recompute).
+struct TcSparse {
+    const int* row_ptr;
+    const int* col_idx;
+    const void* vals;
+    int g, cout, splits;
+};
+
 struct TcLayer {
     const void* x;
     void* y;
@@ -46,6 +54,7 @@ struct TcLayer {
     int k16;
     const int* cols;             // input channel per entry of the tile's column list (null: all channels in order)
     const int* chan;             // output channel of row i of the tiles (null: i itself; -1: padding)
+    const TcSparse* sparse;      // device memory
     int* err;
     int first_item;              // items of this layer start here
     TcDiv n_tiles, px_tiles;     // channel tiles, pixel tiles

@@ -211,10 +211,12 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         // one device block: weights, then the small arrays (each on a 256-byte boundary); the inverse
         // column map and the places are needed by the expansion only
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-        const size_t o_tiles = up(bytes), o_cols = o_tiles + up(tiles.size() * sizeof(TcTile)), o_chan = o_cols + up(cols.size() * 4);
+        const TcSparse sparse = {w->d_row_ptr, w->d_col_idx, w->d_vals, w->g, w->cout, splits};
+        const size_t o_tiles = up(bytes), o_sparse = o_tiles + up(tiles.size() * sizeof(TcTile)), o_cols = o_sparse + up(sizeof sparse), o_chan = o_cols + up(cols.size() * 4);
         const size_t o_place = o_chan + up(chan.size() * 4), o_inv = o_place + up(place.size() * 4), end = o_inv + up(inv.size() * 4);
         std::vector<unsigned char> small(end - o_tiles);
         std::memcpy(small.data(), tiles.data(), tiles.size() * sizeof(TcTile));
+        std::memcpy(small.data() + (o_sparse - o_tiles), &sparse, sizeof sparse);
         std::memcpy(small.data() + (o_cols - o_tiles), cols.data(), cols.size() * 4);
         std::memcpy(small.data() + (o_chan - o_tiles), chan.data(), chan.size() * 4);
         std::memcpy(small.data() + (o_place - o_tiles), place.data(), place.size() * 4);
@@ -245,6 +247,7 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         }
         p.b = d;
         p.tiles = reinterpret_cast<TcTile*>(d + o_tiles);
+        p.sparse = reinterpret_cast<TcSparse*>(d + o_sparse);
         p.cols = list ? reinterpret_cast<int*>(d + o_cols) : nullptr;
         p.chan = chan.empty() ? nullptr : reinterpret_cast<int*>(d + o_chan);
         p.uploaded = true;
@@ -316,7 +319,7 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
         return ALCS_ERR_UNSUPPORTED;
     TcLayer& y = *out;
     y.x = p.x; y.y = p.y; y.bias = p.bias; y.res = p.res;
-    y.b = t.b; y.tiles = t.cols || t.k16_min != t.k16_max || t.splits > 1 ? t.tiles : nullptr; y.k16 = t.k16_max; y.cols = t.cols; y.chan = t.chan;
+    y.b = t.b; y.tiles = t.cols || t.k16_min != t.k16_max || t.splits > 1 ? t.tiles : nullptr; y.k16 = t.k16_max; y.cols = t.cols; y.chan = t.chan; y.sparse = t.sparse;
     y.err = w->d_err;
     y.hw = tc_div(p.oh * p.ow);
     y.q = p.n * y.hw.d;

@@ -27,6 +27,7 @@ struct TcPrep {
     TcTile* tiles = nullptr;
     int* cols = nullptr;         // null: every tile takes all columns
     int* chan = nullptr;         // null: identity
+    TcSparse* sparse = nullptr;
 };
 
 // The problem a launch solves (one layer), everything but the weights.

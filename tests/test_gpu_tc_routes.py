@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 from alcs_workloads import rng
-from gpu_util import TOL, assert_parity, check_layer
+from gpu_util import TOL, assert_parity, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -96,3 +96,117 @@ def test_long_predecessor_does_not_exhaust_the_waits_of_its_successor(alcs):
     Yref, A = oracle.conv1x1(W, M, X, None, False, 4, want_scale=True)
     assert_parity(ys.cpu().numpy(), Yref, A, "f32")
     assert alcs.alcs_packed_status(p) == 0 and alcs.alcs_packed_status(q) == 0
+
+
+def _with_specials(X, seed, share=1e-3):
+    """X with infinities of both signs and NaNs among its values: scattered, and one pixel of nothing else."""
+    X = X.copy()
+    flat = X.reshape(-1)
+    u = rng.uniform01(seed, 9, flat.size)
+    for k, v in enumerate((np.inf, -np.inf, np.nan)):
+        flat[(u >= k * share) & (u < (k + 1) * share)] = v
+    X[-1, :, -1] = np.inf
+    return X
+
+
+def _kept_blocks_reference(W, M, X, b, g, residual=None):
+    """Sums over the kept blocks alone, [n, cout, pixels] in float64, and the scale of their finite part.  (The oracle is
+    dense: there 0 times an infinity is NaN for dropped blocks, too.)  W [cout, columns], X [n, columns, pixels]."""
+    cout = W.shape[0]
+    keep = np.repeat(M != 0, g, axis=0)[:cout]
+    Wm, X = np.where(keep, W, 0).astype(np.float64), X.astype(np.float64)
+    finite = np.where(np.isfinite(X), X, 0.0)
+    base = 0.0 if b is None else b[None, :, None].astype(np.float64)
+    Y, A = np.matmul(Wm, finite) + base, np.matmul(np.abs(Wm), np.abs(finite)) + np.abs(base)
+    if residual is not None:
+        Y, A = Y + residual, A + np.abs(residual)
+    hits = lambda w, x: np.matmul(w.astype(np.float64), x.astype(np.float64)) > 0
+    up, down, zero = keep & (Wm > 0), keep & (Wm < 0), keep & (Wm == 0)
+    pos = hits(up, X == np.inf) | hits(down, X == -np.inf)
+    neg = hits(up, X == -np.inf) | hits(down, X == np.inf)
+    nan = hits(keep, np.isnan(X)) | hits(zero, np.isinf(X)) | (pos & neg)
+    Y[pos], Y[neg], Y[nan] = np.inf, -np.inf, np.nan
+    return Y, A
+
+
+def _assert_special(Y, Yref, A, kind, relu=False):
+    """Finite where the kept blocks meet finite values only, else the same infinity, or NaN (which a ReLU makes 0)."""
+    Y = Y.reshape(Yref.shape).astype(np.float64)
+    nan, inf = np.isnan(Yref), np.isinf(Yref)
+    if relu:
+        Yref = np.where(nan, Yref, np.maximum(Yref, 0.0))
+    assert (Y[nan] == 0).all() if relu else np.isnan(Y[nan]).all()
+    assert np.array_equal(Y[inf], Yref[inf])
+    ok = ~nan & ~inf
+    assert (np.abs(Y[ok] - Yref[ok]) <= TOL[kind] * A[ok]).all()
+    assert not ok.all() and ok.any()
+
+
+# n, cin, cout, h, wd, g, density: word and element copies, whole images, sorted rows with column lists, several chunks
+@pytest.mark.parametrize("n,cin,cout,h,wd,g,density", [(3, 100, 150, 14, 14, 4, 0.3), (5, 65, 40, 9, 9, 2, 0.4), (7, 64, 260, 7, 7, 8, 0.3),
+                                                      (2, 300, 128, 16, 16, 4, 0.0), (40, 200, 64, 12, 12, 1, 0.2)])
+@pytest.mark.parametrize("dtype", [np.float32, np.float16])
+@pytest.mark.parametrize("relu", [False, True])
+def test_infinite_and_nan_inputs_touch_kept_blocks_alone(alcs, n, cin, cout, h, wd, g, density, dtype, relu):
+    W, M, X, b = _case(n + cin + cout, n, cin, cout, h * wd, g, density, dtype)
+    if density == 0.0:
+        M = (np.arange(cin)[None, :] < 1 + (np.arange(M.shape[0])[:, None] * 7) ** 2 % cin).astype(np.uint8)
+    X = _with_specials(X, n)
+    Yref, A = _kept_blocks_reference(W, M, X, b, g)
+    for y_f32 in {False, dtype == np.float16}:
+        Y = run_gpu(alcs, W, M, X, b, relu, g, cfg=dict(math_mode=4), y_f32=y_f32, h=h, wd=wd)
+        _assert_special(Y, Yref, A, "f32" if dtype == np.float32 else "f16", relu)
+
+
+@pytest.mark.parametrize("stride,dtype", [(1, np.float32), (2, np.float32), (2, np.float16)])
+def test_infinite_and_nan_inputs_with_stride_and_residual(alcs, stride, dtype):
+    import torch
+    n, cin, cout, h, wd, g = 3, 72, 96, 12, 16, 8
+    W, M, X, b = _case(stride, n, cin, cout, h * wd, g, 0.4, dtype)
+    X = _with_specials(X, 5)
+    oh, ow = -(-h // stride), -(-wd // stride)
+    R = rng.normal(6, 5, n * cout * oh * ow).reshape(n, cout, oh * ow).astype(dtype)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    y = torch.zeros((n, cout, oh * ow), dtype=torch.float32 if dtype == np.float32 else torch.float16, device="cuda")
+    alcs.alcs_spconv1x1_ex(p, torch.from_numpy(X).cuda(), y, n, h, wd, stride, torch.from_numpy(b).cuda(), torch.from_numpy(R).cuda(), 0,
+                           torch.cuda.current_stream(), dict(math_mode=4))
+    torch.cuda.synchronize()
+    Xs = X.reshape(n, cin, h, wd)[:, :, ::stride, ::stride].reshape(n, cin, oh * ow)
+    _assert_special(y.cpu().numpy(), *_kept_blocks_reference(W, M, Xs, b, g, R), "f32" if dtype == np.float32 else "f16")
+
+
+@pytest.mark.parametrize("n,cin,cout,h,w,k,stride,pad", [(1, 200, 20, 7, 7, 3, 1, 1), (3, 20, 130, 14, 14, 3, 2, 1), (2, 33, 40, 9, 8, 3, 1, 0)])
+def test_infinite_and_nan_inputs_of_a_kxk_layer(alcs, n, cin, cout, h, w, k, stride, pad):
+    """(The first is small enough for its columns to be split.)"""
+    import torch
+    g = 4
+    W, M, _, b = _case(n + cin, n, cin * k * k, cout, 1, g, 0.3)
+    X = _with_specials(rng.normal(n + cin, 2, n * cin * h * w).reshape(n, cin, h * w).astype(np.float32), 7, 3e-4).reshape(n, cin, h, w)
+    oh, ow = (h + 2 * pad - k) // stride + 1, (w + 2 * pad - k) // stride + 1
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    y = torch.zeros((n, cout, oh, ow), device="cuda")
+    alcs.alcs_spconv2d(p, torch.from_numpy(X).cuda(), y, n, cin, h, w, k, k, stride, pad, torch.from_numpy(b).cuda(), 0, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    columns = torch.nn.functional.unfold(torch.from_numpy(X), k, padding=pad, stride=stride).numpy()
+    _assert_special(y.cpu().numpy(), *_kept_blocks_reference(W, M, columns, b, g), "f32")
+
+
+def test_infinite_inputs_of_one_layer_of_a_merged_stack(alcs):
+    import torch
+    layers, keep = [], []
+    for i, (n, cin, cout, h) in enumerate([(2, 64, 96, 14), (3, 80, 48, 7), (2, 32, 160, 28)]):
+        W, M, X, b = _case(60 + i, n, cin, cout, h * h, 4, 0.3)
+        if i == 1:
+            X = _with_specials(X, 3)
+        p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+        alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, dict(math_mode=4))
+        layers.append(dict(w=p, x=torch.from_numpy(X).cuda(), y=torch.zeros((n, cout, h * h), device="cuda"), n=n, h=h, wd=h,
+                           bias=torch.from_numpy(b).cuda(), flags=0))
+        keep.append((X, oracle.conv1x1(W, M, X, b, False, 4, want_scale=True) if i != 1 else _kept_blocks_reference(W, M, X, b, 4)))
+    st = alcs.alcs_stack_create(layers, 0)
+    for _ in range(2):
+        alcs.alcs_stack_run(st, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    for L, (X, (Yref, A)) in zip(layers, keep):
+        (assert_parity if np.isfinite(X).all() else _assert_special)(L["y"].cpu().numpy(), Yref, A, "f32")
+    alcs.alcs_stack_destroy(st)
