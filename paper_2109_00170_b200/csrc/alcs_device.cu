@@ -441,7 +441,7 @@ int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>
             }
         }
     }
-    if (allow_tc && hw > 0 && alcs::tc_fits(w->cin, w->cout, q / hw, hw, hw, 1)) {
+    if (allow_tc && hw > 0 && alcs::tc_fits(w, 1, q / hw, hw, hw)) {
         int n[8];
         const int count = tc_widths(w, n);
         for (int i = 0; i < count; ++i) out.push_back(tc_plan(w, n[i], q, di.sms));
@@ -495,7 +495,7 @@ int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg
     DeviceInfo di;
     int rc = device_info(w->device, &di);
     if (rc) return rc;
-    if (hw > 0 && allow_tc && (!c || c->math_mode == 4) && alcs::tc_fits(w->cin, w->cout, q / hw, hw_in, hw, 1)) {
+    if (hw > 0 && allow_tc && (!c || c->math_mode == 4) && alcs::tc_fits(w, 1, q / hw, hw_in, hw)) {
         if (c) {        // the tcgen05 kernel as asked for: row_groups channel tiles
             const int tiles = c->row_groups ? c->row_groups : tc_best(w, q, di.sms).n_rg;
             const int n = ((w->cout + std::max(1, tiles) - 1) / std::max(1, tiles) + 15) / 16 * 16;
@@ -807,7 +807,7 @@ bool tc_strided_ok(const alcs_packed* w, const void* x, int n, int oh, int ow, i
     // (rows of 4-byte copies only, as 16-bit 14x14 images have them, cost more than the gather pass of the other
     // kernels: 31 us against 15 for 231 -> 604 channels, 14 x 14 at stride 2, batch 15, fp16)
     const size_t row = (size_t)wd_in * w->elt();
-    return row % 8 == 0 && (uintptr_t)x % 8 == 0 && alcs::tc_fits(w->cin, w->cout, n, (long long)h_in * wd_in, (long long)oh * ow, 1) &&
+    return row % 8 == 0 && (uintptr_t)x % 8 == 0 && alcs::tc_fits(w, 1, n, (long long)h_in * wd_in, (long long)oh * ow) &&
            alcs::tc_patch_fits(w, tc_problem(x, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
 }
 
@@ -1533,7 +1533,7 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
 {
     auto open = [&](const alcs_stack::Item& it) {
         const alcs_layer& L = it.layer;
-        if (L.stride > 1 || !alcs::tc_fits(L.w->cin, L.w->cout, L.n, (long long)L.h * L.wd, (long long)it.oh * it.ow, 1)) return false;
+        if (L.stride > 1 || !alcs::tc_fits(L.w, 1, L.n, (long long)L.h * L.wd, (long long)it.oh * it.ow)) return false;
         if (fixed_too) return true;
         std::lock_guard<std::mutex> lk(L.w->mu);
         return L.w->tuned.find(alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}) == L.w->tuned.end();

@@ -114,6 +114,7 @@ struct alcs_packed {
     std::vector<int32_t> row_ptr;     // [rows+1]
     std::vector<int32_t> col_idx;     // [nb]
     std::vector<uint8_t> vals;        // [nb*g] elements of dt, raw bytes
+    bool finite = true;               // no infinity or NaN among them (fp32 alone is looked at)
     // device side (valid once uploaded)
     int device = -1;
     int* d_err = nullptr;             // device error word written by a kernel whose bounded wait ran out

@@ -12,6 +12,19 @@
 
 namespace {
 
+bool all_finite(const alcs_packed& p)
+{
+    if (p.dt != ALCS_F32) return true;
+    uint32_t all = 0;       // (no branch in the loop: a few values per cycle)
+    for (size_t i = 0; i + 4 <= p.vals.size(); i += 4) {
+        uint32_t u;
+        std::memcpy(&u, &p.vals[i], 4);
+        all |= ((u & 0x7f800000u) + 0x00800000u) & 0x80000000u;
+    }
+    return all == 0;
+}
+
+
 constexpr uint32_t kMagic = 0x53434C41u;  // "ALCS" little-endian
 constexpr uint32_t kBlobVersion = 1;
 
@@ -673,6 +686,7 @@ ALCS_API int alcs_pack(const void* w, const uint8_t* block_mask, int cout, int c
             }
         }
         p->row_ptr[rows] = k;
+        p->finite = all_finite(*p);
     } catch (const std::bad_alloc&) {
         delete p;
         return ALCS_ERR_ALLOC;
@@ -763,6 +777,7 @@ ALCS_API int alcs_packed_deserialize(const void* buf, size_t nbytes, alcs_packed
         in += (size_t)h.nb * 4;
         p->vals.resize((size_t)h.nb * h.g * es);
         if (!p->vals.empty()) std::memcpy(p->vals.data(), in, p->vals.size());
+        p->finite = all_finite(*p);
     } catch (const std::bad_alloc&) {
         delete p;
         return ALCS_ERR_ALLOC;

@@ -315,7 +315,7 @@ bool tc_whole_images(const alcs_packed* w, const TcProblem& p)
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out)
 {
     const int taps = std::max(1, p.kh * p.kw);
-    if (!tc_fits(w->cin / taps, w->cout, p.n, (long long)p.h_in * p.w_in, (long long)p.oh * p.ow, taps) || (p.kh && !tc_patch_fits(w, p, t.n)))
+    if (!tc_fits(w, taps, p.n, (long long)p.h_in * p.w_in, (long long)p.oh * p.ow) || (p.kh && !tc_patch_fits(w, p, t.n)))
         return ALCS_ERR_UNSUPPORTED;
     TcLayer& y = *out;
     y.x = p.x; y.y = p.y; y.bias = p.bias; y.res = p.res;
@@ -423,7 +423,7 @@ int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st)
 {
     const long long hw = (long long)p.oh * p.ow;
     const int taps = p.kh * p.kw;
-    if (!tc_fits(w->cin / taps, w->cout, p.n, (long long)p.h_in * p.w_in, hw, taps)) return ALCS_ERR_UNSUPPORTED;
+    if (!tc_fits(w, taps, p.n, (long long)p.h_in * p.w_in, hw)) return ALCS_ERR_UNSUPPORTED;
     int sms = 0, smem = 0;
     int rc = device_limits(w->device, &sms, &smem);
     if (rc) return rc;
@@ -480,11 +480,12 @@ int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st)
     return rc;
 }
 
-// 32-bit arithmetic of the kernel: element offsets into X, byte offsets inside the images one tile touches.
-bool tc_fits(int cin, int cout, long long n, long long hw_in, long long hw, int k)
+// 32-bit arithmetic of the kernel: element offsets into X, byte offsets inside the images one tile touches.  fp32 weights that
+// are not finite cannot be split into parts that add up to them.
+bool tc_fits(const alcs_packed* w, int taps, long long n, long long hw_in, long long hw)
 {
-    return n * hw_in * cin < (1ll << 31) - 4096 && ((long long)kTcM / std::max(1ll, hw) + 2) * hw * cout * 4 < (1ll << 32) &&
-           (long long)cin * k < (1 << 20) && n * hw <= (1ll << 30);
+    return n * hw_in * (w->cin / taps) < (1ll << 31) - 4096 && ((long long)kTcM / std::max(1ll, hw) + 2) * hw * w->cout * 4 < (1ll << 32) &&
+           w->cin < (1 << 20) && n * hw <= (1ll << 30) && (w->finite || w->dt != ALCS_F32);
 }
 
 }  // namespace alcs

@@ -48,7 +48,7 @@ int tc_run(const alcs_packed* w, const TcPrep& t, const TcProblem& p, cudaStream
 int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st);      // UNSUPPORTED where patch staging cannot
 bool tc_whole_images(const alcs_packed* w, const TcProblem& p);     // are X's chunks staged as runs of whole images?
 bool tc_patch_fits(const alcs_packed* w, const TcProblem& p, int n);     // can the problem be run by patch staging, n channels per tile?
-bool tc_fits(int cin, int cout, long long n, long long hw_in, long long hw, int k);
+bool tc_fits(const alcs_packed* w, int taps, long long n, long long hw_in, long long hw);       // taps: of the kernel, 1 for pointwise layers
 
 }  // namespace alcs
 

@@ -210,3 +210,36 @@ def test_infinite_inputs_of_one_layer_of_a_merged_stack(alcs):
     for L, (X, (Yref, A)) in zip(layers, keep):
         (assert_parity if np.isfinite(X).all() else _assert_special)(L["y"].cpu().numpy(), Yref, A, "f32")
     alcs.alcs_stack_destroy(st)
+
+
+def test_fp32_weights_that_are_not_finite(alcs):
+    """An infinite weight has no bfloat16 parts that add up to it: such a matrix stays on the other kernels."""
+    import torch
+    n, cin, cout, h, g = 40, 96, 128, 14, 4
+    W, M, X, b = _case(4, n, cin, cout, h * h, g, 0.5)
+    X = np.abs(X) + np.float32(0.1)
+    M[:, 0] = 1
+    W[5, 0], W[70, 0], W[71, 0] = np.inf, -np.inf, np.nan
+    M[3, 1] = 0
+    W[12, 1] = np.nan                       # a dropped block's value is not kept
+    p = alcs.alcs_packed_deserialize(alcs.alcs_packed_serialize(alcs.alcs_pack(W, M, g)))
+    p = alcs.alcs_packed_upload(p, 0)
+    st, xd, bd = torch.cuda.current_stream(), torch.from_numpy(X).cuda(), torch.from_numpy(b).cuda()
+    y = [torch.full((n, cout, h * h), 7.0, device="cuda") for _ in range(3)]
+    alcs.alcs_spconv1x1(p, xd, y[0], n, h, h, bd, 0, st)
+    stack = alcs.alcs_stack_create([dict(w=p, x=xd, y=y[k], n=n, h=h, wd=h, bias=bd, flags=0) for k in (1, 2)], 0)
+    alcs.alcs_stack_run(stack, st)
+    with pytest.raises(alcs.AlcsError) as e:
+        alcs.alcs_spconv1x1(p, xd, y[0], n, h, h, bd, 0, st, dict(math_mode=4))
+    assert e.value.status == alcs.ALCS_ERR_UNSUPPORTED
+    y2 = torch.full((n, cout, h, h), 7.0, device="cuda")
+    alcs.alcs_spconv2d(p, xd, y2, n, cin, h, h, 1, 1, 1, 0, bd, 0, st)
+    torch.cuda.synchronize()
+    other = np.setdiff1d(np.arange(cout), (5, 70, 71))
+    Wf = np.where(np.isfinite(W), W, 0).astype(np.float32)
+    Yref, A = oracle.conv1x1(Wf, M, X, b, False, g, want_scale=True)
+    for t in y + [y2]:
+        Y = t.cpu().numpy().reshape(n, cout, h * h)
+        assert (Y[:, 5] == np.inf).all() and (Y[:, 70] == -np.inf).all() and np.isnan(Y[:, 71]).all()
+        assert_parity(Y[:, other], Yref[:, other], A[:, other], "f32")
+    alcs.alcs_stack_destroy(stack)
