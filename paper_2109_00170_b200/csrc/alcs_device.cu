@@ -2027,20 +2027,25 @@ extern "C" ALCS_API int alcs_spconv1x1_noalloc(const alcs_packed* w, const void*
         auto it = w->plan_cache.find(alcs::ShapeKey{n, h, wd, flags});
         if (it == w->plan_cache.end()) return ALCS_ERR_STATE;
         plan = it->second;
-        if (plan.gather) {      // the small-problem kernel: needs only its resident copy of the storage format
-            if (!w->d_row_ptr) return ALCS_ERR_STATE;
+        if (plan.gather && w->d_row_ptr)      // the small-problem kernel: needs only its resident copy of the storage format
             return launch_gather_plan(w, plan, x, y, n, h, wd, bias, flags, st);
+        if (!plan.gather && !plan.tc_n) {
+            auto si = w->sched.find(alcs::sched_key(plan.kc, plan.n_rg, flavour_of(g_variants[plan.variant].v)));
+            if (si != w->sched.end() && si->second.uploaded) sc = &si->second;
         }
-        if (plan.tc_n) {        // needs no scratch, but what does not fit it is refused whatever kernel the plan names
+        if (!sc) {
+            // The tcgen05 kernel, in the form that the plan names or in any other that is resident: alcs_stack_create
+            // prepares the form of the launch it merged the layer into, the plan is that of a call by itself.  It
+            // needs no scratch, but what does not fit that is refused whatever kernel the plan names.
             const size_t row = (size_t)h * wd * w->elt();
             if (row % 16 != 0 && (size_t)n * w->cin * ((row + 15) / 16 * 16) > ALCS_NOALLOC_SCRATCH_BYTES) return ALCS_ERR_TOO_LARGE;
             const alcs::TcProblem pr = tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd);
-            const alcs::TcPrep* t = alcs::tc_find(w, tc_key(w, plan, pr));
-            return t ? alcs::tc_run(w, *t, pr, st) : ALCS_ERR_STATE;
+            const alcs::TcPrep* t = plan.tc_n ? alcs::tc_find(w, tc_key(w, plan, pr)) : nullptr;
+            if (!t) t = alcs::tc_any_pointwise(w);
+            if (!t) return ALCS_ERR_STATE;
+            rc = alcs::tc_run(w, *t, pr, st);
+            return rc == ALCS_ERR_UNSUPPORTED ? ALCS_ERR_STATE : rc;
         }
-        auto si = w->sched.find(alcs::sched_key(plan.kc, plan.n_rg, flavour_of(g_variants[plan.variant].v)));
-        if (si == w->sched.end() || !si->second.uploaded) return ALCS_ERR_STATE;
-        sc = &si->second;
     }
     DeviceInfo di;
     rc = device_info(w->device, &di);

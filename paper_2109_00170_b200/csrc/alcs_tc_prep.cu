@@ -127,6 +127,15 @@ TcPrep* tc_find(const alcs_packed* w, const TcKey& key)
     return it == w->tc.end() ? nullptr : it->second;
 }
 
+// Any form whose columns are input channels in order or by a list takes every pointwise layer of stride 1.
+const TcPrep* tc_any_pointwise(const alcs_packed* w)
+{
+    const TcPrep* best = nullptr;
+    for (const auto& kv : w->tc)
+        if (kv.first[1] <= 1 && kv.first[2] <= 1 && kv.second->splits == 1 && (!best || kv.second->n > best->n)) best = kv.second;
+    return best;
+}
+
 void tc_free(TcPrep* p)
 {
     if (!p) return;

@@ -39,6 +39,7 @@ struct TcProblem {
 
 int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep** out);
 TcPrep* tc_find(const alcs_packed* w, const TcKey& key);       // already prepared, or null; caller holds w->mu
+const TcPrep* tc_any_pointwise(const alcs_packed* w);          // a prepared form for pointwise layers, or null; caller holds w->mu
 void tc_free(TcPrep* p);
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out);
 double tc_item_us(int dt, int n, int k16);

@@ -243,3 +243,23 @@ def test_fp32_weights_that_are_not_finite(alcs):
         assert (Y[:, 5] == np.inf).all() and (Y[:, 70] == -np.inf).all() and np.isnan(Y[:, 71]).all()
         assert_parity(Y[:, other], Yref[:, other], A[:, other], "f32")
     alcs.alcs_stack_destroy(stack)
+
+
+def test_noalloc_after_stack_create(alcs):
+    """Creating a stack makes its shapes usable without allocation, also where the layers were merged into one launch
+    with other tiles than a layer by itself would get."""
+    import torch
+    layers, keep = [], []
+    for i, (cin, cout, h) in enumerate([(64, 128, 56), (128, 256, 28), (512, 512, 14), (512, 512, 14), (1024, 1024, 7), (256, 256, 28)]):
+        W, M, X, b = _case(80 + i, 1, cin, cout, h * h, 4, 0.2)
+        p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+        layers.append(dict(w=p, x=torch.from_numpy(X).cuda(), y=torch.empty((1, cout, h * h), device="cuda"), n=1, h=h, wd=h,
+                           bias=torch.from_numpy(b).cuda(), flags=alcs.ALCS_RELU))
+        keep.append(oracle.conv1x1(W, M, X, b, True, 4, want_scale=True))
+    st = alcs.alcs_stack_create(layers, 0)
+    for L, (Yref, A) in zip(layers, keep):
+        y = torch.full_like(L["y"], float("nan"))
+        alcs.alcs_spconv1x1_noalloc(L["w"], L["x"], y, 1, L["h"], L["wd"], L["bias"], L["flags"], torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert_parity(y.cpu().numpy(), Yref, A, "f32")
+    alcs.alcs_stack_destroy(st)
