@@ -802,13 +802,14 @@ alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& p
 
 // Can the tcgen05 kernel take a strided layer (whatever the channels per tile)?  The answer is part of the plan's key
 // (kNoTc), which holds the output size alone.
-bool tc_strided_ok(const alcs_packed* w, const void* x, int n, int oh, int ow, int stride, int h_in, int wd_in)
+bool tc_strided_ok(const alcs_packed* w, int n, int oh, int ow, int stride, int h_in, int wd_in)
 {
     // (rows of 4-byte copies only, as 16-bit 14x14 images have them, cost more than the gather pass of the other
     // kernels: 31 us against 15 for 231 -> 604 channels, 14 x 14 at stride 2, batch 15, fp16)
+    // (of the shape alone, so that calls with another X find what the first one prepared)
     const size_t row = (size_t)wd_in * w->elt();
-    return row % 8 == 0 && (uintptr_t)x % 8 == 0 && alcs::tc_fits(w, 1, n, (long long)h_in * wd_in, (long long)oh * ow) &&
-           alcs::tc_patch_fits(w, tc_problem(x, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
+    return row % 8 == 0 && alcs::tc_fits(w, 1, n, (long long)h_in * wd_in, (long long)oh * ow) &&
+           alcs::tc_patch_fits(w, tc_problem(nullptr, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
 }
 
 // Launch the tcgen05 kernel for one layer; strided layers run by patch staging.
@@ -1239,7 +1240,7 @@ ALCS_API int alcs_spconv1x1_ex(const alcs_packed* w, const void* x, void* y, int
         if (rb < yend && yb < rend) return ALCS_ERR_INVALID_ARG;     // the residual may not overlap y
     }
     Plan plan;
-    const bool tc = stride == 1 || tc_strided_ok(w, x, n, oh, ow, stride, h, wd);
+    const bool tc = stride == 1 || tc_strided_ok(w, n, oh, ow, stride, h, wd);
     rc = resolve_plan(w, n, oh, ow, flags | kStagedOnly | (tc ? 0u : kNoTc), q, cfg, &plan, (long long)h * wd);
     if (rc) return rc;
     return launch_plan(w, plan, x, y, n, oh, ow, bias, flags, static_cast<cudaStream_t>(cuda_stream), nullptr, 0,
@@ -1742,7 +1743,7 @@ ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned 
         it.ow = (L.wd + stride - 1) / stride;
         int rc = check_conv_args(L.w, L.x, L.y, L.n, it.oh, it.ow, L.flags, &it.q);
         if (!rc) rc = check_device(L.w);
-        const bool tc = !rc && it.q > 0 && (stride == 1 || tc_strided_ok(L.w, L.x, L.n, it.oh, it.ow, stride, L.h, L.wd));
+        const bool tc = !rc && it.q > 0 && (stride == 1 || tc_strided_ok(L.w, L.n, it.oh, it.ow, stride, L.h, L.wd));
         if (!rc && it.q > 0) rc = resolve_plan(L.w, L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u) | (tc ? 0u : kNoTc), it.q, nullptr, &it.plan, (long long)L.h * L.wd);
         if (rc) { delete s; return rc; }
         s->items.push_back(it);

@@ -416,14 +416,16 @@ __device__ __forceinline__ void copy_patch(const TcLayer& y, const Patch& t, uns
             for (int c = 0; c < nc; ++c) {
                 if (vb == 16) cp_async16(to, from);
                 else if (vb == 8) cp_async_small<8>(to, from, 8);
-                else cp_async_small<4>(to, from, 4);
+                else if (sizeof(raw) == 4 || vb == 4) cp_async_small<4>(to, from, 4);
+                else if constexpr (sizeof(raw) == 2) st_slot(to, ld_x(from));       // (an X that starts on an odd element)
                 to += pitch;
                 from += y.hw_in;
             }
         }
         slot += rows * y.w_in * (unsigned)sizeof(raw);
     }
-    cp_async_arrive(bar);
+    if (sizeof(raw) == 2 && vb == 2) bar_arrive(bar);
+    else cp_async_arrive(bar);
 }
 
 __device__ __forceinline__ void ld_slot(unsigned addr, float& v) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr)); }

@@ -308,16 +308,16 @@ bool tc_patch_fits(const alcs_packed* w, const TcProblem& p, int n)
 {
     if (p.kh * p.kw > 32 || w->cin % (p.kh * p.kw)) return false;
     const PatchPlan pl = patch_plan(w, p);
-    return pl.vec_bytes >= 4 && 2 * 16ll * pl.pitch * (long long)w->elt() <= patch_room(w->dt, n);
+    return 2 * 16ll * pl.pitch * (long long)w->elt() <= patch_room(w->dt, n);
 }
 
 // Small images whose rows do not start on copy boundaries (7x7): a tile takes whole images, of which the columns of
-// a chunk are one run of memory, if those runs keep to 16 bytes.
+// a chunk are one run of memory, if those runs keep to 16 bytes.  A property of the shape alone, since the form of the
+// expanded weights follows from it: an X that does not start on 16 bytes is copied element by element instead.
 bool tc_whole_images(const alcs_packed* w, const TcProblem& p)
 {
     const size_t elt = w->elt(), row = (size_t)p.oh * p.ow * elt;
-    return !p.kh && row % 16 != 0 && (elt == 4 || row % 4 != 0 || (uintptr_t)p.x % 4 != 0) && row <= kTcM * elt && (uintptr_t)p.x % 16 == 0 &&
-           w->cin % 16 == 0;
+    return !p.kh && row % 16 != 0 && (elt == 4 || row % 4 != 0) && row <= kTcM * elt && w->cin % 16 == 0;
 }
 
 // UNSUPPORTED: beyond the kernel's 32-bit offsets, or rows that patch staging cannot copy (see tc_fits, tc_patch_fits).
@@ -358,7 +358,7 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
         int vb = 16;
         while (vb > elt && (((size_t)y.hw.d * elt) % vb || (uintptr_t)p.x % vb)) vb >>= 1;
         y.vec_bytes = vb == 16 || (elt == 2 && vb > elt) ? vb : 0;      // (8 bytes of fp32: as single elements)
-        if (!t.cols && tc_whole_images(w, p)) y.images = kTcM / y.hw.d;
+        if (!t.cols && tc_whole_images(w, p) && (uintptr_t)p.x % 16 == 0) y.images = kTcM / y.hw.d;
     }
     y.ppt = y.images ? y.images * y.hw.d : kTcM;
     y.px_tiles = tc_div((y.q + y.ppt - 1) / y.ppt);

@@ -263,3 +263,41 @@ def test_noalloc_after_stack_create(alcs):
         torch.cuda.synchronize()
         assert_parity(y.cpu().numpy(), Yref, A, "f32")
     alcs.alcs_stack_destroy(st)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float16])
+@pytest.mark.parametrize("n,cin,cout,h,wd,stride", [(5, 64, 40, 7, 7, 1), (3, 80, 48, 14, 14, 1), (2, 64, 48, 12, 16, 2), (3, 100, 260, 9, 8, 2)])
+def test_inputs_that_start_anywhere_take_what_the_first_call_prepared(alcs, n, cin, cout, h, wd, stride, dtype):
+    """After one call for a shape, an X that starts on any element allocates nothing: it can be captured."""
+    import torch
+    g = 8
+    W, M, X, b = _case(n + cin, n, cin, cout, h * wd, g, 0.4, dtype)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    oh, ow = -(-h // stride), -(-wd // stride)
+    room = torch.empty(X.size + 8, dtype=torch.from_numpy(X).dtype, device="cuda")
+    y = torch.empty((n, cout, oh * ow), dtype=room.dtype, device="cuda")
+    bd = torch.from_numpy(b).cuda()
+    side = torch.cuda.Stream()
+    call = lambda x: alcs.alcs_spconv1x1_ex(p, x, y, n, h, wd, stride, bd, None, alcs.ALCS_RELU, side, dict(math_mode=4))
+    Yref, A = oracle.conv1x1_ex(W, M, X.reshape(n, cin, h, wd), b, None, True, g, stride, want_scale=True)
+    for at in range(8):
+        x = room[at:at + X.size]
+        x.copy_(torch.from_numpy(X).reshape(-1))
+        y.fill_(float("nan"))
+        torch.cuda.synchronize()
+        if at == 0:
+            call(x)
+        else:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=side):
+                call(x)
+            graph.replay()
+        torch.cuda.synchronize()
+        assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
+        if stride == 1:
+            alcs.alcs_spconv1x1_set_cfg(p, n, h, wd, alcs.ALCS_RELU, dict(math_mode=4))
+            y.fill_(float("nan"))
+            alcs.alcs_spconv1x1_noalloc(p, x, y, n, h, wd, bd, alcs.ALCS_RELU, torch.cuda.current_stream())
+            torch.cuda.synchronize()
+            assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
+    assert alcs.alcs_packed_status(p) == 0
