@@ -1428,6 +1428,14 @@ ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void*
     const int per = images_per_piece(n, x_image, y_image);
     const unsigned char* const xh = static_cast<const unsigned char*>(x_host);
     unsigned char* const yh = static_cast<unsigned char*>(y_host);
+    // A configuration stored for the call's shape holds for its pieces, too, where it can run them.
+    alcs_launch_cfg stored;
+    bool use_stored = false;
+    if (per < n) {
+        std::lock_guard<std::mutex> lk(w->mu);
+        const auto it = w->tuned.find(alcs::ShapeKey{n, h, wd, flags});
+        if (it != w->tuned.end()) { stored = it->second; use_stored = true; }
+    }
     if (per < n) {
         // The bus carries both directions at once: piece i is downloaded while piece i + 1 is multiplied and piece
         // i + 2 uploaded.  Everything is ordered after what is on cuda_stream now and before what comes next.
@@ -1445,7 +1453,11 @@ ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void*
                 ok(cudaMemcpyAsync(px, xh + x_image * at, x_image * m, cudaMemcpyHostToDevice, pipe->in));
                 ok(cudaEventRecord(pipe->uploaded[i], pipe->in));
                 ok(cudaStreamWaitEvent(st, pipe->uploaded[i], 0));
-                if (e == cudaSuccess) rc = alcs_spconv1x1(w, px, py, m, h, wd, bias_host ? db : nullptr, flags, cuda_stream);
+                const float* const b = bias_host ? db : nullptr;
+                if (e == cudaSuccess) {
+                    rc = alcs_spconv1x1_cfg(w, px, py, m, h, wd, b, flags, use_stored ? &stored : nullptr, cuda_stream);
+                    if (rc == ALCS_ERR_UNSUPPORTED && use_stored) rc = alcs_spconv1x1(w, px, py, m, h, wd, b, flags, cuda_stream);
+                }
                 if (rc) break;
                 ok(cudaEventRecord(pipe->computed[i], st));
                 ok(cudaStreamWaitEvent(pipe->out, pipe->computed[i], 0));

@@ -301,3 +301,25 @@ def test_inputs_that_start_anywhere_take_what_the_first_call_prepared(alcs, n, c
             torch.cuda.synchronize()
             assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
     assert alcs.alcs_packed_status(p) == 0
+
+
+def test_host_call_in_pieces_keeps_the_configuration_of_its_shape(alcs):
+    """The kernels differ in the order of their sums, so equal bits show that the same one ran."""
+    import torch
+    n, cin, cout, h, g = 32, 128, 128, 14, 4
+    W, M, X, _ = _case(2, n, cin, cout, h * h, g, 0.5)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    size = alcs.alcs_spconv1x1_host_workspace(p, n, h, h, 0)
+    ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+    xh, yh = torch.from_numpy(X).pin_memory(), torch.empty((n, cout, h * h)).pin_memory()
+    st, xd = torch.cuda.current_stream(), torch.from_numpy(X).cuda()
+    results = []
+    for cfg in (dict(math_mode=1), dict(math_mode=4, row_groups=2), dict(math_mode=3, pixels_per_lane=2, warps=4)):
+        alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, cfg)
+        alcs.alcs_spconv1x1_host(p, xh, yh, n, h, h, None, 0, ws, size, st)
+        y = torch.empty((n, cout, h * h), device="cuda")
+        alcs.alcs_spconv1x1(p, xd, y, n, h, h, None, 0, st)
+        torch.cuda.synchronize()
+        assert torch.equal(y.cpu(), yh)          # a pixel's sum does not depend on the images beside it
+        results.append(yh.numpy().copy())
+    assert not np.array_equal(results[0], results[1])         # (the kernels do differ in their rounding)
