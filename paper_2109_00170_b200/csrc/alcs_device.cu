@@ -1034,25 +1034,28 @@ struct alcs_stack {
 
 namespace {
 
-// Streams and events with which one alcs_spconv1x1_host call overlaps its uploads, convolutions and downloads.
-// A call takes one from the device's list (or makes one) while it enqueues and puts it back; the list keeps at
-// most kMaxPipes.  Re-recording an event does not disturb waits that were enqueued on its earlier state.
+// Streams and events with which one alcs_spconv1x1_host call overlaps its uploads, convolutions and downloads.  A device
+// has at most kMaxPipes of them.  A call takes one that nobody is enqueueing on and whose copies are either done or
+// those of an earlier call on the same stream, which this one follows anyway: a call never waits for another
+// stream's.  Re-recording an event does not disturb waits that were enqueued on its earlier state.
 constexpr int kPipePieces = 4;
-constexpr size_t kMaxPipes = 8;
+constexpr int kMaxPipes = 8;
 struct CopyPipe {
-    cudaStream_t in = nullptr, out = nullptr;
-    cudaEvent_t start = nullptr, done = nullptr, uploaded[kPipePieces] = {}, computed[kPipePieces] = {};
+    cudaStream_t in = nullptr, out = nullptr, user = nullptr;
+    cudaEvent_t start = nullptr, in_done = nullptr, out_done = nullptr, uploaded[kPipePieces] = {}, computed[kPipePieces] = {};
+    bool leased = false;
     bool make()
     {
         bool ok = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) == cudaSuccess;
         auto event = [&](cudaEvent_t& e) { ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
-        event(start); event(done);
+        event(start); event(in_done); event(out_done);
         for (int i = 0; i < kPipePieces; ++i) { event(uploaded[i]); event(computed[i]); }
         return ok;
     }
+    bool idle() const { return cudaEventQuery(in_done) == cudaSuccess && cudaEventQuery(out_done) == cudaSuccess; }
     ~CopyPipe()
     {
-        for (cudaEvent_t e : {start, done}) if (e) cudaEventDestroy(e);
+        for (cudaEvent_t e : {start, in_done, out_done}) if (e) cudaEventDestroy(e);
         for (int i = 0; i < kPipePieces; ++i) {
             if (uploaded[i]) cudaEventDestroy(uploaded[i]);
             if (computed[i]) cudaEventDestroy(computed[i]);
@@ -1065,24 +1068,42 @@ std::mutex g_pipe_mu;
 std::vector<std::unique_ptr<CopyPipe>>* const g_pipes = new std::vector<std::unique_ptr<CopyPipe>>[64];     // (never destroyed: the CUDA runtime may be gone by then)
 
 struct PipeLease {
-    int dev;
-    std::unique_ptr<CopyPipe> pipe;
-    explicit PipeLease(int d) : dev(d)
+    CopyPipe* pipe = nullptr;       // null: all busy, or st is being captured (whose graph must not hold streams of other calls)
+    PipeLease(int dev, cudaStream_t st)
     {
-        {
+        // (queries and new streams must not end a capture that another thread has under way)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone) {
             std::lock_guard<std::mutex> lk(g_pipe_mu);
-            if (!g_pipes[dev].empty()) { pipe = std::move(g_pipes[dev].back()); g_pipes[dev].pop_back(); }
+            auto& list = g_pipes[dev];
+            for (const bool same : {true, false})
+                for (auto& p : list)
+                    if (!pipe && !p->leased && (same ? p->user == st : p->idle())) pipe = p.get();
+            if (!pipe && list.size() < (size_t)kMaxPipes) {
+                std::unique_ptr<CopyPipe> made(new (std::nothrow) CopyPipe());
+                if (made && made->make()) {
+                    pipe = made.get();
+                    list.push_back(std::move(made));
+                }
+            }
+            if (pipe) {
+                pipe->leased = true;
+                pipe->user = st;
+            }
         }
-        if (!pipe) {
-            pipe.reset(new (std::nothrow) CopyPipe());
-            if (pipe && !pipe->make()) { pipe.reset(); (void)cudaGetLastError(); }
-        }
+        (void)cudaGetLastError();
+        cudaThreadExchangeStreamCaptureMode(&mode);
     }
     ~PipeLease()
     {
+        if (!pipe) return;
         std::lock_guard<std::mutex> lk(g_pipe_mu);
-        if (pipe && g_pipes[dev].size() < kMaxPipes) g_pipes[dev].push_back(std::move(pipe));
+        pipe->leased = false;
     }
+    PipeLease(const PipeLease&) = delete;
+    PipeLease& operator=(const PipeLease&) = delete;
 };
 
 // Images per piece of a host-buffer call: four pieces of at least a megabyte whose X starts on 16-byte
@@ -1439,40 +1460,46 @@ ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void*
     if (per < n) {
         // The bus carries both directions at once: piece i is downloaded while piece i + 1 is multiplied and piece
         // i + 2 uploaded.  Everything is ordered after what is on cuda_stream now and before what comes next.
-        PipeLease lease(w->device);
-        if (CopyPipe* const pipe = lease.pipe.get()) {
-            ALCS_CUDA(cudaEventRecord(pipe->start, st));
-            ALCS_CUDA(cudaStreamWaitEvent(pipe->in, pipe->start, 0));
-            rc = ALCS_OK;
-            cudaError_t e = cudaSuccess;
-            auto ok = [&](cudaError_t c) { if (e == cudaSuccess) e = c; return e == cudaSuccess; };
-            for (int i = 0, at = 0; at < n && rc == ALCS_OK && e == cudaSuccess; ++i, at += per) {
-                const int m = std::min(per, n - at);
-                unsigned char* const px = dx + x_image * at;
-                unsigned char* const py = dy + y_image * at;
-                ok(cudaMemcpyAsync(px, xh + x_image * at, x_image * m, cudaMemcpyHostToDevice, pipe->in));
-                ok(cudaEventRecord(pipe->uploaded[i], pipe->in));
-                ok(cudaStreamWaitEvent(st, pipe->uploaded[i], 0));
-                const float* const b = bias_host ? db : nullptr;
-                if (e == cudaSuccess) {
-                    rc = alcs_spconv1x1_cfg(w, px, py, m, h, wd, b, flags, use_stored ? &stored : nullptr, cuda_stream);
-                    if (rc == ALCS_ERR_UNSUPPORTED && use_stored) rc = alcs_spconv1x1(w, px, py, m, h, wd, b, flags, cuda_stream);
-                }
-                if (rc) break;
-                ok(cudaEventRecord(pipe->computed[i], st));
-                ok(cudaStreamWaitEvent(pipe->out, pipe->computed[i], 0));
-                ok(cudaMemcpyAsync(yh + y_image * at, py, y_image * m, cudaMemcpyDeviceToHost, pipe->out));
-            }
-            // (also on an error: the caller's stream must not run ahead of the copies that were enqueued)
-            for (cudaStream_t s : {pipe->in, pipe->out}) {
-                const cudaError_t a1 = cudaEventRecord(pipe->done, s), a2 = cudaStreamWaitEvent(st, pipe->done, 0);
-                ok(a1);
-                ok(a2);
-            }
-            if (rc) return rc;
-            ALCS_CUDA(e);
-            return ALCS_OK;
+        // Without a pipe the pieces follow one another on cuda_stream.
+        PipeLease lease(w->device, st);
+        CopyPipe* const pipe = lease.pipe;
+        const cudaStream_t in = pipe ? pipe->in : st, out = pipe ? pipe->out : st;
+        rc = ALCS_OK;
+        cudaError_t e = cudaSuccess;
+        auto ok = [&](cudaError_t c) { if (e == cudaSuccess) e = c; };
+        if (pipe) {
+            ok(cudaEventRecord(pipe->start, st));
+            ok(cudaStreamWaitEvent(in, pipe->start, 0));
         }
+        for (int i = 0, at = 0; at < n && rc == ALCS_OK && e == cudaSuccess; ++i, at += per) {
+            const int m = std::min(per, n - at);
+            unsigned char* const px = dx + x_image * at;
+            unsigned char* const py = dy + y_image * at;
+            ok(cudaMemcpyAsync(px, xh + x_image * at, x_image * m, cudaMemcpyHostToDevice, in));
+            if (pipe) {
+                ok(cudaEventRecord(pipe->uploaded[i], in));
+                ok(cudaStreamWaitEvent(st, pipe->uploaded[i], 0));
+            }
+            const float* const b = bias_host ? db : nullptr;
+            if (e == cudaSuccess) {
+                rc = alcs_spconv1x1_cfg(w, px, py, m, h, wd, b, flags, use_stored ? &stored : nullptr, cuda_stream);
+                if (rc == ALCS_ERR_UNSUPPORTED && use_stored) rc = alcs_spconv1x1(w, px, py, m, h, wd, b, flags, cuda_stream);
+            }
+            if (rc) break;
+            if (pipe) {
+                ok(cudaEventRecord(pipe->computed[i], st));
+                ok(cudaStreamWaitEvent(out, pipe->computed[i], 0));
+            }
+            ok(cudaMemcpyAsync(yh + y_image * at, py, y_image * m, cudaMemcpyDeviceToHost, out));
+        }
+        if (pipe) {     // (also on an error: the caller's stream must not run ahead of the copies that were enqueued)
+            const cudaError_t a1 = cudaEventRecord(pipe->in_done, in), a2 = cudaStreamWaitEvent(st, pipe->in_done, 0);
+            const cudaError_t a3 = cudaEventRecord(pipe->out_done, out), a4 = cudaStreamWaitEvent(st, pipe->out_done, 0);
+            for (const cudaError_t c : {a1, a2, a3, a4}) ok(c);
+        }
+        if (rc) return rc;
+        ALCS_CUDA(e);
+        return ALCS_OK;
     }
     ALCS_CUDA(cudaMemcpyAsync(dx, x_host, xb, cudaMemcpyHostToDevice, st));
     rc = alcs_spconv1x1(w, dx, dy, n, h, wd, bias_host ? db : nullptr, flags, cuda_stream);

@@ -323,3 +323,68 @@ def test_host_call_in_pieces_keeps_the_configuration_of_its_shape(alcs):
         assert torch.equal(y.cpu(), yh)          # a pixel's sum does not depend on the images beside it
         results.append(yh.numpy().copy())
     assert not np.array_equal(results[0], results[1])         # (the kernels do differ in their rounding)
+
+
+def _host_case(alcs, n=24, cin=128, cout=160, h=14):
+    import torch
+    W, M, X, b = _case(n, n, cin, cout, h * h, 4, 0.3)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+    size = alcs.alcs_spconv1x1_host_workspace(p, n, h, h, 0)
+    call = lambda x, y, ws, st: alcs.alcs_spconv1x1_host(p, x, y, n, h, h, None, 0, ws, size, st)
+    make = lambda: (torch.from_numpy(X).pin_memory(), torch.full((n, cout, h * h), float("nan")).pin_memory(),
+                    torch.empty(size, dtype=torch.uint8, device="cuda"))
+    return call, make, oracle.conv1x1(W, M, X, None, False, 4, want_scale=True)
+
+
+def test_host_calls_do_not_wait_for_another_stream(alcs):
+    """A call must end although a call on another stream, enqueued before it, cannot start yet.  (Few streams: more
+    than the device has queues would wait for one another whatever the library does.)  Then more streams at once than
+    the library keeps copy streams for."""
+    import torch
+    call, make, (Yref, A) = _host_case(alcs)
+    free, slow, blocked = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Stream()
+    mine, theirs, gate = make(), make(), torch.cuda.Event()
+    call(*mine, free)
+    torch.cuda.synchronize()
+    mine[1].fill_(float("nan"))
+    with torch.cuda.stream(slow):
+        torch.cuda._sleep(1_000_000_000)        # (half a second, on the device)
+        gate.record(slow)
+    blocked.wait_event(gate)
+    call(*theirs, blocked)
+    call(*mine, free)
+    free.synchronize()
+    assert not gate.query()
+    torch.cuda.synchronize()
+    many = [(torch.cuda.Stream(), make()) for _ in range(10)]
+    with torch.cuda.stream(slow):
+        torch.cuda._sleep(100_000_000)
+        gate.record(slow)
+    for s, b in many:
+        s.wait_event(gate)
+        call(*b, s)
+    torch.cuda.synchronize()
+    for b in [mine, theirs] + [b for _, b in many]:
+        assert_parity(b[1].numpy(), Yref, A, "f32")
+
+
+def test_host_call_under_capture(alcs):
+    """The copies of a captured call are its graph's own: another stream's call during the capture is not drawn in."""
+    import torch
+    call, make, (Yref, A) = _host_case(alcs)
+    a, b, side, other = make(), make(), torch.cuda.Stream(), torch.cuda.Stream()
+    call(*a, side)
+    call(*b, other)
+    torch.cuda.synchronize()
+    a[1].fill_(float("nan"))
+    b[1].fill_(float("nan"))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side, capture_error_mode="relaxed"):
+        call(*a, side)
+        call(*b, other)
+    other.synchronize()
+    assert_parity(b[1].numpy(), Yref, A, "f32")
+    assert not np.isfinite(a[1].numpy()).any()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert_parity(a[1].numpy(), Yref, A, "f32")
