@@ -388,3 +388,18 @@ def test_host_call_under_capture(alcs):
     graph.replay()
     torch.cuda.synchronize()
     assert_parity(a[1].numpy(), Yref, A, "f32")
+
+
+def test_host_call_on_pageable_memory(alcs):
+    """Pageable buffers, and a mix of both kinds, take the call in one piece."""
+    import torch
+    call, make, (Yref, A) = _host_case(alcs)
+    x, y, ws = make()
+    xp, yp = x.clone(), torch.empty(y.shape)
+    assert not xp.is_pinned() and not yp.is_pinned()
+    st = torch.cuda.current_stream()
+    for a, b in ((x, y), (xp, yp), (x, yp), (xp, y)):
+        b.fill_(float("nan"))
+        call(a, b, ws, st)
+        torch.cuda.synchronize()
+        assert_parity(b.numpy(), Yref, A, "f32")
