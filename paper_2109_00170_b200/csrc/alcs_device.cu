@@ -1657,13 +1657,14 @@ int stack_scratch(alcs_stack* s, bool any_plan)
         if (it.q > 8 * hw) need = std::max(need, (px + 512) * L.w->cin * (elt + 1));
     }
     if (need <= s->xpad_bytes) return ALCS_OK;
-    if (s->xpad) cudaFree(s->xpad);
-    s->xpad = nullptr;
-    s->xpad_bytes = 0;
-    if (cudaMalloc(&s->xpad, need) != cudaSuccess) {
+    void* room = nullptr;
+    if (cudaMalloc(&room, need) != cudaSuccess) {       // (the old scratch, which a captured graph may name, stays)
         (void)cudaGetLastError();
         return ALCS_ERR_ALLOC;
     }
+    if (s->exec) { cudaGraphExecDestroy(s->exec); s->exec = nullptr; }
+    if (s->xpad) cudaFree(s->xpad);
+    s->xpad = room;
     s->xpad_bytes = need;
     return ALCS_OK;
 }

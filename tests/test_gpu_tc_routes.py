@@ -403,3 +403,39 @@ def test_host_call_on_pageable_memory(alcs):
         call(a, b, ws, st)
         torch.cuda.synchronize()
         assert_parity(b.numpy(), Yref, A, "f32")
+
+
+def test_graph_stack_survives_a_tuning_call_that_finds_no_memory(alcs):
+    """alcs_stack_tune asks for scratch for every plan it may try; without the memory the stack runs on as before."""
+    import torch
+    W, M, X, b = _case(1, 40, 64, 48, 49, 4, 0.4)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+    alcs.alcs_spconv1x1_set_cfg(p, 40, 7, 7, 0, dict(math_mode=1))          # repacks its 7x7 images into the stack's scratch
+    n, cin = 65536, 256
+    V, N, _, _ = _case(2, 1, cin, 16, 49, 4, 0.5)
+    big = alcs.alcs_packed_upload(alcs.alcs_pack(V, N, 4), 0)
+    alcs.alcs_spconv1x1_set_cfg(big, n, 7, 7, 0, dict(math_mode=4))         # 3.3 GB of input, 4.3 GB of scratch for other plans
+    y = torch.empty((40, 48, 49), device="cuda")
+    layers = [dict(w=p, x=torch.from_numpy(X).cuda(), y=y, n=40, h=7, wd=7, bias=None, flags=0),
+              dict(w=big, x=torch.zeros((n, cin, 49), device="cuda"), y=torch.empty((n, 16, 49), device="cuda"), n=n, h=7, wd=7, bias=None, flags=0)]
+    st, s = alcs.alcs_stack_create(layers, alcs.ALCS_STACK_GRAPH), torch.cuda.Stream()
+    alcs.alcs_stack_run(st, s)
+    s.synchronize()
+    Yref, A = oracle.conv1x1(W, M, X, None, False, 4, want_scale=True)
+    assert_parity(y.cpu().numpy(), Yref, A, "f32")
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (2 << 30), dtype=torch.uint8, device="cuda")
+    with pytest.raises(alcs.AlcsError) as e:
+        alcs.alcs_stack_tune(st, 1, s)
+    assert e.value.status == alcs.ALCS_ERR_ALLOC
+    del hog
+    torch.cuda.empty_cache()
+    other = torch.full((1 << 20,), 7.0, device="cuda")          # what a freed block would be given to
+    for _ in range(2):
+        y.fill_(float("nan"))
+        torch.cuda.synchronize()
+        alcs.alcs_stack_run(st, s)
+        s.synchronize()
+        assert_parity(y.cpu().numpy(), Yref, A, "f32")
+    assert (other == 7.0).all()
+    alcs.alcs_stack_destroy(st)
