@@ -1530,7 +1530,7 @@ struct Extent {
 };
 
 struct LayerExtents {
-    Extent x, y, res;
+    Extent x, y, res, bias;
 };
 
 LayerExtents extents(const alcs_stack::Item& it)
@@ -1542,13 +1542,15 @@ LayerExtents extents(const alcs_stack::Item& it)
     r.x = {(uintptr_t)L.x, (uintptr_t)L.x + (size_t)L.n * L.w->cin * L.h * L.wd * xe};
     r.y = {(uintptr_t)L.y, (uintptr_t)L.y + yb};
     r.res = {(uintptr_t)L.residual, L.residual ? (uintptr_t)L.residual + yb : 0};
+    r.bias = {(uintptr_t)L.bias, L.bias ? (uintptr_t)(L.bias + L.w->cout) : 0};
     return r;
 }
 
 // May the two layers run at the same time?
 bool independent(const LayerExtents& a, const LayerExtents& b)
 {
-    return !(a.y.meets(b.x) || a.y.meets(b.res) || a.y.meets(b.y) || b.y.meets(a.x) || b.y.meets(a.res));
+    auto writes_input = [](const Extent& y, const LayerExtents& o) { return y.meets(o.x) || y.meets(o.res) || y.meets(o.bias); };
+    return !(a.y.meets(b.y) || writes_input(a.y, b) || writes_input(b.y, a));
 }
 
 alcs::TcProblem tc_problem(const alcs_stack::Item& it)

@@ -439,3 +439,25 @@ def test_graph_stack_survives_a_tuning_call_that_finds_no_memory(alcs):
         assert_parity(y.cpu().numpy(), Yref, A, "f32")
     assert (other == 7.0).all()
     alcs.alcs_stack_destroy(st)
+
+
+def test_merged_layers_do_not_read_a_bias_that_another_one_writes(alcs):
+    import torch
+    n, cin, cout, h = 2, 64, 64, 14
+    W, M, X, b = _case(9, n, cin, cout, h * h, 4, 0.5)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+    alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, dict(math_mode=4))
+    x = torch.from_numpy(X).cuda()
+    y = [torch.zeros((n, cout, h * h), device="cuda") for _ in range(2)]
+    bias = y[0].view(-1)[:cout]                    # the first channel of the first layer's output
+    st = alcs.alcs_stack_create([dict(w=p, x=x, y=y[0], n=n, h=h, wd=h, bias=torch.from_numpy(b).cuda(), flags=0),
+                                 dict(w=p, x=x, y=y[1], n=n, h=h, wd=h, bias=bias, flags=0)], 0)
+    for _ in range(3):
+        y[0].zero_()
+        alcs.alcs_stack_run(st, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    Y0, A0 = oracle.conv1x1(W, M, X, b, False, 4, want_scale=True)
+    assert_parity(y[0].cpu().numpy(), Y0, A0, "f32")
+    Y1, A1 = oracle.conv1x1(W, M, X, bias.cpu().numpy(), False, 4, want_scale=True)
+    assert_parity(y[1].cpu().numpy(), Y1, A1, "f32")
+    alcs.alcs_stack_destroy(st)
