@@ -983,6 +983,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             asm volatile("griddepcontrol.wait;" ::: "memory");
             // every producer copies whole chunks, the block's chunks in turn
             unsigned n = 0, mine = warp - kProdWarp0;
+            int bulk_phase = -1;        // of its slot, if the last copy there was a bulk one
             Cursor<L> cur(a);
 #pragma unroll 1
             while (ok && cur.step()) {
@@ -1012,11 +1013,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         ok = __all_sync(0xffffffffu, bar_wait(x_empty + 8 * slot, ((mine / S) & 1u) ^ 1u));
                         if (!ok) break;
                         src.chunk(ring0 + slot * kSlot, k * 16, min(NS, k16 - k) * 16, lane, x_full + 8 * slot);
+                        bulk_phase = src.n_img ? (int)((mine / S) & 1u) : -1;
                     }
                     n = end;
                 }
             }
+            // whoever waits for them may have given up: see the copies in flight land before shared memory goes away
             asm volatile("cp.async.wait_all;" ::: "memory");
+            if (!PATCH && bulk_phase >= 0) (void)bar_wait(x_full + 8 * (warp - kProdWarp0), bulk_phase);
         }
         if (warp == kLoadWarp && elect_one()) {
             unsigned stage = 0, ph = 0, used = 0;
@@ -1040,12 +1044,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     if (++stage == (unsigned)a.stages) { stage = 0; ph ^= 1u; }
                 }
             }
-            if (!ok)        // gave up: see the copies in flight land before shared memory goes away
+            // whoever waits for them may have given up: see the copies in flight land before shared memory goes away
 #pragma unroll 1
-                for (unsigned i = 0; i < min(used, (unsigned)a.stages); ++i) {
-                    const unsigned at = (stage + a.stages - 1 - i) % a.stages;
-                    (void)bar_wait(b_full + 8 * at, at < stage ? ph : ph ^ 1u);
-                }
+            for (unsigned i = 0; i < min(used, (unsigned)a.stages); ++i) {
+                const unsigned at = (stage + a.stages - 1 - i) % a.stages;
+                (void)bar_wait(b_full + 8 * at, at < stage ? ph : ph ^ 1u);
+            }
         }
     }
     if (!ok)
