@@ -570,8 +570,8 @@ __device__ __forceinline__ void recompute(const TcArgs<L>& a, unsigned layers, i
 #pragma unroll 1
                 for (int s = 0; s < (PATCH ? y.kw : 1); ++s)
                     if (w.inside(y, r, s))
-#pragma unroll 4
-                        for (int c = c0; c < c1; ++c) bad = bad || special<XT>(__ldg(x + w.at(y, c, r, s)));
+#pragma unroll 8
+                        for (int c = c0; c < c1; ++c) bad |= special<XT>(__ldg(x + w.at(y, c, r, s)));
         }
         unsigned todo = __ballot_sync(0xffffffffu, bad);
         if (!todo) continue;
@@ -889,8 +889,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 #pragma unroll 1
             for (int h = 0; h < out_rows; h += 32) {
                 if (whole) tmem_wait_ld(lo);
-                // (an input that is not finite reaches every channel of the tile, so one of them tells)
-                if (h == 0 && special<float>(lo[0])) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(not_finite), "r"(1u << (L > 1 ? cur.layer : 0)) : "memory");
+                // (an input that is not finite reaches every channel of the tile, so one of them tells; rows that are no
+                // output may hold whatever lay in shared memory)
+                if (h == 0 && live && special<float>(lo[0])) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(not_finite), "r"(1u << (L > 1 ? cur.layer : 0)) : "memory");
                 const unsigned off = lane_off + (any ? 0 : (unsigned)h * pitch);
                 const int rows = min(32, out_rows - h);
                 if (GENERAL && sizeof(XT) == 2 && wide) store32<float>(lo, y, out, res, off, pitch, floor, bias + h * 4, row0 + h, rows, live, any);

@@ -461,3 +461,35 @@ def test_merged_layers_do_not_read_a_bias_that_another_one_writes(alcs):
     Y1, A1 = oracle.conv1x1(W, M, X, bias.cpu().numpy(), False, 4, want_scale=True)
     assert_parity(y[1].cpu().numpy(), Y1, A1, "f32")
     alcs.alcs_stack_destroy(st)
+
+
+def test_rows_that_are_no_output_do_not_count_as_infinite(alcs):
+    """One 7x7 image in a tile that has room for two: what the second one's rows hold is left over from the launch
+    before, here infinities; a call must take as long as it does behind finite inputs (9 us, and 200 when every
+    item was searched for the input that is not there)."""
+    import torch
+    n, cin, h, g = 2, 1024, 7, 8
+    W, M, X, _ = _case(6, n, cin, 64, h * h, g, 0.5, np.float16)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    st, cfg = torch.cuda.current_stream(), dict(math_mode=4)
+    bad = torch.full((n, cin, h * h), float("inf"), dtype=torch.float16, device="cuda")
+    x, y2, y = torch.from_numpy(X).cuda(), torch.empty((n, 64, h * h), dtype=torch.float16, device="cuda"), torch.empty((1, 64, h * h), dtype=torch.float16, device="cuda")
+
+    def us(first):
+        best = 1e9
+        for _ in range(5):
+            alcs.alcs_spconv1x1(p, first, y2, n, h, h, None, 0, st, cfg)
+            torch.cuda.synchronize()
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            for _ in range(10):
+                alcs.alcs_spconv1x1(p, x, y, 1, h, h, None, 0, st, cfg)
+            e[1].record()
+            torch.cuda.synchronize()
+            best = min(best, e[0].elapsed_time(e[1]) * 100)
+        return best
+
+    us(x)
+    assert us(bad) < 3 * us(x) + 20
+    Yref, A = oracle.conv1x1(W, M, X[:1], None, False, g, want_scale=True)
+    assert_parity(y.cpu().numpy(), Yref, A, "f16")
