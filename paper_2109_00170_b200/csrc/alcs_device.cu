@@ -270,11 +270,22 @@ void set_unit_args(ConvArgs& a, const Schedule& sc, int mma)
     a.xch_slots = sc.max_x;
 }
 
-// The small-problem kernel as a plan.  Its cost: a launch, then the longer of two times: the rounds of dependent
-// loads (a warp issues the input vectors of four blocks and waits for them; a thread block's columns take `batches`
-// such rounds) and the bytes of X, which every block row fetches for itself from L2.  The constants are fits to one
-// B200: 4.5 us for 512 -> 512 @14 at batch 1, 3.8 for 731 -> 95 @7, 12 for 512 -> 512 @14 at batch 4, 24 for
-// 512 -> 512 @7 at batch 16.
+// Blocks of the longest block row.  (No lock: a caller may hold w->mu, and every thread computes the same value.)
+int longest_row(const alcs_packed* w)
+{
+    int longest = w->max_row_blocks;
+    if (longest < 0) {
+        longest = 0;
+        for (int r = 0; r < w->rows; ++r) longest = std::max(longest, w->row_ptr[r + 1] - w->row_ptr[r]);
+        w->max_row_blocks = longest;
+    }
+    return longest;
+}
+
+// The small-problem kernel as a plan.  Its cost: a launch, then the longest of: the rounds of dependent loads (a warp
+// issues the input vectors of four blocks and waits for them; a thread block's columns take `batches` such rounds) with
+// each block's start and its sum over the warps, the bytes of X, which every block row fetches for itself from L2, and
+// the arithmetic.  A fit to 1,600 launches of random shapes on one B200: median error 12 %.
 bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const DeviceInfo& di, Plan* out)
 {
     const int sms = di.sms;
@@ -287,32 +298,64 @@ bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const Devic
     pl.variant = -1; pl.gather = 1; pl.gp = p; pl.gks = ks;
     const bool vec = hw % 4 == 0 && p >= 4;
     const double per_row = w->rows ? (double)w->nb / w->rows : 0.0;
-    const double batches = std::ceil(per_row / ks / 4.0);
+    const double batches = std::ceil(per_row / ks / 4.0), longest = std::ceil((double)longest_row(w) / ks / 4.0);
     const double resident = std::max(1, (w->g * p > 16 ? 512 : 1024) / (ks * 32));          // thread blocks per SM
-    const double rounds = std::ceil((double)blocks / (sms * resident));
-    const double batch_us = (p == 2 ? 0.55 : p == 4 ? 0.7 : 0.9) * (vec || p == 2 ? 1.0 : 1.3);
-    const double bytes = (double)w->nb * n * tiles * 32.0 * p * 4;
-    // (every further round of thread blocks pays its own start and its stores: 49 us for 20,000 blocks of 17 -> 169 @56)
-    pl.cost = 1e-6 * (2.6 + std::max(rounds * batches * batch_us + (rounds - 1) * 1.4, bytes / (vec ? 5.5e6 : 3.3e6)));
+    const double rounds = (double)blocks / (sms * resident), share = w->g * p / 32.0;       // of the most outputs a lane can hold
+    const double batch_us = (p == 2 ? 0.74 : p == 4 ? 0.725 : 0.77) * (vec || p == 2 ? 1.0 : 1.08);
+    const double loads = (std::max(1.0, rounds) * (batches * batch_us + 0.078 * ks * share) + rounds * 0.885 +
+                          0.79 * std::max(0.0, longest - batches) * batch_us) * (1.0 + 0.32 * share);
+    const double px = (double)n * tiles * 32.0 * p;
+    const double l2 = (double)w->nb * px * 4 / (vec ? 9.9e6 : 4.4e6), fma = (double)w->nb * w->g * px * 28.1e-6 / sms;
+    const double hbm = (double)n * hw * (w->cin + w->cout) * 4 / 7.0e6;
+    pl.cost = 1e-6 * (2.8 + std::max({loads, l2, fma, hbm}));
     *out = pl;
     return true;
 }
 
-// Fixed cost of a launch of the tcgen05 kernel, first copies and last stores included, in microseconds.
-constexpr double kTcRampUs = 5.0;
-
 // Most images for which the small-problem kernel is considered (beyond, the bytes of X decide against it anyway).
 constexpr long long kGatherImages = 64;
 
-// The tcgen05 kernel with n output channels per tile as a plan, and its cost: rounds of items over the SMs.
-Plan tc_plan(const alcs_packed* w, int n, long long q, int sms)
+// A layer as the planner sees it: output and input size, what the call adds to the convolution.
+struct CallShape {
+    int n, oh, ow, h, wd, stride = 1;
+    bool residual = false;
+    int images() const { return std::max(1, n); }
+    int hw() const { return oh * ow; }
+    long long q() const { return (long long)images() * hw(); }
+};
+
+alcs::TcProblem tc_problem(const void* x, void* y, int n, int h, int wd, const float* bias, unsigned flags, const void* residual, int stride,
+                           int h_in, int wd_in)
+{
+    const int k = stride > 1 ? 1 : 0;
+    return {x, y, bias, residual, n, h, wd, h_in, wd_in, stride, 0, k, k, flags};
+}
+
+// (for estimates: no buffers, any address for a residual)
+alcs::TcProblem tc_problem(const CallShape& c)
+{
+    static const char some = 0;
+    return tc_problem(nullptr, nullptr, c.images(), c.oh, c.ow, nullptr, 0, c.residual ? &some : nullptr, c.stride, c.h, c.wd);
+}
+
+// Can the tcgen05 kernel take the layer (whatever the channels per tile)?  A strided one: rows of 4-byte copies only, as
+// 16-bit 14x14 images have them, cost more than the gather pass of the other kernels (31 us against 15 for 231 -> 604
+// channels, 14 x 14 at stride 2, batch 15, fp16).  The answer follows from the shape and the weights alone, so that calls
+// with another X find what the first one prepared.
+bool tc_ok(const alcs_packed* w, const CallShape& c)
+{
+    if (c.q() <= 0 || !alcs::tc_fits(w, 1, c.images(), (long long)c.h * c.wd, c.hw())) return false;
+    return c.stride == 1 || ((size_t)c.wd * w->elt() % 8 == 0 && alcs::tc_patch_fits(w, tc_problem(c), alcs::kTcMaxN));
+}
+
+// The tcgen05 kernel with n output channels per tile as a plan.
+Plan tc_plan(const alcs_packed* w, int n, const CallShape& c, int sms)
 {
     Plan p;
     p.n_rg = (w->cout + n - 1) / n;
     n = ((w->cout + p.n_rg - 1) / p.n_rg + 15) / 16 * 16;       // (the equal split into that many tiles)
     p.tc_n = n;
-    const long long items = (q + alcs::kTcM - 1) / alcs::kTcM * p.n_rg, rounds = (items + sms - 1) / sms;
-    p.cost = 1e-6 * (kTcRampUs + rounds * alcs::tc_item_us(w->dt, n, (w->cin + 15) / 16));
+    p.cost = 1e-6 * alcs::tc_layer_us(w, tc_problem(c), n, sms);
     return p;
 }
 
@@ -327,16 +370,39 @@ int tc_widths(const alcs_packed* w, int (&n)[8])
     return count;
 }
 
-Plan tc_best(const alcs_packed* w, long long q, int sms)
+Plan tc_best(const alcs_packed* w, const CallShape& c, int sms)
 {
     int n[8];
     const int count = tc_widths(w, n);
-    Plan best = tc_plan(w, n[0], q, sms);
+    Plan best = tc_plan(w, n[0], c, sms);
     for (int i = 1; i < count; ++i) {
-        const Plan p = tc_plan(w, n[i], q, sms);
+        const Plan p = tc_plan(w, n[i], c, sms);
         if (p.cost < best.cost) best = p;
     }
     return best;
+}
+
+// What the planner's own choice among the staged kernels takes, in microseconds, without listing their configurations
+// (which takes up to some tenths of a second): the repacking pass, then the longer of the bytes and the arithmetic, the
+// latency of a work item's chunks and of its longest row.  Fits to 990 launches of random shapes, types and densities on
+// one B200: median errors of 15 to 19 %.
+double staged_us(const alcs_packed* w, const CallShape& c, int sms)
+{
+    struct Fit { double launch, pass, pass_rate, rate, px, row, x, chunk, longest, block[5]; };
+    static const Fit fits[3] = {      // fp32; 16 bits on the CUDA cores; fp16 on mma.sync
+        {4.81, 1.42, 10.0e6, 2.48e6, 0.0120, 34.0e-6, 0.89e-6, 0.90, 0.045, {20.8e-6, 24.0e-6, 28.3e-6, 48.5e-6, 113e-6}},
+        {7.06, 0.43, 4.73e6, 2.00e6, 0.0031, 256e-6, 17.2e-6, 0.85, 0.0355, {25.1e-6, 35.0e-6, 55.7e-6, 65.7e-6, 163e-6}},
+        {7.25, 0.0, 4.89e6, 3.07e6, 0.0, 0.0, 185e-6, 0.40, 0.0045, {14.0e-6, 14.0e-6, 14.0e-6, 19.3e-6, 47.4e-6}}};
+    const Fit& f = fits[w->dt == ALCS_F32 ? 0 : w->dt == ALCS_F16 && w->g >= 4 ? 2 : 1];
+    const double q = (double)c.q(), elt = (double)w->elt(), x_bytes = q * w->cin * elt;
+    const size_t row = (size_t)c.hw() * w->elt();
+    double us = f.launch + f.chunk * w->cin / 64.0 + f.longest * longest_row(w);
+    if (c.stride > 1 || (row % 16 != 0 && row % 16 != 8)) us += f.pass + x_bytes * (1 + c.stride) / f.pass_rate;
+    const int at = w->g == 1 ? 0 : w->g == 2 ? 1 : w->g == 4 ? 2 : w->g == 8 ? 3 : 4;
+    const double work = q * f.px + w->nb * q * f.block[at] + w->rows * q * f.row + x_bytes * f.x * std::max(1.0, w->rows / 32.0);
+    us += std::max(work / sms, (x_bytes + q * w->cout * elt) / f.rate);
+    if (c.residual) us += q * w->cout * (w->dt == ALCS_F32 ? 2.5e-6 : 2.0e-6);
+    return us;
 }
 
 // Can the producers stage the rows of X as they are, with 8-byte copies, where 16-byte copies would need
@@ -346,16 +412,26 @@ bool direct_rows_ok(int hw, int elt) { return ((size_t)hw * elt) % 16 == 8; }
 // How many of the best candidates the tuner times a second time and remembers for alcs_stack_tune.
 constexpr size_t kFinalists = 12;
 
-// Enumerate every valid launch configuration for this shape, cheapest (by the model) first.
-// Internal flag, only ever seen in plan-cache keys: the call has a residual operand or a stride, which
-// the small-problem kernel does not take, so only the staged kernels are listed.
-constexpr unsigned kStagedOnly = 0x10000u;
-// Another one: a strided input that the tcgen05 kernel cannot stage.
-constexpr unsigned kNoTc = 0x20000u;
+// Internal bits of the flags in plan-cache keys, which else hold the output size alone: kExtra says that the call has a
+// residual operand or a stride (which the small-problem kernel does not take), the others which, and how its input
+// rows can be copied.
+constexpr unsigned kExtra = 0x10000u, kResidual = 0x20000u, kStrideShift = 20, kRowShift = 24, kNoTc = 0x80000000u;
 
-// allow_tc: may the tcgen05 kernel be listed (its limits depend on the input, which this function does not see)?
-int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>& out, bool allow_small = true, bool allow_tc = true)
+unsigned key_flags(const alcs_packed* w, unsigned flags, const CallShape& c)
 {
+    if (c.stride == 1 && !c.residual) return flags;
+    const size_t row = (size_t)c.wd * w->elt();
+    const unsigned align = c.stride == 1 ? 0 : row % 16 == 0 ? 2 : row % 8 == 0 ? 1 : 0;
+    return flags | kExtra | (c.residual ? kResidual : 0u) | (unsigned)std::min(c.stride, 15) << kStrideShift | align << kRowShift | (tc_ok(w, c) ? 0u : kNoTc);
+}
+
+// Enumerate every valid launch configuration for this shape, cheapest (by the model) first.
+// quick: the kernels that stage X through shared memory alone, with row-group counts a quarter apart: what a first call
+// can wait for (the full list of a 2048 x 2048 layer takes a second).
+int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>& out, bool quick = false)
+{
+    const long long q = std::max(1ll, c.q());
+    const int hw = c.hw();
     DeviceInfo di;
     int rc = device_info(w->device, &di);
     if (rc) return rc;
@@ -388,7 +464,7 @@ int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>
             const long long tiles = (q + 32 * v.p - 1) / (32 * v.p);
             const int rg_dense = std::min(w->rows, rg_min * 4 + 2);
             const int rg_hi = std::max<long long>(rg_dense, std::min<long long>(w->rows, (2ll * di.sms + tiles - 1) / tiles));
-            for (int n_rg = rg_min; n_rg <= rg_hi; n_rg = n_rg < rg_dense ? n_rg + 1 : std::max(n_rg + 1, n_rg * 5 / 4)) {
+            for (int n_rg = rg_min; n_rg <= rg_hi; n_rg = n_rg < rg_dense && !quick ? n_rg + 1 : std::max(n_rg + 1, n_rg * 5 / 4)) {
                 const int rpg = (w->rows + n_rg - 1) / n_rg;
                 if (rpg == last_rpg || rpg > cap) continue;
                 last_rpg = rpg;
@@ -441,16 +517,16 @@ int enumerate_plans(const alcs_packed* w, long long q, int hw, std::vector<Plan>
             }
         }
     }
-    if (allow_tc && hw > 0 && alcs::tc_fits(w, 1, q / hw, hw, hw)) {
+    if (!quick && tc_ok(w, c)) {
         int n[8];
         const int count = tc_widths(w, n);
-        for (int i = 0; i < count; ++i) out.push_back(tc_plan(w, n[i], q, di.sms));
+        for (int i = 0; i < count; ++i) out.push_back(tc_plan(w, n[i], c, di.sms));
     }
-    if (allow_small && hw > 0 && q / hw <= 8) {        // small batches only: one thread block per (block row, image, pixel tile)
+    if (!quick && c.stride == 1 && !c.residual && hw > 0 && c.images() <= 8) {        // small batches only: one thread block per (block row, image, pixel tile)
         for (int p = 8; p >= 2; p /= 2)
             for (int ks = 4; ks <= 16; ks *= 2) {
                 Plan g;
-                if (gather_plan(w, (int)(q / hw), hw, p, ks, di, &g)) out.push_back(g);
+                if (gather_plan(w, c.images(), hw, p, ks, di, &g)) out.push_back(g);
             }
     }
     std::stable_sort(out.begin(), out.end(), [](const Plan& a, const Plan& b) { return a.cost < b.cost; });
@@ -489,36 +565,53 @@ void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
 }
 
 // Resolve a (possibly partial) configuration into a concrete plan.
-int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg* c, Plan* out, bool allow_small = true, long long hw_in = 0, bool allow_tc = true)
+int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_cfg* c, Plan* out)
 {
-    if (hw_in < hw) hw_in = hw;
     DeviceInfo di;
     int rc = device_info(w->device, &di);
     if (rc) return rc;
-    if (hw > 0 && allow_tc && (!c || c->math_mode == 4) && alcs::tc_fits(w, 1, q / hw, hw_in, hw)) {
-        if (c) {        // the tcgen05 kernel as asked for: row_groups channel tiles
-            const int tiles = c->row_groups ? c->row_groups : tc_best(w, q, di.sms).n_rg;
-            const int n = ((w->cout + std::max(1, tiles) - 1) / std::max(1, tiles) + 15) / 16 * 16;
-            if (n > alcs::kTcMaxN) return ALCS_ERR_UNSUPPORTED;
-            *out = tc_plan(w, n, q, di.sms);
-            return ALCS_OK;
-        }
-        // Nobody asked for anything: the tcgen05 kernel, or the small-problem kernel where a few images leave most
-        // SMs without a tile and the latency of one item's chunk chain is all there is.
-        *out = tc_best(w, q, di.sms);
-        if (allow_small && q / hw <= kGatherImages)
+    const bool allow_small = shape.stride == 1 && !shape.residual;
+    const int hw = shape.hw();
+    const bool tc = (!c || c->math_mode == 4) && tc_ok(w, shape);
+    if (c && c->math_mode == 4) {       // the tcgen05 kernel as asked for: row_groups channel tiles
+        if (!tc) return ALCS_ERR_UNSUPPORTED;
+        const int tiles = c->row_groups ? c->row_groups : tc_best(w, shape, di.sms).n_rg;
+        const int n = ((w->cout + std::max(1, tiles) - 1) / std::max(1, tiles) + 15) / 16 * 16;
+        if (n > alcs::kTcMaxN) return ALCS_ERR_UNSUPPORTED;
+        *out = tc_plan(w, n, shape, di.sms);
+        return ALCS_OK;
+    }
+    if (!c) {
+        // Nobody asked for anything: the tcgen05 kernel; the small-problem kernel where a few images leave most SMs without a
+        // tile and the latency of one item's chunk chain is all there is; or the staged kernels, whose time falls with the
+        // density where the dense tiles' does not, if they are expected to be clearly faster.  Their estimate is the
+        // rougher one, most of all for long calls (512 -> 512 at 14 x 14, batch 256, 10 % kept: 252 us where 100 were
+        // expected, 120 dense), so those have to promise more.  2048 -> 2048 at 7 x 7, batch 32, 5 % kept: 92 us dense, 49.
+        Plan best;
+        best.cost = 1e30;
+        if (tc) best = tc_best(w, shape, di.sms);
+        if (allow_small && hw > 0 && shape.images() <= kGatherImages)
             for (int p = 8; p >= 2; p /= 2)
                 for (int ks = 4; ks <= 16; ks *= 2) {
                     Plan g;
-                    if (gather_plan(w, (int)(q / hw), hw, p, ks, di, &g) && g.cost < out->cost) *out = g;
+                    if (gather_plan(w, shape.images(), hw, p, ks, di, &g) && g.cost < best.cost) best = g;
                 }
+        const double staged = 1e-6 * staged_us(w, shape, di.sms);
+        if (staged * (best.cost < 100e-6 ? 1.15 : 1.5) < best.cost) {
+            std::vector<Plan> list;
+            rc = enumerate_plans(w, shape, list, true);
+            if (rc && (rc != ALCS_ERR_UNSUPPORTED || best.cost >= 1e30)) return rc;
+            if (!rc) {
+                best = list[0];
+                best.cost = staged;
+            }
+        }
+        *out = best;
         return ALCS_OK;
     }
-    if (c && c->math_mode == 4) return ALCS_ERR_UNSUPPORTED;
     std::vector<Plan> all;
-    rc = enumerate_plans(w, q, hw, all, allow_small, allow_tc);
+    rc = enumerate_plans(w, shape, all);
     if (rc) return rc;
-    if (!c) { *out = all[0]; return ALCS_OK; }
     if (c->math_mode == 3 && !allow_small) return ALCS_ERR_UNSUPPORTED;
     if (c->math_mode == 3) {        // the small-problem kernel, with the given (or the best-ranked) shape
         for (const Plan& p : all)
@@ -527,7 +620,7 @@ int cfg_to_plan(const alcs_packed* w, long long q, int hw, const alcs_launch_cfg
                 return ALCS_OK;
             }
         if (hw > 0 && c->pixels_per_lane && c->warps &&
-            gather_plan(w, (int)(q / hw), hw, c->pixels_per_lane, c->warps, di, out)) return ALCS_OK;
+            gather_plan(w, shape.images(), hw, c->pixels_per_lane, c->warps, di, out)) return ALCS_OK;
         return ALCS_ERR_UNSUPPORTED;
     }
     auto variant_ok = [&](const Plan& p) {
@@ -774,22 +867,10 @@ int launch_gather_plan(const alcs_packed* w, const Plan& p, const void* x, void*
     a.tiles = (a.hw + 32 * p.gp - 1) / (32 * p.gp);
     a.relu = (flags & ALCS_RELU) ? 1 : 0;
     a.vec = (p.gp >= 4 && a.hw % 4 == 0 && (uintptr_t)x % 16 == 0) ? 1 : 0;
-    int longest = w->max_row_blocks;        // (no lock: a caller may hold w->mu, and every thread computes the same value)
-    if (longest < 0) {
-        longest = 0;
-        for (int r = 0; r < w->rows; ++r) longest = std::max(longest, w->row_ptr[r + 1] - w->row_ptr[r]);
-        w->max_row_blocks = longest;
-    }
+    const int longest = longest_row(w);
     a.stage_blocks = alcs::gather_stage_blocks(w->g, longest);
     ALCS_CUDA(alcs::launch_gather(w->g, p.gp, p.gks, a, st));
     return ALCS_OK;
-}
-
-alcs::TcProblem tc_problem(const void* x, void* y, int n, int h, int wd, const float* bias, unsigned flags, const void* residual, int stride,
-                           int h_in, int wd_in)
-{
-    const int k = stride > 1 ? 1 : 0;
-    return {x, y, bias, residual, n, h, wd, h_in, wd_in, stride, 0, k, k, flags};
 }
 
 // Which form of the expanded weights a problem takes: strided layers, and small images that are staged as runs of
@@ -798,18 +879,6 @@ alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& p
 {
     const int k = pr.kh || alcs::tc_whole_images(w, pr) ? 1 : 0;
     return {p.tc_n, k, k};
-}
-
-// Can the tcgen05 kernel take a strided layer (whatever the channels per tile)?  The answer is part of the plan's key
-// (kNoTc), which holds the output size alone.
-bool tc_strided_ok(const alcs_packed* w, int n, int oh, int ow, int stride, int h_in, int wd_in)
-{
-    // (rows of 4-byte copies only, as 16-bit 14x14 images have them, cost more than the gather pass of the other
-    // kernels: 31 us against 15 for 231 -> 604 channels, 14 x 14 at stride 2, batch 15, fp16)
-    // (of the shape alone, so that calls with another X find what the first one prepared)
-    const size_t row = (size_t)wd_in * w->elt();
-    return row % 8 == 0 && alcs::tc_fits(w, 1, n, (long long)h_in * wd_in, (long long)oh * ow) &&
-           alcs::tc_patch_fits(w, tc_problem(nullptr, nullptr, n, oh, ow, nullptr, 0, nullptr, stride, h_in, wd_in), alcs::kTcMaxN);
 }
 
 // Launch the tcgen05 kernel for one layer; strided layers run by patch staging.
@@ -946,28 +1015,30 @@ int check_device(const alcs_packed* w)
     return cur == w->device ? ALCS_OK : ALCS_ERR_STATE;
 }
 
-int resolve_plan(const alcs_packed* w, int n, int h, int wd, unsigned flags, long long q,
-                 const alcs_launch_cfg* cfg, Plan* plan, long long hw_in = 0)
+int resolve_plan(const alcs_packed* w, const CallShape& c, unsigned flags, const alcs_launch_cfg* cfg, Plan* plan)
 {
-    alcs::ShapeKey key{n, h, wd, flags};
+    alcs::ShapeKey key{c.n, c.oh, c.ow, key_flags(w, flags, c)};
     if (cfg) {
-        const int c[12] = {cfg->pixels_per_lane, cfg->rows_per_warp, cfg->warps, cfg->chunk_channels,
+        const int v[12] = {cfg->pixels_per_lane, cfg->rows_per_warp, cfg->warps, cfg->chunk_channels,
                            cfg->stages, cfg->row_groups, cfg->min_blocks, cfg->copy_mode, cfg->producer_warps,
                            cfg->math_mode, cfg->consumer_groups, cfg->split_rows};
-        for (int i = 0; i < 12; ++i) key.c[i] = c[i];
+        for (int i = 0; i < 12; ++i) key.c[i] = v[i];
     }
+    alcs_launch_cfg stored;
+    const alcs_launch_cfg* use = cfg;
     {
         std::lock_guard<std::mutex> lk(w->mu);
         auto it = w->plan_cache.find(key);
         if (it != w->plan_cache.end()) { *plan = it->second; return ALCS_OK; }
+        if (!use) {     // a configuration tuned or set for the shape (stored under the public flags)
+            auto t = w->tuned.find(alcs::ShapeKey{c.n, c.oh, c.ow, flags});
+            if (t != w->tuned.end() && !((key.flags & kExtra) && t->second.math_mode == 3) && !((key.flags & kNoTc) && t->second.math_mode == 4)) {
+                stored = t->second;
+                use = &stored;
+            }
+        }
     }
-    const alcs_launch_cfg* use = cfg;
-    if (!use) {     // a configuration tuned or set for the shape (stored under the public flags)
-        auto it = w->tuned.find(alcs::ShapeKey{n, h, wd, flags & ~(kStagedOnly | kNoTc)});
-        if (it != w->tuned.end() && !((flags & kStagedOnly) && it->second.math_mode == 3) &&
-            !((flags & kNoTc) && it->second.math_mode == 4)) use = &it->second;
-    }
-    const int rc = cfg_to_plan(w, q, h * wd, use, plan, !(flags & kStagedOnly), hw_in, !(flags & kNoTc));
+    const int rc = cfg_to_plan(w, c, use, plan);
     if (rc) return rc;
     std::lock_guard<std::mutex> lk(w->mu);
     w->plan_cache[key] = *plan;
@@ -1232,7 +1303,7 @@ ALCS_API int alcs_spconv1x1_cfg(const alcs_packed* w, const void* x, void* y, in
     if (rc) return rc;
     if (q == 0) return ALCS_OK;
     Plan plan;
-    rc = resolve_plan(w, n, h, wd, flags, q, cfg, &plan);
+    rc = resolve_plan(w, {n, h, wd, h, wd}, flags, cfg, &plan);
     if (rc) return rc;
     return launch_plan(w, plan, x, y, n, h, wd, bias, flags, static_cast<cudaStream_t>(cuda_stream));
 }
@@ -1269,8 +1340,7 @@ ALCS_API int alcs_spconv1x1_ex(const alcs_packed* w, const void* x, void* y, int
         if (rb < yend && yb < rend) return ALCS_ERR_INVALID_ARG;     // the residual may not overlap y
     }
     Plan plan;
-    const bool tc = stride == 1 || tc_strided_ok(w, n, oh, ow, stride, h, wd);
-    rc = resolve_plan(w, n, oh, ow, flags | kStagedOnly | (tc ? 0u : kNoTc), q, cfg, &plan, (long long)h * wd);
+    rc = resolve_plan(w, {n, oh, ow, h, wd, stride, residual != nullptr}, flags, cfg, &plan);
     if (rc) return rc;
     return launch_plan(w, plan, x, y, n, oh, ow, bias, flags, static_cast<cudaStream_t>(cuda_stream), nullptr, 0,
                        residual, stride, h, wd);
@@ -1287,7 +1357,7 @@ ALCS_API int alcs_spconv1x1_plan(const alcs_packed* w, int n, int h, int wd, uns
     const long long q = (long long)n * h * wd;
     if ((long long)h * wd > (1ll << 30) || q > (1ll << 30)) return ALCS_ERR_SHAPE;
     Plan plan;
-    const int rc = resolve_plan(w, n, h, wd, flags, std::max(1ll, q), nullptr, &plan);
+    const int rc = resolve_plan(w, {n, h, wd, h, wd}, flags, nullptr, &plan);
     if (rc) return rc;
     plan_to_cfg(plan, out);
     return ALCS_OK;
@@ -1305,7 +1375,7 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
     if (q == 0) return ALCS_OK;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     std::vector<Plan> all;
-    rc = enumerate_plans(w, q, h * wd, all);
+    rc = enumerate_plans(w, {n, h, wd, h, wd}, all);
     if (rc) return rc;
     const size_t max_try = 1200;
     if (all.size() > max_try) all.resize(max_try);
@@ -1412,7 +1482,7 @@ ALCS_API int alcs_spconv1x1_set_cfg(alcs_packed* w, int n, int h, int wd, unsign
     const long long q = (long long)n * h * wd;
     if ((long long)h * wd > (1ll << 30) || q > (1ll << 30)) return ALCS_ERR_SHAPE;
     Plan plan;
-    const int rc = cfg_to_plan(w, std::max(1ll, q), h * wd, cfg, &plan);
+    const int rc = cfg_to_plan(w, {n, h, wd, h, wd}, cfg, &plan);
     if (rc) return rc;
     alcs_launch_cfg full;
     plan_to_cfg(plan, &full);
@@ -1553,6 +1623,12 @@ bool independent(const LayerExtents& a, const LayerExtents& b)
     return !(a.y.meets(b.y) || writes_input(a.y, b) || writes_input(b.y, a));
 }
 
+CallShape call_shape(const alcs_stack::Item& it)
+{
+    const alcs_layer& L = it.layer;
+    return {L.n, it.oh, it.ow, L.h, L.wd, L.stride > 1 ? L.stride : 1, L.residual != nullptr};
+}
+
 alcs::TcProblem tc_problem(const alcs_stack::Item& it)
 {
     const alcs_layer& L = it.layer;
@@ -1578,6 +1654,9 @@ size_t merge_end(const alcs_stack* s, size_t first, F eligible)
     return end;
 }
 
+// Fixed cost of a merged launch, first copies and last stores included, in microseconds.
+constexpr double kMergedRampUs = 5.0;
+
 // Consecutive independent layers whose configuration nobody fixed: one launch of the tcgen05 kernel for all of
 // them, where its estimate is below the sum of the layers' own.  With few items in all, narrower tiles shorten
 // the longest SM's share; with many, wide ones do the least work.
@@ -1586,7 +1665,7 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
 {
     auto open = [&](const alcs_stack::Item& it) {
         const alcs_layer& L = it.layer;
-        if (L.stride > 1 || !alcs::tc_fits(L.w, 1, L.n, (long long)L.h * L.wd, (long long)it.oh * it.ow)) return false;
+        if (L.stride > 1 || !tc_ok(L.w, call_shape(it))) return false;
         if (fixed_too) return true;
         std::lock_guard<std::mutex> lk(L.w->mu);
         return L.w->tuned.find(alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}) == L.w->tuned.end();
@@ -1606,17 +1685,19 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
                 int n[8], at = 0;
                 const int count = tc_widths(w, n);
                 while (at + 1 < count && n[at] > cap) ++at;
-                const double us = alcs::tc_item_us(w->dt, n[at], (w->cin + 15) / 16);
-                total += us * ((it.q + alcs::kTcM - 1) / alcs::kTcM) * ((w->cout + n[at] - 1) / n[at]);
-                longest = std::max(longest, us);
+                const double px = (double)((it.q + alcs::kTcM - 1) / alcs::kTcM);
+                for (const double us : alcs::tc_tiles_us(w, tc_problem(call_shape(it)), n[at])) {
+                    total += us * px;
+                    longest = std::max(longest, us);
+                }
                 widths[k - i] = n[at];
             }
-            const double t = kTcRampUs + std::max(total / di.sms, longest) + 0.25 * longest;
+            const double t = kMergedRampUs + std::max(total / di.sms, longest) + 0.25 * longest;
             if (t < best) { best = t; choice = widths; }
         }
         for (size_t k = i; k < end && !choice.empty(); ++k) {
             alcs_stack::Item& it = s->items[k];
-            it.plan = tc_plan(it.layer.w, choice[k - i], it.q, di.sms);
+            it.plan = tc_plan(it.layer.w, choice[k - i], call_shape(it), di.sms);
         }
         i = end;
     }
@@ -1702,7 +1783,7 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
         if (rc) return rc;
         rc = alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
         if (rc) return rc;
-        for (int k16 : t->k16) us[i].push_back(alcs::tc_item_us(it.layer.w->dt, t->n, k16));
+        for (int k16 : t->k16) us[i].push_back(alcs::tc_tile_us(it.layer.w, tc_problem(it), t->n, k16, t->cols != nullptr, t->chan != nullptr));
     }
     rc = alcs::tc_finish(w0, a, false);
     if (rc) return rc;
@@ -1796,8 +1877,7 @@ ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned 
         it.ow = (L.wd + stride - 1) / stride;
         int rc = check_conv_args(L.w, L.x, L.y, L.n, it.oh, it.ow, L.flags, &it.q);
         if (!rc) rc = check_device(L.w);
-        const bool tc = !rc && it.q > 0 && (stride == 1 || tc_strided_ok(L.w, L.n, it.oh, it.ow, stride, L.h, L.wd));
-        if (!rc && it.q > 0) rc = resolve_plan(L.w, L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u) | (tc ? 0u : kNoTc), it.q, nullptr, &it.plan, (long long)L.h * L.wd);
+        if (!rc && it.q > 0) rc = resolve_plan(L.w, call_shape(it), L.flags, nullptr, &it.plan);
         if (rc) { delete s; return rc; }
         s->items.push_back(it);
     }
@@ -1914,7 +1994,7 @@ int stack_candidates(const alcs_stack::Item& it, std::vector<Plan>& out)
     const bool small = !extra && it.oh * it.ow > 0 && it.q / ((long long)it.oh * it.ow) <= 8;
     if (had && !small) return ALCS_OK;
     std::vector<Plan> all;
-    const int rc = enumerate_plans(L.w, it.q, it.oh * it.ow, all, !extra);
+    const int rc = enumerate_plans(L.w, call_shape(it), all);
     if (rc) return rc;
     for (size_t i = 0; i < all.size(); ++i) {
         if (!((!had && i < 8) || all[i].gather) || (L.stride > 1 && all[i].tc_n)) continue;
@@ -1998,10 +2078,10 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
         const alcs_layer& L = it.layer;
         alcs_launch_cfg c;
         plan_to_cfg(it.plan, &c);
-        const bool extra = (L.stride > 1) || L.residual;
+        const alcs::ShapeKey key{L.n, it.oh, it.ow, key_flags(L.w, L.flags, call_shape(it))};
         std::lock_guard<std::mutex> lk(L.w->mu);
         L.w->tuned[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}] = c;
-        L.w->plan_cache[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags | (extra ? kStagedOnly : 0u)}] = it.plan;
+        L.w->plan_cache[key] = it.plan;
     }
     cur = time_stack(s, st, e0, e1, reps);      // (also leaves a graph stack captured with the chosen plans)
     if (cur < 0) return ALCS_ERR_CUDA;

@@ -6,7 +6,9 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <numeric>
 
@@ -376,6 +378,137 @@ double tc_item_us(int dt, int n, int k16)
     const int nch = (k16 * 16 + tc_kc(dt) - 1) / tc_kc(dt);
     const double chunk = dt == ALCS_F32 ? std::max(0.95, 0.1 + 0.0096 * n) : std::max(0.9, 0.3 + 0.006 * n);
     return nch * chunk + 0.3 + 0.005 * n;
+}
+
+namespace {
+
+// What one item costs, in microseconds: least-squares fits (of the logarithm) to 2,500 launches of random shapes, types and
+// densities on one B200; the median error is 7 %, one in ten is off by more than 25 %.
+struct TileFit {
+    double ramp;                 // a launch, with its first and last item's latencies that nothing overlaps
+    double mma, mma_n;           // a 16-column step on the tensor cores: mma + mma_n * channels
+    double list;                 // a step that follows a column list, beyond its copies
+    double store, store_n;       // bias, activation and stores: store + store_n * channels, ...
+    double sorted, res;          // ... store_n times this where every row's channel is looked up, and with a residual
+    double tail;                 // share of a tile's stores behind the last item
+    double copy[5], first[5];    // a step's copies, and the first chunk's latency per step: 16, 8, 4 bytes, elements, whole images
+};
+constexpr TileFit kTileFit[2] = {
+    {2.0, 0.217, 0.0011, 0.062, 0.75, 0.0100, 4.2, 8.0, 0.53, {0.258, 0.510, 0.510, 0.510, 0.317}, {0.75, 1.51, 1.51, 1.51, 0.38}},
+    {2.15, 0.097, 0.00096, 0.089, 0.745, 0.0086, 6.0, 9.0, 0.91, {0.187, 0.190, 0.282, 0.467, 0.108}, {0.36, 0.49, 0.59, 1.74, 0.0}}};
+// Patch staging: a step on the tensor cores; reading and splitting a step's values; one copy instruction of a warp.
+constexpr double kPatchRamp = 3.75, kPatchMma[2] = {0.195, 0.097}, kPatchMmaN = 0.00098, kPatchConvert[2] = {0.233, 0.15}, kPatchCopy = 0.0231,
+                 kPatchFirst = 0.24;
+constexpr double kBytesPerUs = 7.0e6;
+
+int copy_kind(const alcs_packed* w, const TcProblem& p)
+{
+    if (tc_whole_images(w, p)) return 4;
+    const size_t row = (size_t)p.oh * p.ow * w->elt();
+    return row % 16 == 0 ? 0 : w->dt == ALCS_F32 ? 3 : row % 8 == 0 ? 1 : row % 4 == 0 ? 2 : 3;
+}
+
+double store_us(const alcs_packed* w, const TcProblem& p, int n, bool sorted)
+{
+    const TileFit& f = kTileFit[w->dt != ALCS_F32];
+    return f.store + f.store_n * n * std::max(sorted ? f.sorted : 1.0, p.res ? f.res : 1.0);
+}
+
+// Copy instructions of a warp for one block of 16 channels of the widest patch.  (Of an aligned X: no estimate depends on
+// where X starts.)
+double patch_copies(const alcs_packed* w, TcProblem p)
+{
+    p.x = nullptr;
+    const PatchPlan pl = patch_plan(w, p);
+    return 16.0 * pl.pitch * (double)w->elt() / pl.vec_bytes / 32.0;
+}
+
+// Channel tiles as tc_prepare would lay them out, from the lengths of the block rows: a tile of rows that keep a share
+// d_r of the columns at random keeps 1 - prod(1 - d_r) of them.
+struct TileGuess {
+    std::vector<int> k16;
+    bool list = false, sorted = false;
+};
+
+TileGuess guess_tiles(const alcs_packed* w, const TcProblem& p, int n)
+{
+    const int rpt = n / w->g, tiles = (w->rows + rpt - 1) / rpt, dense16 = (w->cin + 15) / 16;
+    std::vector<int> len(w->rows);
+    for (int r = 0; r < w->rows; ++r) len[r] = w->row_ptr[r + 1] - w->row_ptr[r];
+    auto steps = [&](std::vector<int>& out) {
+        long long sum = 0;
+        out.resize(tiles);
+        for (int t = 0; t < tiles; ++t) {
+            double none = 1.0;
+            int any = 0;
+            for (int r = t * rpt; r < std::min(w->rows, (t + 1) * rpt); ++r) {
+                none *= 1.0 - (double)len[r] / w->cin;
+                any |= len[r];
+            }
+            out[t] = any ? std::max(1, (int)std::ceil(w->cin * (1.0 - none) / 16.0)) : 0;
+            sum += out[t];
+        }
+        return sum;
+    };
+    TileGuess g;
+    long long sum = steps(g.k16);
+    const bool lists = !p.kh && !tc_whole_images(w, p);
+    if (lists && skewed(*w)) {
+        std::vector<int> k16;
+        std::sort(len.begin(), len.end(), std::greater<int>());
+        const long long s = steps(k16);
+        if (s * 20 <= sum * 19) { g.k16.swap(k16); g.sorted = true; sum = s; }
+    }
+    g.list = lists && sum * 10 <= (long long)dense16 * tiles * 9;
+    if (!g.list)
+        for (int& k : g.k16) k = k ? dense16 : 0;
+    return g;
+}
+
+}  // namespace
+
+double tc_tile_us(const alcs_packed* w, const TcProblem& p, int n, int k16, bool list, bool sorted)
+{
+    const int half = w->dt != ALCS_F32;
+    const TileFit& f = kTileFit[half];
+    const double store = store_us(w, p, n, sorted);
+    if (k16 == 0) return 1.5 * store;
+    if (p.kh)
+        return k16 * std::max({kPatchConvert[half], kPatchMma[half] + kPatchMmaN * n, kPatchCopy * patch_copies(w, p) / (p.kh * p.kw)}) + store;
+    const double work = k16 * std::max(f.copy[copy_kind(w, p)] + (list ? f.list : 0.0), f.mma + f.mma_n * n);
+    // (the epilogue adds up the chunk sums of a long item and then stores: a residual's loads are not hidden there)
+    return p.res && k16 * 16 > 2 * tc_kc(w->dt) ? work + 0.65 * store : std::max(work, store);
+}
+
+std::vector<double> tc_tiles_us(const alcs_packed* w, const TcProblem& p, int n)
+{
+    const TileGuess g = guess_tiles(w, p, n);
+    std::vector<double> us;
+    for (int k16 : g.k16) us.push_back(tc_tile_us(w, p, n, k16, g.list, g.sorted));
+    return us;
+}
+
+double tc_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms)
+{
+    const TileFit& f = kTileFit[w->dt != ALCS_F32];
+    const TileGuess g = guess_tiles(w, p, n);
+    const long long hw = (long long)p.oh * p.ow, q = hw * std::max(1, p.n);
+    const int ppt = !p.kh && tc_whole_images(w, p) ? (int)(kTcM / hw * hw) : kTcM, kind = copy_kind(w, p);
+    const double px = (double)((q + ppt - 1) / ppt);
+    double sum = 0, longest = 0;
+    int k_max = 0;
+    for (int k16 : g.k16) {
+        const double t = tc_tile_us(w, p, n, k16, g.list, g.sorted);
+        sum += t;
+        longest = std::max(longest, t);
+        k_max = std::max(k_max, k16);
+    }
+    const double rounds = std::ceil(px * g.k16.size() / sms);
+    const double main = std::max(rounds * sum / g.k16.size(), longest);
+    const double bytes = (double)q * (w->cin + w->cout * (p.res ? 2.0 : 1.0)) * w->elt();
+    if (p.kh) return std::max(kPatchRamp + main + kPatchFirst * std::min(k_max, 4), kPatchRamp + bytes / kBytesPerUs);
+    const double first = f.first[kind] * std::min(k_max, tc_kc(w->dt) / 16);
+    return std::max(f.ramp + main + first + f.tail * store_us(w, p, n, g.sorted), f.ramp + bytes / kBytesPerUs);
 }
 
 // Number items and choose the ring depth for the a.n_layers layers filled in.

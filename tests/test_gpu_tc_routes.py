@@ -493,3 +493,43 @@ def test_rows_that_are_no_output_do_not_count_as_infinite(alcs):
     assert us(bad) < 3 * us(x) + 20
     Yref, A = oracle.conv1x1(W, M, X[:1], None, False, g, want_scale=True)
     assert_parity(y.cpu().numpy(), Yref, A, "f16")
+
+
+def _modes(alcs, sparsity, n, cin, cout, h, g, dtype=np.float32):
+    W, M, _, _ = _case(1, 1, cin, cout, 1, g, 1.0 - sparsity, dtype)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    return alcs.alcs_spconv1x1_plan(p, n, h, h, 0)["math_mode"]
+
+
+def test_sparse_layers_leave_the_dense_tiles_to_the_dense_ones(alcs):
+    """The tcgen05 kernel's time hardly depends on the density, the CUDA cores' does: 92 us against 49 for 2048 -> 2048
+    at 7x7, batch 32, 5 % kept, and 92 against 220 with half of the blocks kept."""
+    assert _modes(alcs, 0.95, 32, 2048, 2048, 7, 4) == 1
+    assert _modes(alcs, 0.5, 32, 2048, 2048, 7, 4) == 4
+    assert _modes(alcs, 0.8, 64, 512, 512, 14, 4) == 4
+    assert _modes(alcs, 0.5, 64, 512, 512, 14, 8, np.float16) == 4
+
+
+# n, cin, cout, h, wd, g, stride, residual, density: strided rows of 8-byte copies and residuals that the staged kernels take
+# sooner than plain layers, of every element type's path
+@pytest.mark.parametrize("n,cin,cout,h,wd,g,stride,residual,density", [(8, 512, 512, 14, 14, 4, 2, False, 0.2), (32, 256, 512, 14, 14, 4, 3, True, 0.03),
+                                                                      (64, 32, 64, 56, 56, 8, 1, True, 0.2), (4, 1024, 256, 14, 14, 1, 2, True, 0.03)])
+@pytest.mark.parametrize("dtype", [np.float32, np.float16])
+def test_planned_strided_and_residual_layers(alcs, n, cin, cout, h, wd, g, stride, residual, density, dtype):
+    import torch
+    W, M, X, b = _case(n + stride, n, cin, cout, h * wd, g, density, dtype)
+    oh, ow = -(-h // stride), -(-wd // stride)
+    R = rng.normal(6, 5, n * cout * oh * ow).reshape(n, cout, oh * ow).astype(dtype) if residual else None
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    xd, bd, rd = torch.from_numpy(X).cuda(), torch.from_numpy(b).cuda(), None if R is None else torch.from_numpy(R).cuda()
+    Yref, A = oracle.conv1x1_ex(W, M, X.reshape(n, cin, h, wd), b, R, True, g, stride, want_scale=True)
+    y = torch.full((n, cout, oh * ow), float("nan"), dtype=xd.dtype, device="cuda")
+    alcs.alcs_spconv1x1_ex(p, xd, y, n, h, wd, stride, bd, rd, alcs.ALCS_RELU, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
+    stack = alcs.alcs_stack_create([dict(w=p, x=xd, y=y, n=n, h=h, wd=wd, bias=bd, flags=alcs.ALCS_RELU, residual=rd, stride=stride)], 0)
+    y.fill_(float("nan"))
+    alcs.alcs_stack_run(stack, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
+    alcs.alcs_stack_destroy(stack)
