@@ -133,11 +133,14 @@ struct alcs_packed {
     mutable std::map<std::array<int, 8>, alcs::Schedule> sched2d;
     // expanded weights of the tcgen05 kernel, by {channels per tile, kh, kw} (alcs_tc_prep.h)
     mutable std::map<std::array<int, 3>, alcs::TcPrep*> tc;
+    // which kernel a k x k layer runs on, by {n, cin, h, w, kh, kw, stride, pad}: channels per tile of the tcgen05 kernel
+    // (0: the CUDA cores) and parts of its columns
+    mutable std::map<std::array<int, 8>, std::array<int, 2>> conv2d_choice;
     mutable std::map<alcs::ShapeKey, alcs_launch_cfg> tuned;   // filled by alcs_spconv1x1_tune, alcs_spconv1x1_set_cfg, alcs_stack_tune
     // the best few plans of the last alcs_spconv1x1_tune per shape, best first: what alcs_stack_tune tries in context
     mutable std::map<alcs::ShapeKey, std::vector<alcs::Plan>> finalists;
     mutable std::map<alcs::ShapeKey, alcs::Plan> plan_cache;   // resolved plans, by shape
-    mutable std::mutex mu;                                      // guards plan_cache and sched
+    mutable std::mutex mu;                                      // guards the maps
     size_t elt() const { return dt == ALCS_F32 ? 4 : 2; }
 };
 

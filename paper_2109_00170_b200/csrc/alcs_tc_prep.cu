@@ -369,17 +369,6 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
     return ALCS_OK;
 }
 
-// How long one item takes, in microseconds, by type, channels per tile and 16-column steps: per chunk the MMAs
-// (24 of n / 2 cycles in fp32; the tensor cores run at about 1.55 GHz under that load) or the staging and
-// conversion of X, whichever is longer, plus the part of the store that nothing overlaps.  Measured: 1.33 / 1.03 /
-// 0.95 us per fp32 chunk at n = 128 / 64 / 32.
-double tc_item_us(int dt, int n, int k16)
-{
-    const int nch = (k16 * 16 + tc_kc(dt) - 1) / tc_kc(dt);
-    const double chunk = dt == ALCS_F32 ? std::max(0.95, 0.1 + 0.0096 * n) : std::max(0.9, 0.3 + 0.006 * n);
-    return nch * chunk + 0.3 + 0.005 * n;
-}
-
 namespace {
 
 // What one item costs, in microseconds: least-squares fits (of the logarithm) to 2,500 launches of random shapes, types and
@@ -561,20 +550,18 @@ int tc_run(const alcs_packed* w, const TcPrep& t, const TcProblem& p, cudaStream
     return rc ? rc : tc_launch(w, a, p.kh > 0, st);
 }
 
-int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st)
+// The width, and the number of parts the channels are split into, that take the least time: rounds of items over
+// the SMs, and for split columns the partial sums' way through memory and one more launch (5 us, then 2.8 TB/s).
+// Small batches leave most SMs idle otherwise: one 7 x 7 image of 512 channels is a chain of 72 chunks.
+double tc_conv2d_choose(const alcs_packed* w, const TcProblem& p, int sms, int* n_out, int* splits_out)
 {
     const long long hw = (long long)p.oh * p.ow;
     const int taps = p.kh * p.kw;
-    if (!tc_fits(w, taps, p.n, (long long)p.h_in * p.w_in, hw)) return ALCS_ERR_UNSUPPORTED;
-    int sms = 0, smem = 0;
-    int rc = device_limits(w->device, &sms, &smem);
-    if (rc) return rc;
-    // The width, and the number of parts the channels are split into, that take the least time: rounds of items over
-    // the SMs, and for split columns the partial sums' way through memory and one more launch (3 us, then 2 TB/s each
-    // way).  Small batches leave most SMs idle otherwise: one 7 x 7 image of 512 channels is a chain of 72 chunks.
+    *n_out = 0;
+    *splits_out = 1;
+    if (!tc_fits(w, taps, p.n, (long long)p.h_in * p.w_in, hw)) return 0;
     const int blocks = (w->cin / taps + 15) / 16;
     const long long px = (p.n * hw + kTcM - 1) / kTcM;
-    int n = 0, splits = 1;
     double best = 0;
     for (int want = kTcMaxN; want >= 16; want -= 16) {
         const int want_tiles = (w->cout + want - 1) / want, v = ((w->cout + want_tiles - 1) / want_tiles + 15) / 16 * 16;
@@ -586,11 +573,20 @@ int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st)
             const double bytes = (double)s * tiles * v * p.n * hw * 4;
             if (s > 1 && (bytes > (32 << 20) || (double)p.n * hw * w->cout > 1e9)) break;
             const long long items = px * tiles * s;
-            const double us = (double)((items + sms - 1) / sms) * tc_item_us(w->dt, v, part * taps) + (s > 1 ? 3.0 + bytes / 1.0e6 : 0.0);
-            if (n == 0 || us < best * 0.95) { n = v; splits = s; best = us; }
+            const double us = kPatchRamp + kPatchFirst * std::min(part * taps, 4) +
+                              (double)((items + sms - 1) / sms) * tc_tile_us(w, p, v, part * taps, false, false) + (s > 1 ? 5.2 + bytes / 2.8e6 : 0.0);
+            if (*n_out == 0 || us < best * 0.95) { *n_out = v; *splits_out = s; best = us; }
         }
     }
-    if (n == 0) return ALCS_ERR_UNSUPPORTED;
+    return best;
+}
+
+int tc_conv2d(const alcs_packed* w, const TcProblem& p, int n, int splits, cudaStream_t st)
+{
+    const long long hw = (long long)p.oh * p.ow;
+    int sms = 0, smem = 0;
+    int rc = device_limits(w->device, &sms, &smem);
+    if (rc) return rc;
     TcPrep* t = nullptr;
     rc = tc_prepare(w, {n, p.kh, p.kw, splits}, st, &t);
     if (rc) return rc;

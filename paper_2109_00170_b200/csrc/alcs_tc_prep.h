@@ -42,7 +42,6 @@ TcPrep* tc_find(const alcs_packed* w, const TcKey& key);       // already prepar
 const TcPrep* tc_any_pointwise(const alcs_packed* w);          // a prepared form for pointwise layers, or null; caller holds w->mu
 void tc_free(TcPrep* p);
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out);
-double tc_item_us(int dt, int n, int k16);
 // Estimates, in microseconds, from the shape and the weights alone.
 double tc_tile_us(const alcs_packed* w, const TcProblem& p, int n, int k16, bool list, bool sorted);
 std::vector<double> tc_tiles_us(const alcs_packed* w, const TcProblem& p, int n);        // of every channel tile, as tc_prepare would make them
@@ -50,7 +49,9 @@ double tc_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms);
 int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a, bool patch);
 int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool patch, cudaStream_t st);
 int tc_run(const alcs_packed* w, const TcPrep& t, const TcProblem& p, cudaStream_t st);      // one layer, prepared
-int tc_conv2d(const alcs_packed* w, const TcProblem& p, cudaStream_t st);      // UNSUPPORTED where patch staging cannot
+// Channels per tile and parts of the columns for a k x k layer (n = 0: not for this kernel), and the time they take.
+double tc_conv2d_choose(const alcs_packed* w, const TcProblem& p, int sms, int* n, int* splits);
+int tc_conv2d(const alcs_packed* w, const TcProblem& p, int n, int splits, cudaStream_t st);
 bool tc_whole_images(const alcs_packed* w, const TcProblem& p);     // are X's chunks staged as runs of whole images?
 bool tc_patch_fits(const alcs_packed* w, const TcProblem& p, int n);     // can the problem be run by patch staging, n channels per tile?
 bool tc_fits(const alcs_packed* w, int taps, long long n, long long hw_in, long long hw);       // taps: of the kernel, 1 for pointwise layers

@@ -175,12 +175,12 @@ def test_infinite_and_nan_inputs_with_stride_and_residual(alcs, stride, dtype):
     _assert_special(y.cpu().numpy(), *_kept_blocks_reference(W, M, Xs, b, g, R), "f32" if dtype == np.float32 else "f16")
 
 
-@pytest.mark.parametrize("n,cin,cout,h,w,k,stride,pad", [(1, 200, 20, 7, 7, 3, 1, 1), (3, 20, 130, 14, 14, 3, 2, 1), (2, 33, 40, 9, 8, 3, 1, 0)])
+@pytest.mark.parametrize("n,cin,cout,h,w,k,stride,pad", [(1, 200, 200, 7, 7, 3, 1, 1), (30, 40, 130, 14, 14, 3, 2, 1), (20, 65, 140, 9, 8, 3, 1, 0)])
 def test_infinite_and_nan_inputs_of_a_kxk_layer(alcs, n, cin, cout, h, w, k, stride, pad):
-    """(The first is small enough for its columns to be split.)"""
+    """(The first is small enough for its columns to be split; dense enough for the tensor cores.)"""
     import torch
-    g = 4
-    W, M, _, b = _case(n + cin, n, cin * k * k, cout, 1, g, 0.3)
+    g = 1
+    W, M, _, b = _case(n + cin, n, cin * k * k, cout, 1, g, 0.8)
     X = _with_specials(rng.normal(n + cin, 2, n * cin * h * w).reshape(n, cin, h * w).astype(np.float32), 7, 3e-4).reshape(n, cin, h, w)
     oh, ow = (h + 2 * pad - k) // stride + 1, (w + 2 * pad - k) // stride + 1
     p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
@@ -533,3 +533,62 @@ def test_planned_strided_and_residual_layers(alcs, n, cin, cout, h, wd, g, strid
     torch.cuda.synchronize()
     assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
     alcs.alcs_stack_destroy(stack)
+
+
+def _conv2d(alcs, p, X, b, cout, k, stride, pad, cfg=None):
+    import torch
+    n, cin, h, w = X.shape
+    oh, ow = (h + 2 * pad - k[0]) // stride + 1, (w + 2 * pad - k[1]) // stride + 1
+    y = torch.full((n, cout, oh, ow), float("nan"), device="cuda")
+    alcs.alcs_spconv2d(p, torch.from_numpy(X).cuda(), y, n, cin, h, w, k[0], k[1], stride, pad, torch.from_numpy(b).cuda(), 0,
+                       torch.cuda.current_stream(), cfg)
+    torch.cuda.synchronize()
+    return y.cpu().numpy()
+
+
+_CONV_CFG = ("positions_per_lane", "strip_rows", "row_groups", "chunk_channels", "images_per_item")
+
+
+# n, cin, cout, h, w, kh, kw, stride, pad: patches of one and of several images, rows copied by 16, 8 and 4 bytes, channel
+# blocks with a remainder, borders on every side; dense enough for the tensor cores to be chosen
+@pytest.mark.parametrize("n,cin,cout,h,w,kh,kw,stride,pad", [(8, 40, 160, 14, 14, 3, 3, 1, 1), (100, 65, 150, 9, 8, 3, 3, 2, 1), (4, 129, 300, 7, 7, 3, 3, 1, 1),
+                                                            (12, 24, 130, 28, 30, 1, 3, 1, 1), (3, 100, 136, 12, 12, 5, 5, 1, 2), (8, 130, 160, 11, 8, 1, 1, 1, 0)])
+def test_dense_kxk_layers_on_the_tensor_cores_and_sparse_ones_not(alcs, n, cin, cout, h, w, kh, kw, stride, pad):
+    g, X = 1, rng.normal(n + cin, 2, n * cin * h * w).reshape(n, cin, h, w).astype(np.float32)
+    for density in (1.0, 0.005):
+        W, M, _, b = _case(n + cin + h, n, cin * kh * kw, cout, 1, g, density)
+        p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+        plan = alcs.alcs_spconv2d_plan(p, n, cin, h, w, kh, kw, stride, pad)
+        cores = _conv2d(alcs, p, X, b, cout, (kh, kw), stride, pad, {k: plan[k] for k in _CONV_CFG})
+        Y = _conv2d(alcs, p, X, b, cout, (kh, kw), stride, pad)
+        Yref, A = oracle.conv2d(W.reshape(cout, cin, kh, kw), M, X, b, False, g, stride, pad, want_scale=True)
+        assert_parity(cores, Yref, A, "f32")
+        assert_parity(Y, Yref, A, "f32")
+        # (the kernels differ in the order of their sums, so the bits show which one ran)
+        if density == 1.0:
+            assert not np.array_equal(Y, cores)
+
+
+@pytest.mark.parametrize("n,cin,cout,h", [(1, 512, 512, 7), (16, 96, 96, 14)])
+def test_kxk_layer_under_capture(alcs, n, cin, cout, h):
+    """The first takes split columns, whose partial sums are the graph's own memory; replays see new inputs."""
+    import torch
+    g = 4
+    W, M, _, b = _case(n + cin, n, cin * 9, cout, 1, g, 0.5)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    X = rng.normal(3, 2, 2 * n * cin * h * h).reshape(2, n, cin, h, h).astype(np.float32)
+    x, y, bd, side = torch.from_numpy(X[0]).cuda(), torch.zeros((n, cout, h, h), device="cuda"), torch.from_numpy(b).cuda(), torch.cuda.Stream()
+    call = lambda: alcs.alcs_spconv2d(p, x, y, n, cin, h, h, 3, 3, 1, 1, bd, 0, side)
+    side.wait_stream(torch.cuda.current_stream())
+    call()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        call()
+    for i in (1, 0, 1):
+        x.copy_(torch.from_numpy(X[i]))
+        y.fill_(float("nan"))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        Yref, A = oracle.conv2d(W.reshape(cout, cin, 3, 3), M, X[i], b, False, g, 1, 1, want_scale=True)
+        assert_parity(y.cpu().numpy(), Yref, A, "f32")
