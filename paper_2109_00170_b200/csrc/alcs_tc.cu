@@ -493,19 +493,30 @@ __device__ __forceinline__ void store32(float (&v)[32], const TcLayer& y, char* 
     }
 }
 
-// An item whose tile keeps no block: bias and residual alone.
+// An item whose tile keeps no block: bias and residual alone, four channels at a time (one at a time, each waited for its
+// loads: 230 us for 60 -> 644 channels, 56 x 56, batch 22, fp16, 1 % kept, most of whose tiles are empty).
 template <typename YT>
 __device__ __forceinline__ void store_bias(const TcLayer& y, char* out, const char* res, unsigned lane_off, int row0, int rows, bool live)
 {
     const unsigned pitch = (unsigned)y.hw.d * (unsigned)sizeof(YT);
 #pragma unroll 1
-    for (int j = 0; j < rows; ++j) {
-        const int c = channel_of(y, row0 + j);
-        if (live && c >= 0) {
-            float v = y.bias ? __ldg(y.bias + c) : 0.0f;
-            if (res) v += (float)__ldg(reinterpret_cast<const YT*>(res + (lane_off + c * pitch)));
-            put(reinterpret_cast<YT*>(out + (lane_off + c * pitch)), y.relu ? fmaxf(v, 0.0f) : v);
+    for (int j = 0; j < rows; j += 4) {
+        int c[4];
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k] = live && j + k < rows ? channel_of(y, row0 + j + k) : -1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = y.bias && c[k] >= 0 ? __ldg(y.bias + c[k]) : 0.0f;
+        if (res) {
+            YT r[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) r[k] = __ldg(reinterpret_cast<const YT*>(res + (live ? lane_off + max(c[k], 0) * pitch : 0)));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] += (float)r[k];
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (c[k] >= 0) put(reinterpret_cast<YT*>(out + (lane_off + c[k] * pitch)), y.relu ? fmaxf(v[k], 0.0f) : v[k]);
     }
 }
 

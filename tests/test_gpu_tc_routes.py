@@ -592,3 +592,24 @@ def test_kxk_layer_under_capture(alcs, n, cin, cout, h):
         torch.cuda.synchronize()
         Yref, A = oracle.conv2d(W.reshape(cout, cin, 3, 3), M, X[i], b, False, g, 1, 1, want_scale=True)
         assert_parity(y.cpu().numpy(), Yref, A, "f32")
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float16])
+@pytest.mark.parametrize("residual", [False, True])
+def test_mostly_empty_channel_tiles(alcs, dtype, residual):
+    """Tiles that keep nothing are bias and residual alone, for channel counts that do not end on four, and beside tiles
+    that keep something, in and out of order of length."""
+    import torch
+    n, cin, cout, h, g = 3, 60, 158, 14, 2
+    W, M, X, b = _case(5, n, cin, cout, h * h, g, 0.5, dtype)
+    M[8:] = 0
+    M[70, 3] = 1
+    R = rng.normal(6, 5, n * cout * h * h).reshape(n, cout, h * h).astype(dtype)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    for tiles in (2, 5, 10):
+        y = torch.full((n, cout, h * h), float("nan"), dtype=torch.from_numpy(X).dtype, device="cuda")
+        alcs.alcs_spconv1x1_ex(p, torch.from_numpy(X).cuda(), y, n, h, h, 1, torch.from_numpy(b).cuda(), torch.from_numpy(R).cuda() if residual else None,
+                               alcs.ALCS_RELU, torch.cuda.current_stream(), dict(math_mode=4, row_groups=tiles))
+        torch.cuda.synchronize()
+        Yref, A = oracle.conv1x1_ex(W, M, X.reshape(n, cin, h, h), b, R if residual else None, True, g, 1, want_scale=True)
+        assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
