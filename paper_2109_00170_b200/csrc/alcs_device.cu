@@ -522,7 +522,7 @@ int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>&
         const int count = tc_widths(w, n);
         for (int i = 0; i < count; ++i) out.push_back(tc_plan(w, n[i], c, di.sms));
     }
-    if (!quick && c.stride == 1 && !c.residual && hw > 0 && c.images() <= 8) {        // small batches only: one thread block per (block row, image, pixel tile)
+    if (!quick && c.stride == 1 && !c.residual && hw > 0 && c.images() <= kGatherImages) {        // small batches only: one thread block per (block row, image, pixel tile)
         for (int p = 8; p >= 2; p /= 2)
             for (int ks = 4; ks <= 16; ks *= 2) {
                 Plan g;
@@ -1991,7 +1991,7 @@ int stack_candidates(const alcs_stack::Item& it, std::vector<Plan>& out)
                 if (!(extra && p.gather) && !(L.stride > 1 && p.tc_n)) out.push_back(p);
     }
     const bool had = !out.empty();
-    const bool small = !extra && it.oh * it.ow > 0 && it.q / ((long long)it.oh * it.ow) <= 8;
+    const bool small = !extra && it.oh * it.ow > 0 && it.q / ((long long)it.oh * it.ow) <= kGatherImages;
     if (had && !small) return ALCS_OK;
     std::vector<Plan> all;
     const int rc = enumerate_plans(L.w, call_shape(it), all);

@@ -613,3 +613,20 @@ def test_mostly_empty_channel_tiles(alcs, dtype, residual):
         torch.cuda.synchronize()
         Yref, A = oracle.conv1x1_ex(W, M, X.reshape(n, cin, h, h), b, R if residual else None, True, g, 1, want_scale=True)
         assert_parity(y.cpu().numpy(), Yref, A, "f32" if dtype == np.float32 else "f16")
+
+
+def test_tuner_lists_what_an_untuned_call_may_run(alcs):
+    """The planner considers the small-problem kernel for up to 64 images; so must the list that the tuner times (which is
+    also where a configuration that names the kernel alone looks for its shape)."""
+    import torch
+    n, cin, cout, h, g = 24, 57, 48, 14, 16
+    W, M, X, b = _case(3, n, cin, cout, h * h, g, 0.1)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    x, y, st = torch.from_numpy(X).cuda(), torch.empty((n, cout, h * h), device="cuda"), torch.cuda.current_stream()
+    alcs.alcs_spconv1x1(p, x, y, n, h, h, None, 0, st, dict(math_mode=3))
+    torch.cuda.synchronize()
+    Yref, A = oracle.conv1x1(W, M, X, None, False, g, want_scale=True)
+    assert_parity(y.cpu().numpy(), Yref, A, "f32")
+    alcs.alcs_spconv1x1_tune(p, x, y, n, h, h, None, 0, st)
+    torch.cuda.synchronize()
+    assert_parity(y.cpu().numpy(), Yref, A, "f32")
