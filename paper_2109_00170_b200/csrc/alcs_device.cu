@@ -1447,9 +1447,11 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
     if (best_i < 0) return ALCS_ERR_CUDA;
     alcs_launch_cfg c;
     plan_to_cfg(all[best_i], &c);
+    all[best_i].cost = 1e-3 * best_ms;
     {
         std::lock_guard<std::mutex> lk(w->mu);
         w->tuned[alcs::ShapeKey{n, h, wd, flags}] = c;
+        w->tuned_alone.insert(alcs::ShapeKey{n, h, wd, flags});
         w->plan_cache[alcs::ShapeKey{n, h, wd, flags}] = all[best_i];
         std::vector<Plan>& fin = w->finalists[alcs::ShapeKey{n, h, wd, flags}];
         fin.clear();
@@ -1489,6 +1491,7 @@ ALCS_API int alcs_spconv1x1_set_cfg(alcs_packed* w, int n, int h, int wd, unsign
     std::lock_guard<std::mutex> lk(w->mu);
     const alcs::ShapeKey key{n, h, wd, flags};
     w->tuned[key] = full;
+    w->tuned_alone.erase(key);
     w->plan_cache[key] = plan;
     return ALCS_OK;
 }
@@ -1657,8 +1660,8 @@ size_t merge_end(const alcs_stack* s, size_t first, F eligible)
 // Fixed cost of a merged launch, first copies and last stores included, in microseconds.
 constexpr double kMergedRampUs = 5.0;
 
-// Consecutive independent layers whose configuration nobody fixed: one launch of the tcgen05 kernel for all of
-// them, where its estimate is below the sum of the layers' own.  With few items in all, narrower tiles shorten
+// Consecutive independent layers whose configuration nobody fixed for the stack: one launch of the tcgen05 kernel for
+// all of them, where its estimate is below the sum of the layers' own (measured ones, after alcs_spconv1x1_tune).  With few items in all, narrower tiles shorten
 // the longest SM's share; with many, wide ones do the least work.
 // fixed_too: of whatever was fixed, too (alcs_stack_tune).
 void stack_merge(alcs_stack* s, bool fixed_too = false)
@@ -1667,8 +1670,9 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
         const alcs_layer& L = it.layer;
         if (L.stride > 1 || !tc_ok(L.w, call_shape(it))) return false;
         if (fixed_too) return true;
+        const alcs::ShapeKey key{L.n, it.oh, it.ow, L.flags};
         std::lock_guard<std::mutex> lk(L.w->mu);
-        return L.w->tuned.find(alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}) == L.w->tuned.end();
+        return L.w->tuned.find(key) == L.w->tuned.end() || L.w->tuned_alone.count(key) != 0;
     };
     for (size_t i = 0; i < s->items.size();) {
         const size_t end = s->items[i].q ? merge_end(s, i, open) : i;
@@ -2081,6 +2085,7 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
         const alcs::ShapeKey key{L.n, it.oh, it.ow, key_flags(L.w, L.flags, call_shape(it))};
         std::lock_guard<std::mutex> lk(L.w->mu);
         L.w->tuned[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}] = c;
+        L.w->tuned_alone.erase(alcs::ShapeKey{L.n, it.oh, it.ow, L.flags});
         L.w->plan_cache[key] = it.plan;
     }
     cur = time_stack(s, st, e0, e1, reps);      // (also leaves a graph stack captured with the chosen plans)

@@ -7,6 +7,8 @@
 #include <array>
 #include <cstdint>
 #include <map>
+#include <memory>
+#include <set>
 #include <mutex>
 #include <tuple>
 #include <vector>
@@ -137,6 +139,9 @@ struct alcs_packed {
     // (0: the CUDA cores) and parts of its columns
     mutable std::map<std::array<int, 8>, std::array<int, 2>> conv2d_choice;
     mutable std::map<alcs::ShapeKey, alcs_launch_cfg> tuned;   // filled by alcs_spconv1x1_tune, alcs_spconv1x1_set_cfg, alcs_stack_tune
+    // those of `tuned` that alcs_spconv1x1_tune measured (its plan's cost is the time): the best for a call by itself, which
+    // a stack may run otherwise
+    mutable std::set<alcs::ShapeKey> tuned_alone;
     // the best few plans of the last alcs_spconv1x1_tune per shape, best first: what alcs_stack_tune tries in context
     mutable std::map<alcs::ShapeKey, std::vector<alcs::Plan>> finalists;
     mutable std::map<alcs::ShapeKey, alcs::Plan> plan_cache;   // resolved plans, by shape

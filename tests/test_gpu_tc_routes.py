@@ -630,3 +630,28 @@ def test_tuner_lists_what_an_untuned_call_may_run(alcs):
     alcs.alcs_spconv1x1_tune(p, x, y, n, h, h, None, 0, st)
     torch.cuda.synchronize()
     assert_parity(y.cpu().numpy(), Yref, A, "f32")
+
+
+def test_stack_of_tuned_layers_is_still_one_launch(alcs):
+    """A layer tuned by itself may run otherwise in a stack: 13 layers of one image, tuned one by one, took 63 us in launches
+    of their own against 23 in one.  A configuration that was set holds."""
+    import torch
+    layers, keep, st = [], [], torch.cuda.current_stream()
+    for i, (cin, cout, h) in enumerate([(128, 256, 28), (256, 256, 28), (512, 512, 14), (512, 512, 14), (512, 1024, 7), (1024, 1024, 7)]):
+        W, M, X, b = _case(90 + i, 1, cin, cout, h * h, 4, 0.2)
+        p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 4), 0)
+        x, y, bd = torch.from_numpy(X).cuda(), torch.empty((1, cout, h * h), device="cuda"), torch.from_numpy(b).cuda()
+        alcs.alcs_spconv1x1_tune(p, x, y, 1, h, h, bd, alcs.ALCS_RELU, st)
+        layers.append(dict(w=p, x=x, y=y, n=1, h=h, wd=h, bias=bd, flags=alcs.ALCS_RELU))
+        keep.append(oracle.conv1x1(W, M, X, b, True, 4, want_scale=True))
+    stack = alcs.alcs_stack_create(layers, 0)
+    assert {alcs.alcs_stack_layer_cfg(stack, i)["math_mode"] for i in range(len(layers))} == {4}
+    alcs.alcs_stack_run(stack, st)
+    torch.cuda.synchronize()
+    for L, (Yref, A) in zip(layers, keep):
+        assert_parity(L["y"].cpu().numpy(), Yref, A, "f32")
+    alcs.alcs_stack_destroy(stack)
+    alcs.alcs_spconv1x1_set_cfg(layers[2]["w"], 1, 14, 14, alcs.ALCS_RELU, dict(math_mode=3, pixels_per_lane=2, warps=4))
+    stack = alcs.alcs_stack_create(layers, 0)
+    assert alcs.alcs_stack_layer_cfg(stack, 2)["math_mode"] == 3
+    alcs.alcs_stack_destroy(stack)
