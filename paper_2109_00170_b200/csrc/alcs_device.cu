@@ -884,7 +884,7 @@ alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& p
 // Launch the tcgen05 kernel for one layer; strided layers run by patch staging.
 int launch_tc_plan(const alcs_packed* w, const Plan& p, const alcs::TcProblem& pr, cudaStream_t st)
 {
-    alcs::TcPrep* t = nullptr;
+    alcs::TcForm t;
     const int rc = alcs::tc_prepare(w, tc_key(w, p, pr), st, &t);
     return rc ? rc : alcs::tc_run(w, *t, pr, st);
 }
@@ -1092,6 +1092,7 @@ struct alcs_stack {
         int first, count;
         std::unique_ptr<alcs::TcArgs<alcs::kTcMaxLayers>> args;
         int* sched = nullptr;       // device
+        std::vector<alcs::TcForm> forms;        // what args refer to
     };
     std::vector<Run> runs;
     bool runs_valid = false;
@@ -1251,7 +1252,7 @@ ALCS_API void alcs_packed_free(alcs_packed* p)
         if (cudaGetDevice(&prev) == cudaSuccess && cudaSetDevice(p->device) == cudaSuccess) {
             for (auto& kv : p->sched) free_schedule_device(kv.second);
             for (auto& kv : p->sched2d) free_schedule_device(kv.second);
-            for (auto& kv : p->tc) alcs::tc_free(kv.second);
+            p->tc.clear();
             cudaFree(p->d_err);
             cudaFree(p->d_xpad);
             cudaFree(p->d_row_ptr);      // (the other two arrays lie in the same block)
@@ -1374,6 +1375,7 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
     if (rc) return rc;
     if (q == 0) return ALCS_OK;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    const alcs::TcForms forms = alcs::tc_forms(w);
     std::vector<Plan> all;
     rc = enumerate_plans(w, {n, h, wd, h, wd}, all);
     if (rc) return rc;
@@ -1469,6 +1471,7 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
                 if (!used) { free_schedule_device(kv.second); kv.second.n_rg = 0; }
             }
     }
+    alcs::tc_release(w, forms);         // the expanded weights of the widths that did not win
     // leave y holding the result of the chosen configuration
     rc = launch_plan(w, all[best_i], x, y, n, h, wd, bias, flags, st);
     if (best) *best = c;
@@ -1717,7 +1720,7 @@ int stack_make_resident(alcs_stack* s)
         if (it.plan.gather) {
             rc = ensure_canonical_on_device(w, nullptr);
         } else if (it.plan.tc_n) {
-            alcs::TcPrep* t = nullptr;
+            alcs::TcForm t;
             rc = alcs::tc_prepare(w, tc_key(w, it.plan, tc_problem(it)), nullptr, &t);
         } else {
             Schedule* sc = get_schedule(w, it.plan.kc, it.plan.n_rg, true, flavour_of(g_variants[it.plan.variant].v));
@@ -1782,11 +1785,12 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
     std::vector<std::vector<double>> us(run.count);       // per layer and channel tile
     for (int i = 0; i < run.count; ++i) {
         const auto& it = s->items[first + i];
-        alcs::TcPrep* t = nullptr;
+        alcs::TcForm t;
         rc = alcs::tc_prepare(it.layer.w, tc_key(it.layer.w, it.plan, tc_problem(it)), nullptr, &t);
         if (rc) return rc;
         rc = alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
         if (rc) return rc;
+        run.forms.push_back(t);
         for (int k16 : t->k16) us[i].push_back(alcs::tc_tile_us(it.layer.w, tc_problem(it), t->n, k16, t->cols != nullptr, t->chan != nullptr));
     }
     rc = alcs::tc_finish(w0, a, false);
@@ -2026,6 +2030,9 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
     struct Done { cudaEvent_t a, b; ~Done() { cudaEventDestroy(a); cudaEventDestroy(b); } } done{e0, e1};
     const int scratch_rc = stack_scratch(s, true);
     if (scratch_rc) return scratch_rc;
+    std::map<const alcs_packed*, alcs::TcForms> forms;
+    for (const auto& it : s->items)
+        if (!forms.count(it.layer.w)) forms[it.layer.w] = alcs::tc_forms(it.layer.w);
     double cur = time_stack(s, st, e0, e1, 3);
     if (cur < 0) return ALCS_ERR_CUDA;
     const int reps = (int)std::min(100.0, std::max(3.0, 3000.0 / std::max(cur, 1.0)));     // batches of about 3 ms
@@ -2090,6 +2097,7 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
     }
     cur = time_stack(s, st, e0, e1, reps);      // (also leaves a graph stack captured with the chosen plans)
     if (cur < 0) return ALCS_ERR_CUDA;
+    for (const auto& f : forms) alcs::tc_release(f.first, f.second);
     if (us_after) *us_after = cur;
     return ALCS_OK;
 }
@@ -2179,7 +2187,7 @@ extern "C" ALCS_API int alcs_spconv1x1_noalloc(const alcs_packed* w, const void*
             const size_t row = (size_t)h * wd * w->elt();
             if (row % 16 != 0 && (size_t)n * w->cin * ((row + 15) / 16 * 16) > ALCS_NOALLOC_SCRATCH_BYTES) return ALCS_ERR_TOO_LARGE;
             const alcs::TcProblem pr = tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd);
-            const alcs::TcPrep* t = plan.tc_n ? alcs::tc_find(w, tc_key(w, plan, pr)) : nullptr;
+            const alcs::TcPrep* t = plan.tc_n ? alcs::tc_find(w, tc_key(w, plan, pr)).get() : nullptr;
             if (!t) t = alcs::tc_any_pointwise(w);
             if (!t) return ALCS_ERR_STATE;
             rc = alcs::tc_run(w, *t, pr, st);

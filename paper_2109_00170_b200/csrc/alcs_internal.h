@@ -133,8 +133,8 @@ struct alcs_packed {
     // plane, plane pitch, stride, kh, kw, channels per chunk}: the column offsets baked into them depend
     // on the geometry
     mutable std::map<std::array<int, 8>, alcs::Schedule> sched2d;
-    // expanded weights of the tcgen05 kernel, by {channels per tile, kh, kw} (alcs_tc_prep.h)
-    mutable std::map<std::array<int, 3>, alcs::TcPrep*> tc;
+    // expanded weights of the tcgen05 kernel, by {channels per tile, kh, kw, splits} (alcs_tc_prep.h); stacks share them
+    mutable std::map<std::array<int, 4>, std::shared_ptr<alcs::TcPrep>> tc;
     // which kernel a k x k layer runs on, by {n, cin, h, w, kh, kw, stride, pad}: channels per tile of the tcgen05 kernel
     // (0: the CUDA cores) and parts of its columns
     mutable std::map<std::array<int, 8>, std::array<int, 2>> conv2d_choice;

@@ -123,9 +123,9 @@ bool skewed(const alcs_packed& w)
 
 }  // namespace
 
-TcPrep* tc_find(const alcs_packed* w, const TcKey& key)
+TcForm tc_find(const alcs_packed* w, const TcKey& key)
 {
-    auto it = w->tc.find({key.n + key.splits * 1024, key.kh, key.kw});
+    auto it = w->tc.find(key.id());
     return it == w->tc.end() ? nullptr : it->second;
 }
 
@@ -134,18 +134,30 @@ const TcPrep* tc_any_pointwise(const alcs_packed* w)
 {
     const TcPrep* best = nullptr;
     for (const auto& kv : w->tc)
-        if (kv.first[1] <= 1 && kv.first[2] <= 1 && kv.second->splits == 1 && (!best || kv.second->n > best->n)) best = kv.second;
+        if (kv.first[1] <= 1 && kv.first[2] <= 1 && kv.second->splits == 1 && (!best || kv.second->n > best->n)) best = kv.second.get();
     return best;
 }
 
-void tc_free(TcPrep* p)
+TcForms tc_forms(const alcs_packed* w)
 {
-    if (!p) return;
-    cudaFree(p->b);
-    delete p;
+    std::lock_guard<std::mutex> lk(w->mu);
+    TcForms keys;
+    for (const auto& kv : w->tc) keys.push_back(kv.first);
+    return keys;
 }
 
-int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep** out)
+void tc_release(const alcs_packed* w, const TcForms& before)
+{
+    std::lock_guard<std::mutex> lk(w->mu);
+    for (auto it = w->tc.begin(); it != w->tc.end();) {
+        bool keep = it->first[1] > 1 || it->first[2] > 1 || it->first[3] > 1 || it->second.use_count() > 1 ||
+                    std::find(before.begin(), before.end(), it->first) != before.end();
+        for (const auto& pc : w->plan_cache) keep = keep || pc.second.tc_n == it->first[0];
+        it = keep ? std::next(it) : w->tc.erase(it);        // (cudaFree waits for whatever still runs)
+    }
+}
+
+int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcForm* out)
 {
     {
         std::lock_guard<std::mutex> lk(w->mu);
@@ -262,9 +274,11 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep**
         p.cols = list ? reinterpret_cast<int*>(d + o_cols) : nullptr;
         p.chan = chan.empty() ? nullptr : reinterpret_cast<int*>(d + o_chan);
         p.uploaded = true;
-        TcPrep* kept = new TcPrep(p);
-        w->tc[{key.n + key.splits * 1024, key.kh, key.kw}] = kept;
-        *out = kept;
+        *out = TcForm(new TcPrep(p), [](TcPrep* f) {
+            cudaFree(f->b);
+            delete f;
+        });
+        w->tc[key.id()] = *out;
     } catch (const std::bad_alloc&) {
         return ALCS_ERR_ALLOC;
     }
@@ -587,7 +601,7 @@ int tc_conv2d(const alcs_packed* w, const TcProblem& p, int n, int splits, cudaS
     int sms = 0, smem = 0;
     int rc = device_limits(w->device, &sms, &smem);
     if (rc) return rc;
-    TcPrep* t = nullptr;
+    TcForm t;
     rc = tc_prepare(w, {n, p.kh, p.kw, splits}, st, &t);
     if (rc) return rc;
     if (splits == 1) return tc_run(w, *t, p, st);

@@ -2,6 +2,8 @@
 #ifndef ALCS_TC_PREP_H_
 #define ALCS_TC_PREP_H_
 
+#include <array>
+#include <memory>
 #include <vector>
 
 #include "alcs_internal.h"
@@ -14,6 +16,7 @@ namespace alcs {
 struct TcKey {
     int n, kh, kw;
     int splits = 1;      // patch staging: parts the channel blocks are split into, a tile of its own each
+    std::array<int, 4> id() const { return {n, kh, kw, splits}; }
 };
 
 struct TcPrep {
@@ -37,10 +40,14 @@ struct TcProblem {
     unsigned flags;
 };
 
-int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcPrep** out);
-TcPrep* tc_find(const alcs_packed* w, const TcKey& key);       // already prepared, or null; caller holds w->mu
+using TcForm = std::shared_ptr<TcPrep>;
+int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcForm* out);
+TcForm tc_find(const alcs_packed* w, const TcKey& key);        // already prepared, or null; caller holds w->mu
 const TcPrep* tc_any_pointwise(const alcs_packed* w);          // a prepared form for pointwise layers, or null; caller holds w->mu
-void tc_free(TcPrep* p);
+// Release the pointwise forms that are not among `before` (keys), in no cached plan and in no stack.
+using TcForms = std::vector<std::array<int, 4>>;
+TcForms tc_forms(const alcs_packed* w);
+void tc_release(const alcs_packed* w, const TcForms& before);
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out);
 // Estimates, in microseconds, from the shape and the weights alone.
 double tc_tile_us(const alcs_packed* w, const TcProblem& p, int n, int k16, bool list, bool sorted);

@@ -655,3 +655,35 @@ def test_stack_of_tuned_layers_is_still_one_launch(alcs):
     stack = alcs.alcs_stack_create(layers, 0)
     assert alcs.alcs_stack_layer_cfg(stack, 2)["math_mode"] == 3
     alcs.alcs_stack_destroy(stack)
+
+
+def test_tuning_releases_the_expanded_weights_that_lost(alcs):
+    """25 MB for every width of a 2048 x 2048 layer in fp32, eight widths tried; forms that were there before stay."""
+    import torch
+    st, g = torch.cuda.current_stream(), 4
+
+    def layer(n, cin, cout, h):
+        W, M, X, _ = _case(3, n, cin, cout, h * h, g, 0.5)
+        p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+        return p, W, M, X, torch.from_numpy(X).cuda(), torch.empty((n, cout, h * h), device="cuda")
+
+    p, *_, x, y = layer(4, 256, 256, 14)
+    alcs.alcs_spconv1x1_tune(p, x, y, 4, 14, 14, None, 0, st)          # (loads the kernels that are timed)
+    p, W, M, X, x, y = layer(4, 2048, 2048, 14)
+    alcs.alcs_spconv1x1(p, x, y, 4, 14, 14, None, 0, st, dict(math_mode=4, row_groups=16))
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        alcs.alcs_spconv1x1(p, x, y, 4, 14, 14, None, 0, side, dict(math_mode=4, row_groups=16))
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    alcs.alcs_spconv1x1_tune(p, x, y, 4, 14, 14, None, 0, st)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] < 80 << 20
+    Yref, A = oracle.conv1x1(W, M, X, None, False, g, want_scale=True)
+    assert_parity(y.cpu().numpy(), Yref, A, "f32")
+    y.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert_parity(y.cpu().numpy(), Yref, A, "f32")
