@@ -307,7 +307,7 @@ bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const Devic
     const double px = (double)n * tiles * 32.0 * p;
     const double l2 = (double)w->nb * px * 4 / (vec ? 9.9e6 : 4.4e6), fma = (double)w->nb * w->g * px * 28.1e-6 / sms;
     const double hbm = (double)n * hw * (w->cin + w->cout) * 4 / 7.0e6;
-    pl.cost = 1e-6 * (2.8 + std::max({loads, l2, fma, hbm}));
+    pl.cost = 1e-6 * (2.0 + std::max({loads, l2, fma, hbm}));
     *out = pl;
     return true;
 }
@@ -412,6 +412,27 @@ bool direct_rows_ok(int hw, int elt) { return ((size_t)hw * elt) % 16 == 8; }
 // How many of the best candidates the tuner times a second time and remembers for alcs_stack_tune.
 constexpr size_t kFinalists = 12;
 
+// Schedules a first call builds to choose among.
+constexpr size_t kQuickSchedules = 3;
+
+// The sizes of a schedule without building it, for rows of equal length: a segment (block row, chunk) of `len` blocks takes
+// about len / 2 + 1/4 pair records, or len / 16 + 1/2 step records.
+Schedule guess_schedule(const alcs_packed* w, const KernelVariant& v, int kc, int n_rg)
+{
+    Schedule s;
+    const int cap = v.nw / v.groups * v.rw;
+    s.kc = kc;
+    s.nch = (w->cin + kc - 1) / kc;
+    s.n_rg = v.mma ? std::max(1, std::min(n_rg, w->rows)) : std::max(std::max(1, (w->rows + cap - 1) / cap), std::min(n_rg, w->rows));
+    s.rpg = v.mma ? (w->rows + s.n_rg - 1) / s.n_rg : cap;
+    s.ros = 4 * s.rpg;
+    const double segments = (double)w->rows * s.nch, len = w->nb / segments, per = v.mma ? 16.0 : 2.0;
+    const double records = segments * std::min(len, len / per + 0.5 * (1.0 - 1.0 / per));
+    s.n_rec = (int)(records * (v.mma ? alcs::step_record_bytes(v.g) : alcs::record_bytes(v.g)) / 16.0);
+    s.wcap = (int)(1.2 * s.n_rec / ((double)s.n_rg * s.nch)) + 16;
+    return s;
+}
+
 // Internal bits of the flags in plan-cache keys, which else hold the output size alone: kExtra says that the call has a
 // residual operand or a stride (which the small-problem kernel does not take), the others which, and how its input
 // rows can be copied.
@@ -426,8 +447,9 @@ unsigned key_flags(const alcs_packed* w, unsigned flags, const CallShape& c)
 }
 
 // Enumerate every valid launch configuration for this shape, cheapest (by the model) first.
-// quick: the kernels that stage X through shared memory alone, with row-group counts a quarter apart: what a first call
-// can wait for (the full list of a 2048 x 2048 layer takes a second).
+// quick: the kernels that stage X through shared memory alone, ranked by guessed schedules; the first few are then built and
+// the best of those is put in front.  For a first call, which cannot wait for all schedules to be built (a second or
+// more for a 2048 x 2048 layer).
 int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>& out, bool quick = false)
 {
     const long long q = std::max(1ll, c.q());
@@ -444,7 +466,7 @@ int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>&
     out.clear();
     for (size_t vi = 0; vi < g_variants.size(); ++vi) {
         const KernelVariant& v = g_variants[vi].v;
-        if (v.is_f16 != (int)w->dt || v.g != w->g) continue;
+        if (v.is_f16 != (int)w->dt || v.g != w->g || (quick && v.split)) continue;
         rc = prepare_variant(g_variants[vi], w->device);
         if (rc) return rc;
         const int cap = v.nw / v.groups * v.rw;
@@ -468,7 +490,8 @@ int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>&
                 const int rpg = (w->rows + n_rg - 1) / n_rg;
                 if (rpg == last_rpg || rpg > cap) continue;
                 last_rpg = rpg;
-                const Schedule* sc = get_schedule(w, kc, n_rg, false, flavour_of(v));
+                const Schedule guess = quick ? guess_schedule(w, v, kc, n_rg) : Schedule();
+                const Schedule* sc = quick ? &guess : get_schedule(w, kc, n_rg, false, flavour_of(v));
                 if (!sc) return ALCS_ERR_ALLOC;
                 if (v.split && sc->max_x == 0) continue;        // nothing to split: the plain variant covers it
                 const StageLayout L = stage_layout(v, *sc, elt);
@@ -530,6 +553,28 @@ int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>&
             }
     }
     std::stable_sort(out.begin(), out.end(), [](const Plan& a, const Plan& b) { return a.cost < b.cost; });
+    if (quick && !out.empty()) {
+        Plan best;
+        best.cost = 1e30;
+        std::vector<std::array<int, 3>> built;
+        for (const Plan& guess : out) {
+            const std::array<int, 3> key = {guess.variant, guess.kc, guess.n_rg};
+            if (std::find(built.begin(), built.end(), key) != built.end()) continue;
+            if (built.size() >= kQuickSchedules && best.cost < 1e30) break;
+            built.push_back(key);
+            const KernelVariant& v = g_variants[guess.variant].v;
+            const Schedule* sc = get_schedule(w, guess.kc, guess.n_rg, false, flavour_of(v));
+            if (!sc) return ALCS_ERR_ALLOC;
+            Plan p = guess;
+            p.n_rg = sc->n_rg;
+            p.smem = plan_smem(stage_layout(v, *sc, elt), p.stages);
+            if (p.smem > (size_t)smem_max || (p.occ = occupancy_of(g_variants[p.variant], p.smem)) < 1) continue;
+            p.cost = guess.cost * model_cost(w, v, *sc, q, di, p.occ) / model_cost(w, v, guess_schedule(w, v, guess.kc, guess.n_rg), q, di, guess.occ);
+            if (p.cost < best.cost) best = p;
+        }
+        if (best.cost >= 1e30) return ALCS_ERR_UNSUPPORTED;
+        out.assign(1, best);
+    }
     return out.empty() ? ALCS_ERR_UNSUPPORTED : ALCS_OK;
 }
 
@@ -1880,7 +1925,6 @@ ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned 
         it.layer = L;
         if (L.stride < 0) { delete s; return ALCS_ERR_INVALID_ARG; }
         const int stride = L.stride > 1 ? L.stride : 1;
-        const bool extra = stride > 1 || L.residual;
         it.oh = (L.h + stride - 1) / stride;
         it.ow = (L.wd + stride - 1) / stride;
         int rc = check_conv_args(L.w, L.x, L.y, L.n, it.oh, it.ow, L.flags, &it.q);
