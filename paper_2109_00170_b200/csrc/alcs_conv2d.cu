@@ -325,7 +325,8 @@ extern "C" ALCS_API int alcs_spconv2d_cfg(const alcs_packed* w, const void* x, v
         const std::array<int, 2> on = kernel_of(w, g, pr, sms, smem_optin);
         if (on[0]) {
             rc = alcs::tc_conv2d(w, pr, on[0], on[1], st);
-            if (rc != ALCS_ERR_UNSUPPORTED) return rc;
+            if (rc != ALCS_ERR_UNSUPPORTED && rc != ALCS_ERR_ALLOC && rc != ALCS_ERR_SHAPE) return rc;
+            // (no memory for the expanded weights or the partial sums, or too many of them: the CUDA cores need none)
         }
     }
     Conv2dPlan p;

@@ -578,6 +578,19 @@ int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>&
     return out.empty() ? ALCS_ERR_UNSUPPORTED : ALCS_OK;
 }
 
+// The staged kernels' plan for a call without a configuration: of the quick list, or, should no guessed schedule have fitted
+// shared memory, of the full one.
+int staged_best(const alcs_packed* w, const CallShape& c, Plan* out)
+{
+    std::vector<Plan> list;
+    int rc = enumerate_plans(w, c, list, true);
+    if (rc == ALCS_ERR_UNSUPPORTED) rc = enumerate_plans(w, c, list);
+    if (rc) return rc;
+    for (const Plan& p : list)
+        if (!p.tc_n && !p.gather) { *out = p; return ALCS_OK; }
+    return ALCS_ERR_UNSUPPORTED;
+}
+
 void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
 {
     if (p.gather) {
@@ -634,7 +647,16 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
         // expected, 120 dense), so those have to promise more.  2048 -> 2048 at 7 x 7, batch 32, 5 % kept: 92 us dense, 49.
         Plan best;
         best.cost = 1e30;
-        if (tc) best = tc_best(w, shape, di.sms);
+        if (tc) {
+            const alcs::TcForms forms = alcs::tc_forms(w);
+            int n[8];
+            const int count = tc_widths(w, n);
+            for (int i = 0; i < count; ++i) {
+                if (!alcs::tc_form_free(w, forms, {n[i], 0, 0})) continue;
+                const Plan p = tc_plan(w, n[i], shape, di.sms);
+                if (p.cost < best.cost) best = p;
+            }
+        }
         if (allow_small && hw > 0 && shape.images() <= kGatherImages)
             for (int p = 8; p >= 2; p /= 2)
                 for (int ks = 4; ks <= 16; ks *= 2) {
@@ -643,11 +665,11 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
                 }
         const double staged = 1e-6 * staged_us(w, shape, di.sms);
         if (staged * (best.cost < 100e-6 ? 1.15 : 1.5) < best.cost) {
-            std::vector<Plan> list;
-            rc = enumerate_plans(w, shape, list, true);
+            Plan p;
+            rc = staged_best(w, shape, &p);
             if (rc && (rc != ALCS_ERR_UNSUPPORTED || best.cost >= 1e30)) return rc;
             if (!rc) {
-                best = list[0];
+                best = p;
                 best.cost = staged;
             }
         }
@@ -1090,6 +1112,21 @@ int resolve_plan(const alcs_packed* w, const CallShape& c, unsigned flags, const
     return ALCS_OK;
 }
 
+// The plan of a call by default whose expanded weights found no memory: the staged kernels, for later calls of the shape, too.
+bool no_room(const Plan& plan, const alcs_launch_cfg* cfg, int rc)
+{
+    return plan.tc_n && !cfg && (rc == ALCS_ERR_ALLOC || rc == ALCS_ERR_SHAPE);
+}
+
+int staged_instead(const alcs_packed* w, const CallShape& c, unsigned flags, Plan* plan)
+{
+    const int rc = staged_best(w, c, plan);
+    if (rc) return rc;
+    std::lock_guard<std::mutex> lk(w->mu);
+    w->plan_cache[alcs::ShapeKey{c.n, c.oh, c.ow, key_flags(w, flags, c)}] = *plan;
+    return ALCS_OK;
+}
+
 }  // namespace
 
 // The same helpers for the other translation units of the library (alcs_internal.h).
@@ -1349,9 +1386,13 @@ ALCS_API int alcs_spconv1x1_cfg(const alcs_packed* w, const void* x, void* y, in
     if (rc) return rc;
     if (q == 0) return ALCS_OK;
     Plan plan;
-    rc = resolve_plan(w, {n, h, wd, h, wd}, flags, cfg, &plan);
+    const CallShape shape{n, h, wd, h, wd};
+    rc = resolve_plan(w, shape, flags, cfg, &plan);
     if (rc) return rc;
-    return launch_plan(w, plan, x, y, n, h, wd, bias, flags, static_cast<cudaStream_t>(cuda_stream));
+    rc = launch_plan(w, plan, x, y, n, h, wd, bias, flags, static_cast<cudaStream_t>(cuda_stream));
+    if (no_room(plan, cfg, rc) && (rc = staged_instead(w, shape, flags, &plan)) == ALCS_OK)
+        rc = launch_plan(w, plan, x, y, n, h, wd, bias, flags, static_cast<cudaStream_t>(cuda_stream));
+    return rc;
 }
 
 ALCS_API int alcs_spconv1x1(const alcs_packed* w, const void* x, void* y, int n, int h, int wd,
@@ -1386,10 +1427,13 @@ ALCS_API int alcs_spconv1x1_ex(const alcs_packed* w, const void* x, void* y, int
         if (rb < yend && yb < rend) return ALCS_ERR_INVALID_ARG;     // the residual may not overlap y
     }
     Plan plan;
-    rc = resolve_plan(w, {n, oh, ow, h, wd, stride, residual != nullptr}, flags, cfg, &plan);
+    const CallShape shape{n, oh, ow, h, wd, stride, residual != nullptr};
+    rc = resolve_plan(w, shape, flags, cfg, &plan);
     if (rc) return rc;
-    return launch_plan(w, plan, x, y, n, oh, ow, bias, flags, static_cast<cudaStream_t>(cuda_stream), nullptr, 0,
-                       residual, stride, h, wd);
+    auto launch = [&] { return launch_plan(w, plan, x, y, n, oh, ow, bias, flags, static_cast<cudaStream_t>(cuda_stream), nullptr, 0, residual, stride, h, wd); };
+    rc = launch();
+    if (no_room(plan, cfg, rc) && (rc = staged_instead(w, shape, flags, &plan)) == ALCS_OK) rc = launch();
+    return rc;
 }
 
 ALCS_API int alcs_spconv1x1_plan(const alcs_packed* w, int n, int h, int wd, unsigned flags,
@@ -1716,7 +1760,7 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
 {
     auto open = [&](const alcs_stack::Item& it) {
         const alcs_layer& L = it.layer;
-        if (L.stride > 1 || !tc_ok(L.w, call_shape(it))) return false;
+        if (L.stride > 1 || !tc_ok(L.w, call_shape(it)) || (long long)L.w->rows * L.w->g * L.w->cin > alcs::kTcMaxWeights) return false;
         if (fixed_too) return true;
         const alcs::ShapeKey key{L.n, it.oh, it.ow, L.flags};
         std::lock_guard<std::mutex> lk(L.w->mu);
@@ -1767,7 +1811,9 @@ int stack_make_resident(alcs_stack* s)
         } else if (it.plan.tc_n) {
             alcs::TcForm t;
             rc = alcs::tc_prepare(w, tc_key(w, it.plan, tc_problem(it)), nullptr, &t);
-        } else {
+            if (no_room(it.plan, nullptr, rc)) rc = staged_instead(w, call_shape(it), it.layer.flags, &it.plan);
+        }
+        if (!rc && !it.plan.gather && !it.plan.tc_n) {
             Schedule* sc = get_schedule(w, it.plan.kc, it.plan.n_rg, true, flavour_of(g_variants[it.plan.variant].v));
             rc = sc ? upload_schedule(w, sc, nullptr) : ALCS_ERR_ALLOC;
         }

@@ -146,6 +146,19 @@ TcForms tc_forms(const alcs_packed* w)
     return keys;
 }
 
+bool tc_form_free(const alcs_packed* w, const TcForms& forms, const TcKey& key)
+{
+    if ((long long)w->rows * w->g * w->cin > kTcMaxWeights) return false;
+    int same = 0;
+    for (const auto& f : forms) {
+        // (a pointwise layer's two forms, of all columns and of lists, go together)
+        const bool size = key.kh <= 1 && key.kw <= 1 ? f[1] <= 1 && f[2] <= 1 : f[1] == key.kh && f[2] == key.kw;
+        if (size && f[0] == key.n && f[3] == key.splits) return true;
+        same += size;
+    }
+    return same < kTcMaxForms;
+}
+
 void tc_release(const alcs_packed* w, const TcForms& before)
 {
     std::lock_guard<std::mutex> lk(w->mu);
@@ -576,6 +589,7 @@ double tc_conv2d_choose(const alcs_packed* w, const TcProblem& p, int sms, int* 
     if (!tc_fits(w, taps, p.n, (long long)p.h_in * p.w_in, hw)) return 0;
     const int blocks = (w->cin / taps + 15) / 16;
     const long long px = (p.n * hw + kTcM - 1) / kTcM;
+    const TcForms forms = tc_forms(w);
     double best = 0;
     for (int want = kTcMaxN; want >= 16; want -= 16) {
         const int want_tiles = (w->cout + want - 1) / want, v = ((w->cout + want_tiles - 1) / want_tiles + 15) / 16 * 16;
@@ -586,6 +600,7 @@ double tc_conv2d_choose(const alcs_packed* w, const TcProblem& p, int sms, int* 
             if ((blocks + part - 1) / part != s) continue;
             const double bytes = (double)s * tiles * v * p.n * hw * 4;
             if (s > 1 && (bytes > (32 << 20) || (double)p.n * hw * w->cout > 1e9)) break;
+            if (!tc_form_free(w, forms, {v, p.kh, p.kw, s})) continue;
             const long long items = px * tiles * s;
             const double us = kPatchRamp + kPatchFirst * std::min(part * taps, 4) +
                               (double)((items + sms - 1) / sms) * tc_tile_us(w, p, v, part * taps, false, false) + (s > 1 ? 5.2 + bytes / 2.8e6 : 0.0);

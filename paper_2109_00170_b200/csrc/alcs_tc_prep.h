@@ -47,6 +47,11 @@ const TcPrep* tc_any_pointwise(const alcs_packed* w);          // a prepared for
 // Release the pointwise forms that are not among `before` (keys), in no cached plan and in no stack.
 using TcForms = std::vector<std::array<int, 4>>;
 TcForms tc_forms(const alcs_packed* w);
+// What a call that asks for no kernel may spend on expanded weights (6 bytes per dense weight in fp32, 2 in 16 bits): matrices of
+// at most kTcMaxWeights, and kTcMaxForms forms per kernel size, beyond which a further batch size takes one that is there.
+constexpr long long kTcMaxWeights = 1ll << 26;
+constexpr int kTcMaxForms = 4;
+bool tc_form_free(const alcs_packed* w, const TcForms& forms, const TcKey& key);       // may `key` be chosen?
 void tc_release(const alcs_packed* w, const TcForms& before);
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out);
 // Estimates, in microseconds, from the shape and the weights alone.

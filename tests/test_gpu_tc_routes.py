@@ -687,3 +687,48 @@ def test_tuning_releases_the_expanded_weights_that_lost(alcs):
     graph.replay()
     torch.cuda.synchronize()
     assert_parity(y.cpu().numpy(), Yref, A, "f32")
+
+
+def test_very_large_matrices_are_not_expanded(alcs):
+    """67 million weights, a thousandth of them kept, would take 400 MB as dense tiles: by default they stay as they are."""
+    import torch
+    n, c, h, g = 4, 8208, 7, 4
+    M = (rng.uniform01(1, 3, c // g * c) < 0.001).astype(np.uint8).reshape(c // g, c)
+    W = np.repeat(rng.normal(1, 1, c).astype(np.float32)[None, :], c, axis=0)
+    X = rng.normal(1, 2, n * c * h * h).reshape(n, c, h * h).astype(np.float32)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    y, x = torch.empty((n, c, h * h), device="cuda"), torch.from_numpy(X).cuda()
+    before = torch.cuda.mem_get_info()[0]
+    alcs.alcs_spconv1x1(p, x, y, n, h, h, None, 0, torch.cuda.current_stream())
+    assert alcs.alcs_spconv1x1_plan(p, n, h, h, 0)["math_mode"] != 4
+    y2 = torch.empty((n, c, h, h), device="cuda")
+    alcs.alcs_spconv2d(p, x, y2, n, c, h, h, 1, 1, 1, 0, None, 0, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] < 350 << 20
+    idx = np.arange(0, y.numel(), 997, dtype=np.int64)
+    Yref = oracle.conv1x1_points(W, M, X, idx)
+    Yref, A = Yref if isinstance(Yref, tuple) else (Yref, None)
+    for t in (y, y2):
+        d = np.abs(t.cpu().numpy().reshape(-1)[idx].astype(np.float64) - Yref)
+        assert (d <= TOL["f32"] * (A if A is not None else np.abs(Yref).max())).all()
+
+
+def test_forms_of_the_expanded_weights_are_bounded(alcs):
+    """Calls of many batch sizes share a few forms: 14 MB each for 512 x 512 x 3 x 3."""
+    import torch
+    cin, cout, h, g = 512, 512, 7, 4
+    W, M, _, _ = _case(3, 1, cin * 9, cout, 1, g, 0.5)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    X = rng.normal(4, 2, 64 * cin * h * h).reshape(64, cin, h, h).astype(np.float32)
+    x, y, st = torch.from_numpy(X).cuda(), torch.empty((64, cout, h, h), device="cuda"), torch.cuda.current_stream()
+    call = lambda n: alcs.alcs_spconv2d(p, x, y, n, cin, h, h, 3, 3, 1, 1, None, 0, st)
+    call(1)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for n in list(range(2, 64)) + [64]:
+        call(n)
+    torch.cuda.synchronize()
+    # three more forms, and what the pool of the partial sums keeps (64 MB)
+    assert before - torch.cuda.mem_get_info()[0] < (3 * 15 + 64 + 16) << 20
+    Yref, A = oracle.conv2d(W.reshape(cout, cin, 3, 3), M, X[-2:], None, False, g, 1, 1, want_scale=True)
+    assert_parity(y[-2:].cpu().numpy(), Yref, A, "f32")
