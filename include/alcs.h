@@ -58,7 +58,7 @@ typedef enum {
     ALCS_F16 = 1,               /* IEEE binary16 weights and activations, fp32 accumulation         */
     ALCS_BF16 = 2               /* bfloat16 weights and activations, fp32 accumulation; by the paper's rule
                                    (Section 3.2.1: group size = register bits / element bits) a 16-bit type
-                                   doubles the group size of fp32, as binary16 does.  CUDA-core kernels only. */
+                                   doubles the group size of fp32, as binary16 does.  CUDA cores or tcgen05; no mma.sync kernel. */
 } alcs_dtype;
 
 /* Bits of the `flags` argument of the convolution entry points. */
@@ -188,7 +188,8 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     tiles of X; fp32 operands are split exactly into three bfloat16 parts each.  Only row_groups
  *                     (the number of channel tiles, each of at most 128 channels) applies; no scratch is used.  Outputs of
  *                     pixels with infinite or NaN inputs are computed from the storage format instead, so that such values
- *                     reach the channels that keep a block of theirs and no others, as with the other kernels (slowly)
+ *                     reach the channels that keep a block of theirs and no others, as with the other kernels (slowly); fp32
+ *                     matrices that keep an infinite or NaN weight are refused (UNSUPPORTED)
  *   consumer_groups   1 = all consumer warps work on one work item at a time; 2 = two halves of the
  *                     consumer warps take the thread block's work items alternately (tensor-core
  *                     kernels only), so that one half multiplies while the other half stores
@@ -232,13 +233,19 @@ ALCS_API int alcs_variant_get(int index, alcs_dtype* dt, int* g, alcs_launch_cfg
  * alcs_spconv1x1: x device [n][cin][h*wd], y device [n][cout][h*wd], both contiguous NCHW of the
  * packed dtype (y fp32 if ALCS_Y_F32); bias device fp32 [cout] or NULL; flags = ALCS_RELU |
  * ALCS_Y_F32.  x and y must not overlap and must be aligned to their element size.  16-byte
- * aligned buffers with h*wd a multiple of 4 (fp32) or 8 (fp16) are used in place.  If the rows of
- * x are not a multiple of 16 bytes long (h*wd = 49, ...) x is first repacked, by a small kernel on
- * the same stream, into scratch memory owned by w (allocated or grown by the first call that
- * needs it; n*cin*round_up(h*wd)*element bytes) and y is stored element by element; results are
- * identical.  Because that scratch belongs to w, two such convolutions with the SAME w must not
- * run concurrently on different streams.  Enqueues one kernel on cuda_stream;
- * no allocation and no synchronisation once this shape has been seen (see alcs_packed_upload).  n == 0 or h*wd == 0 is a successful no-op.
+ * aligned buffers with h*wd a multiple of 4 (fp32) or 8 (fp16) are used in place.
+ * Without a configuration the library chooses, once per shape, between the tcgen05 kernel, the small-problem kernel and
+ * the kernels that stage x through shared memory (math_mode 4, 3, 1 and 2 of alcs_launch_cfg; alcs_spconv1x1_plan
+ * tells which).  The first two read x in place whatever the length of its rows; if a staged kernel runs and the rows
+ * of x are not a multiple of 16 bytes long (h*wd = 49, ...), x is first repacked, by a small kernel on the same stream,
+ * into scratch memory owned by w (allocated or grown by the first call that needs it; n*cin*round_up(h*wd)*element
+ * bytes).  Because that scratch belongs to w, two such convolutions with the SAME w must not run concurrently on
+ * different streams.  Enqueues one kernel, or that pass and one kernel, on cuda_stream; no allocation and no
+ * synchronisation once this shape has been seen (see alcs_packed_upload), wherever x starts.  The tcgen05 kernel's
+ * expanded weights take 6 bytes (fp32) or 2 bytes per weight of the dense matrix and form; by default at most four forms are
+ * made per matrix and kernel size, and none for a matrix of more than 2^26 weights or where memory is short.
+ * Infinite and NaN inputs reach the channels that keep a block of theirs and no others; such pixels are slow on the
+ * tcgen05 kernel.  ReLU turns NaN into 0.  n == 0 or h*wd == 0 is a successful no-op.
  * Errors: INVALID_ARG, SHAPE (n*channels*pixels beyond int32 tiles), UNSUPPORTED (g), STATE (not
  * uploaded / wrong current device), CUDA.
  */
@@ -254,8 +261,9 @@ ALCS_API int alcs_spconv1x1(const alcs_packed* w, const void* x, void* y, int n,
  * oh < ceil(h/stride), ow < ceil(wd/stride).  x device [n][cin][h][wd]; y and residual device
  * [n][cout][oh*ow] of the same element type (the packed dtype, or fp32 with ALCS_Y_F32); residual may be
  * NULL; it must not overlap y.  stride = 1 with residual = NULL is alcs_spconv1x1_cfg.  With stride > 1
- * the pixels that are read are first gathered, by a small kernel on the same stream, into the scratch
- * memory owned by w (see alcs_spconv1x1); the residual is read straight from the caller's buffer in the
+ * the staged kernels first gather the pixels that are read, by a small kernel on the same stream, into the scratch
+ * memory owned by w (see alcs_spconv1x1); the tcgen05 kernel, which takes input rows of a multiple of 8 bytes, reads x
+ * in place; the residual is read straight from the caller's buffer in the
  * epilogue, added in fp32 before ReLU and before the single rounding of an fp16 output.  cfg may be
  * NULL.  Errors as alcs_spconv1x1, plus INVALID_ARG for stride < 1.
  */
@@ -290,7 +298,8 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
 /*
  * alcs_spconv1x1_set_cfg: make later alcs_spconv1x1 / alcs_stack_create calls with this
  * (n, h, wd, flags) use the given configuration, e.g. one that alcs_spconv1x1_tune found in an
- * earlier process.  Fields left 0 are chosen by the library.  Host only; returns UNSUPPORTED if no
+ * earlier process.  Fields left 0 are chosen by the library.  A stack runs such a layer as configured, while one
+ * that alcs_spconv1x1_tune measured by itself may be merged with others where that is faster.  Host only; returns UNSUPPORTED if no
  * compiled kernel variant fits it.
  */
 ALCS_API int alcs_spconv1x1_set_cfg(alcs_packed* w, int n, int h, int wd, unsigned flags,
@@ -300,9 +309,11 @@ ALCS_API int alcs_spconv1x1_set_cfg(alcs_packed* w, int n, int h, int wd, unsign
  * alcs_spconv1x1_host: the same operation on HOST buffers x_host / y_host / bias_host, staged
  * through a caller-provided device workspace of at least alcs_spconv1x1_host_workspace() bytes
  * (256-byte aligned).  Enqueues H2D copies, the kernel and the D2H copy on cuda_stream and
- * returns without synchronising; use pinned host memory for truly asynchronous copies.  A call of a megabyte or
- * more is cut into up to four pieces by images, whose uploads and downloads run on two streams of the library's own
- * beside the convolutions, ordered by events after what is on cuda_stream and before what follows on it.
+ * returns without synchronising; use pinned host memory for truly asynchronous copies.  A call on pinned buffers
+ * of 2 MB and more (x and y together) is cut into up to four pieces of at least a megabyte by images, whose uploads and
+ * downloads run on two streams of the library's own beside the convolutions, ordered by events after what is on
+ * cuda_stream and before what follows on it (on cuda_stream itself while that is being captured).  A configuration stored
+ * for the call's shape holds for its pieces.
  */
 ALCS_API size_t alcs_spconv1x1_host_workspace(const alcs_packed* w, int n, int h, int wd, unsigned flags);
 ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void* y_host, int n, int h,
@@ -319,8 +330,9 @@ ALCS_API int alcs_spconv1x1_host(const alcs_packed* w, const void* x_host, void*
  * call for a shape uploads the launch schedule, and inputs whose rows are not a multiple of 16
  * bytes long (h*wd = 49, ...) are repacked into scratch that w allocates or grows on demand.  This
  * entry point never calls cudaMalloc, cudaFree or any other allocating routine:
- *   - the launch schedule for (n, h, wd, flags) must already be on the device, i.e. alcs_spconv1x1,
- *     alcs_spconv1x1_tune or alcs_stack_create has been called once for that shape during set-up;
+ *   - what the kernel for (n, h, wd, flags) needs must already be on the device, i.e. alcs_spconv1x1,
+ *     alcs_spconv1x1_tune or alcs_stack_create has been called once for that shape during set-up (a layer that a stack
+ *     merged into one launch runs here on the weights of that launch);
  *     otherwise the call fails with ALCS_ERR_STATE and launches nothing;
  *   - the repacked copy of x goes into one fixed array of ALCS_NOALLOC_SCRATCH_BYTES bytes that is
  *     part of the library image (every GPU that loads the library holds it until the process exits).
@@ -391,19 +403,20 @@ ALCS_API int alcs_probe_segment_loop(int g, int pixels_per_lane, int rows_per_wa
  * alcs_spconv2d: x device [n][cin][h][wd], y device [n][cout][oh][ow] with
  * oh = (h + 2*pad - kh)/stride + 1 (ow likewise), contiguous NCHW fp32, 4-byte aligned, not
  * overlapping; bias device fp32 [cout] or NULL; flags = ALCS_RELU or 0.  Enqueues one kernel on
- * cuda_stream.  The first call for a new geometry builds that geometry's launch schedule, allocates
- * device memory owned by w for it and waits for its upload; later calls with the same geometry do
- * neither.  n == 0 is a successful no-op.
+ * cuda_stream, or two with the partial sums of a split layer between them, which are taken from and returned to a
+ * stream-ordered pool of the library's own (under stream capture: memory of the graph).  The first call for a new
+ * geometry prepares the weights, allocates device memory owned by w for it and waits for its upload; later calls with
+ * the same geometry do neither.  n == 0 is a successful no-op.
  * Errors: INVALID_ARG (null or misaligned or overlapping buffers, non-positive sizes, unknown
  * flags), SHAPE (cin*kh*kw is not the packed column count, kernel larger than the padded image,
  * more than 2^31-1 elements), UNSUPPORTED (fp16 weights, g outside {1,2,4,8,16}, stride > 2,
  * kernels wider than 8*stride+1, or so many input channels that not even a one-row strip of all of
  * them fits in shared memory), STATE, ALLOC, CUDA.
  *
- * alcs_spconv2d runs on the fifth-generation tensor cores (as math_mode 4 of alcs_launch_cfg) wherever the input
- * rows that 128 output pixels need fit shared memory for 16 channels at a time, kernels of at most 32 taps; else, and
- * with an explicit configuration, on the CUDA-core kernel.  alcs_spconv2d_plan reports the CUDA-core kernel's launch
- * configuration (host only).
+ * alcs_spconv2d runs on the fifth-generation tensor cores (as math_mode 4 of alcs_launch_cfg) where the input rows that
+ * 128 output pixels need fit shared memory for 16 channels at a time, for kernels of at most 32 taps, unless so few blocks
+ * are kept that the CUDA-core kernel is expected to be faster; else, and with an explicit configuration, on that one.
+ * alcs_spconv2d_plan reports the launch configuration that the CUDA-core kernel takes where it runs (host only).
  * ------------------------------------------------------------------------------------------- */
 typedef struct {
     int positions_per_lane;     /* output positions per lane (2, 4 or 8)                           */

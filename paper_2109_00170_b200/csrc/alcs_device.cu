@@ -307,7 +307,11 @@ bool gather_plan(const alcs_packed* w, int n, int hw, int p, int ks, const Devic
     const double px = (double)n * tiles * 32.0 * p;
     const double l2 = (double)w->nb * px * 4 / (vec ? 9.9e6 : 4.4e6), fma = (double)w->nb * w->g * px * 28.1e-6 / sms;
     const double hbm = (double)n * hw * (w->cin + w->cout) * 4 / 7.0e6;
-    pl.cost = 1e-6 * (2.0 + std::max({loads, l2, fma, hbm}));
+    // (a second fit, by whole waves of thread blocks, is the better one where there are several of them: 18 us, not 12, for
+    // 96 -> 160 channels at 13x13, batch 48; the longer one counts)
+    const double waves = std::ceil(rounds), wave_us = (p == 2 ? 0.55 : p == 4 ? 0.7 : 0.9) * (vec || p == 2 ? 1.0 : 1.3);
+    const double by_waves = std::max(waves * batches * wave_us + (waves - 1) * 1.4, (double)w->nb * px * 4 / (vec ? 5.5e6 : 3.3e6));
+    pl.cost = 1e-6 * std::max(2.0 + std::max({loads, l2, fma, hbm}), 2.6 + by_waves);
     *out = pl;
     return true;
 }
@@ -397,11 +401,12 @@ double staged_us(const alcs_packed* w, const CallShape& c, int sms)
     const double q = (double)c.q(), elt = (double)w->elt(), x_bytes = q * w->cin * elt;
     const size_t row = (size_t)c.hw() * w->elt();
     double us = f.launch + f.chunk * w->cin / 64.0 + f.longest * longest_row(w);
-    if (c.stride > 1 || (row % 16 != 0 && row % 16 != 8)) us += f.pass + x_bytes * (1 + c.stride) / f.pass_rate;
+    // (the pass over a strided input reads single elements)
+    if (c.stride > 1 || (row % 16 != 0 && row % 16 != 8)) us += f.pass + x_bytes * (1 + c.stride) / (c.stride > 1 ? std::min(f.pass_rate, 4.0e6) : f.pass_rate);
     const int at = w->g == 1 ? 0 : w->g == 2 ? 1 : w->g == 4 ? 2 : w->g == 8 ? 3 : 4;
     const double work = q * f.px + w->nb * q * f.block[at] + w->rows * q * f.row + x_bytes * f.x * std::max(1.0, w->rows / 32.0);
     us += std::max(work / sms, (x_bytes + q * w->cout * elt) / f.rate);
-    if (c.residual) us += q * w->cout * (w->dt == ALCS_F32 ? 2.5e-6 : 2.0e-6);
+    if (c.residual) us += q * w->cout * (w->dt == ALCS_F32 ? 3.2e-6 : 2.0e-6);
     return us;
 }
 
@@ -412,8 +417,8 @@ bool direct_rows_ok(int hw, int elt) { return ((size_t)hw * elt) % 16 == 8; }
 // How many of the best candidates the tuner times a second time and remembers for alcs_stack_tune.
 constexpr size_t kFinalists = 12;
 
-// Schedules a first call builds to choose among.
-constexpr size_t kQuickSchedules = 3;
+// Schedules a first call builds to choose among: about a millisecond's worth, and at least three.
+size_t quick_schedules(const alcs_packed* w) { return (size_t)std::max(3, std::min(24, 500000 / std::max(1, w->nb))); }
 
 // The sizes of a schedule without building it, for rows of equal length: a segment (block row, chunk) of `len` blocks takes
 // about len / 2 + 1/4 pair records, or len / 16 + 1/2 step records.
@@ -560,7 +565,7 @@ int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>&
         for (const Plan& guess : out) {
             const std::array<int, 3> key = {guess.variant, guess.kc, guess.n_rg};
             if (std::find(built.begin(), built.end(), key) != built.end()) continue;
-            if (built.size() >= kQuickSchedules && best.cost < 1e30) break;
+            if (built.size() >= quick_schedules(w) && best.cost < 1e30) break;
             built.push_back(key);
             const KernelVariant& v = g_variants[guess.variant].v;
             const Schedule* sc = get_schedule(w, guess.kc, guess.n_rg, false, flavour_of(v));
@@ -1882,7 +1887,7 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
         rc = alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
         if (rc) return rc;
         run.forms.push_back(t);
-        for (int k16 : t->k16) us[i].push_back(alcs::tc_tile_us(it.layer.w, tc_problem(it), t->n, k16, t->cols != nullptr, t->chan != nullptr));
+        for (int k16 : t->k16) us[i].push_back(alcs::tc_merged_item_us(it.layer.w->dt, t->n, k16));
     }
     rc = alcs::tc_finish(w0, a, false);
     if (rc) return rc;

@@ -412,12 +412,17 @@ __device__ __forceinline__ void copy_patch(const TcLayer& y, const Patch& t, uns
             }
             const raw* from = src + at;
             unsigned to = slot + p * vb;
+            if constexpr (sizeof(raw) == 2)
+                if (vb == 2) {      // (an X that starts on an odd element)
+#pragma unroll 1
+                    for (int c = 0; c < nc; ++c) st_slot(to + c * pitch, ld_x(from + (size_t)c * y.hw_in));
+                    continue;
+                }
 #pragma unroll 4
             for (int c = 0; c < nc; ++c) {
                 if (vb == 16) cp_async16(to, from);
                 else if (vb == 8) cp_async_small<8>(to, from, 8);
-                else if (sizeof(raw) == 4 || vb == 4) cp_async_small<4>(to, from, 4);
-                else if constexpr (sizeof(raw) == 2) st_slot(to, ld_x(from));       // (an X that starts on an odd element)
+                else cp_async_small<4>(to, from, 4);
                 to += pitch;
                 from += y.hw_in;
             }
@@ -678,7 +683,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 
     if (warp < kConvWarps) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConvRegs));
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         const unsigned quad = (unsigned)(warp & 3);
         const int s0_ = warp >> 2, row = quad * 32 + lane;       // a warp takes every fourth 16-column step
         unsigned i = 0, slot = 0, xph = 0, buf = 0, aph = 1;
@@ -715,6 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             for (int k16 = cur.t.k16; k16 > 0; k16 -= NS, ++i) {
                 const unsigned my_a = tmem_a + (quad << 21) + buf * AB;      // lanes 32 * quad ...
                 const int ns = min(NS, k16);
+                if (i == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
                 ok = (PATCH || bar_wait(x_full + 8 * slot, xph)) && bar_wait(a_empty + 8 * buf, aph);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -934,7 +939,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProdRegs));
         constexpr int kIssuers = E::group == 1 ? 2 : 1;
         if (warp >= kMmaWarp && warp < kMmaWarp + kIssuers && elect_one()) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");
             const unsigned me = warp - kMmaWarp;
             unsigned n_chunk = 0, n_grp = 0, stage = 0, ph = 0, buf = 0, aph = 0;
             Cursor<L> cur(a);
@@ -954,6 +958,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     if (kIssuers == 1 || (n_chunk & 1u) == me) {
                         const int ns = min(NS, k16 - NS * c);
                         const unsigned d = n_grp & 1u;
+                        if (n_chunk == me) asm volatile("griddepcontrol.wait;" ::: "memory");
                         ok = (!first || bar_wait(d_empty + 8 * d, ((n_grp >> 1) & 1u) ^ 1u)) && bar_wait(b_full + 8 * stage, ph) &&
                              bar_wait(a_full + 8 * buf, aph);
                         // all a chunk needs is there: when the other issuer's chunk has been issued, this one follows it

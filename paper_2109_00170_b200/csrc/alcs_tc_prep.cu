@@ -496,6 +496,15 @@ double tc_tile_us(const alcs_packed* w, const TcProblem& p, int n, int k16, bool
     return p.res && k16 * 16 > 2 * tc_kc(w->dt) ? work + 0.65 * store : std::max(work, store);
 }
 
+// An item among those of other layers in one launch, where staging, tensor cores and stores of different items overlap: what
+// the list of a merged launch is made from (ResNet-50's layers in fp16: 99 us; dealt by tc_tile_us, 108).
+double tc_merged_item_us(int dt, int n, int k16)
+{
+    const int nch = (k16 * 16 + tc_kc(dt) - 1) / tc_kc(dt);
+    const double chunk = dt == ALCS_F32 ? std::max(0.95, 0.1 + 0.0096 * n) : std::max(0.9, 0.3 + 0.006 * n);
+    return nch * chunk + 0.3 + 0.005 * n;
+}
+
 std::vector<double> tc_tiles_us(const alcs_packed* w, const TcProblem& p, int n)
 {
     const TileGuess g = guess_tiles(w, p, n);

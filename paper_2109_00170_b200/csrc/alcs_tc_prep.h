@@ -57,6 +57,7 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
 // Estimates, in microseconds, from the shape and the weights alone.
 double tc_tile_us(const alcs_packed* w, const TcProblem& p, int n, int k16, bool list, bool sorted);
 std::vector<double> tc_tiles_us(const alcs_packed* w, const TcProblem& p, int n);        // of every channel tile, as tc_prepare would make them
+double tc_merged_item_us(int dt, int n, int k16);
 double tc_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms);
 int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a, bool patch);
 int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool patch, cudaStream_t st);
