@@ -173,7 +173,8 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     after the other and a work item stages them with a few large bulk (TMA) copies: the
  *                     staging then costs the kernel next to no instructions, at the price of one more pass
  *                     over X where its rows would not have needed repacking.  Batches of more than 8 images
- *   producer_warps    warps of the thread block that only move data (1..4)
+ *   producer_warps    warps of the thread block that only move data (1..4); math_mode 4: 8 names the kernel for 16-bit operands
+ *                     that multiplies X as it lies in memory (stride 1), 0 leaves the choice of kernel to the library
  *   math_mode         1 = fp32 FMA on the CUDA cores; 2 = tensor cores (fp16 weights and activations
  *                     only): 16 kept blocks of a block row times the 16 input rows they select is a
  *                     dense 16 x g by 16 x pixels contraction, run as warp-level MMA with fp32
@@ -186,7 +187,7 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     4 = fifth-generation tensor cores: the kept blocks of a tile of output channels are expanded
  *                     (once per packed matrix, on the device) to dense weight tiles and multiplied with 128-pixel
  *                     tiles of X; fp32 operands are split exactly into three bfloat16 parts each.  Only row_groups
- *                     (the number of channel tiles, each of at most 128 channels) applies; no scratch is used.  Outputs of
+ *                     (the number of channel tiles, each of at most 128 channels) and producer_warps apply; no scratch is used.  Outputs of
  *                     pixels with infinite or NaN inputs are computed from the storage format instead, so that such values
  *                     reach the channels that keep a block of theirs and no others, as with the other kernels (slowly); fp32
  *                     matrices that keep an infinite or NaN weight are refused (UNSUPPORTED)
@@ -527,7 +528,7 @@ typedef struct {
  * largest such layer, released by alcs_stack_destroy): nothing a captured graph refers to is freed
  * or moved by later alcs_spconv1x1 calls with the same packed matrices, at any batch size.
  * Consecutive layers on the fifth-generation tensor-core kernel (math_mode 4, up to 16 of one element type) none of
- * which reads or writes what another one writes run as ONE launch, whose items (128 pixels x a channel tile) are
+ * which reads or writes what another one writes run as ONE launch, whose items (a tile of pixels x a channel tile) are
  * dealt to the SMs by a list made when the stack is created; layers that do touch each other's buffers keep
  * their order.  Two runs
  * of the same stack must not overlap on the GPU (they share that scratch and the outputs).

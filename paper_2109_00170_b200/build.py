@@ -19,9 +19,9 @@ CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libalcs.so")
 
-SOURCES = ["alcs_pack.cpp", "alcs_device.cu", "alcs_conv2d.cu", "alcs_project.cu", "alcs_gather.cu", "alcs_probe.cu", "alcs_tc.cu", "alcs_tc_prep.cu", "alcs_variants_f32_g4.cu",
+SOURCES = ["alcs_pack.cpp", "alcs_device.cu", "alcs_conv2d.cu", "alcs_project.cu", "alcs_gather.cu", "alcs_probe.cu", "alcs_tc.cu", "alcs_tc16.cu", "alcs_tc_prep.cu", "alcs_variants_f32_g4.cu",
            "alcs_variants_f32_other.cu", "alcs_variants_f16.cu", "alcs_variants_f16_mma.cu", "alcs_variants_bf16.cu"]
-HEADERS = ["alcs_internal.h", "alcs_kernels.cuh", "alcs_mma.cuh", "alcs_conv2d.cuh", "alcs_gather.h", "alcs_tc.h", "alcs_tc_prep.h"]
+HEADERS = ["alcs_internal.h", "alcs_kernels.cuh", "alcs_mma.cuh", "alcs_conv2d.cuh", "alcs_gather.h", "alcs_tc.h", "alcs_tc.cuh", "alcs_tc_prep.h"]
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC,-Wall,-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),

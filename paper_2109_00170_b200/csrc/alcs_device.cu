@@ -352,7 +352,12 @@ bool tc_ok(const alcs_packed* w, const CallShape& c)
     return c.stride == 1 || ((size_t)c.wd * w->elt() % 8 == 0 && alcs::tc_patch_fits(w, tc_problem(c), alcs::kTcMaxN));
 }
 
-// The tcgen05 kernel with n output channels per tile as a plan.
+// alcs_tc16.cu takes 16-bit operands at stride 1.
+bool tc16_ok(const alcs_packed* w, const CallShape& c) { return w->dt != ALCS_F32 && c.stride == 1; }
+constexpr int kTc16Producers = 8;        // producer_warps of a configuration that names it
+
+// The tcgen05 kernels with n output channels per tile as a plan: the one that is expected to be faster.  Its estimate has to be clearly
+// lower for alcs_tc16.cu where rows must be picked apart (43 x 780 -> 139 @7 with a residual: 27 us where 17 were expected).
 Plan tc_plan(const alcs_packed* w, int n, const CallShape& c, int sms)
 {
     Plan p;
@@ -360,6 +365,15 @@ Plan tc_plan(const alcs_packed* w, int n, const CallShape& c, int sms)
     n = ((w->cout + p.n_rg - 1) / p.n_rg + 15) / 16 * 16;       // (the equal split into that many tiles)
     p.tc_n = n;
     p.cost = 1e-6 * alcs::tc_layer_us(w, tc_problem(c), n, sms);
+    if (tc16_ok(w, c)) {
+        int px;
+        const double us = 1e-6 * alcs::tc16_layer_us(w, tc_problem(c), n, sms, &px);
+        const bool direct = (size_t)c.hw() * w->elt() % 8 == 0;
+        if (us * (direct ? 1.05 : 1.3) < p.cost) {
+            p.tc_px = px;
+            if (direct) p.cost = us;        // (else the staged kernels stay where they were chosen: 156 -> 43 @7, batch 11: 12 us, not 16)
+        }
+    }
     return p;
 }
 
@@ -610,6 +624,7 @@ void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
         c->pixels_per_lane = 1;
         c->math_mode = 4;
         c->row_groups = p.n_rg;
+        c->producer_warps = p.tc_px ? kTc16Producers : 0;
         return;
     }
     const KernelVariant& v = g_variants[p.variant].v;
@@ -642,6 +657,7 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
         const int n = ((w->cout + std::max(1, tiles) - 1) / std::max(1, tiles) + 15) / 16 * 16;
         if (n > alcs::kTcMaxN) return ALCS_ERR_UNSUPPORTED;
         *out = tc_plan(w, n, shape, di.sms);
+        if (c->producer_warps == kTc16Producers && !out->tc_px && tc16_ok(w, shape)) (void)alcs::tc16_layer_us(w, tc_problem(shape), out->tc_n, di.sms, &out->tc_px);
         return ALCS_OK;
     }
     if (!c) {
@@ -954,8 +970,9 @@ alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& p
 }
 
 // Launch the tcgen05 kernel for one layer; strided layers run by patch staging.
-int launch_tc_plan(const alcs_packed* w, const Plan& p, const alcs::TcProblem& pr, cudaStream_t st)
+int launch_tc_plan(const alcs_packed* w, const Plan& p, alcs::TcProblem pr, cudaStream_t st)
 {
+    pr.pixels = p.tc_px;
     alcs::TcForm t;
     const int rc = alcs::tc_prepare(w, tc_key(w, p, pr), st, &t);
     return rc ? rc : alcs::tc_run(w, *t, pr, st);
@@ -1757,7 +1774,7 @@ size_t merge_end(const alcs_stack* s, size_t first, F eligible)
 // Fixed cost of a merged launch, first copies and last stores included, in microseconds.
 constexpr double kMergedRampUs = 5.0;
 
-// Consecutive independent layers whose configuration nobody fixed for the stack: one launch of the tcgen05 kernel for
+// Consecutive independent layers whose configuration nobody fixed for the stack: one launch of a tcgen05 kernel for
 // all of them, where its estimate is below the sum of the layers' own (measured ones, after alcs_spconv1x1_tune).  With few items in all, narrower tiles shorten
 // the longest SM's share; with many, wide ones do the least work.
 // fixed_too: of whatever was fixed, too (alcs_stack_tune).
@@ -1775,30 +1792,67 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
         const size_t end = s->items[i].q ? merge_end(s, i, open) : i;
         DeviceInfo di;
         if (end - i < 2 || device_info(s->items[i].layer.w->device, &di)) { i = std::max(end, i + 1); continue; }
+        std::vector<int> widths(end - i), pixels(end - i), choice, choice_px;
+        // Layers [from, to) in one launch of one of the two kernels: the widths (and pixels) that take the least, and the time.
+        auto together = [&](size_t from, size_t to, bool sixteen) {
+            double best = 0;
+            std::vector<int> n_of(to - from), px_of(to - from);
+            for (int cap = alcs::kTcMaxN; cap >= (sixteen ? 32 : 16); cap /= 2)
+                for (int cap_px = sixteen ? alcs::kTc16Pixels : alcs::kTcM; cap_px >= (sixteen ? 32 : alcs::kTcM); cap_px /= 2) {
+                    double total = 0, longest = 0;
+                    for (size_t k = from; k < to; ++k) {
+                        const alcs_stack::Item& it = s->items[k];
+                        const alcs_packed* w = it.layer.w;
+                        const alcs::TcProblem pr = tc_problem(call_shape(it));
+                        int n[8], at = 0;
+                        const int count = tc_widths(w, n);
+                        while (at + 1 < count && n[at] > cap) ++at;
+                        std::vector<double> us;
+                        int px = alcs::kTcM;
+                        if (sixteen) {
+                            const std::vector<int> steps = alcs::tc_tile_steps(w, pr, n[at]);
+                            px = alcs::tc16_capped(w, pr, steps.empty() ? 0 : *std::max_element(steps.begin(), steps.end()), cap_px);
+                            for (int k16 : steps) us.push_back(alcs::tc16_item_us(w, pr, n[at], k16, px));
+                        } else {
+                            us = alcs::tc_tiles_us(w, pr, n[at]);
+                        }
+                        for (const double t : us) {
+                            total += t * (double)((it.q + px - 1) / px);
+                            longest = std::max(longest, t);
+                        }
+                        n_of[k - from] = n[at];
+                        px_of[k - from] = sixteen ? px : 0;
+                    }
+                    const double t = kMergedRampUs + std::max(total / di.sms, longest) + 0.25 * longest;
+                    if (best > 0 && t >= best) continue;
+                    best = t;
+                    std::copy(n_of.begin(), n_of.end(), widths.begin() + (from - i));
+                    std::copy(px_of.begin(), px_of.end(), pixels.begin() + (from - i));
+                }
+            return best;
+        };
         double best = 0;
         for (size_t k = i; k < end; ++k) best += s->items[k].plan.cost * 1e6;
-        std::vector<int> choice, widths(end - i);
-        for (int cap = alcs::kTcMaxN; cap >= 16; cap /= 2) {
-            double total = 0, longest = 0;
-            for (size_t k = i; k < end; ++k) {
-                const alcs_stack::Item& it = s->items[k];
-                const alcs_packed* w = it.layer.w;
-                int n[8], at = 0;
-                const int count = tc_widths(w, n);
-                while (at + 1 < count && n[at] > cap) ++at;
-                const double px = (double)((it.q + alcs::kTcM - 1) / alcs::kTcM);
-                for (const double us : alcs::tc_tiles_us(w, tc_problem(call_shape(it)), n[at])) {
-                    total += us * px;
-                    longest = std::max(longest, us);
-                }
-                widths[k - i] = n[at];
+        const double one = together(i, end, false);
+        if (one < best) { best = one; choice = widths; choice_px = pixels; }
+        // 16-bit operands: layers whose rows can be copied as they are on alcs_tc16.cu, a launch per sequence of layers of one kind
+        // (several launches have to promise a tenth: the estimates are that good)
+        auto direct = [&](size_t k) { return (size_t)s->items[k].oh * s->items[k].ow * s->items[k].layer.w->elt() % 8 == 0; };
+        if (s->items[i].layer.w->dt != ALCS_F32) {
+            double t = 0;
+            int launches = 0;
+            bool any = false;
+            for (size_t from = i, to; from < end; from = to, ++launches) {
+                for (to = from + 1; to < end && direct(to) == direct(from);) ++to;
+                t += together(from, to, direct(from));
+                any = any || direct(from);
             }
-            const double t = kMergedRampUs + std::max(total / di.sms, longest) + 0.25 * longest;
-            if (t < best) { best = t; choice = widths; }
+            if (any && t * (launches > 1 ? 1.1 : 1.0) < best) { best = t; choice = widths; choice_px = pixels; }
         }
         for (size_t k = i; k < end && !choice.empty(); ++k) {
             alcs_stack::Item& it = s->items[k];
             it.plan = tc_plan(it.layer.w, choice[k - i], call_shape(it), di.sms);
+            it.plan.tc_px = choice_px[k - i];
         }
         i = end;
     }
@@ -1878,16 +1932,23 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
     run.args.reset(new alcs::TcArgs<alcs::kTcMaxLayers>());
     alcs::TcArgs<alcs::kTcMaxLayers>& a = *run.args;
     a.n_layers = run.count;
-    std::vector<std::vector<double>> us(run.count);       // per layer and channel tile
     for (int i = 0; i < run.count; ++i) {
         const auto& it = s->items[first + i];
         alcs::TcForm t;
         rc = alcs::tc_prepare(it.layer.w, tc_key(it.layer.w, it.plan, tc_problem(it)), nullptr, &t);
         if (rc) return rc;
-        rc = alcs::tc_fill(it.layer.w, *t, tc_problem(it), &a.layer[i]);
-        if (rc) return rc;
         run.forms.push_back(t);
-        for (int k16 : t->k16) us[i].push_back(alcs::tc_merged_item_us(it.layer.w->dt, t->n, k16));
+    }
+    std::vector<std::vector<double>> us(run.count);       // per layer and channel tile
+    for (int i = 0; i < run.count; ++i) {
+        const auto& it = s->items[first + i];
+        const alcs::TcForm& t = run.forms[i];
+        alcs::TcProblem pr = tc_problem(it);
+        pr.pixels = it.plan.tc_px ? alcs::tc16_capped(it.layer.w, pr, t->k16_max, it.plan.tc_px) : 0;
+        rc = alcs::tc_fill(it.layer.w, *t, pr, &a.layer[i]);
+        if (rc) return rc;
+        for (int k16 : t->k16)
+            us[i].push_back(pr.pixels ? alcs::tc16_item_us(it.layer.w, pr, t->n, k16, a.layer[i].ppt) : alcs::tc_merged_item_us(w0->dt, t->n, k16));
     }
     rc = alcs::tc_finish(w0, a, false);
     if (rc) return rc;
@@ -1900,7 +1961,7 @@ int build_merged(alcs_stack* s, size_t first, size_t end)
             for (int k = 0; k < y.n_tiles.d * y.px_tiles.d; ++k)
                 items.emplace_back(us[i][y.tile_major ? k / y.px_tiles.d : k % y.n_tiles.d], y.first_item + k);
         }
-        if (a.n_items <= 16 * blocks)
+        if (a.n_items <= 16 * blocks || a.layer[0].n_px)
             std::stable_sort(items.begin(), items.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
         std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<std::pair<double, int>>> idle;
         for (int b = 0; b < blocks; ++b) idle.emplace(0.0, b);
@@ -1939,7 +2000,8 @@ int build_runs(alcs_stack* s)
     auto on_tc = [](const alcs_stack::Item& it) { return it.plan.tc_n != 0 && it.layer.stride <= 1; };
     for (size_t i = 0; i < s->items.size();) {
         if (s->items[i].q == 0) { ++i; continue; }
-        const size_t end = merge_end(s, i, on_tc);
+        // (layers of one kernel)
+        const size_t end = merge_end(s, i, [&](const alcs_stack::Item& it) { return on_tc(it) && !it.plan.tc_px == !s->items[i].plan.tc_px; });
         if (end > i) {
             const int rc = build_merged(s, i, end);
             if (rc) { drop_runs(s); return rc; }
@@ -2053,7 +2115,7 @@ namespace {
 bool same_plan(const Plan& a, const Plan& b)
 {
     return a.variant == b.variant && a.kc == b.kc && a.n_rg == b.n_rg && a.stages == b.stages && a.bulk == b.bulk &&
-           a.gather == b.gather && a.gp == b.gp && a.gks == b.gks && a.tc_n == b.tc_n;
+           a.gather == b.gather && a.gp == b.gp && a.gks == b.gks && a.tc_n == b.tc_n && a.tc_px == b.tc_px;
 }
 
 // Run time of one pass over the whole stack in microseconds, as alcs_stack_run runs it (a graph stack
@@ -2281,7 +2343,8 @@ extern "C" ALCS_API int alcs_spconv1x1_noalloc(const alcs_packed* w, const void*
             // needs no scratch, but what does not fit that is refused whatever kernel the plan names.
             const size_t row = (size_t)h * wd * w->elt();
             if (row % 16 != 0 && (size_t)n * w->cin * ((row + 15) / 16 * 16) > ALCS_NOALLOC_SCRATCH_BYTES) return ALCS_ERR_TOO_LARGE;
-            const alcs::TcProblem pr = tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd);
+            alcs::TcProblem pr = tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd);
+            pr.pixels = plan.tc_px;
             const alcs::TcPrep* t = plan.tc_n ? alcs::tc_find(w, tc_key(w, plan, pr)).get() : nullptr;
             if (!t) t = alcs::tc_any_pointwise(w);
             if (!t) return ALCS_ERR_STATE;

@@ -90,8 +90,9 @@ struct Plan {
     // the small-problem kernel (no staging, reads the canonical format): variant is -1, and
     int gather = 0;        // 1 selects it,
     int gp = 0, gks = 0;   // pixels per lane and warps per thread block (shares of one block row's columns)
-    // the tcgen05 kernel (alcs_tc.cu): variant is -1, and
-    int tc_n = 0;          // output channels per tile (0: not this kernel)
+    // the tcgen05 kernels: variant is -1, and
+    int tc_n = 0;          // output channels per tile (0: not these kernels)
+    int tc_px = 0;         // pixels per tile on alcs_tc16.cu (0: alcs_tc.cu)
 };
 
 // Key of the plan cache: the problem shape plus the requested configuration (all zero = automatic).

@@ -73,8 +73,11 @@ struct TcLayer {
     TcDiv w_vec;                 // copies per image row
     int oh, row_step;            // input rows are taken every row_step
     int blocks, pitch;
-    int vec_bytes;               // bytes of one copy of X: 16, 8, 4; 0: element by element
-    int ppt;                     // pixels per tile: kTcM, or those of ...
+    int vec_bytes;               // bytes of one copy of X: 16, 8, 4; 0: element by element; kTcRaw: see alcs_tc16.cu
+    // alcs_tc16.cu: pixels of the MMA (ppt rounded up to a multiple of 32; 0: the other kernel); bytes of one store, and of one load of the
+    // residual; kTcRaw: bytes of a chunk's rows, between the runs of a row, between rows
+    int n_px, y_vec, res_vec, raw_bytes, raw_pitch, raw_row;
+    int ppt;                     // pixels per tile: kTcM (alcs_tc16.cu: up to kTc16Pixels), or those of ...
     int images;                  // ... this many whole images, staged as runs of memory (0: not so)
     int n_img;
     int relu, y32;               // y32: fp32 output of 16-bit operands
@@ -86,9 +89,23 @@ struct TcArgs {
     const int* sched;            // null: thread block b takes items b, b + grid, ...; else its items are sched[b], sched[b + grid], ... until -1
     int stages;                  // weight stages in shared memory
     int stage_bytes;
-    int slots, slot_bytes;       // patch staging: X ring
+    int slots, slot_bytes;       // patch staging: X ring; alcs_tc16.cu: slot_bytes of weights in front of a stage's X
+    int raw_slots, raw_bytes;    // alcs_tc16.cu: rows fetched as they are
     TcLayer layer[L];
 };
+
+// alcs_tc16.cu: a stage holds kTc16Chunk columns of the weights and of X; kTc16Fixed bytes of shared memory
+// in front of the stages.
+constexpr int kTc16Chunk = 64, kTc16Header = 1024, kTc16Staging = 32 * 128, kTc16Fixed = kTc16Header + 16 * kTc16Staging;
+constexpr int kTc16Pixels = 256;     // at most, per tile; half of it where a tile's columns take several accumulators
+constexpr int kTc16Group = 16;       // 16-column steps per accumulator
+constexpr int kTcRaw = 1;            // X is fetched by 16-byte words and picked apart in shared memory
+constexpr int kTc16RawMost = 48 * 1024;        // bytes of a chunk's rows
+constexpr int kTc16Raw = kTc16Pixels / 2;      // most pixels per tile then
+constexpr int tc16_weight_bytes(int n) { return kTc16Chunk * n * 2; }
+constexpr int tc16_stage_bytes(int n, int px) { return tc16_weight_bytes(n) + (px + 63) / 64 * (64 * kTc16Chunk * 2); }
+cudaError_t launch_tc16(int dt, const TcArgs<kTcMaxLayers>& a, int blocks, cudaStream_t st);
+cudaError_t prepare_tc16(int dt);
 
 // Sum of the partial results of a layer whose columns were split: part[image][tile][split][n][hw] over the splits in
 // order, bias, ReLU.

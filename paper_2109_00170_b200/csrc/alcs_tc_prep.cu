@@ -185,7 +185,8 @@ int tc_prepare(const alcs_packed* w, const TcKey& key, cudaStream_t st, TcForm* 
         std::lock_guard<std::mutex> lk(mu);
         bool& r = ready[w->device & 63][(int)w->dt];
         if (!r) {
-            const cudaError_t e = prepare_tc(w->dt);
+            cudaError_t e = prepare_tc(w->dt);
+            if (e == cudaSuccess && w->dt != ALCS_F32) e = prepare_tc16(w->dt);
             if (e != cudaSuccess) return cuda_fail(e);
             r = true;
         }
@@ -349,6 +350,43 @@ bool tc_whole_images(const alcs_packed* w, const TcProblem& p)
     return !p.kh && row % 16 != 0 && (elt == 4 || row % 4 != 0) && row <= kTcM * elt && w->cin % 16 == 0;
 }
 
+// Rows fetched as they are: a tile's runs of consecutive pixels, of an image each, in whole 16-byte words.
+void tc16_raw(const TcProblem& p, int pixels, int* pitch, int* row)
+{
+    const long long hw = (long long)p.oh * p.ow, runs = std::min<long long>(std::max(1, p.n), (pixels - 2) / hw + 2);
+    *pitch = (int)((std::min<long long>(hw, pixels) * 2 + 14 + 15) / 16 * 16);
+    *row = (int)(runs * *pitch);
+}
+
+int tc16_raw_bytes(const TcProblem& p, int pixels)
+{
+    int pitch, row;
+    tc16_raw(p, pixels, &pitch, &row);
+    return kTc16Chunk * row;
+}
+
+// Pixels per tile that a layer can take, the most first.
+std::vector<int> tc16_tiles(const alcs_packed* w, const TcProblem& p, int k16_max)
+{
+    int most = k16_max > kTc16Group ? kTc16Pixels / 2 : kTc16Pixels;
+    std::vector<int> px;
+    if ((size_t)p.oh * p.ow * w->elt() % 8 != 0) {
+        most = std::min(most, kTc16Raw);
+        while (most > 32 && tc16_raw_bytes(p, most) > kTc16RawMost) most -= 32;
+    }
+    for (; most >= 32; most -= 32) px.push_back(most);
+    return px;
+}
+
+// The most pixels per tile that are no more than `cap`.
+int tc16_capped(const alcs_packed* w, const TcProblem& p, int k16_max, int cap)
+{
+    const std::vector<int> px = tc16_tiles(w, p, k16_max);
+    for (int v : px)
+        if (v <= cap) return v;
+    return px.back();
+}
+
 // UNSUPPORTED: beyond the kernel's 32-bit offsets, or rows that patch staging cannot copy (see tc_fits, tc_patch_fits).
 int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* out)
 {
@@ -374,6 +412,33 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
     y.n_img = p.n;
     y.images = 0;
     const int elt = (int)w->elt();
+    y.n_px = 0;
+    if (p.pixels) {
+        const int e = (p.flags & ALCS_Y_F32) ? 4 : 2;
+        // the widest piece that keeps to one image and to its alignment
+        auto widest = [&](size_t row, const void* at, int least) {
+            int v = 16;
+            while (v > least && (row % v || (uintptr_t)at % v)) v >>= 1;
+            return v;
+        };
+        const size_t hw = (size_t)y.hw.d;
+        const int v = widest(hw * elt, p.x, elt);
+        y.vec_bytes = v >= 8 ? v : kTcRaw;
+        y.y_vec = widest(hw * e, p.y, e);
+        y.res_vec = p.res ? widest(hw * e, p.res, e) : 16;
+        y.ppt = t.k16_max > kTc16Group ? std::min(p.pixels, kTc16Pixels / 2) : p.pixels;
+        if (y.vec_bytes == kTcRaw) {
+            // (an X that does not start where its copies would have to takes fewer pixels per tile)
+            if (y.ppt > kTc16Raw || tc16_raw_bytes(p, y.ppt) > kTc16RawMost) y.ppt = 32;
+            tc16_raw(p, y.ppt, &y.raw_pitch, &y.raw_row);
+            y.raw_bytes = kTc16Chunk * y.raw_row;
+        }
+        y.n_px = y.ppt;
+        y.px_tiles = tc_div((y.q + y.ppt - 1) / y.ppt);
+        y.relu = (p.flags & ALCS_RELU) ? 1 : 0;
+        y.y32 = e == 4;
+        return ALCS_OK;
+    }
     if (p.kh) {
         const PatchPlan pl = patch_plan(w, p);
         y.taps = tc_div(p.kh * p.kw); y.kwd = tc_div(p.kw);
@@ -536,6 +601,47 @@ double tc_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms)
     return std::max(f.ramp + main + first + f.tail * store_us(w, p, n, g.sorted), f.ramp + bytes / kBytesPerUs);
 }
 
+// alcs_tc16.cu: least-squares fits (of the logarithm) to 1,087 launches of random shapes, densities and tile sizes on one B200; median
+// error 9 %, and the tile sizes they choose take 2 % more than the best of those measured.  A chunk: by how X is copied (16 bytes,
+// 8, rows fetched as they are), or by its bytes; the stores of 128 pixels by their width.
+double tc16_item_us(const alcs_packed* w, const TcProblem& p, int n, int k16, int pixels)
+{
+    const size_t hw = (size_t)p.oh * p.ow, row = hw * w->elt(), e = (p.flags & ALCS_Y_F32) ? 4 : 2;
+    const double px = pixels, store_px[4] = {0.68 * e / 2.0, 0.96, 1.5, 2.14};
+    const int width = hw * e % 16 == 0 ? 0 : hw * e % 8 == 0 ? 1 : hw * e % 4 == 0 ? 2 : 3;
+    const double store = 1.25 + px / 128.0 * store_px[width] * (p.res ? 3.0 : 1.0);
+    double chunk = row % 16 == 0 ? 0.41 + 0.00027 * px : row % 8 == 0 ? 0.41 + 0.0024 * px : 2.6;
+    if (k16 * 16 < w->cin) chunk += 0.1;        // (a column list)
+    chunk = std::max(chunk, 0.0024 * px + 0.0019 * n);
+    return std::max((k16 + 3) / 4 * chunk, store);
+}
+
+double tc16_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms, int* pixels)
+{
+    const std::vector<int> k16 = tc_tile_steps(w, p, n);
+    const long long q = (long long)std::max(1, p.n) * p.oh * p.ow;
+    const int k_max = k16.empty() ? 0 : *std::max_element(k16.begin(), k16.end());
+    const bool raw = (size_t)p.oh * p.ow * w->elt() % 8 != 0;
+    double best = 0;
+    *pixels = 0;
+    for (int px : tc16_tiles(w, p, k_max)) {
+        const double tiles = (double)((q + px - 1) / px);
+        double sum = 0, longest = 0;
+        for (int k : k16) {
+            const double us = tc16_item_us(w, p, n, k, px);
+            sum += us;
+            longest = std::max(longest, us);
+        }
+        const double rounds = std::ceil(tiles * k16.size() / sms);
+        const double us = 2.3 + (raw ? 3.0 : 0.0) + std::max(rounds * sum / k16.size(), longest) + 1.2 * std::min(longest, 1.25 + px / 128.0 * 0.7);
+        if (!*pixels || us < best * 0.98) { best = us; *pixels = px; }
+    }
+    const double bytes = (double)q * (w->cin + w->cout * (p.res ? 2.0 : 1.0)) * w->elt();
+    return std::max(best, 2.0 + bytes / kBytesPerUs);
+}
+
+std::vector<int> tc_tile_steps(const alcs_packed* w, const TcProblem& p, int n) { return guess_tiles(w, p, n).k16; }
+
 // Number items and choose the ring depth for the a.n_layers layers filled in.
 int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a, bool patch)
 {
@@ -552,6 +658,25 @@ int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a, bool patch)
     if (items > 0x7fffffffll) return ALCS_ERR_SHAPE;
     a.n_items = (int)items;
     a.sched = nullptr;
+    a.raw_slots = a.raw_bytes = 0;
+    if (a.layer[0].n_px) {
+        int px = 32;
+        for (int i = 0; i < a.n_layers; ++i) px = std::max(px, a.layer[i].n_px);
+        a.slots = 0;
+        a.slot_bytes = tc16_weight_bytes(n);
+        a.stage_bytes = tc16_stage_bytes(n, px);
+        int room = std::min(smem, 227 * 1024) - kTc16Fixed;
+        a.raw_slots = a.raw_bytes = 0;
+        for (int i = 0; i < a.n_layers; ++i)
+            if (a.layer[i].vec_bytes == kTcRaw) a.raw_bytes = std::max(a.raw_bytes, (a.layer[i].raw_bytes + 127) / 128 * 128);
+        if (a.raw_bytes) {      // two stages, then slots, as many as there is room for: what is in flight is there
+            a.raw_slots = std::min(4, (room - 2 * a.stage_bytes) / a.raw_bytes);
+            if (a.raw_slots < 1) return ALCS_ERR_UNSUPPORTED;
+            room -= a.raw_slots * a.raw_bytes;
+        }
+        a.stages = std::min(8, room / a.stage_bytes);
+        return a.stages >= 2 ? ALCS_OK : ALCS_ERR_UNSUPPORTED;
+    }
     a.stage_bytes = tc_stage_bytes(w->dt, n);
     int room = std::min(smem, 227 * 1024) - kTcHeaderBytes;
     a.slots = a.slot_bytes = 0;
@@ -573,7 +698,7 @@ int tc_launch(const alcs_packed* w, const TcArgs<kTcMaxLayers>& a, bool patch, c
     int sms = 0, smem = 0;
     const int rc = device_limits(w->device, &sms, &smem);
     if (rc) return rc;
-    const cudaError_t e = launch_tc(w->dt, patch, a, std::min(a.n_items, sms), st);
+    const cudaError_t e = a.layer[0].n_px ? launch_tc16(w->dt, a, std::min(a.n_items, sms), st) : launch_tc(w->dt, patch, a, std::min(a.n_items, sms), st);
     return e == cudaSuccess ? ALCS_OK : cuda_fail(e);
 }
 

@@ -1,0 +1,137 @@
+"""GPU parity of the tcgen05 kernel for 16-bit operands (math_mode 4, producer_warps 8) against the oracle at the sizes where
+its tiles, accumulators, copies and stores change."""
+import numpy as np
+import pytest
+
+import oracle
+from alcs_workloads import rng
+from gpu_util import TOL, assert_parity, check_layer
+
+pytestmark = pytest.mark.gpu
+CFG = dict(math_mode=4, producer_warps=8)
+
+
+def _case(seed, n, cin, cout, hw, g, density, dtype=np.float16):
+    rows = (cout + g - 1) // g
+    W = (rng.normal(seed, 1, cout * cin) * cin ** -0.5).reshape(cout, cin).astype(dtype)
+    X = np.abs(rng.normal(seed, 2, n * cin * hw)).reshape(n, cin, hw).astype(dtype)
+    M = (rng.uniform01(seed, 3, rows * cin) < density).astype(np.uint8).reshape(rows, cin)
+    return W, M, X, (0.1 * rng.normal(seed, 4, cout)).astype(np.float32)
+
+
+# n, cin, cout, h, wd, g, density: one pixel; ends of pixel tiles (31 .. 33, 255 .. 257 pixels); columns around a chunk and around an
+# accumulator (63 .. 65, 255 .. 257); channels around a tile and around a warp's 32; copies of 16, 8 bytes and fetched rows, images that
+# end inside a copy; column lists; more items than SMs, with one accumulator and with several
+SHAPES = [(1, 16, 8, 1, 1, 8, 1.0), (1, 63, 127, 31, 1, 8, 0.4), (2, 64, 128, 4, 4, 8, 0.4), (1, 65, 129, 33, 1, 8, 0.4), (1, 255, 33, 255, 1, 1, 0.3),
+          (1, 256, 31, 16, 16, 16, 0.3), (1, 257, 130, 257, 1, 8, 0.3), (3, 40, 72, 14, 14, 8, 0.3), (5, 100, 64, 7, 7, 8, 0.4), (4, 48, 40, 9, 6, 8, 0.4),
+          (3, 520, 96, 17, 23, 8, 0.2), (7, 300, 64, 6, 6, 4, 0.02), (24, 64, 256, 28, 28, 8, 0.25), (30, 272, 260, 14, 14, 8, 0.25), (9, 16, 16, 56, 56, 8, 1.0)]
+
+
+@pytest.mark.parametrize("n,cin,cout,h,wd,g,density", SHAPES)
+def test_shapes(alcs, n, cin, cout, h, wd, g, density):
+    W, M, X, b = _case(n + cin + cout, n, cin, cout, h * wd, g, density)
+    for tiles in sorted({0, -(-cout // 16)}):
+        check_layer(alcs, W, M, X, b, True, g, cfg=dict(CFG, row_groups=tiles), h=h, wd=wd)
+    # fp32 output: the products are exact, so the fp32 tolerance holds
+    Y = check_layer(alcs, W, M, X, None, False, g, cfg=CFG, h=h, wd=wd, y_f32=True)
+    assert Y <= TOL["f32"]
+
+
+def _device_call(alcs, W, M, X, b, g, h, wd, res, bf16, y_f32, x_off=0, y_off=0):
+    """One residual call with X and Y starting `off` elements into their buffers; returns Y and what lies around it."""
+    import torch
+    dev = torch.device("cuda:0")
+    tdt = torch.bfloat16 if bf16 else torch.float16
+    Wt = torch.from_numpy(W.astype(np.float32)).to(tdt)
+    p = alcs.alcs_pack(Wt.view(torch.int16).numpy().view(np.uint16), M, g, bf16=True) if bf16 else alcs.alcs_pack(Wt.numpy(), M, g)
+    alcs.alcs_packed_upload(p, 0)
+    n, cin, hw = X.shape
+    xb = torch.zeros(X.size + x_off + 8, dtype=tdt, device=dev)
+    xb[x_off:x_off + X.size] = torch.from_numpy(X.astype(np.float32)).to(dev).to(tdt).reshape(-1)
+    ydt = torch.float32 if y_f32 else tdt
+    size = n * W.shape[0] * hw
+    yb = torch.full((size + y_off + 32,), 7.0, dtype=ydt, device=dev)
+    rt = None if res is None else torch.from_numpy(res).to(dev).to(ydt).contiguous()
+    flags = alcs.ALCS_RELU | (alcs.ALCS_Y_F32 if y_f32 else 0)
+    alcs.alcs_spconv1x1_ex(p, xb[x_off:], yb[y_off:], n, h, wd, 1, torch.from_numpy(b).to(dev), rt, flags, torch.cuda.current_stream(), CFG)
+    torch.cuda.synchronize()
+    assert alcs.alcs_packed_status(p) == 0
+    y = yb.float().cpu().numpy()
+    assert (y[:y_off] == 7).all() and (y[y_off + size:] == 7).all(), "stored outside Y"
+    x = xb[x_off:x_off + X.size].float().cpu().numpy().reshape(X.shape)
+    return y[y_off:y_off + size].reshape(n, W.shape[0], hw), Wt.float().numpy(), x, None if rt is None else rt.float().cpu().numpy()
+
+
+@pytest.mark.parametrize("n,cin,cout,h,wd", [(3, 64, 136, 7, 7), (2, 48, 40, 14, 14), (4, 272, 96, 8, 8), (2, 33, 260, 11, 13), (40, 40, 136, 16, 16)])
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("y_f32", [False, True])
+@pytest.mark.parametrize("offsets", [(0, 0), (4, 2), (1, 1)])
+def test_residual_types_and_alignments(alcs, n, cin, cout, h, wd, bf16, y_f32, offsets):
+    """Residual, output types, and buffers that start anywhere.  One rounding of the output: 2^-11 of it in fp16, 2^-8 in bfloat16
+    (half of the last place kept, doubled), beside the fp32 sum's tolerance."""
+    g, hw = 8, h * wd
+    W, M, X, b = _case(cin + cout, n, cin, cout, hw, g, 0.4, np.float32)
+    res = rng.normal(9, 5, n * cout * hw).reshape(n, cout, hw).astype(np.float32)
+    Y, Wr, Xr, Rr = _device_call(alcs, W, M, X, b, g, h, wd, res, bf16, y_f32, *offsets)
+    Yref, A = oracle.conv1x1(Wr, M, Xr, b, False, g, want_scale=True)
+    Yref, A = np.maximum(Yref + Rr, 0.0), A + np.abs(Rr)
+    assert np.isfinite(Y).all()
+    unit = 0.0 if y_f32 else 2.0 ** -8 if bf16 else 2.0 ** -11
+    assert (np.abs(Y - Yref) <= TOL["f32"] * A + unit * np.abs(Yref)).all()
+
+
+def test_rows_that_keep_nothing_and_skewed_rows(alcs):
+    n, cin, cout, h, g = 6, 300, 256, 14, 8
+    W, M, X, b = _case(5, n, cin, cout, h * h, g, 0.05)
+    M[3::2] = 0
+    M[0] = 1
+    for tiles in (2, 8, 16):
+        check_layer(alcs, W, M, X, b, True, g, cfg=dict(CFG, row_groups=tiles), h=h, wd=h)
+    M[:] = 0
+    Y = check_layer(alcs, W, M, X, b, True, g, cfg=CFG, h=h, wd=h)
+    assert Y <= 2.0 ** -11
+
+
+@pytest.mark.parametrize("h,cin", [(14, 64), (7, 300), (8, 272)])
+def test_infinite_and_nan_inputs_touch_kept_blocks_alone(alcs, h, cin):
+    n, cout, g = 3, 136, 8
+    W, M, X, b = _case(31, n, cin, cout, h * h, g, 0.3)
+    X[1, 5, 3] = np.inf
+    X[2, 7, h * h - 1] = np.nan
+    import torch
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    x, y = torch.from_numpy(X).cuda(), torch.empty(n, cout, h * h, dtype=torch.float16, device="cuda")
+    alcs.alcs_spconv1x1(p, x, y, n, h, h, torch.from_numpy(b).cuda(), 0, torch.cuda.current_stream(), CFG)
+    torch.cuda.synchronize()
+    Y = y.float().cpu().numpy()
+    kept = np.repeat(M, g, axis=0)[:cout].astype(bool)
+    Xf = X.copy()
+    Xf[1, 5, 3] = Xf[2, 7, h * h - 1] = 0
+    Yref, A = oracle.conv1x1(W, M, Xf, b, False, g, want_scale=True)
+    bad = np.zeros(Y.shape, bool)
+    bad[1, kept[:, 5] & (W[:, 5] != 0), 3] = True
+    bad[2, kept[:, 7], h * h - 1] = True
+    assert not np.isfinite(Y[bad]).any()
+    assert_parity(np.where(bad, 0, Y), np.where(bad, 0, Yref), A, "f16")
+
+
+@pytest.mark.parametrize("sizes", [[(64, 96, 14), (272, 40, 8), (32, 160, 28)], [(48, 64, 16), (100, 64, 7), (64, 32, 14)]])
+@pytest.mark.parametrize("graph", [False, True])
+def test_merged_stack(alcs, sizes, graph):
+    """Layers of one launch, and layers of the two tensor-core kernels one behind the other."""
+    import torch
+    n, g = 6, 8
+    layers, want = [], []
+    for i, (cin, cout, h) in enumerate(sizes):
+        W, M, X, b = _case(100 + i, n, cin, cout, h * h, g, 0.4)
+        p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+        layers.append(dict(w=p, x=torch.from_numpy(X).cuda(), y=torch.full((n, cout, h * h), float("nan"), dtype=torch.float16, device="cuda"),
+                           n=n, h=h, wd=h, bias=torch.from_numpy(b).cuda(), flags=alcs.ALCS_RELU))
+        want.append(oracle.conv1x1(W, M, X, b, True, g, want_scale=True))
+    s = alcs.alcs_stack_create(layers, alcs.ALCS_STACK_GRAPH if graph else 0)
+    for _ in range(2):
+        alcs.alcs_stack_run(s, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    for L, (Yref, A) in zip(layers, want):
+        assert_parity(L["y"].cpu().numpy(), Yref, A, "f16")
+        assert alcs.alcs_packed_status(L["w"]) == 0
