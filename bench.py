@@ -508,10 +508,11 @@ def bench_conv2d(args):
 def stack_launches(specs, cfgs):
     """Kernel launches of one pass over the stack: consecutive layers on the tcgen05 kernel (math_mode 4) share a
     launch, up to 16 of them; the benchmark's layers have buffers of their own, so nothing keeps them apart."""
-    total, run = 0, 0
+    total, run, kind = 0, 0, None
     for sp, cfg in zip(specs, cfgs):
-        if cfg.get("math_mode") == 4:
-            total, run = (total + 1, 1) if run in (0, 16) else (total, run + 1)
+        if cfg.get("math_mode") == 4:       # (two kernels: producer_warps names the one for 16-bit operands)
+            total, run = (total + 1, 1) if run in (0, 16) or cfg.get("producer_warps", 0) != kind else (total, run + 1)
+            kind = cfg.get("producer_warps", 0)
         else:
             total, run = total + kernels_per_layer(sp, cfg), 0
     return total
