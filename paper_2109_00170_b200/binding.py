@@ -1,5 +1,5 @@
-"""Thin ctypes binding of libalcs.so: argument marshalling only, same names as the C ABI
-(include/alcs.h).  Every step of the convolution runs in the library's CUDA kernels; there is no
+"""Thin binding of libalcs.so: argument marshalling only, same names as the C ABI
+(include/alcs.h); through ctypes, and for the calls that a program makes once per layer through _alcs_call (C).  Every step of the convolution runs in the library's CUDA kernels; there is no
 Python or CPU fallback, and loading fails loudly if the shared object has not been built.
 """
 from __future__ import annotations
@@ -83,11 +83,12 @@ class Layer(C.Structure):
 
 
 _lib = None
+_call = None      # the C marshalling of the per-layer calls, bound to _lib's functions
 
 
 def lib():
     """Load libalcs.so once.  Raises if it is missing: there is nothing to fall back to."""
-    global _lib
+    global _lib, _call
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -140,7 +141,12 @@ def lib():
         f = getattr(L, name)
         if f.restype is C.c_int and name not in ("alcs_version",):
             f.restype = i
-    _lib = L
+    try:
+        from . import _alcs_call as native
+    except ImportError as e:
+        raise RuntimeError("_alcs_call not found or not loadable: build it with `python -m paper_2109_00170_b200.build`") from e
+    native.bind(*(C.cast(getattr(L, name), vp).value for name in ("alcs_spconv1x1", "alcs_spconv1x1_ex", "alcs_spconv2d", "alcs_stack_run")))
+    _lib, _call = L, native
     return L
 
 
@@ -187,6 +193,10 @@ class Packed:
         if not self._h:
             raise AlcsError(ALCS_ERR_STATE, "Packed (freed)")
         return self._h
+
+    @property
+    def address(self) -> int:
+        return self._h.value or self.handle
 
     def free(self):
         if self._h:
@@ -304,18 +314,24 @@ def alcs_variant_get(index: int) -> dict:
 def alcs_spconv1x1(w: Packed, x, y, n: int, h: int, wd: int, bias=None, flags: int = 0, stream=None,
                    cfg=None):
     """x, y, bias: device tensors (anything with data_ptr()) or raw device addresses."""
-    c = _cfg(cfg)
-    if c is None:
-        st = lib().alcs_spconv1x1(w.handle, _addr(x), _addr(y), n, h, wd, _addr(bias), flags, _stream(stream))
+    if cfg is None:
+        st = (_call or (lib(), _call)[1]).spconv1x1(w.address, x, y, n, h, wd, bias, flags, stream)
     else:
+        c = _cfg(cfg)
         st = lib().alcs_spconv1x1_cfg(w.handle, _addr(x), _addr(y), n, h, wd, _addr(bias), flags,
                                       C.byref(c), _stream(stream))
-    _check(st, "alcs_spconv1x1")
+    if st != ALCS_OK:
+        _check(st, "alcs_spconv1x1")
 
 
 def alcs_spconv1x1_ex(w: Packed, x, y, n: int, h: int, wd: int, stride: int = 1, bias=None, residual=None,
                       flags: int = 0, stream=None, cfg=None):
     """Strided pointwise convolution with a residual operand added before the activation."""
+    if cfg is None:
+        st = (_call or (lib(), _call)[1]).spconv1x1_ex(w.address, x, y, n, h, wd, stride, bias, residual, flags, stream)
+        if st != ALCS_OK:
+            _check(st, "alcs_spconv1x1_ex")
+        return
     c = _cfg(cfg)
     _check(lib().alcs_spconv1x1_ex(w.handle, _addr(x), _addr(y), n, h, wd, stride, _addr(bias), _addr(residual), flags,
                                    C.byref(c) if c is not None else None, _stream(stream)), "alcs_spconv1x1_ex")
@@ -366,8 +382,8 @@ def alcs_spconv2d(w: Packed, x, y, n: int, cin: int, h: int, wd: int, kh: int, k
     """General k x k convolution: x [n,cin,h,wd], y [n,cout,oh,ow] fp32 device tensors; w packed from
     the flattened filters [cout, cin*kh*kw].  cfg: optional dict of alcs_conv2d_cfg fields to fix."""
     if cfg is None:
-        _check(lib().alcs_spconv2d(w.handle, _addr(x), _addr(y), n, cin, h, wd, kh, kw, stride, pad, _addr(bias),
-                                   flags, _stream(stream)), "alcs_spconv2d")
+        _check((_call or (lib(), _call)[1]).spconv2d(w.address, x, y, n, cin, h, wd, kh, kw, stride, pad, bias, flags, stream),
+               "alcs_spconv2d")
     else:
         c = Conv2dCfg(**{k: int(v) for k, v in cfg.items()})
         _check(lib().alcs_spconv2d_cfg(w.handle, _addr(x), _addr(y), n, cin, h, wd, kh, kw, stride, pad, _addr(bias),
@@ -479,6 +495,10 @@ class Stack:
             raise AlcsError(ALCS_ERR_STATE, "Stack (destroyed)")
         return self._h
 
+    @property
+    def address(self) -> int:
+        return self._h.value or self.handle
+
     def destroy(self):
         if self._h:
             lib().alcs_stack_destroy(self._h)
@@ -503,7 +523,7 @@ def alcs_stack_create(layers: Sequence[dict], stack_flags: int = 0) -> Stack:
 
 
 def alcs_stack_run(s: Stack, stream=None):
-    _check(lib().alcs_stack_run(s.handle, _stream(stream)), "alcs_stack_run")
+    _check((_call or (lib(), _call)[1]).stack_run(s.address, stream), "alcs_stack_run")
 
 
 def alcs_stack_tune(s: Stack, passes: int = 0, stream=None):

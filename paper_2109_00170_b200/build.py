@@ -1,4 +1,5 @@
-"""Build libalcs.so (the C-ABI library with the sm_100a kernels) in-tree with nvcc.
+"""Build libalcs.so (the C-ABI library with the sm_100a kernels) in-tree with nvcc, and _alcs_call.so, a helper of the
+Python binding, with gcc.
 
     python -m paper_2109_00170_b200.build [--force]
 
@@ -12,12 +13,14 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libalcs.so")
+CALL = os.path.join(PKG, "_alcs_call.so")       # the binding's most frequent calls, marshalled in C
 
 SOURCES = ["alcs_pack.cpp", "alcs_device.cu", "alcs_conv2d.cu", "alcs_project.cu", "alcs_gather.cu", "alcs_probe.cu", "alcs_tc.cu", "alcs_tc16.cu", "alcs_tc_prep.cu", "alcs_variants_f32_g4.cu",
            "alcs_variants_f32_other.cu", "alcs_variants_f16.cu", "alcs_variants_f16_mma.cu", "alcs_variants_bf16.cu"]
@@ -58,8 +61,21 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _build_call(force: bool) -> None:
+    src = os.path.join(CSRC, "alcs_call.c")
+    if not force and os.path.exists(CALL) and os.path.getmtime(CALL) >= os.path.getmtime(src):
+        return
+    tmp = CALL + f".tmp{os.getpid()}"
+    r = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"], src, "-o", tmp],
+                       capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"gcc failed on alcs_call.c:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, CALL)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile (if stale) and return the path of libalcs.so."""
+    _build_call(force)
     os.makedirs(OBJ, exist_ok=True)
     if force:
         for f in os.listdir(OBJ):
