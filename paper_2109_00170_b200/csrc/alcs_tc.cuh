@@ -112,8 +112,9 @@ template <> struct Elem<__nv_bfloat16> {
 __device__ __forceinline__ int div_of(int n, const TcDiv& d) { return (int)((unsigned long long)(unsigned)n * d.mul >> d.shift); }
 
 // A role's walk over the block's items.  Where the tiles differ, what the next item needs from the tile table
-// is loaded one item ahead, and from the list of items two ahead: no step waits for memory.
-template <int L>
+// is loaded one item ahead.  AHEAD: from the list of items two ahead, so that no step waits for memory; of use to short items
+// (the other kernel's merged launches lose 1 % by it: a register and a load more in every role).
+template <int L, bool AHEAD = false>
 struct Cursor {
     const TcArgs<L>& a;
     int item, next_item, after = -1, at, layer = 0, next_layer = 0;
@@ -122,7 +123,7 @@ struct Cursor {
     __device__ __forceinline__ explicit Cursor(const TcArgs<L>& a_) : a(a_), at(blockIdx.x)
     {
         next_item = L > 1 && a.sched ? __ldg(a.sched + at) : at;
-        if (L > 1 && a.sched) after = __ldg(a.sched + at + gridDim.x);
+        if (AHEAD && L > 1 && a.sched) after = __ldg(a.sched + at + gridDim.x);
         peek();
     }
     __device__ __forceinline__ const TcLayer& of() const { return a.layer[L > 1 ? layer : 0]; }
@@ -166,11 +167,11 @@ struct Cursor {
         if (!has_next()) return false;
         item = next_item;
         at += gridDim.x;
-        if (L > 1 && a.sched) {         // (the list ends with a row of -1)
+        if (AHEAD && L > 1 && a.sched) {        // (the list ends with a row of -1)
             next_item = after;
             if (has_next()) after = __ldg(a.sched + at + gridDim.x);
         } else {
-            next_item = at;
+            next_item = L > 1 && a.sched ? __ldg(a.sched + at) : at;
         }
         layer = next_layer;
         t = next;

@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc16_kernel(const __grid_constant
         const unsigned staging = staging0 + warp * kStagingBytes, my_row = staging + lane * 128;
         unsigned n_grp = 0;
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        Cursor<L> cur(a);
+        Cursor<L, true> cur(a);
 #pragma unroll 1
         while (ok && cur.step()) {
             const TcLayer& y = cur.of();
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc16_kernel(const __grid_constant
             const int pw = warp - kProdWarp0;
             unsigned stage = 0, ph = 1, slot = 0, raw_ph = 0;
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            Cursor<L> cur(a);
+            Cursor<L, true> cur(a);
 #pragma unroll 1
             while (ok && cur.step()) {
                 const TcLayer& y = cur.of();
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc16_kernel(const __grid_constant
             const int k_mine = (warp - kRawWarp0) * (kChunk / kRawWarps);
             unsigned slot = 0, ph = 1;
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            Cursor<L> cur(a);
+            Cursor<L, true> cur(a);
 #pragma unroll 1
             while (ok && cur.step()) {
                 const TcLayer& y = cur.of();
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc16_kernel(const __grid_constant
             if (elect_one()) {
                 unsigned n_grp = 0, stage = 0, ph = 0;
                 bool first_wait = true;
-                Cursor<L> cur(a);
+                Cursor<L, true> cur(a);
 #pragma unroll 1
                 while (ok && cur.step()) {
                     const int k16 = cur.t.k16, n = cur.of().n, pixels = cur.of().n_px;
@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc16_kernel(const __grid_constant
         } else if (warp == kLoadWarp) {
             if (elect_one()) {
                 unsigned stage = 0, ph = 1, used = 0;
-                Cursor<L> cur(a);
+                Cursor<L, true> cur(a);
 #pragma unroll 1
                 while (ok && cur.step()) {
                     const TcLayer& y = cur.of();
