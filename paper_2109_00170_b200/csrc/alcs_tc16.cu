@@ -210,9 +210,11 @@ struct Fetch {
             word[i] = (w - run * per_run) * 16;
         }
     }
-    __device__ __forceinline__ void rows(const TcLayer& y, unsigned to, int k, int lane) const
+    // Fetch 16 rows; did this lane store elements itself?
+    __device__ __forceinline__ bool rows(const TcLayer& y, unsigned to, int k, int lane) const
     {
         to += lane * 16;
+        bool stored = false;
 #pragma unroll 1
         for (int r0 = 0; r0 < kChunk / kRawWarps; r0 += 4) {
             unsigned at[4][2];
@@ -229,6 +231,7 @@ struct Fetch {
                     edge = edge || (wanted && !inside);
                 }
             }
+            stored = stored || edge;
             if (edge)
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
@@ -241,6 +244,7 @@ struct Fetch {
                                 asm volatile("st.shared.u16 [%0], %1;" ::"r"(to + (r0 + r) * y.raw_row + i * 512 + (b - at[r][i])), "h"(v) : "memory");
                             }
         }
+        return stored;
     }
 };
 
@@ -572,8 +576,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc16_kernel(const __grid_constant
                 for (int k0 = 0; k0 < cur.t.k16 * 16; k0 += kChunk) {
                     ok = __all_sync(0xffffffffu, bar_wait(raw_empty + 8 * slot, ph));
                     if (!ok) break;
-                    if (k0 + k_mine < cur.t.k16 * 16) f.rows(y, raw0 + slot * a.raw_bytes + k_mine * y.raw_row, k0 + k_mine, lane);
-                    cp_async_arrive(raw_full + 8 * slot);
+                    const bool stored = k0 + k_mine < cur.t.k16 * 16 && f.rows(y, raw0 + slot * a.raw_bytes + k_mine * y.raw_row, k0 + k_mine, lane);
+                    if (stored) {
+                        // The arrival of copies says nothing of a thread's own stores; an ordinary one orders both, once the copies are done.
+                        asm volatile("cp.async.wait_all;" ::: "memory");
+                        bar_arrive(raw_full + 8 * slot);
+                    } else {
+                        cp_async_arrive(raw_full + 8 * slot);
+                    }
                     if (++slot == R) { slot = 0; ph ^= 1u; }
                 }
             }

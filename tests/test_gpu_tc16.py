@@ -37,7 +37,7 @@ def test_shapes(alcs, n, cin, cout, h, wd, g, density):
     assert Y <= TOL["f32"]
 
 
-def _device_call(alcs, W, M, X, b, g, h, wd, res, bf16, y_f32, x_off=0, y_off=0):
+def _device_call(alcs, W, M, X, b, g, h, wd, res, bf16, y_f32, x_off=0, y_off=0, cfg=CFG):
     """One residual call with X and Y starting `off` elements into their buffers; returns Y and what lies around it."""
     import torch
     dev = torch.device("cuda:0")
@@ -53,7 +53,7 @@ def _device_call(alcs, W, M, X, b, g, h, wd, res, bf16, y_f32, x_off=0, y_off=0)
     yb = torch.full((size + y_off + 32,), 7.0, dtype=ydt, device=dev)
     rt = None if res is None else torch.from_numpy(res).to(dev).to(ydt).contiguous()
     flags = alcs.ALCS_RELU | (alcs.ALCS_Y_F32 if y_f32 else 0)
-    alcs.alcs_spconv1x1_ex(p, xb[x_off:], yb[y_off:], n, h, wd, 1, torch.from_numpy(b).to(dev), rt, flags, torch.cuda.current_stream(), CFG)
+    alcs.alcs_spconv1x1_ex(p, xb[x_off:], yb[y_off:], n, h, wd, 1, torch.from_numpy(b).to(dev), rt, flags, torch.cuda.current_stream(), cfg)
     torch.cuda.synchronize()
     assert alcs.alcs_packed_status(p) == 0
     y = yb.float().cpu().numpy()
@@ -78,6 +78,19 @@ def test_residual_types_and_alignments(alcs, n, cin, cout, h, wd, bf16, y_f32, o
     assert np.isfinite(Y).all()
     unit = 0.0 if y_f32 else 2.0 ** -8 if bf16 else 2.0 ** -11
     assert (np.abs(Y - Yref) <= TOL["f32"] * A + unit * np.abs(Yref)).all()
+
+
+@pytest.mark.parametrize("x_off", [0, 1, 3, 7])
+@pytest.mark.parametrize("n,hw", [(1, 49), (2, 63), (3, 131)])
+def test_ends_of_x_in_slots_used_again(alcs, n, hw, x_off):
+    """Words that reach beyond X are stored element by element, to slots that held other rows before: six chunks, sixteen channel
+    tiles, and other values at the second call."""
+    g, cin, cout = 8, 384, 256
+    for seed in (3, 4):
+        W, M, X, b = _case(seed, n, cin, cout, hw, g, 0.4, np.float32)
+        Y, Wr, Xr, _ = _device_call(alcs, W, M, X, b, g, hw, 1, None, False, True, x_off, cfg=dict(CFG, row_groups=16))
+        Yref, A = oracle.conv1x1(Wr, M, Xr, b, True, g, want_scale=True)
+        assert (np.abs(Y - Yref) <= TOL["f32"] * A).all()
 
 
 def test_rows_that_keep_nothing_and_skewed_rows(alcs):
