@@ -1,5 +1,6 @@
 """Thin binding of libalcs.so: argument marshalling only, same names as the C ABI
-(include/alcs.h); through ctypes, and for the calls that a program makes once per layer through _alcs_call (C).  Every step of the convolution runs in the library's CUDA kernels; there is no
+(include/alcs.h); through ctypes, and for the plain form of the calls
+that a program makes once per layer through _alcs_call (C).  Every step of the convolution runs in the library's CUDA kernels; there is no
 Python or CPU fallback, and loading fails loudly if the shared object has not been built.
 """
 from __future__ import annotations
@@ -86,6 +87,16 @@ _lib = None
 _call = None      # the C marshalling of the per-layer calls, bound to _lib's functions
 
 
+class _NoCall:
+    """In the place of _alcs_call: no call is plain, ctypes makes all of them."""
+
+    @staticmethod
+    def _none(*args):
+        return None
+
+    spconv1x1 = spconv1x1_ex = spconv2d = stack_run = _none
+
+
 def lib():
     """Load libalcs.so once.  Raises if it is missing: there is nothing to fall back to."""
     global _lib, _call
@@ -150,6 +161,11 @@ def lib():
     return L
 
 
+def _native():
+    """_alcs_call: its functions return the status, or None for a call that they leave to ctypes."""
+    return _call or (lib(), _call)[1]
+
+
 def _check(status: int, where: str):
     if status != ALCS_OK:
         raise AlcsError(status, where)
@@ -193,10 +209,6 @@ class Packed:
         if not self._h:
             raise AlcsError(ALCS_ERR_STATE, "Packed (freed)")
         return self._h
-
-    @property
-    def address(self) -> int:
-        return self._h.value or self.handle
 
     def free(self):
         if self._h:
@@ -315,7 +327,9 @@ def alcs_spconv1x1(w: Packed, x, y, n: int, h: int, wd: int, bias=None, flags: i
                    cfg=None):
     """x, y, bias: device tensors (anything with data_ptr()) or raw device addresses."""
     if cfg is None:
-        st = (_call or (lib(), _call)[1]).spconv1x1(w.address, x, y, n, h, wd, bias, flags, stream)
+        st = _native().spconv1x1(w.handle, x, y, n, h, wd, bias, flags, stream)
+        if st is None:
+            st = lib().alcs_spconv1x1(w.handle, _addr(x), _addr(y), n, h, wd, _addr(bias), flags, _stream(stream))
     else:
         c = _cfg(cfg)
         st = lib().alcs_spconv1x1_cfg(w.handle, _addr(x), _addr(y), n, h, wd, _addr(bias), flags,
@@ -327,10 +341,9 @@ def alcs_spconv1x1(w: Packed, x, y, n: int, h: int, wd: int, bias=None, flags: i
 def alcs_spconv1x1_ex(w: Packed, x, y, n: int, h: int, wd: int, stride: int = 1, bias=None, residual=None,
                       flags: int = 0, stream=None, cfg=None):
     """Strided pointwise convolution with a residual operand added before the activation."""
-    if cfg is None:
-        st = (_call or (lib(), _call)[1]).spconv1x1_ex(w.address, x, y, n, h, wd, stride, bias, residual, flags, stream)
-        if st != ALCS_OK:
-            _check(st, "alcs_spconv1x1_ex")
+    st = _native().spconv1x1_ex(w.handle, x, y, n, h, wd, stride, bias, residual, flags, stream) if cfg is None else None
+    if st is not None:
+        _check(st, "alcs_spconv1x1_ex")
         return
     c = _cfg(cfg)
     _check(lib().alcs_spconv1x1_ex(w.handle, _addr(x), _addr(y), n, h, wd, stride, _addr(bias), _addr(residual), flags,
@@ -382,8 +395,11 @@ def alcs_spconv2d(w: Packed, x, y, n: int, cin: int, h: int, wd: int, kh: int, k
     """General k x k convolution: x [n,cin,h,wd], y [n,cout,oh,ow] fp32 device tensors; w packed from
     the flattened filters [cout, cin*kh*kw].  cfg: optional dict of alcs_conv2d_cfg fields to fix."""
     if cfg is None:
-        _check((_call or (lib(), _call)[1]).spconv2d(w.address, x, y, n, cin, h, wd, kh, kw, stride, pad, bias, flags, stream),
-               "alcs_spconv2d")
+        st = _native().spconv2d(w.handle, x, y, n, cin, h, wd, kh, kw, stride, pad, bias, flags, stream)
+        if st is None:
+            st = lib().alcs_spconv2d(w.handle, _addr(x), _addr(y), n, cin, h, wd, kh, kw, stride, pad, _addr(bias),
+                                     flags, _stream(stream))
+        _check(st, "alcs_spconv2d")
     else:
         c = Conv2dCfg(**{k: int(v) for k, v in cfg.items()})
         _check(lib().alcs_spconv2d_cfg(w.handle, _addr(x), _addr(y), n, cin, h, wd, kh, kw, stride, pad, _addr(bias),
@@ -495,10 +511,6 @@ class Stack:
             raise AlcsError(ALCS_ERR_STATE, "Stack (destroyed)")
         return self._h
 
-    @property
-    def address(self) -> int:
-        return self._h.value or self.handle
-
     def destroy(self):
         if self._h:
             lib().alcs_stack_destroy(self._h)
@@ -523,7 +535,10 @@ def alcs_stack_create(layers: Sequence[dict], stack_flags: int = 0) -> Stack:
 
 
 def alcs_stack_run(s: Stack, stream=None):
-    _check((_call or (lib(), _call)[1]).stack_run(s.address, stream), "alcs_stack_run")
+    st = _native().stack_run(s.handle, stream)
+    if st is None:
+        st = lib().alcs_stack_run(s.handle, _stream(stream))
+    _check(st, "alcs_stack_run")
 
 
 def alcs_stack_tune(s: Stack, passes: int = 0, stream=None):
