@@ -1,6 +1,6 @@
 """Thin binding of libalcs.so: argument marshalling only, same names as the C ABI
 (include/alcs.h); through ctypes, and for the plain form of the calls
-that a program makes once per layer through _alcs_call (C).  Every step of the convolution runs in the library's CUDA kernels; there is no
+that a program makes once per layer through _alcs_call (C), where that has been built.  Every step of the convolution runs in the library's CUDA kernels; there is no
 Python or CPU fallback, and loading fails loudly if the shared object has not been built.
 """
 from __future__ import annotations
@@ -88,7 +88,7 @@ _call = None      # the C marshalling of the per-layer calls, bound to _lib's fu
 
 
 class _NoCall:
-    """In the place of _alcs_call: no call is plain, ctypes makes all of them."""
+    """In the place of _alcs_call where it has not been built for this Python: no call is plain, ctypes makes all of them."""
 
     @staticmethod
     def _none(*args):
@@ -154,9 +154,9 @@ def lib():
             f.restype = i
     try:
         from . import _alcs_call as native
-    except ImportError as e:
-        raise RuntimeError("_alcs_call not found or not loadable: build it with `python -m paper_2109_00170_b200.build`") from e
-    native.bind(*(C.cast(getattr(L, name), vp).value for name in ("alcs_spconv1x1", "alcs_spconv1x1_ex", "alcs_spconv2d", "alcs_stack_run")))
+        native.bind(*(C.cast(getattr(L, name), vp).value for name in ("alcs_spconv1x1", "alcs_spconv1x1_ex", "alcs_spconv2d", "alcs_stack_run")))
+    except ImportError:
+        native = _NoCall
     _lib, _call = L, native
     return L
 

@@ -128,3 +128,27 @@ def test_same_through_both_ways(monkeypatch, name):
         assert getattr(native, name)(plain[0].handle, *plain[1:-1], np.int64(1)) is None
     finally:
         native.bind(*(C.cast(getattr(real, n), VP).value for n in names))
+
+
+def test_works_without_the_helper(monkeypatch, tmp_path):
+    """No _alcs_call for this Python: the library loads and every call goes through ctypes; nor does a missing compiler stop the build."""
+    import sys
+    import sysconfig
+
+    import paper_2109_00170_b200 as A
+    from paper_2109_00170_b200 import build
+    monkeypatch.setattr(B, "_lib", None)
+    monkeypatch.setattr(B, "_call", None)
+    monkeypatch.delattr(A, "_alcs_call", raising=False)
+    monkeypatch.setitem(sys.modules, "paper_2109_00170_b200._alcs_call", None)        # importing it raises ImportError
+    assert B.lib() is not None and B._call is B._NoCall
+    p = A.alcs_pack(np.ones((4, 4), np.float32), np.ones((1, 4), np.uint8), 4)
+    with pytest.raises(B.AlcsError):         # (not on a device)
+        A.alcs_spconv1x1(p, 4096, 8192, 1, 1, 1)
+    assert build.CALL.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    monkeypatch.setattr(build, "CALL", str(tmp_path / "helper.so"))
+    monkeypatch.setenv("CC", str(tmp_path / "no-such-compiler"))
+    build._build_call(True)
+    monkeypatch.setenv("CC", "false")
+    build._build_call(True)
+    assert not list(tmp_path.iterdir())
