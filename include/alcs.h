@@ -173,8 +173,9 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     after the other and a work item stages them with a few large bulk (TMA) copies: the
  *                     staging then costs the kernel next to no instructions, at the price of one more pass
  *                     over X where its rows would not have needed repacking.  Batches of more than 8 images
- *   producer_warps    warps of the thread block that only move data (1..4); math_mode 4: 8 names the kernel for 16-bit operands
- *                     that multiplies X as it lies in memory (stride 1), 0 leaves the choice of kernel to the library
+ *   producer_warps    warps of the thread block that only move data (1..4).  math_mode 4 has two kernels for 16-bit operands at
+ *                     stride 1: 8 names the one that multiplies X as it lies in memory, 4 the one that takes it apart;
+ *                     any other value leaves the choice to the library.  Other layers have one kernel, whatever it says
  *   math_mode         1 = fp32 FMA on the CUDA cores; 2 = tensor cores (fp16 weights and activations
  *                     only): 16 kept blocks of a block row times the 16 input rows they select is a
  *                     dense 16 x g by 16 x pixels contraction, run as warp-level MMA with fp32
@@ -187,7 +188,9 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     4 = fifth-generation tensor cores: the kept blocks of a tile of output channels are expanded
  *                     (once per packed matrix, on the device) to dense weight tiles and multiplied with 128-pixel
  *                     tiles of X; fp32 operands are split exactly into three bfloat16 parts each.  Only row_groups
- *                     (the number of channel tiles, each of at most 128 channels) and producer_warps apply; no scratch is used.  Outputs of
+ *                     (the number of channel tiles, each of at most 128 channels), producer_warps and, with producer_warps 8,
+ *                     pixels_per_lane apply (pixels per tile, 32 to 256: the most multiples of 32 that are no more and that the layer
+ *                     can take; less than 32: the library chooses); no scratch is used.  Outputs of
  *                     pixels with infinite or NaN inputs are computed from the storage format instead, so that such values
  *                     reach the channels that keep a block of theirs and no others, as with the other kernels (slowly); fp32
  *                     matrices that keep an infinite or NaN weight are refused (UNSUPPORTED)

@@ -354,24 +354,33 @@ bool tc_ok(const alcs_packed* w, const CallShape& c)
 
 // alcs_tc16.cu takes 16-bit operands at stride 1.
 bool tc16_ok(const alcs_packed* w, const CallShape& c) { return w->dt != ALCS_F32 && c.stride == 1; }
-constexpr int kTc16Producers = 8;        // producer_warps of a configuration that names it
+// producer_warps of a configuration that names the kernel of such a layer: alcs_tc.cu, alcs_tc16.cu.  Its pixels_per_lane are
+// pixels per tile then (a lane of the accumulator is a channel).
+constexpr int kTcProducers = 4, kTc16Producers = 8;
 
-// The tcgen05 kernels with n output channels per tile as a plan: the one that is expected to be faster.  Its estimate has to be clearly
-// lower for alcs_tc16.cu where rows must be picked apart (43 x 780 -> 139 @7 with a residual: 27 us where 17 were expected).
-Plan tc_plan(const alcs_packed* w, int n, const CallShape& c, int sms)
+// The tcgen05 kernel that is named with n output channels per tile as a plan: alcs_tc.cu, or alcs_tc16.cu with the most pixels per tile
+// that are no more than `pixels`, or with those that are expected to take the least.
+constexpr int kAnyPixels = -1;
+Plan tc_plan_on(const alcs_packed* w, int n, const CallShape& c, int sms, int pixels)
 {
     Plan p;
     p.n_rg = (w->cout + n - 1) / n;
-    n = ((w->cout + p.n_rg - 1) / p.n_rg + 15) / 16 * 16;       // (the equal split into that many tiles)
-    p.tc_n = n;
-    p.cost = 1e-6 * alcs::tc_layer_us(w, tc_problem(c), n, sms);
+    p.tc_n = ((w->cout + p.n_rg - 1) / p.n_rg + 15) / 16 * 16;       // (the equal split into that many tiles)
+    p.cost = 1e-6 * (pixels ? alcs::tc16_layer_us(w, tc_problem(c), p.tc_n, sms, std::max(0, pixels), &p.tc_px) : alcs::tc_layer_us(w, tc_problem(c), p.tc_n, sms));
+    return p;
+}
+
+// The one that is expected to be faster.  Its estimate has to be clearly
+// lower for alcs_tc16.cu where rows must be picked apart (43 x 780 -> 139 @7 with a residual: 27 us where 17 were expected).
+Plan tc_plan(const alcs_packed* w, int n, const CallShape& c, int sms)
+{
+    Plan p = tc_plan_on(w, n, c, sms, 0);
     if (tc16_ok(w, c)) {
-        int px;
-        const double us = 1e-6 * alcs::tc16_layer_us(w, tc_problem(c), n, sms, &px);
+        Plan other = tc_plan_on(w, n, c, sms, kAnyPixels);
         const bool direct = (size_t)c.hw() * w->elt() % 8 == 0;
-        if (us * (direct ? 1.05 : 1.3) < p.cost) {
-            p.tc_px = px;
-            if (direct) p.cost = us;        // (else the staged kernels stay where they were chosen: 156 -> 43 @7, batch 11: 12 us, not 16)
+        if (other.cost * (direct ? 1.05 : 1.3) < p.cost) {
+            if (!direct) other.cost = p.cost;        // (the staged kernels stay where they were chosen: 156 -> 43 @7, batch 11: 12 us, not 16)
+            p = other;
         }
     }
     return p;
@@ -388,13 +397,14 @@ int tc_widths(const alcs_packed* w, int (&n)[8])
     return count;
 }
 
-Plan tc_best(const alcs_packed* w, const CallShape& c, int sms)
+template <typename F>
+Plan tc_best(const alcs_packed* w, F of_width)
 {
     int n[8];
     const int count = tc_widths(w, n);
-    Plan best = tc_plan(w, n[0], c, sms);
+    Plan best = of_width(n[0]);
     for (int i = 1; i < count; ++i) {
-        const Plan p = tc_plan(w, n[i], c, sms);
+        const Plan p = of_width(n[i]);
         if (p.cost < best.cost) best = p;
     }
     return best;
@@ -610,7 +620,7 @@ int staged_best(const alcs_packed* w, const CallShape& c, Plan* out)
     return ALCS_ERR_UNSUPPORTED;
 }
 
-void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
+void plan_to_cfg(const alcs_packed* w, const CallShape& shape, const Plan& p, alcs_launch_cfg* c)
 {
     if (p.gather) {
         std::memset(c, 0, sizeof *c);
@@ -621,10 +631,10 @@ void plan_to_cfg(const Plan& p, alcs_launch_cfg* c)
     }
     if (p.tc_n) {
         std::memset(c, 0, sizeof *c);
-        c->pixels_per_lane = 1;
+        c->pixels_per_lane = p.tc_px ? p.tc_px : 1;
         c->math_mode = 4;
         c->row_groups = p.n_rg;
-        c->producer_warps = p.tc_px ? kTc16Producers : 0;
+        c->producer_warps = p.tc_px ? kTc16Producers : tc16_ok(w, shape) ? kTcProducers : 0;
         return;
     }
     const KernelVariant& v = g_variants[p.variant].v;
@@ -653,11 +663,19 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
     const bool tc = (!c || c->math_mode == 4) && tc_ok(w, shape);
     if (c && c->math_mode == 4) {       // the tcgen05 kernel as asked for: row_groups channel tiles
         if (!tc) return ALCS_ERR_UNSUPPORTED;
-        const int tiles = c->row_groups ? c->row_groups : tc_best(w, shape, di.sms).n_rg;
-        const int n = ((w->cout + std::max(1, tiles) - 1) / std::max(1, tiles) + 15) / 16 * 16;
+        const int named = tc16_ok(w, shape) ? c->producer_warps : 0;       // (the others have one kernel)
+        auto of_width = [&](int n) {
+            return named == kTcProducers ? tc_plan_on(w, n, shape, di.sms, 0)
+                 : named == kTc16Producers ? tc_plan_on(w, n, shape, di.sms, c->pixels_per_lane >= 32 ? c->pixels_per_lane : kAnyPixels)
+                 : tc_plan(w, n, shape, di.sms);
+        };
+        if (!c->row_groups) {
+            *out = tc_best(w, of_width);
+            return ALCS_OK;
+        }
+        const int tiles = std::max(1, c->row_groups), n = ((w->cout + tiles - 1) / tiles + 15) / 16 * 16;
         if (n > alcs::kTcMaxN) return ALCS_ERR_UNSUPPORTED;
-        *out = tc_plan(w, n, shape, di.sms);
-        if (c->producer_warps == kTc16Producers && !out->tc_px && tc16_ok(w, shape)) (void)alcs::tc16_layer_us(w, tc_problem(shape), out->tc_n, di.sms, &out->tc_px);
+        *out = of_width(n);
         return ALCS_OK;
     }
     if (!c) {
@@ -1471,7 +1489,7 @@ ALCS_API int alcs_spconv1x1_plan(const alcs_packed* w, int n, int h, int wd, uns
     Plan plan;
     const int rc = resolve_plan(w, {n, h, wd, h, wd}, flags, nullptr, &plan);
     if (rc) return rc;
-    plan_to_cfg(plan, out);
+    plan_to_cfg(w, {n, h, wd, h, wd}, plan, out);
     return ALCS_OK;
 }
 
@@ -1559,7 +1577,7 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
     if (e != cudaSuccess) { alcs::set_cuda_error_text(cudaGetErrorString(e)); return ALCS_ERR_CUDA; }
     if (best_i < 0) return ALCS_ERR_CUDA;
     alcs_launch_cfg c;
-    plan_to_cfg(all[best_i], &c);
+    plan_to_cfg(w, {n, h, wd, h, wd}, all[best_i], &c);
     all[best_i].cost = 1e-3 * best_ms;
     {
         std::lock_guard<std::mutex> lk(w->mu);
@@ -1601,7 +1619,7 @@ ALCS_API int alcs_spconv1x1_set_cfg(alcs_packed* w, int n, int h, int wd, unsign
     const int rc = cfg_to_plan(w, {n, h, wd, h, wd}, cfg, &plan);
     if (rc) return rc;
     alcs_launch_cfg full;
-    plan_to_cfg(plan, &full);
+    plan_to_cfg(w, {n, h, wd, h, wd}, plan, &full);
     std::lock_guard<std::mutex> lk(w->mu);
     const alcs::ShapeKey key{n, h, wd, flags};
     w->tuned[key] = full;
@@ -1851,8 +1869,7 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
         }
         for (size_t k = i; k < end && !choice.empty(); ++k) {
             alcs_stack::Item& it = s->items[k];
-            it.plan = tc_plan(it.layer.w, choice[k - i], call_shape(it), di.sms);
-            it.plan.tc_px = choice_px[k - i];
+            it.plan = tc_plan_on(it.layer.w, choice[k - i], call_shape(it), di.sms, choice_px[k - i]);
         }
         i = end;
     }
@@ -2245,7 +2262,7 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
         if (it.q == 0) continue;
         const alcs_layer& L = it.layer;
         alcs_launch_cfg c;
-        plan_to_cfg(it.plan, &c);
+        plan_to_cfg(L.w, call_shape(it), it.plan, &c);
         const alcs::ShapeKey key{L.n, it.oh, it.ow, key_flags(L.w, L.flags, call_shape(it))};
         std::lock_guard<std::mutex> lk(L.w->mu);
         L.w->tuned[alcs::ShapeKey{L.n, it.oh, it.ow, L.flags}] = c;
@@ -2264,7 +2281,7 @@ ALCS_API int alcs_stack_layer_cfg(const alcs_stack* s, int layer, alcs_launch_cf
     if (!s || !out || layer < 0 || layer >= (int)s->items.size()) return ALCS_ERR_INVALID_ARG;
     std::memset(out, 0, sizeof *out);
     if (s->items[layer].q == 0) return ALCS_OK;
-    plan_to_cfg(s->items[layer].plan, out);
+    plan_to_cfg(s->items[layer].layer.w, call_shape(s->items[layer]), s->items[layer].plan, out);
     return ALCS_OK;
 }
 

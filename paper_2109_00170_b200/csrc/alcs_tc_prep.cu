@@ -616,7 +616,7 @@ double tc16_item_us(const alcs_packed* w, const TcProblem& p, int n, int k16, in
     return std::max((k16 + 3) / 4 * chunk, store);
 }
 
-double tc16_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms, int* pixels)
+double tc16_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms, int cap, int* pixels)
 {
     const std::vector<int> k16 = tc_tile_steps(w, p, n);
     const long long q = (long long)std::max(1, p.n) * p.oh * p.ow;
@@ -624,7 +624,7 @@ double tc16_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms, i
     const bool raw = (size_t)p.oh * p.ow * w->elt() % 8 != 0;
     double best = 0;
     *pixels = 0;
-    for (int px : tc16_tiles(w, p, k_max)) {
+    for (int px : cap ? std::vector<int>{tc16_capped(w, p, k_max, cap)} : tc16_tiles(w, p, k_max)) {
         const double tiles = (double)((q + px - 1) / px);
         double sum = 0, longest = 0;
         for (int k : k16) {

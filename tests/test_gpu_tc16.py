@@ -148,3 +148,59 @@ def test_merged_stack(alcs, sizes, graph):
     for L, (Yref, A) in zip(layers, want):
         assert_parity(L["y"].cpu().numpy(), Yref, A, "f16")
         assert alcs.alcs_packed_status(L["w"]) == 0
+
+
+@pytest.mark.parametrize("cin,h", [(64, 14), (300, 14), (64, 7), (300, 9)])
+def test_configurations_say_what_runs(alcs, cin, h):
+    """What plan() and a stack report names the kernel, its channel tiles and its pixels per tile, so that it can be fixed again."""
+    n, cout, g = 4, 136, 8
+    W, M, X, b = _case(cin + h, n, cin, cout, h * h, g, 0.4)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    most = (256 if h == 14 else 128) if cin == 64 else 128
+    asked = [(0, 0), (4, 0), (8, 0), (8, 1)] + [(8, px) for px in (32, 64, 96, 100, 128, 256, 1000)]
+    for producers, px in asked:
+        for tiles in (0, 2, 5):
+            cfg = dict(math_mode=4, producer_warps=producers, pixels_per_lane=px, row_groups=tiles)
+            alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, cfg)
+            plan = alcs.alcs_spconv1x1_plan(p, n, h, h)
+            assert plan["math_mode"] == 4 and (not tiles or plan["row_groups"] == tiles)
+            assert plan["producer_warps"] == producers if producers else plan["producer_warps"] in (4, 8)
+            if producers == 8:
+                assert plan["pixels_per_lane"] in ([min(px // 32 * 32, most)] if px >= 32 else range(32, most + 1, 32))
+            alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, plan)
+            assert alcs.alcs_spconv1x1_plan(p, n, h, h) == plan
+            check_layer(alcs, W, M, X, b, False, g, cfg=plan, h=h, wd=h, packed=p)
+    # in a stack, beside a layer on the other kernel
+    import torch
+    x, ys = torch.from_numpy(X).cuda(), [torch.empty(n, cout, h * h, dtype=torch.float16, device="cuda") for _ in range(3)]
+    qs = [alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0) for _ in range(3)]
+    want = [dict(math_mode=4, producer_warps=8, pixels_per_lane=64, row_groups=2), dict(math_mode=4, producer_warps=4, pixels_per_lane=1, row_groups=3),
+            dict(math_mode=4, producer_warps=8, pixels_per_lane=32, row_groups=9)]
+    for q, cfg in zip(qs, want):
+        alcs.alcs_spconv1x1_set_cfg(q, n, h, h, 0, cfg)
+    s = alcs.alcs_stack_create([dict(w=q, x=x, y=y, n=n, h=h, wd=h, bias=None, flags=0) for q, y in zip(qs, ys)], 0)
+    for i, cfg in enumerate(want):
+        got = alcs.alcs_stack_layer_cfg(s, i)
+        assert {k: got[k] for k in cfg} == cfg
+    alcs.alcs_stack_run(s, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    Yref, A = oracle.conv1x1(W, M, X, None, False, g, want_scale=True)
+    for y in ys:
+        assert_parity(y.cpu().numpy(), Yref, A, "f16")
+
+
+def test_layers_of_one_kernel_take_any_producers(alcs):
+    """fp32 and strided layers have one tcgen05 kernel: producer_warps says nothing there, as ever."""
+    import torch
+    W, M, X, b = _case(3, 2, 64, 72, 14 * 14, 8, 0.5, np.float32)
+    for producers in (0, 4, 8):
+        check_layer(alcs, W, M, X, b, True, 8, cfg=dict(math_mode=4, producer_warps=producers), h=14, wd=14)
+    W, M, X, b = _case(4, 2, 64, 72, 16 * 16, 8, 0.5)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 8), 0)
+    x, y = torch.from_numpy(X).cuda(), torch.empty(2, 72, 64, dtype=torch.float16, device="cuda")
+    ref = None
+    for producers in (0, 4, 8):
+        alcs.alcs_spconv1x1_ex(p, x, y, 2, 16, 16, 2, None, None, 0, torch.cuda.current_stream(), dict(math_mode=4, producer_warps=producers))
+        torch.cuda.synchronize()
+        ref = y.clone() if ref is None else ref
+        assert torch.equal(y, ref)
