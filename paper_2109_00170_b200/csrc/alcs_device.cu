@@ -386,6 +386,21 @@ Plan tc_plan(const alcs_packed* w, int n, const CallShape& c, int sms)
     return p;
 }
 
+// What a tuner compares with n output channels per tile: both kernels, and of alcs_tc16.cu a few heights beside the one that is expected to
+// be the best (the estimate's median error is 9 %, the heights next to it differ by less).
+void tc_plans(const alcs_packed* w, int n, const CallShape& c, int sms, std::vector<Plan>& out)
+{
+    out.push_back(tc_plan_on(w, n, c, sms, 0));
+    if (!tc16_ok(w, c)) return;
+    std::vector<int> px;
+    for (int want : {kAnyPixels, alcs::kTc16Pixels, alcs::kTc16Pixels / 2, alcs::kTc16Pixels / 4}) {
+        const Plan p = tc_plan_on(w, n, c, sms, want);
+        if (std::find(px.begin(), px.end(), p.tc_px) != px.end()) continue;
+        px.push_back(p.tc_px);
+        out.push_back(p);
+    }
+}
+
 // Channels per tile worth considering: the equal split of cout into as many tiles as each multiple of 16 asks for.
 int tc_widths(const alcs_packed* w, int (&n)[8])
 {
@@ -572,7 +587,7 @@ int enumerate_plans(const alcs_packed* w, const CallShape& c, std::vector<Plan>&
     if (!quick && tc_ok(w, c)) {
         int n[8];
         const int count = tc_widths(w, n);
-        for (int i = 0; i < count; ++i) out.push_back(tc_plan(w, n[i], c, di.sms));
+        for (int i = 0; i < count; ++i) tc_plans(w, n[i], c, di.sms, out);
     }
     if (!quick && c.stride == 1 && !c.residual && hw > 0 && c.images() <= kGatherImages) {        // small batches only: one thread block per (block row, image, pixel tile)
         for (int p = 8; p >= 2; p /= 2)
@@ -1795,13 +1810,14 @@ constexpr double kMergedRampUs = 5.0;
 // Consecutive independent layers whose configuration nobody fixed for the stack: one launch of a tcgen05 kernel for
 // all of them, where its estimate is below the sum of the layers' own (measured ones, after alcs_spconv1x1_tune).  With few items in all, narrower tiles shorten
 // the longest SM's share; with many, wide ones do the least work.
-// fixed_too: of whatever was fixed, too (alcs_stack_tune).
-void stack_merge(alcs_stack* s, bool fixed_too = false)
+// by: what decides; alcs_stack_tune measures both ways, of whatever was fixed, too.
+enum class MergeBy { estimates, one_launch, kernels };
+void stack_merge(alcs_stack* s, MergeBy by = MergeBy::estimates)
 {
     auto open = [&](const alcs_stack::Item& it) {
         const alcs_layer& L = it.layer;
         if (L.stride > 1 || !tc_ok(L.w, call_shape(it)) || (long long)L.w->rows * L.w->g * L.w->cin > alcs::kTcMaxWeights) return false;
-        if (fixed_too) return true;
+        if (by != MergeBy::estimates) return true;
         const alcs::ShapeKey key{L.n, it.oh, it.ow, L.flags};
         std::lock_guard<std::mutex> lk(L.w->mu);
         return L.w->tuned.find(key) == L.w->tuned.end() || L.w->tuned_alone.count(key) != 0;
@@ -1851,12 +1867,12 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
         };
         double best = 0;
         for (size_t k = i; k < end; ++k) best += s->items[k].plan.cost * 1e6;
-        const double one = together(i, end, false);
-        if (one < best) { best = one; choice = widths; choice_px = pixels; }
+        const double one = by == MergeBy::kernels ? 0 : together(i, end, false);
+        if (by == MergeBy::one_launch || (by == MergeBy::estimates && one < best)) { best = one; choice = widths; choice_px = pixels; }
         // 16-bit operands: layers whose rows can be copied as they are on alcs_tc16.cu, a launch per sequence of layers of one kind
         // (several launches have to promise a tenth: the estimates are that good)
         auto direct = [&](size_t k) { return (size_t)s->items[k].oh * s->items[k].ow * s->items[k].layer.w->elt() % 8 == 0; };
-        if (s->items[i].layer.w->dt != ALCS_F32) {
+        if (by != MergeBy::one_launch && s->items[i].layer.w->dt != ALCS_F32) {
             double t = 0;
             int launches = 0;
             bool any = false;
@@ -1865,7 +1881,7 @@ void stack_merge(alcs_stack* s, bool fixed_too = false)
                 t += together(from, to, direct(from));
                 any = any || direct(from);
             }
-            if (any && t * (launches > 1 ? 1.1 : 1.0) < best) { best = t; choice = widths; choice_px = pixels; }
+            if (any && (by == MergeBy::kernels || t * (launches > 1 ? 1.1 : 1.0) < best)) { best = t; choice = widths; choice_px = pixels; }
         }
         for (size_t k = i; k < end && !choice.empty(); ++k) {
             alcs_stack::Item& it = s->items[k];
@@ -2178,8 +2194,14 @@ int stack_candidates(const alcs_stack::Item& it, std::vector<Plan>& out)
     std::vector<Plan> all;
     const int rc = enumerate_plans(L.w, call_shape(it), all);
     if (rc) return rc;
+    int ranked = 0;
+    std::vector<int> widths;
     for (size_t i = 0; i < all.size(); ++i) {
-        if (!((!had && i < 8) || all[i].gather) || (L.stride > 1 && all[i].tc_n)) continue;
+        // (the tcgen05 kernels with as many channels per tile count once)
+        const bool again = all[i].tc_n && std::find(widths.begin(), widths.end(), all[i].tc_n) != widths.end();
+        if (all[i].tc_n && !again) widths.push_back(all[i].tc_n);
+        ranked += !again;
+        if (!((!had && ranked <= 8) || all[i].gather) || (L.stride > 1 && all[i].tc_n)) continue;
         bool dup = false;
         for (const Plan& p : out) dup |= same_plan(p, all[i]);
         if (!dup) out.push_back(all[i]);
@@ -2213,10 +2235,14 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
     cur = time_stack(s, st, e0, e1, reps);
     if (cur < 0) return ALCS_ERR_CUDA;
     if (us_before) *us_before = cur;
-    {   // one launch for all independent layers: no sequence of single-layer changes leads there
+    for (MergeBy by : {MergeBy::one_launch, MergeBy::kernels}) {
+        // one launch for all independent layers, or for each sequence of one kernel: no sequence of single-layer changes leads there
         std::vector<Plan> keep;
+        bool changed = false;
         for (const auto& it : s->items) keep.push_back(it.plan);
-        stack_merge(s, true);
+        stack_merge(s, by);
+        for (size_t i = 0; i < keep.size(); ++i) changed |= !same_plan(keep[i], s->items[i].plan);
+        if (!changed) continue;
         const double t = time_stack(s, st, e0, e1, reps);
         if (t > 0 && t < cur * 0.996) cur = t;
         else

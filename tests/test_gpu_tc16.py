@@ -204,3 +204,32 @@ def test_layers_of_one_kernel_take_any_producers(alcs):
         torch.cuda.synchronize()
         ref = y.clone() if ref is None else ref
         assert torch.equal(y, ref)
+
+
+@pytest.mark.parametrize("stack", [False, True])
+def test_tuners_compare_the_two_kernels(alcs, stack):
+    """X starts on an odd word here, which rows fetched as they are pay for (49 us and more where the other kernel takes 25; for an aligned X
+    it is the slower one): only a tuner that times both kernels finds out."""
+    import torch
+    n, cin, cout, h, g = 38, 78, 1300, 20, 8
+    W, M, X, b = _case(12, n, cin, cout, h * h, g, 0.25, np.float32)
+    Wt, st = torch.from_numpy(W).to(torch.bfloat16), torch.cuda.current_stream()
+    x = torch.zeros(X.size + 8, dtype=torch.bfloat16, device="cuda")[2:2 + X.size]
+    x.copy_(torch.from_numpy(X).reshape(-1))
+    Yref, A = oracle.conv1x1(Wt.float().numpy(), M, x.float().cpu().numpy().reshape(X.shape), None, False, g, want_scale=True)
+    ps = [alcs.alcs_packed_upload(alcs.alcs_pack(Wt.view(torch.int16).numpy().view(np.uint16), M, g, bf16=True), 0) for _ in range(2 if stack else 1)]
+    ys = [torch.empty(n, cout, h * h, dtype=torch.bfloat16, device="cuda") for _ in ps]
+    if stack:
+        for p in ps:
+            alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, dict(math_mode=4, producer_warps=8))
+        s = alcs.alcs_stack_create([dict(w=p, x=x, y=y, n=n, h=h, wd=h, bias=None, flags=0) for p, y in zip(ps, ys)], 0)
+        alcs.alcs_stack_tune(s, 1, st)
+        alcs.alcs_stack_run(s, st)
+        assert all(alcs.alcs_stack_layer_cfg(s, i)["producer_warps"] == 4 for i in range(2))
+    else:
+        alcs.alcs_spconv1x1_tune(ps[0], x, ys[0], n, h, h, None, 0, st)
+    torch.cuda.synchronize()
+    for p, y in zip(ps, ys):
+        cfg = alcs.alcs_spconv1x1_plan(p, n, h, h)
+        assert (cfg["math_mode"], cfg["producer_warps"]) == (4, 4)
+        assert (np.abs(y.float().cpu().numpy() - Yref) <= TOL["f32"] * A + 2.0 ** -8 * np.abs(Yref)).all()
