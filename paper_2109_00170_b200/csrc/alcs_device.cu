@@ -323,6 +323,7 @@ constexpr long long kGatherImages = 64;
 struct CallShape {
     int n, oh, ow, h, wd, stride = 1;
     bool residual = false;
+    bool y32 = false;       // fp32 output of 16-bit operands
     int images() const { return std::max(1, n); }
     int hw() const { return oh * ow; }
     long long q() const { return (long long)images() * hw(); }
@@ -335,11 +336,14 @@ alcs::TcProblem tc_problem(const void* x, void* y, int n, int h, int wd, const f
     return {x, y, bias, residual, n, h, wd, h_in, wd_in, stride, 0, k, k, flags};
 }
 
+// A pointwise layer of n images of h x wd pixels.
+CallShape pointwise(int n, int h, int wd, unsigned flags) { return {n, h, wd, h, wd, 1, false, (flags & ALCS_Y_F32) != 0}; }
+
 // (for estimates: no buffers, any address for a residual)
 alcs::TcProblem tc_problem(const CallShape& c)
 {
     static const char some = 0;
-    return tc_problem(nullptr, nullptr, c.images(), c.oh, c.ow, nullptr, 0, c.residual ? &some : nullptr, c.stride, c.h, c.wd);
+    return tc_problem(nullptr, nullptr, c.images(), c.oh, c.ow, nullptr, c.y32 ? ALCS_Y_F32 : 0, c.residual ? &some : nullptr, c.stride, c.h, c.wd);
 }
 
 // Can the tcgen05 kernel take the layer (whatever the channels per tile)?  A strided one: rows of 4-byte copies only, as
@@ -1441,7 +1445,7 @@ ALCS_API int alcs_spconv1x1_cfg(const alcs_packed* w, const void* x, void* y, in
     if (rc) return rc;
     if (q == 0) return ALCS_OK;
     Plan plan;
-    const CallShape shape{n, h, wd, h, wd};
+    const CallShape shape = pointwise(n, h, wd, flags);
     rc = resolve_plan(w, shape, flags, cfg, &plan);
     if (rc) return rc;
     rc = launch_plan(w, plan, x, y, n, h, wd, bias, flags, static_cast<cudaStream_t>(cuda_stream));
@@ -1482,7 +1486,7 @@ ALCS_API int alcs_spconv1x1_ex(const alcs_packed* w, const void* x, void* y, int
         if (rb < yend && yb < rend) return ALCS_ERR_INVALID_ARG;     // the residual may not overlap y
     }
     Plan plan;
-    const CallShape shape{n, oh, ow, h, wd, stride, residual != nullptr};
+    const CallShape shape{n, oh, ow, h, wd, stride, residual != nullptr, (flags & ALCS_Y_F32) != 0};
     rc = resolve_plan(w, shape, flags, cfg, &plan);
     if (rc) return rc;
     auto launch = [&] { return launch_plan(w, plan, x, y, n, oh, ow, bias, flags, static_cast<cudaStream_t>(cuda_stream), nullptr, 0, residual, stride, h, wd); };
@@ -1502,9 +1506,9 @@ ALCS_API int alcs_spconv1x1_plan(const alcs_packed* w, int n, int h, int wd, uns
     const long long q = (long long)n * h * wd;
     if ((long long)h * wd > (1ll << 30) || q > (1ll << 30)) return ALCS_ERR_SHAPE;
     Plan plan;
-    const int rc = resolve_plan(w, {n, h, wd, h, wd}, flags, nullptr, &plan);
+    const int rc = resolve_plan(w, pointwise(n, h, wd, flags), flags, nullptr, &plan);
     if (rc) return rc;
-    plan_to_cfg(w, {n, h, wd, h, wd}, plan, out);
+    plan_to_cfg(w, pointwise(n, h, wd, flags), plan, out);
     return ALCS_OK;
 }
 
@@ -1521,7 +1525,7 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const alcs::TcForms forms = alcs::tc_forms(w);
     std::vector<Plan> all;
-    rc = enumerate_plans(w, {n, h, wd, h, wd}, all);
+    rc = enumerate_plans(w, pointwise(n, h, wd, flags), all);
     if (rc) return rc;
     const size_t max_try = 1200;
     if (all.size() > max_try) all.resize(max_try);
@@ -1592,7 +1596,7 @@ ALCS_API int alcs_spconv1x1_tune(alcs_packed* w, const void* x, void* y, int n, 
     if (e != cudaSuccess) { alcs::set_cuda_error_text(cudaGetErrorString(e)); return ALCS_ERR_CUDA; }
     if (best_i < 0) return ALCS_ERR_CUDA;
     alcs_launch_cfg c;
-    plan_to_cfg(w, {n, h, wd, h, wd}, all[best_i], &c);
+    plan_to_cfg(w, pointwise(n, h, wd, flags), all[best_i], &c);
     all[best_i].cost = 1e-3 * best_ms;
     {
         std::lock_guard<std::mutex> lk(w->mu);
@@ -1631,10 +1635,10 @@ ALCS_API int alcs_spconv1x1_set_cfg(alcs_packed* w, int n, int h, int wd, unsign
     const long long q = (long long)n * h * wd;
     if ((long long)h * wd > (1ll << 30) || q > (1ll << 30)) return ALCS_ERR_SHAPE;
     Plan plan;
-    const int rc = cfg_to_plan(w, {n, h, wd, h, wd}, cfg, &plan);
+    const int rc = cfg_to_plan(w, pointwise(n, h, wd, flags), cfg, &plan);
     if (rc) return rc;
     alcs_launch_cfg full;
-    plan_to_cfg(w, {n, h, wd, h, wd}, plan, &full);
+    plan_to_cfg(w, pointwise(n, h, wd, flags), plan, &full);
     std::lock_guard<std::mutex> lk(w->mu);
     const alcs::ShapeKey key{n, h, wd, flags};
     w->tuned[key] = full;
@@ -1776,7 +1780,7 @@ bool independent(const LayerExtents& a, const LayerExtents& b)
 CallShape call_shape(const alcs_stack::Item& it)
 {
     const alcs_layer& L = it.layer;
-    return {L.n, it.oh, it.ow, L.h, L.wd, L.stride > 1 ? L.stride : 1, L.residual != nullptr};
+    return {L.n, it.oh, it.ow, L.h, L.wd, L.stride > 1 ? L.stride : 1, L.residual != nullptr, (L.flags & ALCS_Y_F32) != 0};
 }
 
 alcs::TcProblem tc_problem(const alcs_stack::Item& it)

@@ -495,6 +495,13 @@ double store_us(const alcs_packed* w, const TcProblem& p, int n, bool sorted)
     return f.store + f.store_n * n * std::max(sorted ? f.sorted : 1.0, p.res ? f.res : 1.0);
 }
 
+// X, Y and the residual, once.
+double layer_bytes(const alcs_packed* w, const TcProblem& p)
+{
+    const double q = (double)std::max(1, p.n) * p.oh * p.ow, y_elt = (p.flags & ALCS_Y_F32) ? 4.0 : (double)w->elt();
+    return q * (w->cin * (double)w->elt() + w->cout * y_elt * (p.res ? 2.0 : 1.0));
+}
+
 // Copy instructions of a warp for one block of 16 channels of the widest patch.  (Of an aligned X: no estimate depends on
 // where X starts.)
 double patch_copies(const alcs_packed* w, TcProblem p)
@@ -595,7 +602,7 @@ double tc_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms)
     }
     const double rounds = std::ceil(px * g.k16.size() / sms);
     const double main = std::max(rounds * sum / g.k16.size(), longest);
-    const double bytes = (double)q * (w->cin + w->cout * (p.res ? 2.0 : 1.0)) * w->elt();
+    const double bytes = layer_bytes(w, p);
     if (p.kh) return std::max(kPatchRamp + main + kPatchFirst * std::min(k_max, 4), kPatchRamp + bytes / kBytesPerUs);
     const double first = f.first[kind] * std::min(k_max, tc_kc(w->dt) / 16);
     return std::max(f.ramp + main + first + f.tail * store_us(w, p, n, g.sorted), f.ramp + bytes / kBytesPerUs);
@@ -636,7 +643,7 @@ double tc16_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms, i
         const double us = 2.3 + (raw ? 3.0 : 0.0) + std::max(rounds * sum / k16.size(), longest) + 1.2 * std::min(longest, 1.25 + px / 128.0 * 0.7);
         if (!*pixels || us < best * 0.98) { best = us; *pixels = px; }
     }
-    const double bytes = (double)q * (w->cin + w->cout * (p.res ? 2.0 : 1.0)) * w->elt();
+    const double bytes = layer_bytes(w, p);
     return std::max(best, 2.0 + bytes / kBytesPerUs);
 }
 
