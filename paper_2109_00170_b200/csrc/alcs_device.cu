@@ -374,20 +374,33 @@ Plan tc_plan_on(const alcs_packed* w, int n, const CallShape& c, int sms, int pi
     return p;
 }
 
-// The one that is expected to be faster.  Its estimate has to be clearly
-// lower for alcs_tc16.cu where rows must be picked apart (43 x 780 -> 139 @7 with a residual: 27 us where 17 were expected).
-Plan tc_plan(const alcs_packed* w, int n, const CallShape& c, int sms)
+// Of these channels per tile, the plan that is expected to be the fastest; the two kernels are compared at the best of their own.
+// Rows that alcs_tc16.cu picks apart have to promise 30 %: its estimate is 19 % off there (median), and no measure of the shape, output
+// channels least of all, tells the layers that gain from those that don't.  200 layers of random shapes with such rows, against
+// alcs_tc.cu alone: 31 chosen, 1.05 times as fast (geometric mean over all), none more than 4 % slower; at 20 %, 52 chosen, 1.06,
+// six slower by up to 29 %.  Rows copied as they are, 5 %: 80 layers, 50 chosen, 1.28, one slower (7 %).
+// against: what the staged kernels have to beat, the estimate of alcs_tc.cu where rows are picked apart (156 -> 43 @7, batch 11: 16 us
+// where 9 are expected, 12 staged).
+Plan tc_best(const alcs_packed* w, const int* n, int count, const CallShape& c, int sms, double* against = nullptr)
 {
-    Plan p = tc_plan_on(w, n, c, sms, 0);
-    if (tc16_ok(w, c)) {
-        Plan other = tc_plan_on(w, n, c, sms, kAnyPixels);
-        const bool direct = (size_t)c.hw() * w->elt() % 8 == 0;
-        if (other.cost * (direct ? 1.05 : 1.3) < p.cost) {
-            if (!direct) other.cost = p.cost;        // (the staged kernels stay where they were chosen: 156 -> 43 @7, batch 11: 12 us, not 16)
-            p = other;
+    auto best_on = [&](int pixels) {
+        Plan best = tc_plan_on(w, n[0], c, sms, pixels);
+        for (int i = 1; i < count; ++i) {
+            const Plan p = tc_plan_on(w, n[i], c, sms, pixels);
+            if (p.cost < best.cost) best = p;
         }
+        return best;
+    };
+    Plan best = best_on(0);
+    if (against) *against = best.cost;
+    if (!tc16_ok(w, c)) return best;
+    const bool direct = (size_t)c.hw() * w->elt() % 8 == 0;
+    const Plan other = best_on(kAnyPixels);
+    if (other.cost * (direct ? 1.05 : 1.3) < best.cost) {
+        best = other;
+        if (against && direct) *against = best.cost;
     }
-    return p;
+    return best;
 }
 
 // What a tuner compares with n output channels per tile: both kernels, and of alcs_tc16.cu a few heights beside the one that is expected to
@@ -414,19 +427,6 @@ int tc_widths(const alcs_packed* w, int (&n)[8])
         if (!count || v != n[count - 1]) n[count++] = v;
     }
     return count;
-}
-
-template <typename F>
-Plan tc_best(const alcs_packed* w, F of_width)
-{
-    int n[8];
-    const int count = tc_widths(w, n);
-    Plan best = of_width(n[0]);
-    for (int i = 1; i < count; ++i) {
-        const Plan p = of_width(n[i]);
-        if (p.cost < best.cost) best = p;
-    }
-    return best;
 }
 
 // What the planner's own choice among the staged kernels takes, in microseconds, without listing their configurations
@@ -682,19 +682,23 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
     const bool tc = (!c || c->math_mode == 4) && tc_ok(w, shape);
     if (c && c->math_mode == 4) {       // the tcgen05 kernel as asked for: row_groups channel tiles
         if (!tc) return ALCS_ERR_UNSUPPORTED;
+        int n[8], count = tc_widths(w, n);
+        if (c->row_groups) {
+            const int tiles = std::max(1, c->row_groups);
+            n[0] = ((w->cout + tiles - 1) / tiles + 15) / 16 * 16;
+            count = 1;
+            if (n[0] > alcs::kTcMaxN) return ALCS_ERR_UNSUPPORTED;
+        }
         const int named = tc16_ok(w, shape) ? c->producer_warps : 0;       // (the others have one kernel)
-        auto of_width = [&](int n) {
-            return named == kTcProducers ? tc_plan_on(w, n, shape, di.sms, 0)
-                 : named == kTc16Producers ? tc_plan_on(w, n, shape, di.sms, c->pixels_per_lane >= 32 ? c->pixels_per_lane : kAnyPixels)
-                 : tc_plan(w, n, shape, di.sms);
-        };
-        if (!c->row_groups) {
-            *out = tc_best(w, of_width);
+        if (named != kTcProducers && named != kTc16Producers) {
+            *out = tc_best(w, n, count, shape, di.sms);
             return ALCS_OK;
         }
-        const int tiles = std::max(1, c->row_groups), n = ((w->cout + tiles - 1) / tiles + 15) / 16 * 16;
-        if (n > alcs::kTcMaxN) return ALCS_ERR_UNSUPPORTED;
-        *out = of_width(n);
+        const int pixels = named == kTcProducers ? 0 : c->pixels_per_lane >= 32 ? c->pixels_per_lane : kAnyPixels;
+        for (int i = 0; i < count; ++i) {
+            const Plan p = tc_plan_on(w, n[i], shape, di.sms, pixels);
+            if (!i || p.cost < out->cost) *out = p;
+        }
         return ALCS_OK;
     }
     if (!c) {
@@ -704,25 +708,25 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
         // rougher one, most of all for long calls (512 -> 512 at 14 x 14, batch 256, 10 % kept: 252 us where 100 were
         // expected, 120 dense), so those have to promise more.  2048 -> 2048 at 7 x 7, batch 32, 5 % kept: 92 us dense, 49.
         Plan best;
-        best.cost = 1e30;
+        double against = best.cost = 1e30;
         if (tc) {
             const alcs::TcForms forms = alcs::tc_forms(w);
-            int n[8];
-            const int count = tc_widths(w, n);
-            for (int i = 0; i < count; ++i) {
-                if (!alcs::tc_form_free(w, forms, {n[i], 0, 0})) continue;
-                const Plan p = tc_plan(w, n[i], shape, di.sms);
-                if (p.cost < best.cost) best = p;
-            }
+            int n[8], count = 0;
+            for (int i = 0, all = tc_widths(w, n); i < all; ++i)
+                if (alcs::tc_form_free(w, forms, {n[i], 0, 0})) n[count++] = n[i];
+            if (count) best = tc_best(w, n, count, shape, di.sms, &against);
         }
         if (allow_small && hw > 0 && shape.images() <= kGatherImages)
             for (int p = 8; p >= 2; p /= 2)
                 for (int ks = 4; ks <= 16; ks *= 2) {
                     Plan g;
-                    if (gather_plan(w, shape.images(), hw, p, ks, di, &g) && g.cost < best.cost) best = g;
+                    if (gather_plan(w, shape.images(), hw, p, ks, di, &g) && g.cost < best.cost) {
+                        best = g;
+                        against = g.cost;
+                    }
                 }
         const double staged = 1e-6 * staged_us(w, shape, di.sms);
-        if (staged * (best.cost < 100e-6 ? 1.15 : 1.5) < best.cost) {
+        if (staged * (against < 100e-6 ? 1.15 : 1.5) < against) {
             Plan p;
             rc = staged_best(w, shape, &p);
             if (rc && (rc != ALCS_ERR_UNSUPPORTED || best.cost >= 1e30)) return rc;

@@ -253,3 +253,17 @@ def test_planner_knows_the_output_type(alcs):
         cfg = alcs.alcs_stack_layer_cfg(s, 0)
         chosen.append(cfg["math_mode"] == 4 and cfg["producer_warps"] == 8)
     assert chosen == [True, False]
+
+
+@pytest.mark.parametrize("n,cin,cout,h,w,density", [(31, 173, 247, 11, 13, 0.335), (3, 145, 578, 21, 21, 0.426), (16, 128, 256, 28, 28, 0.3), (8, 256, 96, 14, 14, 0.4),
+                                                    (9, 64, 80, 7, 7, 0.4)])
+def test_planned_tiles_are_the_best_of_their_kernel(alcs, n, cin, cout, h, w, density):
+    """The width of the channel tiles follows from the estimate of the kernel that runs (217 images of 204 -> 115 channels @7x7 with a
+    residual: 27 us with the 48 channels that suit the other kernel, 17 with 115)."""
+    W, M, X, b = _case(8, n, cin, cout, h * w, 8, density)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, 8), 0)
+    plan = alcs.alcs_spconv1x1_plan(p, n, h, w)
+    if plan["math_mode"] == 4:
+        alcs.alcs_spconv1x1_set_cfg(p, n, h, w, 0, dict(math_mode=4, producer_warps=plan["producer_warps"]))
+        assert alcs.alcs_spconv1x1_plan(p, n, h, w) == plan
+    check_layer(alcs, W, M, X, b, True, 8, h=h, wd=w)
