@@ -381,6 +381,7 @@ Plan tc_plan_on(const alcs_packed* w, int n, const CallShape& c, int sms, int pi
 // six slower by up to 29 %.  Rows copied as they are, 5 %: 80 layers, 50 chosen, 1.28, one slower (7 %).
 // against: what the staged kernels have to beat, the estimate of alcs_tc.cu where rows are picked apart (156 -> 43 @7, batch 11: 16 us
 // where 9 are expected, 12 staged).
+constexpr double kRawMargin = 1.3, kDirectMargin = 1.05;
 Plan tc_best(const alcs_packed* w, const int* n, int count, const CallShape& c, int sms, double* against = nullptr)
 {
     auto best_on = [&](int pixels) {
@@ -396,7 +397,7 @@ Plan tc_best(const alcs_packed* w, const int* n, int count, const CallShape& c, 
     if (!tc16_ok(w, c)) return best;
     const bool direct = (size_t)c.hw() * w->elt() % 8 == 0;
     const Plan other = best_on(kAnyPixels);
-    if (other.cost * (direct ? 1.05 : 1.3) < best.cost) {
+    if (other.cost * (direct ? kDirectMargin : kRawMargin) < best.cost) {
         best = other;
         if (against && direct) *against = best.cost;
     }
@@ -411,7 +412,8 @@ void tc_plans(const alcs_packed* w, int n, const CallShape& c, int sms, std::vec
     if (!tc16_ok(w, c)) return;
     std::vector<int> px;
     for (int want : {kAnyPixels, alcs::kTc16Pixels, alcs::kTc16Pixels / 2, alcs::kTc16Pixels / 4}) {
-        const Plan p = tc_plan_on(w, n, c, sms, want);
+        Plan p = tc_plan_on(w, n, c, sms, want);
+        p.tc_named = true;
         if (std::find(px.begin(), px.end(), p.tc_px) != px.end()) continue;
         px.push_back(p.tc_px);
         out.push_back(p);
@@ -699,6 +701,7 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
             const Plan p = tc_plan_on(w, n[i], shape, di.sms, pixels);
             if (!i || p.cost < out->cost) *out = p;
         }
+        out->tc_named = true;
         return ALCS_OK;
     }
     if (!c) {
@@ -1010,10 +1013,23 @@ alcs::TcKey tc_key(const alcs_packed* w, const Plan& p, const alcs::TcProblem& p
     return {p.tc_n, k, k};
 }
 
+// Pixels per tile on alcs_tc16.cu (0: alcs_tc.cu) for a call with the X of `pr`.  A plan is made for rows that can be copied as they
+// are, where their length allows it; where X starts elsewhere they have to be picked apart, which the other kernel, whose
+// expanded weights are the same, is mostly the better one at: 80 layers with X on an odd multiple of 2 or 4 bytes, up to 6.2 times as
+// fast; by the rule for odd rows (tc_best) 14 of 55 stay here and none is slower than there.
+int tc_pixels(const alcs_packed* w, const Plan& p, const alcs::TcProblem& pr)
+{
+    if (!p.tc_px || p.tc_named || (size_t)pr.oh * pr.ow * w->elt() % 8 != 0 || alcs::tc16_direct(w, pr)) return p.tc_px;
+    DeviceInfo di;
+    int px;
+    if (device_info(w->device, &di)) return 0;
+    return alcs::tc16_layer_us(w, pr, p.tc_n, di.sms, 0, &px) * kRawMargin < alcs::tc_layer_us(w, pr, p.tc_n, di.sms) ? px : 0;
+}
+
 // Launch the tcgen05 kernel for one layer; strided layers run by patch staging.
 int launch_tc_plan(const alcs_packed* w, const Plan& p, alcs::TcProblem pr, cudaStream_t st)
 {
-    pr.pixels = p.tc_px;
+    pr.pixels = tc_pixels(w, p, pr);
     alcs::TcForm t;
     const int rc = alcs::tc_prepare(w, tc_key(w, p, pr), st, &t);
     return rc ? rc : alcs::tc_run(w, *t, pr, st);
@@ -1845,7 +1861,7 @@ void stack_merge(alcs_stack* s, MergeBy by = MergeBy::estimates)
                     for (size_t k = from; k < to; ++k) {
                         const alcs_stack::Item& it = s->items[k];
                         const alcs_packed* w = it.layer.w;
-                        const alcs::TcProblem pr = tc_problem(call_shape(it));
+                        const alcs::TcProblem pr = tc_problem(it);
                         int n[8], at = 0;
                         const int count = tc_widths(w, n);
                         while (at + 1 < count && n[at] > cap) ++at;
@@ -1879,7 +1895,7 @@ void stack_merge(alcs_stack* s, MergeBy by = MergeBy::estimates)
         if (by == MergeBy::one_launch || (by == MergeBy::estimates && one < best)) { best = one; choice = widths; choice_px = pixels; }
         // 16-bit operands: layers whose rows can be copied as they are on alcs_tc16.cu, a launch per sequence of layers of one kind
         // (several launches have to promise a tenth: the estimates are that good)
-        auto direct = [&](size_t k) { return (size_t)s->items[k].oh * s->items[k].ow * s->items[k].layer.w->elt() % 8 == 0; };
+        auto direct = [&](size_t k) { return alcs::tc16_direct(s->items[k].layer.w, tc_problem(s->items[k])); };
         if (by != MergeBy::one_launch && s->items[i].layer.w->dt != ALCS_F32) {
             double t = 0;
             int launches = 0;
@@ -2084,6 +2100,7 @@ ALCS_API int alcs_stack_create(const alcs_layer* layers, int n_layers, unsigned 
         int rc = check_conv_args(L.w, L.x, L.y, L.n, it.oh, it.ow, L.flags, &it.q);
         if (!rc) rc = check_device(L.w);
         if (!rc && it.q > 0) rc = resolve_plan(L.w, call_shape(it), L.flags, nullptr, &it.plan);
+        if (!rc && it.q > 0) it.plan.tc_px = tc_pixels(L.w, it.plan, tc_problem(it));
         if (rc) { delete s; return rc; }
         s->items.push_back(it);
     }
@@ -2296,6 +2313,7 @@ ALCS_API int alcs_stack_tune(alcs_stack* s, int passes, void* cuda_stream, doubl
         if (it.q == 0) continue;
         const alcs_layer& L = it.layer;
         alcs_launch_cfg c;
+        it.plan.tc_named = tc16_ok(L.w, call_shape(it));
         plan_to_cfg(L.w, call_shape(it), it.plan, &c);
         const alcs::ShapeKey key{L.n, it.oh, it.ow, key_flags(L.w, L.flags, call_shape(it))};
         std::lock_guard<std::mutex> lk(L.w->mu);
@@ -2395,7 +2413,7 @@ extern "C" ALCS_API int alcs_spconv1x1_noalloc(const alcs_packed* w, const void*
             const size_t row = (size_t)h * wd * w->elt();
             if (row % 16 != 0 && (size_t)n * w->cin * ((row + 15) / 16 * 16) > ALCS_NOALLOC_SCRATCH_BYTES) return ALCS_ERR_TOO_LARGE;
             alcs::TcProblem pr = tc_problem(x, y, n, h, wd, bias, flags, nullptr, 1, h, wd);
-            pr.pixels = plan.tc_px;
+            pr.pixels = tc_pixels(w, plan, pr);
             const alcs::TcPrep* t = plan.tc_n ? alcs::tc_find(w, tc_key(w, plan, pr)).get() : nullptr;
             if (!t) t = alcs::tc_any_pointwise(w);
             if (!t) return ALCS_ERR_STATE;

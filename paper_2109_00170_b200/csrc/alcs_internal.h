@@ -93,6 +93,7 @@ struct Plan {
     // the tcgen05 kernels: variant is -1, and
     int tc_n = 0;          // output channels per tile (0: not these kernels)
     int tc_px = 0;         // pixels per tile on alcs_tc16.cu (0: alcs_tc.cu)
+    bool tc_named = false; // a configuration or a tuner chose the kernel, whatever X a call has
 };
 
 // Key of the plan cache: the problem shape plus the requested configuration (all zero = automatic).

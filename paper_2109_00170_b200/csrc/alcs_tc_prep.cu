@@ -350,6 +350,23 @@ bool tc_whole_images(const alcs_packed* w, const TcProblem& p)
     return !p.kh && row % 16 != 0 && (elt == 4 || row % 4 != 0) && row <= kTcM * elt && w->cin % 16 == 0;
 }
 
+namespace {
+
+// Bytes of the widest piece (16 ... elt) of rows of `row` bytes that start at `at` that keeps to one row and to its alignment.
+int widest(size_t row, const void* at, int elt)
+{
+    int v = 16;
+    while (v > elt && (row % v || (uintptr_t)at % v)) v >>= 1;
+    return v;
+}
+
+// How alcs_tc16.cu copies X: 16 or 8 bytes at a time; less: rows fetched as they are.
+int x_piece(const alcs_packed* w, const TcProblem& p) { return widest((size_t)p.oh * p.ow * w->elt(), p.x, (int)w->elt()); }
+
+}  // namespace
+
+bool tc16_direct(const alcs_packed* w, const TcProblem& p) { return x_piece(w, p) >= 8; }
+
 // Rows fetched as they are: a tile's runs of consecutive pixels, of an image each, in whole 16-byte words.
 void tc16_raw(const TcProblem& p, int pixels, int* pitch, int* row)
 {
@@ -365,26 +382,25 @@ int tc16_raw_bytes(const TcProblem& p, int pixels)
     return kTc16Chunk * row;
 }
 
-// Pixels per tile that a layer can take, the most first.
-std::vector<int> tc16_tiles(const alcs_packed* w, const TcProblem& p, int k16_max)
+namespace {
+
+// The most pixels per tile that a layer can take.
+int tc16_most(const alcs_packed* w, const TcProblem& p, int k16_max)
 {
     int most = k16_max > kTc16Group ? kTc16Pixels / 2 : kTc16Pixels;
-    std::vector<int> px;
-    if ((size_t)p.oh * p.ow * w->elt() % 8 != 0) {
+    if (!tc16_direct(w, p)) {
         most = std::min(most, kTc16Raw);
         while (most > 32 && tc16_raw_bytes(p, most) > kTc16RawMost) most -= 32;
     }
-    for (; most >= 32; most -= 32) px.push_back(most);
-    return px;
+    return most;
 }
+
+}  // namespace
 
 // The most pixels per tile that are no more than `cap`.
 int tc16_capped(const alcs_packed* w, const TcProblem& p, int k16_max, int cap)
 {
-    const std::vector<int> px = tc16_tiles(w, p, k16_max);
-    for (int v : px)
-        if (v <= cap) return v;
-    return px.back();
+    return std::max(32, std::min(tc16_most(w, p, k16_max), cap / 32 * 32));
 }
 
 // UNSUPPORTED: beyond the kernel's 32-bit offsets, or rows that patch staging cannot copy (see tc_fits, tc_patch_fits).
@@ -415,21 +431,13 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
     y.n_px = 0;
     if (p.pixels) {
         const int e = (p.flags & ALCS_Y_F32) ? 4 : 2;
-        // the widest piece that keeps to one image and to its alignment
-        auto widest = [&](size_t row, const void* at, int least) {
-            int v = 16;
-            while (v > least && (row % v || (uintptr_t)at % v)) v >>= 1;
-            return v;
-        };
-        const size_t hw = (size_t)y.hw.d;
-        const int v = widest(hw * elt, p.x, elt);
+        const size_t row = (size_t)y.hw.d * e;
+        const int v = x_piece(w, p);
         y.vec_bytes = v >= 8 ? v : kTcRaw;
-        y.y_vec = widest(hw * e, p.y, e);
-        y.res_vec = p.res ? widest(hw * e, p.res, e) : 16;
-        y.ppt = t.k16_max > kTc16Group ? std::min(p.pixels, kTc16Pixels / 2) : p.pixels;
+        y.y_vec = widest(row, p.y, e);
+        y.res_vec = p.res ? widest(row, p.res, e) : 16;
+        y.ppt = tc16_capped(w, p, t.k16_max, p.pixels);      // (the weights, or an X that starts anywhere, may allow less than was planned)
         if (y.vec_bytes == kTcRaw) {
-            // (an X that does not start where its copies would have to takes fewer pixels per tile)
-            if (y.ppt > kTc16Raw || tc16_raw_bytes(p, y.ppt) > kTc16RawMost) y.ppt = 32;
             tc16_raw(p, y.ppt, &y.raw_pitch, &y.raw_row);
             y.raw_bytes = kTc16Chunk * y.raw_row;
         }
@@ -485,8 +493,8 @@ constexpr double kBytesPerUs = 7.0e6;
 int copy_kind(const alcs_packed* w, const TcProblem& p)
 {
     if (tc_whole_images(w, p)) return 4;
-    const size_t row = (size_t)p.oh * p.ow * w->elt();
-    return row % 16 == 0 ? 0 : w->dt == ALCS_F32 ? 3 : row % 8 == 0 ? 1 : row % 4 == 0 ? 2 : 3;
+    const int v = x_piece(w, p);
+    return v == 16 ? 0 : w->dt == ALCS_F32 || v < 4 ? 3 : v == 8 ? 1 : 2;
 }
 
 double store_us(const alcs_packed* w, const TcProblem& p, int n, bool sorted)
@@ -502,8 +510,7 @@ double layer_bytes(const alcs_packed* w, const TcProblem& p)
     return q * (w->cin * (double)w->elt() + w->cout * y_elt * (p.res ? 2.0 : 1.0));
 }
 
-// Copy instructions of a warp for one block of 16 channels of the widest patch.  (Of an aligned X: no estimate depends on
-// where X starts.)
+// Copy instructions of a warp for one block of 16 channels of the widest patch, of an aligned X.
 double patch_copies(const alcs_packed* w, TcProblem p)
 {
     p.x = nullptr;
@@ -613,11 +620,12 @@ double tc_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms)
 // 8, rows fetched as they are), or by its bytes; the stores of 128 pixels by their width.
 double tc16_item_us(const alcs_packed* w, const TcProblem& p, int n, int k16, int pixels)
 {
-    const size_t hw = (size_t)p.oh * p.ow, row = hw * w->elt(), e = (p.flags & ALCS_Y_F32) ? 4 : 2;
+    const size_t hw = (size_t)p.oh * p.ow, e = (p.flags & ALCS_Y_F32) ? 4 : 2;
+    const int v = x_piece(w, p);
     const double px = pixels, store_px[4] = {0.68 * e / 2.0, 0.96, 1.5, 2.14};
     const int width = hw * e % 16 == 0 ? 0 : hw * e % 8 == 0 ? 1 : hw * e % 4 == 0 ? 2 : 3;
     const double store = 1.25 + px / 128.0 * store_px[width] * (p.res ? 3.0 : 1.0);
-    double chunk = row % 16 == 0 ? 0.41 + 0.00027 * px : row % 8 == 0 ? 0.41 + 0.0024 * px : 2.6;
+    double chunk = v == 16 ? 0.41 + 0.00027 * px : v == 8 ? 0.41 + 0.0024 * px : 2.6;
     if (k16 * 16 < w->cin) chunk += 0.1;        // (a column list)
     chunk = std::max(chunk, 0.0024 * px + 0.0019 * n);
     return std::max((k16 + 3) / 4 * chunk, store);
@@ -628,10 +636,11 @@ double tc16_layer_us(const alcs_packed* w, const TcProblem& p, int n, int sms, i
     const std::vector<int> k16 = tc_tile_steps(w, p, n);
     const long long q = (long long)std::max(1, p.n) * p.oh * p.ow;
     const int k_max = k16.empty() ? 0 : *std::max_element(k16.begin(), k16.end());
-    const bool raw = (size_t)p.oh * p.ow * w->elt() % 8 != 0;
+    const bool raw = !tc16_direct(w, p);
     double best = 0;
     *pixels = 0;
-    for (int px : cap ? std::vector<int>{tc16_capped(w, p, k_max, cap)} : tc16_tiles(w, p, k_max)) {
+    const int most = cap ? tc16_capped(w, p, k_max, cap) : tc16_most(w, p, k_max);
+    for (int px = most; px >= (cap ? most : 32); px -= 32) {
         const double tiles = (double)((q + px - 1) / px);
         double sum = 0, longest = 0;
         for (int k : k16) {

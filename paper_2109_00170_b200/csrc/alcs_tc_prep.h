@@ -59,6 +59,7 @@ int tc_fill(const alcs_packed* w, const TcPrep& t, const TcProblem& p, TcLayer* 
 double tc_tile_us(const alcs_packed* w, const TcProblem& p, int n, int k16, bool list, bool sorted);
 std::vector<double> tc_tiles_us(const alcs_packed* w, const TcProblem& p, int n);        // of every channel tile, as tc_prepare would make them
 double tc_merged_item_us(int dt, int n, int k16);
+bool tc16_direct(const alcs_packed* w, const TcProblem& p);       // alcs_tc16.cu copies the rows of X to where they are multiplied
 // alcs_tc16.cu (16-bit operands, stride 1): of an item; of a layer on its own with the pixels per tile that take the least, or (cap) with the
 // most that are no more than `cap`; those.
 double tc16_item_us(const alcs_packed* w, const TcProblem& p, int n, int k16, int pixels);

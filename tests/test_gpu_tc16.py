@@ -267,3 +267,40 @@ def test_planned_tiles_are_the_best_of_their_kernel(alcs, n, cin, cout, h, w, de
         alcs.alcs_spconv1x1_set_cfg(p, n, h, w, 0, dict(math_mode=4, producer_warps=plan["producer_warps"]))
         assert alcs.alcs_spconv1x1_plan(p, n, h, w) == plan
     check_layer(alcs, W, M, X, b, True, 8, h=h, wd=w)
+
+
+def test_inputs_that_start_on_odd_words(alcs):
+    """A layer planned for rows copied as they are, whose X does not start where such copies can: 38 images of 78 -> 1300 channels @20x20 took
+    153 us with 32 pixels per tile on the kernel that then picks rows apart, 49 with 128, 25 on the other one."""
+    import torch
+    n, cin, cout, h, g = 38, 78, 1300, 20, 8
+    W, M, X, b = _case(12, n, cin, cout, h * h, g, 0.25)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    st, bd = torch.cuda.current_stream(), torch.from_numpy(b).cuda()
+    x = torch.zeros(X.size + 8, dtype=torch.float16, device="cuda")[2:2 + X.size]
+    x.copy_(torch.from_numpy(X).reshape(-1))
+    y = torch.empty(n, cout, h * h, dtype=torch.float16, device="cuda")
+    Yref, A = oracle.conv1x1(W, M, X, b, False, g, want_scale=True)
+    assert alcs.alcs_spconv1x1_plan(p, n, h, h)["producer_warps"] == 8
+    took = {}
+    for cfg in (None, dict(CFG, pixels_per_lane=256), dict(CFG, pixels_per_lane=128), dict(CFG, pixels_per_lane=32), dict(math_mode=4, producer_warps=4)):
+        for _ in range(3):
+            y.fill_(float("nan"))
+            alcs.alcs_spconv1x1(p, x, y, n, h, h, bd, 0, st, cfg)
+        a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            alcs.alcs_spconv1x1(p, x, y, n, h, h, bd, 0, st, cfg)
+        e.record()
+        torch.cuda.synchronize()
+        took[tuple(cfg.values()) if cfg else None] = a.elapsed_time(e)
+        assert_parity(y.cpu().numpy(), Yref, A, "f16")
+    times = list(took.values())
+    assert times[1] < 1.5 * times[2] < 1.5 * times[3] and times[0] < 1.3 * times[4], took
+    s = alcs.alcs_stack_create([dict(w=p, x=x, y=y, n=n, h=h, wd=h, bias=bd, flags=0)], 0)
+    assert alcs.alcs_stack_layer_cfg(s, 0)["producer_warps"] == 4
+    # without allocation, and in a captured graph
+    y.fill_(float("nan"))
+    alcs.alcs_spconv1x1_noalloc(p, x, y, n, h, h, bd, 0, st)
+    torch.cuda.synchronize()
+    assert_parity(y.cpu().numpy(), Yref, A, "f16")
