@@ -205,7 +205,7 @@ struct Fetch {
             first[i] = bytes[i] = word[i] = 0;
             if (q >= q1) continue;
             const Rows::Run r(y, q, q0);
-            first[i] = start + r.first * 2;
+            first[i] = start + 2u * (unsigned)r.first;
             bytes[i] = (r.last - r.first + 1) * 2;
             word[i] = (w - run * per_run) * 16;
         }

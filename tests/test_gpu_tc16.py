@@ -304,3 +304,24 @@ def test_inputs_that_start_on_odd_words(alcs):
     alcs.alcs_spconv1x1_noalloc(p, x, y, n, h, h, bd, 0, st)
     torch.cuda.synchronize()
     assert_parity(y.cpu().numpy(), Yref, A, "f16")
+
+
+def test_more_than_2_to_the_30_elements(alcs):
+    """Byte offsets of rows picked apart pass 2^31: the last images of 1.18e9 elements, against the same images by themselves."""
+    import torch
+    n, cin, cout, hw, g = 18000, 16, 8, 4097, 8
+    assert n * cin * hw > 2 ** 30
+    W, M, _, b = _case(2, 1, cin, cout, 8, g, 0.5)
+    p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+    st, bd = torch.cuda.current_stream(), torch.from_numpy(b).cuda()
+    x = torch.empty(n, cin, hw, dtype=torch.float16, device="cuda").uniform_(0, 1, generator=torch.Generator("cuda").manual_seed(1))
+    y = torch.empty(n, cout, hw, dtype=torch.float16, device="cuda")
+    alcs.alcs_spconv1x1(p, x, y, n, hw, 1, bd, 0, st, CFG)
+    for first in (0, n // 2, n - 3):
+        few = torch.empty(3, cout, hw, dtype=torch.float16, device="cuda")
+        alcs.alcs_spconv1x1(p, x[first:first + 3].clone(), few, 3, hw, 1, bd, 0, st, CFG)
+        torch.cuda.synchronize()
+        assert torch.equal(y[first:first + 3], few)
+    Yref, A = oracle.conv1x1(W, M, x[-3:].cpu().numpy(), b, False, g, want_scale=True)
+    assert_parity(few.cpu().numpy(), Yref, A, "f16")
+    assert alcs.alcs_packed_status(p) == 0
