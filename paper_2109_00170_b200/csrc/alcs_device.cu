@@ -1893,8 +1893,10 @@ void stack_merge(alcs_stack* s, MergeBy by = MergeBy::estimates)
         for (size_t k = i; k < end; ++k) best += s->items[k].plan.cost * 1e6;
         const double one = by == MergeBy::kernels ? 0 : together(i, end, false);
         if (by == MergeBy::one_launch || (by == MergeBy::estimates && one < best)) { best = one; choice = widths; choice_px = pixels; }
-        // 16-bit operands: layers whose rows can be copied as they are on alcs_tc16.cu, a launch per sequence of layers of one kind
-        // (several launches have to promise a tenth: the estimates are that good)
+        // 16-bit operands: layers whose rows can be copied as they are on alcs_tc16.cu, a launch per sequence of layers of one kind.
+        // Several launches have to promise a tenth, as the estimates favour them: of 80 stacks of pointwise layers (two networks, inputs of
+        // 160 to 288, batches of 1 to 48) 8 run so, 2 to 19 % faster than in one launch; were all of them to run so, others would
+        // gain up to 24 % and lose up to 43 %.
         auto direct = [&](size_t k) { return alcs::tc16_direct(s->items[k].layer.w, tc_problem(s->items[k])); };
         if (by != MergeBy::one_launch && s->items[i].layer.w->dt != ALCS_F32) {
             double t = 0;

@@ -682,7 +682,6 @@ int tc_finish(const alcs_packed* w, TcArgs<kTcMaxLayers>& a, bool patch)
         a.slot_bytes = tc16_weight_bytes(n);
         a.stage_bytes = tc16_stage_bytes(n, px);
         int room = std::min(smem, 227 * 1024) - kTc16Fixed;
-        a.raw_slots = a.raw_bytes = 0;
         for (int i = 0; i < a.n_layers; ++i)
             if (a.layer[i].vec_bytes == kTcRaw) a.raw_bytes = std::max(a.raw_bytes, (a.layer[i].raw_bytes + 127) / 128 * 128);
         if (a.raw_bytes) {      // two stages, then slots, as many as there is room for: what is in flight is there
