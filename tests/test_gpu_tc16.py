@@ -128,9 +128,16 @@ def test_infinite_and_nan_inputs_touch_kept_blocks_alone(alcs, h, cin):
     assert_parity(np.where(bad, 0, Y), np.where(bad, 0, Yref), A, "f16")
 
 
+def _kernels(alcs, s, count):
+    cfgs = [alcs.alcs_stack_layer_cfg(s, i) for i in range(count)]
+    assert all(c["math_mode"] == 4 for c in cfgs)
+    return [c["producer_warps"] for c in cfgs]
+
+
 @pytest.mark.parametrize("sizes", [[(64, 96, 14), (272, 40, 8), (32, 160, 28)], [(48, 64, 16), (100, 64, 7), (64, 32, 14)]])
+@pytest.mark.parametrize("kernels", [[8, 8, 8], [8, 4, 8], [4, 8, 8]])
 @pytest.mark.parametrize("graph", [False, True])
-def test_merged_stack(alcs, sizes, graph):
+def test_merged_stack(alcs, sizes, kernels, graph):
     """Layers of one launch, and layers of the two tensor-core kernels one behind the other."""
     import torch
     n, g = 6, 8
@@ -138,15 +145,85 @@ def test_merged_stack(alcs, sizes, graph):
     for i, (cin, cout, h) in enumerate(sizes):
         W, M, X, b = _case(100 + i, n, cin, cout, h * h, g, 0.4)
         p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+        alcs.alcs_spconv1x1_set_cfg(p, n, h, h, alcs.ALCS_RELU, dict(math_mode=4, producer_warps=kernels[i]))
         layers.append(dict(w=p, x=torch.from_numpy(X).cuda(), y=torch.full((n, cout, h * h), float("nan"), dtype=torch.float16, device="cuda"),
                            n=n, h=h, wd=h, bias=torch.from_numpy(b).cuda(), flags=alcs.ALCS_RELU))
         want.append(oracle.conv1x1(W, M, X, b, True, g, want_scale=True))
     s = alcs.alcs_stack_create(layers, alcs.ALCS_STACK_GRAPH if graph else 0)
+    assert _kernels(alcs, s, 3) == kernels
     for _ in range(2):
         alcs.alcs_stack_run(s, torch.cuda.current_stream())
     torch.cuda.synchronize()
     for L, (Yref, A) in zip(layers, want):
         assert_parity(L["y"].cpu().numpy(), Yref, A, "f16")
+        assert alcs.alcs_packed_status(L["w"]) == 0
+
+
+def test_stack_that_runs_as_two_launches(alcs):
+    """ResNet-50's pointwise layers at 224: the two of 7x7 images run on the other kernel, in a launch of their own."""
+    import torch
+    from alcs_workloads.layers import RESNET50_BOTTLENECK_PW
+    n, g, gen = 32, 8, torch.Generator("cuda").manual_seed(5)
+    layers, ws = [], []
+    for i, (cin, cout, h) in enumerate(RESNET50_BOTTLENECK_PW):
+        W, M, _, b = _case(200 + i, 1, cin, cout, 1, g, 0.25)
+        p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
+        x = torch.randn(n, cin, h * h, generator=gen, device="cuda").abs_().half()
+        layers.append(dict(w=p, x=x, y=torch.full((n, cout, h * h), float("nan"), dtype=torch.float16, device="cuda"), n=n, h=h, wd=h,
+                           bias=torch.from_numpy(b).cuda(), flags=0))
+        ws.append(torch.from_numpy(W.astype(np.float64) * np.repeat(M, g, axis=0)[:cout]).cuda())
+    s = alcs.alcs_stack_create(layers, 0)
+    assert _kernels(alcs, s, len(layers)) == [4 if h == 7 else 8 for _, _, h in RESNET50_BOTTLENECK_PW]
+    alcs.alcs_stack_run(s, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    for L, W in zip(layers, ws):
+        x, b = L["x"].double(), L["bias"].double()[:, None]
+        Yref, A = W @ x + b, W.abs() @ x + b.abs()
+        assert ((L["y"].double() - Yref).abs() <= TOL["f32"] * A + 2.0 ** -11 * Yref.abs() + 2.0 ** -25).all()
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+def test_merged_launch_of_unlike_layers(alcs, bf16):
+    """One launch of the kernel with a residual, fp32 output, an X that starts on an odd element and infinite and NaN inputs, in different
+    layers: each keeps to itself."""
+    import torch
+    n, g, dt = 5, 8, torch.bfloat16 if bf16 else torch.float16
+    kinds = ["plain", "residual", "y_f32", "odd start", "not finite", "y_f32 residual", "plain"]
+    sizes = [(64, 96, 14), (272, 136, 8), (32, 160, 28), (100, 72, 10), (300, 136, 14), (64, 40, 12), (48, 64, 16)]
+    layers, refs, st = [], [], torch.cuda.current_stream()
+    for i, (kind, (cin, cout, h)) in enumerate(zip(kinds, sizes)):
+        W, M, X, b = _case(300 + i, n, cin, cout, h * h, g, 0.4, np.float32)
+        Wt = torch.from_numpy(W).to(dt)
+        p = alcs.alcs_pack(Wt.view(torch.int16).numpy().view(np.uint16), M, g, bf16=True) if bf16 else alcs.alcs_pack(Wt.numpy(), M, g)
+        alcs.alcs_packed_upload(p, 0)
+        flags = alcs.ALCS_Y_F32 if "y_f32" in kind else 0
+        alcs.alcs_spconv1x1_set_cfg(p, n, h, h, flags, CFG)
+        off = 1 if kind == "odd start" else 0
+        x = torch.zeros(X.size + 8, dtype=dt, device="cuda")[off:off + X.size].view(X.shape)
+        x.copy_(torch.from_numpy(X))
+        if kind == "not finite":
+            x[1, 5, 3], x[2, 7, h * h - 1] = float("inf"), float("nan")
+        ydt = torch.float32 if flags else dt
+        res = torch.from_numpy(rng.normal(9, i, n * cout * h * h).astype(np.float32)).cuda().to(ydt).view(n, cout, h * h) if "residual" in kind else None
+        layers.append(dict(w=p, x=x, y=torch.full((n, cout, h * h), 7.0, dtype=ydt, device="cuda"), n=n, h=h, wd=h, bias=torch.from_numpy(b).cuda(),
+                           flags=flags, residual=res))
+        refs.append((Wt.double().cuda() * torch.from_numpy(np.repeat(M, g, axis=0)[:cout]).cuda(), M))
+    s = alcs.alcs_stack_create(layers, 0)
+    assert _kernels(alcs, s, len(layers)) == [8] * len(layers)
+    alcs.alcs_stack_run(s, st)
+    torch.cuda.synchronize()
+    for kind, L, (W, M) in zip(kinds, layers, refs):
+        x, b, bad = L["x"].double(), L["bias"].double()[:, None], torch.zeros_like(L["y"], dtype=torch.bool)
+        if kind == "not finite":
+            kept = torch.from_numpy(np.repeat(M, g, axis=0)[:W.shape[0]]).cuda().bool()
+            bad[1, :, 3], bad[2, :, -1] = kept[:, 5] & (W[:, 5] != 0), kept[:, 7]
+            x = torch.where(x.isfinite(), x, torch.zeros_like(x))
+        Yref, A = W @ x + b, W.abs() @ x.abs() + b.abs()
+        if L["residual"] is not None:
+            Yref, A = Yref + L["residual"].double(), A + L["residual"].double().abs()
+        y, unit = L["y"].double(), 0.0 if L["y"].dtype == torch.float32 else 2.0 ** -8 if bf16 else 2.0 ** -11
+        assert not y[bad].isfinite().any() and (bad.any() or kind != "not finite")
+        assert ((y - Yref).abs() <= TOL["f32"] * A + unit * Yref.abs() + 2.0 ** -25)[~bad].all(), kind
         assert alcs.alcs_packed_status(L["w"]) == 0
 
 
