@@ -530,8 +530,8 @@ typedef struct {
  * the STACK owns (allocated by alcs_stack_create with the layers' device current, sized for its
  * largest such layer, released by alcs_stack_destroy): nothing a captured graph refers to is freed
  * or moved by later alcs_spconv1x1 calls with the same packed matrices, at any batch size.
- * Consecutive layers on the fifth-generation tensor-core kernel (math_mode 4, up to 16 of one element type) none of
- * which reads or writes what another one writes run as ONE launch, whose items (a tile of pixels x a channel tile) are
+ * Consecutive layers on one of the fifth-generation tensor-core kernels (math_mode 4, up to 16 of one element type) none of
+ * which reads or writes what another one writes run as ONE launch per kernel, whose items (a tile of pixels x a channel tile) are
  * dealt to the SMs by a list made when the stack is created; layers that do touch each other's buffers keep
  * their order.  Two runs
  * of the same stack must not overlap on the GPU (they share that scratch and the outputs).

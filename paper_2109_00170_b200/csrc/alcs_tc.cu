@@ -1,5 +1,6 @@
-// Convolution on the fifth-generation tensor cores (tcgen05), sm_100a: fp32 operands, k x k kernels and strides, and small images
-// of 16-bit operands that are staged whole (the other 16-bit layers: alcs_tc16.cu).
+// Convolution on the fifth-generation tensor cores (tcgen05), sm_100a: fp32 operands, k x k kernels, strides, and those 16-bit
+// layers at stride 1 that alcs_tc16.cu is not expected to be faster at (small images staged whole, most rows of odd length, layers
+// of few pixels: half of the layers of random shape).
 //
 // A work item is (128 output pixels) x (n output channels).  The item's pruned weights are expanded
 // to a dense [columns][n] tile (columns that no row of the tile keeps are left out), so that the item
@@ -492,8 +493,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 if constexpr (kEarly) {
                     // The values are read, and their slot is given back, while the buffer they go to is still being multiplied: what is
                     // left between the end of that and the next multiplication is the split and its stores (917 cycles a chunk
-                    // instead of 1,390; 3x3 layers of ResNet-18, batch 32: 354 -> 341 us, 512 -> 512 @14 with skewed rows, batch
-                    // 256: 132.3 -> 130.6 us.  In merged launches, whose items are short, it is 3 % slower.)
+                    // instead of 1,390; 3x3 layers of ResNet-18, batch 32: 354 -> 341 us; pointwise layers gain 1 %, about the noise.
+                    // In merged launches, whose items are short, it is 3 % slower.)
                     raw v[16];
                     if (!PATCH) ok = __all_sync(0xffffffffu, bar_wait(x_full + 8 * slot, xph));
                     if (ok && s0_ < ns) load(s0_, v);

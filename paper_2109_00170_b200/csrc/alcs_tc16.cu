@@ -19,6 +19,9 @@
 // 256 columns per accumulator, as the tensor core cuts off when it adds to its fp32 accumulator; longer sums are added up in
 // registers with round to nearest.
 //
+// Registers: 64 per thread at launch (see kEpiRegs), of which the compiler spills 42 bytes (66 in merged launches); nothing says that
+// it costs time, and no split of the block's registers among the roles leaves more for all of them.
+//
 // Roles (32 warps, one thread block per SM, persistent over items):
 //   warps 0-15   epilogue: bias, residual, activation, stores, while the next item is multiplied (two accumulators); a warp takes
 //                32 channels and a half or a quarter of the pixels
