@@ -189,8 +189,8 @@ ALCS_API void alcs_packed_free(alcs_packed* p);
  *                     (once per packed matrix, on the device) to dense weight tiles and multiplied with 128-pixel
  *                     tiles of X; fp32 operands are split exactly into three bfloat16 parts each.  Only row_groups
  *                     (the number of channel tiles, each of at most 128 channels), producer_warps and, with producer_warps 8,
- *                     pixels_per_lane apply (pixels per tile, 32 to 256: the most multiples of 32 that are no more and that the layer
- *                     can take; less than 32: the library chooses); no scratch is used.  Outputs of
+ *                     warps apply (32 pixels of a tile each, 1 to 8: as many as that or as the layer can take; 0: the library
+ *                     chooses); no scratch is used.  Outputs of
  *                     pixels with infinite or NaN inputs are computed from the storage format instead, so that such values
  *                     reach the channels that keep a block of theirs and no others, as with the other kernels (slowly); fp32
  *                     matrices that keep an infinite or NaN weight are refused (UNSUPPORTED)

@@ -358,8 +358,8 @@ bool tc_ok(const alcs_packed* w, const CallShape& c)
 
 // alcs_tc16.cu takes 16-bit operands at stride 1.
 bool tc16_ok(const alcs_packed* w, const CallShape& c) { return w->dt != ALCS_F32 && c.stride == 1; }
-// producer_warps of a configuration that names the kernel of such a layer: alcs_tc.cu, alcs_tc16.cu.  Its pixels_per_lane are
-// pixels per tile then (a lane of the accumulator is a channel).
+// producer_warps of a configuration that names the kernel of such a layer: alcs_tc.cu, alcs_tc16.cu.  Its `warps` are 32 pixels of the
+// tile each then (with pixels_per_lane 1, as the staged kernels count).
 constexpr int kTcProducers = 4, kTc16Producers = 8;
 
 // The tcgen05 kernel that is named with n output channels per tile as a plan: alcs_tc.cu, or alcs_tc16.cu with the most pixels per tile
@@ -652,7 +652,8 @@ void plan_to_cfg(const alcs_packed* w, const CallShape& shape, const Plan& p, al
     }
     if (p.tc_n) {
         std::memset(c, 0, sizeof *c);
-        c->pixels_per_lane = p.tc_px ? p.tc_px : 1;
+        c->pixels_per_lane = 1;
+        c->warps = p.tc_px / 32;
         c->math_mode = 4;
         c->row_groups = p.n_rg;
         c->producer_warps = p.tc_px ? kTc16Producers : tc16_ok(w, shape) ? kTcProducers : 0;
@@ -696,7 +697,7 @@ int cfg_to_plan(const alcs_packed* w, const CallShape& shape, const alcs_launch_
             *out = tc_best(w, n, count, shape, di.sms);
             return ALCS_OK;
         }
-        const int pixels = named == kTcProducers ? 0 : c->pixels_per_lane >= 32 ? c->pixels_per_lane : kAnyPixels;
+        const int pixels = named == kTcProducers ? 0 : c->warps > 0 ? 32 * std::min(c->warps, alcs::kTc16Pixels / 32) : kAnyPixels;
         for (int i = 0; i < count; ++i) {
             const Plan p = tc_plan_on(w, n[i], shape, di.sms, pixels);
             if (!i || p.cost < out->cost) *out = p;

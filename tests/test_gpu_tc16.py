@@ -234,16 +234,19 @@ def test_configurations_say_what_runs(alcs, cin, h):
     W, M, X, b = _case(cin + h, n, cin, cout, h * h, g, 0.4)
     p = alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0)
     most = (256 if h == 14 else 128) if cin == 64 else 128
-    asked = [(0, 0), (4, 0), (8, 0), (8, 1)] + [(8, px) for px in (32, 64, 96, 100, 128, 256, 1000)]
-    for producers, px in asked:
+    asked = [(0, 0), (4, 0), (8, 0), (8, -1)] + [(8, warps) for warps in (1, 2, 3, 4, 8, 100)]
+    for producers, warps in asked:
         for tiles in (0, 2, 5):
-            cfg = dict(math_mode=4, producer_warps=producers, pixels_per_lane=px, row_groups=tiles)
+            cfg = dict(math_mode=4, producer_warps=producers, pixels_per_lane=1, warps=warps, row_groups=tiles)
             alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, cfg)
             plan = alcs.alcs_spconv1x1_plan(p, n, h, h)
             assert plan["math_mode"] == 4 and (not tiles or plan["row_groups"] == tiles)
             assert plan["producer_warps"] == producers if producers else plan["producer_warps"] in (4, 8)
             if producers == 8:
-                assert plan["pixels_per_lane"] in ([min(px // 32 * 32, most)] if px >= 32 else range(32, most + 1, 32))
+                assert plan["warps"] in ([min(warps, most // 32)] if warps > 0 else range(1, most // 32 + 1))
+            else:
+                assert plan["warps"] == 0 or plan["producer_warps"] == 8
+            assert plan["pixels_per_lane"] == 1
             alcs.alcs_spconv1x1_set_cfg(p, n, h, h, 0, plan)
             assert alcs.alcs_spconv1x1_plan(p, n, h, h) == plan
             check_layer(alcs, W, M, X, b, False, g, cfg=plan, h=h, wd=h, packed=p)
@@ -251,8 +254,8 @@ def test_configurations_say_what_runs(alcs, cin, h):
     import torch
     x, ys = torch.from_numpy(X).cuda(), [torch.empty(n, cout, h * h, dtype=torch.float16, device="cuda") for _ in range(3)]
     qs = [alcs.alcs_packed_upload(alcs.alcs_pack(W, M, g), 0) for _ in range(3)]
-    want = [dict(math_mode=4, producer_warps=8, pixels_per_lane=64, row_groups=2), dict(math_mode=4, producer_warps=4, pixels_per_lane=1, row_groups=3),
-            dict(math_mode=4, producer_warps=8, pixels_per_lane=32, row_groups=9)]
+    want = [dict(math_mode=4, producer_warps=8, warps=2, row_groups=2), dict(math_mode=4, producer_warps=4, warps=0, row_groups=3),
+            dict(math_mode=4, producer_warps=8, warps=1, row_groups=9)]
     for q, cfg in zip(qs, want):
         alcs.alcs_spconv1x1_set_cfg(q, n, h, h, 0, cfg)
     s = alcs.alcs_stack_create([dict(w=q, x=x, y=y, n=n, h=h, wd=h, bias=None, flags=0) for q, y in zip(qs, ys)], 0)
@@ -360,7 +363,7 @@ def test_inputs_that_start_on_odd_words(alcs):
     Yref, A = oracle.conv1x1(W, M, X, b, False, g, want_scale=True)
     assert alcs.alcs_spconv1x1_plan(p, n, h, h)["producer_warps"] == 8
     took = {}
-    for cfg in (None, dict(CFG, pixels_per_lane=256), dict(CFG, pixels_per_lane=128), dict(CFG, pixels_per_lane=32), dict(math_mode=4, producer_warps=4)):
+    for cfg in (None, dict(CFG, warps=8), dict(CFG, warps=4), dict(CFG, warps=1), dict(math_mode=4, producer_warps=4)):
         for _ in range(3):
             y.fill_(float("nan"))
             alcs.alcs_spconv1x1(p, x, y, n, h, h, bd, 0, st, cfg)
