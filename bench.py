@@ -765,7 +765,7 @@ def main():
     else:
         ach = stats[dom]["flops"] / (per_layer_ms[dom] * 1e-3) / 1e12
         roof = {"bound": "alu", "achieved": ach, "peak": fp32_tf, "unit": "TFLOP/s", "frac": ach / fp32_tf}
-    roof.update({"traffic": stored_traffic(d["layer"], d["cfg"]), "kernel": {2: "spconv1x1_mma_kernel", 3: "gather_kernel", 4: "tc_kernel"}.get(d["cfg"].get("math_mode"), "spconv1x1_kernel"), "layer": d["layer"],
+    roof.update({"traffic": stored_traffic(d["layer"], d["cfg"]), "kernel": {2: "spconv1x1_mma_kernel", 3: "gather_kernel", 4: "tc16_kernel" if d["cfg"].get("producer_warps") == 8 else "tc_kernel"}.get(d["cfg"].get("math_mode"), "spconv1x1_kernel"), "layer": d["layer"],
                  "algorithmic_bytes": stats[dom]["bytes"], "algorithmic_flops": stats[dom]["flops"],
                  "peak_source": f"HBM {peak_src}; fp32 = {SM_COUNT} SMs x {FP32_LANES} lanes x 2 x {sm_max:.0f} MHz"})
     # the fp32 peak as this GPU delivers it from registers, measured now (a few hundred microseconds)
