@@ -644,6 +644,8 @@ def main():
         else:       # forced configuration: one explicit call per layer
             for L in layers:
                 A.alcs_spconv1x1(L["w"], L["x"], L["y"], L["n"], L["h"], L["wd"], L["bias"], L["flags"], stream, L["cfg"])
+    # (what the stack runs: merged layers may run otherwise than by themselves)
+    run_cfgs = [A.alcs_stack_layer_cfg(stack, i) if stack is not None else st["cfg"] for i, st in enumerate(stats)]
     total_flops = sum(st["flops"] for st in stats)
     total_bytes = sum(st["bytes"] for st in stats)
     hbm_gbs, peak_src, fp32_tf, sm_max = peaks()
@@ -799,7 +801,7 @@ def main():
                            "frac": round(sum_roof / sum_us, 4), "min_layer_frac": min(r["frac"] for r in rows),
                            "step_frac": round(sum_roof / (ms_step * 1e3), 4),
                            "us_per_layer": round(ms_step * 1e3 / nl, 2)},
-        "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": stack_launches(specs, [st["cfg"] for st in stats]) * args.steps,
+        "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": stack_launches(specs, run_cfgs) * args.steps,
         "clocks": clocks,
         "batch1": batch1, "layers": rows,
     }

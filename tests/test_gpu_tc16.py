@@ -367,13 +367,16 @@ def test_inputs_that_start_on_odd_words(alcs):
         for _ in range(3):
             y.fill_(float("nan"))
             alcs.alcs_spconv1x1(p, x, y, n, h, h, bd, 0, st, cfg)
-        a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        a.record()
-        for _ in range(20):
-            alcs.alcs_spconv1x1(p, x, y, n, h, h, bd, 0, st, cfg)
-        e.record()
-        torch.cuda.synchronize()
-        took[tuple(cfg.values()) if cfg else None] = a.elapsed_time(e)
+        best = []
+        for _ in range(5):
+            a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                alcs.alcs_spconv1x1(p, x, y, n, h, h, bd, 0, st, cfg)
+            e.record()
+            torch.cuda.synchronize()
+            best.append(a.elapsed_time(e))
+        took[tuple(cfg.values()) if cfg else None] = min(best)
         assert_parity(y.cpu().numpy(), Yref, A, "f16")
     times = list(took.values())
     assert times[1] < 1.5 * times[2] < 1.5 * times[3] and times[0] < 1.3 * times[4], took
